@@ -69,6 +69,8 @@ int host_step_resources(HostStepResources** out) {
 
 __global__ void meta_reorder_kernel(const uint16_t* __restrict__ meta, uint8_t* __restrict__ meta_hw, int64_t R,
                                     int64_t K) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t words = K >> 4;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= R * words) return;
@@ -80,6 +82,8 @@ __global__ void meta_reorder_kernel(const uint16_t* __restrict__ meta, uint8_t* 
 __global__ void pack_like_kernel(const uint16_t* __restrict__ dense, const uint16_t* __restrict__ meta,
                                  const uint8_t* __restrict__ colidx, uint16_t* __restrict__ vals, int64_t T,
                                  int64_t F, int V, int Mv) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t G = F / Mv, words = G >> 2;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= T * words) return;
@@ -217,19 +221,16 @@ void trace_mark(cudaStream_t s) {
 int launch_meta_reorder(const void* meta, void* meta_hw, int64_t R, int64_t K, cudaStream_t s) {
   const int64_t n = R * (K >> 4);
   if (n == 0) return SF_OK;
-  meta_reorder_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const uint16_t*)meta, (uint8_t*)meta_hw, R, K);
-  SF_LAUNCH_CHECK();
-  return SF_OK;
+  return launch_pdl(meta_reorder_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, s, (const uint16_t*)meta,
+                    (uint8_t*)meta_hw, R, K);
 }
 
 int launch_pack_like(const void* dense, const void* meta, const void* colidx, void* vals, int64_t T, int64_t F,
                      int V, int Mv, cudaStream_t s) {
   const int64_t n = T * (F / Mv / 4);
   if (n == 0) return SF_OK;
-  pack_like_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const uint16_t*)dense, (const uint16_t*)meta,
-                                                               (const uint8_t*)colidx, (uint16_t*)vals, T, F, V, Mv);
-  SF_LAUNCH_CHECK();
-  return SF_OK;
+  return launch_pdl(pack_like_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, s, (const uint16_t*)dense,
+                    (const uint16_t*)meta, (const uint8_t*)colidx, (uint16_t*)vals, T, F, V, Mv);
 }
 
 }  // namespace sf

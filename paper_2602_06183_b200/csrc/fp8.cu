@@ -23,6 +23,8 @@ constexpr size_t kStatusBytes8 = 256;
 // One thread converts 16 consecutive elements of a row: two 128-bit loads, one 128-bit store.
 __global__ void __launch_bounds__(256)
 quantize_fp8_kernel(const uint4* __restrict__ X, int64_t rows, int cols, int64_t ld, float scale, uint4* __restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
   const int chunks = cols >> 4;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= rows * chunks) return;
@@ -51,6 +53,8 @@ prune24_fp8_kernel(const uint4* __restrict__ W, int64_t rows, int cols, int64_t 
   __shared__ Top2Entry lut[16];
   top2_lut_init(lut, threadIdx.x);
   __syncthreads();
+  pdl_wait();
+  pdl_trigger();
   const uint32_t upr = (uint32_t)cols >> 3;                       // units per row
   const int64_t total = rows * (int64_t)upr;
   const int64_t base = (int64_t)blockIdx.x * (256 * kUnitsPerThread) + threadIdx.x;
@@ -98,6 +102,8 @@ prune24_fp8_kernel(const uint4* __restrict__ W, int64_t rows, int cols, int64_t 
 }
 
 __global__ void meta_reorder8_kernel(const uint16_t* __restrict__ meta, uint8_t* __restrict__ meta_hw, int64_t R, int64_t K) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t words = K >> 4;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= R * words) return;
@@ -120,10 +126,8 @@ int sf_fp8_quantize(const void* X, int64_t rows, int64_t cols, int64_t ld, float
   if (ld < cols || ld % 8 != 0 || !aligned16(X) || !aligned16(Xq)) return SF_ERR_ALIGN;
   SF_TRY(check_arch());
   const int64_t n = rows * (cols >> 4);
-  quantize_fp8_kernel<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>((const uint4*)X, rows, (int)cols, ld,
-                                                                                 scale, (uint4*)Xq);
-  SF_LAUNCH_CHECK();
-  return SF_OK;
+  return launch_pdl(quantize_fp8_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, (cudaStream_t)stream,
+                    (const uint4*)X, rows, (int)cols, ld, scale, (uint4*)Xq);
 }
 
 int sf_prune24_fp8_sizes(int64_t rows, int64_t cols, int group_dim, size_t* vals_bytes, size_t* meta_bytes) {
@@ -153,14 +157,8 @@ int sf_prune24_compress_fp8(const void* W, int64_t rows, int64_t cols, int64_t l
   if ((n + per_cta - 1) / per_cta > 0x7FFFFFFF) return SF_ERR_SHAPE;
   const unsigned grid = (unsigned)((n + per_cta - 1) / per_cta);
   cudaStream_t s = (cudaStream_t)stream;
-  if (prune_mode == 0)
-    prune24_fp8_kernel<false><<<grid, 256, 0, s>>>((const uint4*)W, rows, (int)cols, ld, scale, (uint32_t*)vals,
-                                                   (uint32_t*)meta, (uint2*)dense_out);
-  else
-    prune24_fp8_kernel<true><<<grid, 256, 0, s>>>((const uint4*)W, rows, (int)cols, ld, scale, (uint32_t*)vals,
-                                                  (uint32_t*)meta, (uint2*)dense_out);
-  SF_LAUNCH_CHECK();
-  return SF_OK;
+  return launch_pdl(prune_mode == 0 ? prune24_fp8_kernel<false> : prune24_fp8_kernel<true>, dim3(grid), 256, 0, s,
+                    (const uint4*)W, rows, (int)cols, ld, scale, (uint32_t*)vals, (uint32_t*)meta, (uint2*)dense_out);
 }
 
 int sf_gemm_fp8_workspace_size(int64_t Mr, int64_t K, size_t* bytes) {
@@ -191,8 +189,7 @@ int sf_gemm_fp8_sparse24(const void* a_vals, const void* a_meta, const void* B, 
   cudaStream_t s = (cudaStream_t)stream;
   uint8_t* hw = reinterpret_cast<uint8_t*>(workspace) + kStatusBytes8;
   const int64_t n = Mr * (K >> 4);
-  meta_reorder8_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const uint16_t*)a_meta, hw, Mr, K);
-  SF_LAUNCH_CHECK();
+  SF_TRY(launch_pdl(meta_reorder8_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, s, (const uint16_t*)a_meta, hw, Mr, K));
   return gemm_fp8(true, a_vals, hw, B, Mr, Nc, K, alpha, C, Nc, (int*)workspace, s);
 }
 

@@ -545,6 +545,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_wait();
+  pdl_trigger();
   const uint32_t tmem_base = ctl->tmem_base;
 
   if (warp == 0) {
@@ -864,7 +866,6 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   const uint32_t rank = cluster_ctarank();               // 0 = leader
   const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
   const int num_m_tiles = args.num_m_tiles, num_n_tiles_ = args.num_n_tiles;   // 256-row tiles
-  const int num_tiles = args.tile_table ? __ldg(args.num_tiles_dev) : num_m_tiles * num_n_tiles_;
   const int nkb_full = (int)(args.K / kBK);
 
   if (threadIdx.x == 0) {
@@ -899,6 +900,9 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   __syncthreads();
   cluster_sync_all();                                    // both CTAs' barriers and TMEM are ready
   tc_fence_after();
+  pdl_wait();                                            // everything above overlaps the previous kernel's tail
+  pdl_trigger();
+  const int num_tiles = args.tile_table ? __ldg(args.num_tiles_dev) : num_m_tiles * num_n_tiles_;
   const uint32_t tmem_base = ctl->tmem_base;
 
   if (warp == 0) {
@@ -1192,9 +1196,8 @@ int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const GemmArgs& a, 
   }
   const int tiles = a.num_m_tiles * a.num_n_tiles;
   const int grid = tiles < sm_count() ? tiles : sm_count();
-  kern<<<grid, kMode == MODE_VENOM ? kThreadsVenom : kThreads, smem_bytes(kMode != MODE_DENSE), s>>>(ta, tb, a);
-  SF_LAUNCH_CHECK();
-  return SF_OK;
+  return launch_pdl(kern, dim3(grid), kMode == MODE_VENOM ? kThreadsVenom : kThreads, smem_bytes(kMode != MODE_DENSE), s,
+                    ta, tb, a);
 }
 
 template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false>
@@ -1217,9 +1220,7 @@ int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
                                  : a.num_m_tiles * a.num_n_tiles;
   const int max_pairs = sm_count() / 2;
   const int pairs = tiles < max_pairs ? tiles : max_pairs;
-  kern<<<2 * pairs, threads2(kEpi, kExpand), smem, s>>>(ta, tb, tm, tpk ? *tpk : ta, a);
-  SF_LAUNCH_CHECK();
-  return SF_OK;
+  return launch_pdl(kern, dim3(2 * pairs), threads2(kEpi, kExpand), smem, s, ta, tb, tm, tpk ? *tpk : ta, a);
 }
 
 // Tile width of the two-accumulator 2:4 variant (transposed-output products): 2 x 224 accumulator

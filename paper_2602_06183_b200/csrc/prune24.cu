@@ -35,6 +35,8 @@ prune24_rows_kernel(const uint4* __restrict__ W, int64_t rows, int cols, int64_t
   __shared__ Top2Entry lut[16];
   top2_lut_init(lut, threadIdx.x);
   __syncthreads();
+  pdl_wait();
+  pdl_trigger();
   const int words_per_row = cols >> 4;                           // 16-element chunks per row
   const int kw = (int)blockIdx.x * 32 + (int)(threadIdx.x & 31);
   const int64_t r = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * kRowsPerCta + (threadIdx.x >> 5);
@@ -105,7 +107,7 @@ template <bool kSoft, bool kFp8 = false>
 __global__ void __launch_bounds__(256)
 prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64_t Rc,
                     uint16_t* __restrict__ vals, uint16_t* __restrict__ meta, uint8_t* __restrict__ meta_hw,
-                    uint16_t* __restrict__ dense_out, int panels_x, int num_panels, float scale = 1.f) {
+                    uint16_t* __restrict__ dense_out, int panels_x, int num_panels, float scale) {
   using namespace ptx;
   extern __shared__ uint8_t cols_smem_raw[];
   uint8_t* cols_smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(cols_smem_raw) + 127) & ~uintptr_t(127));
@@ -134,6 +136,10 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64
     for (int sl = 0; sl < kColsSlots; ++sl) mbar_init(&full[sl], 1);
     *abort_flag = 0;
     fence_mbar_init();
+  }
+  pdl_wait();
+  pdl_trigger();
+  if (tid == 0) {
     for (int d = 0; d < kColsSlots - 1; ++d) issue(d);
   }
   __syncthreads();
@@ -256,6 +262,8 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64
 __global__ void __launch_bounds__(256)
 transpose_kernel(const uint16_t* __restrict__ in, uint16_t* __restrict__ out, int64_t rows, int64_t cols) {
   __shared__ uint16_t t[64][64 + 2];
+  pdl_wait();
+  pdl_trigger();
   const int64_t r0 = (int64_t)blockIdx.y * 64, c0 = (int64_t)blockIdx.x * 64;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;                // 32 x 8
   for (int i = ty; i < 64; i += 8) {
@@ -292,6 +300,8 @@ transpose_kernel(const uint16_t* __restrict__ in, uint16_t* __restrict__ out, in
 __global__ void __launch_bounds__(256)
 transpose64_kernel(const uint16_t* __restrict__ in, uint16_t* __restrict__ out, int64_t rows, int64_t cols) {
   __shared__ uint32_t t[64 * 33];
+  pdl_wait();
+  pdl_trigger();
   const int64_t r0 = (int64_t)blockIdx.y * 64, c0 = (int64_t)blockIdx.x * 64;
   const int tid = threadIdx.x;
 #pragma unroll
@@ -330,12 +340,9 @@ int launch_prune24(const void* W, int64_t rows, int64_t cols, int64_t ld, int gr
     const int64_t gz = (row_ctas + gy - 1) / gy;
     if (gz > 65535) return SF_ERR_SHAPE;
     dim3 grid((unsigned)(((cols >> 4) + 31) / 32), (unsigned)gy, (unsigned)gz);
-    if (prune_mode == 0)
-      prune24_rows_kernel<false><<<grid, 256, 0, s>>>((const uint4*)W, rows, (int)cols, ld, (uint4*)vals,
-                                                      (uint16_t*)meta, (uint8_t*)meta_hw, (uint4*)dense_out);
-    else
-      prune24_rows_kernel<true><<<grid, 256, 0, s>>>((const uint4*)W, rows, (int)cols, ld, (uint4*)vals,
-                                                     (uint16_t*)meta, (uint8_t*)meta_hw, (uint4*)dense_out);
+    return launch_pdl(prune_mode == 0 ? prune24_rows_kernel<false> : prune24_rows_kernel<true>, grid, 256, 0, s,
+                      (const uint4*)W, rows, (int)cols, ld, (uint4*)vals, (uint16_t*)meta, (uint8_t*)meta_hw,
+                      (uint4*)dense_out);
   } else {
     const int64_t px = (cols + kPanelC - 1) / kPanelC, py = (rows + kPanelK - 1) / kPanelK;
     if (px * py > (int64_t)1 << 30) return SF_ERR_SHAPE;
@@ -356,15 +363,10 @@ int launch_prune24(const void* W, int64_t rows, int64_t cols, int64_t ld, int gr
     if (st != SF_OK) return st;
     const int resident = sms[dev] * kColsCtasPerSm;
     const unsigned grid = (unsigned)(num_panels < resident ? num_panels : resident);
-    if (prune_mode == 0)
-      prune24_cols_kernel<false><<<grid, 256, kColsSmemBytes, s>>>(tm, rows, cols, (uint16_t*)vals, (uint16_t*)meta,
-                                                                   (uint8_t*)meta_hw, (uint16_t*)dense_out, (int)px, num_panels);
-    else
-      prune24_cols_kernel<true><<<grid, 256, kColsSmemBytes, s>>>(tm, rows, cols, (uint16_t*)vals, (uint16_t*)meta,
-                                                                  (uint8_t*)meta_hw, (uint16_t*)dense_out, (int)px, num_panels);
+    return launch_pdl(prune_mode == 0 ? prune24_cols_kernel<false> : prune24_cols_kernel<true>, dim3(grid), 256,
+                      kColsSmemBytes, s, tm, rows, cols, (uint16_t*)vals, (uint16_t*)meta, (uint8_t*)meta_hw,
+                      (uint16_t*)dense_out, (int)px, num_panels, 1.f);
   }
-  SF_LAUNCH_CHECK();
-  return SF_OK;
 }
 
 int launch_prune24_cols_fp8(const void* W, int64_t rows, int64_t cols, int64_t ld, int prune_mode, float scale, void* vals,
@@ -389,25 +391,16 @@ int launch_prune24_cols_fp8(const void* W, int64_t rows, int64_t cols, int64_t l
   if (st != SF_OK) return st;
   const int resident = sms[dev] * kColsCtasPerSm;
   const unsigned grid = (unsigned)(num_panels < resident ? num_panels : resident);
-  if (prune_mode == 0)
-    prune24_cols_kernel<false, true><<<grid, 256, kColsSmemBytes, s>>>(tm, rows, cols, (uint16_t*)vals, (uint16_t*)meta, nullptr,
-                                                                       nullptr, (int)px, num_panels, scale);
-  else
-    prune24_cols_kernel<true, true><<<grid, 256, kColsSmemBytes, s>>>(tm, rows, cols, (uint16_t*)vals, (uint16_t*)meta, nullptr,
-                                                                      nullptr, (int)px, num_panels, scale);
-  SF_LAUNCH_CHECK();
-  return SF_OK;
+  return launch_pdl(prune_mode == 0 ? prune24_cols_kernel<false, true> : prune24_cols_kernel<true, true>, dim3(grid), 256,
+                    kColsSmemBytes, s, tm, rows, cols, (uint16_t*)vals, (uint16_t*)meta, (uint8_t*)nullptr,
+                    (uint16_t*)nullptr, (int)px, num_panels, scale);
 }
 
 int launch_transpose(const void* in, void* out, int64_t rows, int64_t cols, cudaStream_t s) {
   if (rows == 0 || cols == 0) return SF_OK;
   dim3 grid((unsigned)((cols + 63) / 64), (unsigned)((rows + 63) / 64));
-  if (rows % 64 == 0 && cols % 64 == 0)
-    transpose64_kernel<<<grid, 256, 0, s>>>((const uint16_t*)in, (uint16_t*)out, rows, cols);
-  else
-    transpose_kernel<<<grid, 256, 0, s>>>((const uint16_t*)in, (uint16_t*)out, rows, cols);
-  SF_LAUNCH_CHECK();
-  return SF_OK;
+  return launch_pdl(rows % 64 == 0 && cols % 64 == 0 ? transpose64_kernel : transpose_kernel, grid, 256, 0, s,
+                    (const uint16_t*)in, (uint16_t*)out, rows, cols);
 }
 
 }  // namespace sf

@@ -37,6 +37,8 @@ constexpr int kRouteTokens = 2;
 __global__ void __launch_bounds__(256, 2)
 route_kernel(const uint16_t* __restrict__ X, const uint16_t* __restrict__ means, int T, int D, int E,
              int* __restrict__ expert, float* __restrict__ logits) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int t0 = ((int)blockIdx.x * 8 + (threadIdx.x >> 5)) * kRouteTokens;
   if (t0 >= T) return;
@@ -132,6 +134,8 @@ __global__ void __launch_bounds__(1024)
 group_kernel(const int* __restrict__ expert, int T, int E, int rows_max, int* __restrict__ row_of_token,
              int* __restrict__ src_of_row, int* __restrict__ seg) {
   extern __shared__ int gsm[];
+  pdl_wait();
+  pdl_trigger();
   int* cnt = gsm;                          // [E][1024]
   int* sseg = gsm + E * 1024;              // [E + 1]
   const int tid = threadIdx.x;
@@ -199,6 +203,8 @@ tile_tables_kernel(const int* __restrict__ seg, int E, int D, int F, GemmTile* _
                    int* __restrict__ counts) {
   __shared__ int baseA[kMaxExperts + 1], baseB[kMaxExperts + 1], baseC[kMaxExperts + 1];
   const int Fe = F / E, fm = Fe / 256, dm = D / 256;
+  pdl_wait();
+  pdl_trigger();
   if (threadIdx.x == 0) {
     baseA[0] = baseB[0] = baseC[0] = 0;
     for (int e = 0; e < E; ++e) {
@@ -238,6 +244,8 @@ tile_tables_kernel(const int* __restrict__ seg, int E, int D, int F, GemmTile* _
 __global__ void __launch_bounds__(256)
 gather_rows_kernel(const uint4* __restrict__ in, const int* __restrict__ src, uint4* __restrict__ out, int rows,
                    int row_u4) {
+  pdl_wait();
+  pdl_trigger();
   const int r = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= rows) return;
   const int s = __ldg(src + r);
@@ -332,18 +340,14 @@ int check_ptrs(std::initializer_list<const void*> ps) {
 
 int launch_route(const void* X, const void* means, int64_t T, int64_t D, int E, void* expert, void* logits,
                  cudaStream_t s) {
-  route_kernel<<<(unsigned)((T + 8 * kRouteTokens - 1) / (8 * kRouteTokens)), 256, 0, s>>>((const uint16_t*)X, (const uint16_t*)means, (int)T, (int)D, E,
-                                                       (int*)expert, (float*)logits);
-  SF_LAUNCH_CHECK();
-  return SF_OK;
+  return launch_pdl(route_kernel, dim3((unsigned)((T + 8 * kRouteTokens - 1) / (8 * kRouteTokens))), 256, 0, s,
+                    (const uint16_t*)X, (const uint16_t*)means, (int)T, (int)D, E, (int*)expert, (float*)logits);
 }
 
 int launch_gather_rows(const void* in, const int* src, void* out, int64_t rows, int64_t cols, cudaStream_t s) {
   if (rows == 0 || cols == 0) return SF_OK;
-  gather_rows_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>((const uint4*)in, src, (uint4*)out, (int)rows,
-                                                               (int)(cols / 8));
-  SF_LAUNCH_CHECK();
-  return SF_OK;
+  return launch_pdl(gather_rows_kernel, dim3((unsigned)((rows + 7) / 8)), 256, 0, s, (const uint4*)in, src, (uint4*)out,
+                    (int)rows, (int)(cols / 8));
 }
 
 }  // namespace
@@ -417,12 +421,10 @@ int sf_routed_ffn_fwd(const sf_router_desc* desc, const void* X, const void* W1,
                                      (kMaxExperts * 1024 + kMaxExperts + 1) * 4));
     if (dev >= 0 && dev < 64) attr_done[dev] = true;
   }
-  group_kernel<<<1, 1024, gsm, s>>>(expert, (int)d.T, d.E, (int)L.rows_max, (int*)at(fwd_ctx, L.row_of_token), src, seg);
-  SF_LAUNCH_CHECK();
-  tile_tables_kernel<<<1, 256, 0, s>>>(seg, d.E, (int)d.D, (int)d.F, (GemmTile*)at(fwd_ctx, L.tabA),
-                                       (GemmTile*)at(fwd_ctx, L.tabB), (GemmTile*)at(fwd_ctx, L.tabC),
-                                       (GemmTile*)at(fwd_ctx, L.tabD), counts);
-  SF_LAUNCH_CHECK();
+  SF_TRY(launch_pdl(group_kernel, dim3(1), 1024, gsm, s, expert, (int)d.T, d.E, (int)L.rows_max,
+                    (int*)at(fwd_ctx, L.row_of_token), src, seg));
+  SF_TRY(launch_pdl(tile_tables_kernel, dim3(1), 256, 0, s, seg, d.E, (int)d.D, (int)d.F, (GemmTile*)at(fwd_ctx, L.tabA),
+                    (GemmTile*)at(fwd_ctx, L.tabB), (GemmTile*)at(fwd_ctx, L.tabC), (GemmTile*)at(fwd_ctx, L.tabD), counts));
   SF_TRY(launch_gather_rows(X, src, at(fwd_ctx, L.xp), L.rows_max, d.D, s));
   trace_mark(s);
   // step 3: y1 = Xp W1s[expert]^T with SquaredReLU and the 2:4 selection in the epilogue

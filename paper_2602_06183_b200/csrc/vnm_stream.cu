@@ -68,6 +68,8 @@ vnm_stream_kernel(const __grid_constant__ CUtensorMap tmapP, int64_t T, int64_t 
     fence_mbar_init();
   }
   __syncthreads();
+  pdl_wait();
+  pdl_trigger();
 
   if (warp == 0) {
     // =========================== producer ===========================
@@ -283,10 +285,8 @@ static int launch_stream_t(const void* P, int64_t T, int64_t F, int64_t ld, int 
   const int per_sm = smem <= 110 * 1024 ? 2 : 1;
   const int64_t resident = (int64_t)sms[dev] * per_sm;
   const unsigned grid = (unsigned)(nstrips < resident ? nstrips : resident);
-  vnm_stream_kernel<kSW, kM><<<grid, kThreadsS, smem, s>>>(tm, T, F, V, apply_sqrelu, (uint16_t*)vals, (uint16_t*)meta,
-                                                           (uint8_t*)colidx, (uint16_t*)relu_vals);
-  SF_LAUNCH_CHECK();
-  return SF_OK;
+  return launch_pdl(vnm_stream_kernel<kSW, kM>, dim3(grid), kThreadsS, smem, s, tm, T, F, V, apply_sqrelu,
+                    (uint16_t*)vals, (uint16_t*)meta, (uint8_t*)colidx, (uint16_t*)relu_vals);
 }
 
 int launch_vnm_stream(const void* P, int64_t T, int64_t F, int64_t ld, int V, int M, int apply_sqrelu, void* vals,
