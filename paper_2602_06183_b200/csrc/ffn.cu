@@ -78,35 +78,11 @@ __global__ void meta_reorder_kernel(const uint16_t* __restrict__ meta, uint8_t* 
   *reinterpret_cast<uint16_t*>(meta_hw + meta_hw_offset(m, kw, K)) = meta[idx];
 }
 
-// vals[t, 2g + j] = dense[t, g*Mv + colidx[t/V, g, pos_j]] with pos from the canonical nibble.
-__global__ void pack_like_kernel(const uint16_t* __restrict__ dense, const uint16_t* __restrict__ meta,
-                                 const uint8_t* __restrict__ colidx, uint16_t* __restrict__ vals, int64_t T,
-                                 int64_t F, int V, int Mv) {
-  pdl_wait();
-  pdl_trigger();
-  const int64_t G = F / Mv, words = G >> 2;
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= T * words) return;
-  const int64_t t = idx / words, kw = idx - t * words;
-  const uint32_t mw = meta[idx];
-  const uint4 c16 = *reinterpret_cast<const uint4*>(colidx + (((t / V) * G) + kw * 4) * 4);
-  const uint32_t cw[4] = {c16.x, c16.y, c16.z, c16.w};
-  uint32_t out[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const uint32_t nib = (mw >> (4 * j)) & 0xFu;
-    const uint32_t ca = (cw[j] >> (8 * (nib & 3u))) & 0xFFu, cb = (cw[j] >> (8 * (nib >> 2))) & 0xFFu;
-    const uint16_t* grp = dense + t * F + (kw * 4 + j) * Mv;
-    out[j] = (uint32_t)grp[ca] | ((uint32_t)grp[cb] << 16);
-  }
-  *reinterpret_cast<uint4*>(vals + t * (2 * G) + kw * 8) = make_uint4(out[0], out[1], out[2], out[3]);
-}
-
 // ---- context / workspace carving ---------------------------------------------------------------
 
 struct SparseLayout {
   // forward context
-  size_t y2_vals, relu_vals, meta, meta_hw, colidx, y2_dense, relu_dense, w2t, y1, vals24, meta24, meta24_hw, relu24,
+  size_t y2_vals, relu_vals, meta, meta_hw, colidx, y2_dense, w2t, y1, vals24, meta24, meta24_hw, relu24,
       ctx_total;
   // workspace (after the status block)
   size_t w1_vals, w1_meta, w1_meta_hw, ws_y1, w2_vals, w2_meta, w2_meta_hw, dy1_dense, dy1_vals, dy1_vals24,
@@ -146,21 +122,20 @@ SparseLayout sparse_layout(const sf_ffn_desc& d) {
     L.meta24 = take(T * F / 8);
     L.meta24_hw = take(T * F / 8);
     L.y2_dense = L.expand ? kNone : take(T * F * 2);
-    L.meta_hw = L.relu_dense = L.w2t = kNone;
+    L.meta_hw = L.w2t = kNone;
   } else {
     L.meta_hw = take(T * G / 2);
     L.y2_dense = take(T * F * 2);
-    L.relu_dense = take(T * F * 2);
     L.w2t = L.plain24 ? kNone : take(F * D * 2);
     L.vals24 = L.y2_vals; L.meta24 = L.meta; L.meta24_hw = L.meta_hw;   // M == 4: the packed form is already 2:4
-    L.relu24 = kNone;
+    L.relu24 = L.relu_vals;
   }
   L.ctx_total = o;
   o = kStatusBytes;
   L.w1_vals = take(F * D);
   L.w1_meta = take(F * D / 8);
   L.w1_meta_hw = take(F * D / 8);
-  L.ws_y1 = ((d.flags & SF_FFN_SAVE_Y1) || L.fused) ? kNone : take(T * F * 2);
+  L.ws_y1 = ((d.flags & SF_FFN_SAVE_Y1) || L.fused || d.M == 4) ? kNone : take(T * F * 2);
   L.w2_vals = take(F * D);
   L.w2_meta = take(F * D / 8);
   L.w2_meta_hw = take(F * D / 8);
@@ -225,14 +200,6 @@ int launch_meta_reorder(const void* meta, void* meta_hw, int64_t R, int64_t K, c
                     (uint8_t*)meta_hw, R, K);
 }
 
-int launch_pack_like(const void* dense, const void* meta, const void* colidx, void* vals, int64_t T, int64_t F,
-                     int V, int Mv, cudaStream_t s) {
-  const int64_t n = T * (F / Mv / 4);
-  if (n == 0) return SF_OK;
-  return launch_pdl(pack_like_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, s, (const uint16_t*)dense,
-                    (const uint16_t*)meta, (const uint8_t*)colidx, (uint16_t*)vals, T, F, V, Mv);
-}
-
 }  // namespace sf
 
 using namespace sf;
@@ -276,7 +243,7 @@ int sf_gemm_sparse24(const void* a_vals, const void* a_meta, const void* B, void
   cudaStream_t s = (cudaStream_t)stream;
   uint8_t* hw = at(workspace, kStatusBytes);
   SF_TRY(launch_meta_reorder(a_meta, hw, Mr, K, s));
-  return gemm_sparse24(a_vals, hw, B, true, Mr, Nc, K, EPI_STORE_T, Ct, Mr, nullptr, 0, (int*)workspace, s);
+  return gemm_sparse24(a_vals, hw, B, true, Mr, Nc, K, EPI_STORE_T, Ct, Mr, (int*)workspace, s);
 }
 
 int sf_gemm_sparse24_rm(const void* a_vals, const void* a_meta, const void* B, int b_kmajor, void* C, int64_t Mr,
@@ -290,7 +257,7 @@ int sf_gemm_sparse24_rm(const void* a_vals, const void* a_meta, const void* B, i
   cudaStream_t s = (cudaStream_t)stream;
   uint8_t* hw = at(workspace, kStatusBytes);
   SF_TRY(launch_meta_reorder(a_meta, hw, Mr, K, s));
-  return gemm_sparse24(a_vals, hw, B, b_kmajor != 0, Mr, Nc, K, EPI_STORE, C, Nc, nullptr, 0, (int*)workspace, s);
+  return gemm_sparse24(a_vals, hw, B, b_kmajor != 0, Mr, Nc, K, EPI_STORE, C, Nc, (int*)workspace, s);
 }
 
 int sf_gemm_venom(const void* a_vals, const void* a_meta, const void* colidx, const void* Bt, void* C, int64_t T,
@@ -370,21 +337,29 @@ int sf_sparse_ffn_fwd(const sf_ffn_desc* desc, const void* X, const void* W1, co
                               status, s));
     trace_mark(s);
     trace_mark(s);      // (the sparsify interval is empty on this path)
+  } else if (d.M == 4) {
+    // the same with groups of four: every block keeps all its columns, the row-wise 2:4 choice is all there is
+    Act24Out out{at(fwd_ctx, L.y2_vals), at(fwd_ctx, L.relu_vals), at(fwd_ctx, L.meta), at(fwd_ctx, L.meta_hw),
+                 at(fwd_ctx, L.y2_dense), save_y1 ? (void*)at(fwd_ctx, L.y1) : nullptr};
+    SF_TRY(gemm_sparse24_act4(at(workspace, L.w1_vals), at(workspace, L.w1_meta_hw), X, d.F, d.T, d.D, d.V, out,
+                              at(fwd_ctx, L.colidx), status, s));
+    trace_mark(s);
+    trace_mark(s);
   } else {
     void* y1 = save_y1 ? (void*)at(fwd_ctx, L.y1) : (void*)at(workspace, L.ws_y1);
     SF_TRY(gemm_sparse24(at(workspace, L.w1_vals), at(workspace, L.w1_meta_hw), X, true, d.F, d.T, d.D, EPI_STORE_T,
-                         y1, d.F, nullptr, 0, status, s));
+                         y1, d.F, status, s));
     trace_mark(s);
     // lines 5-6: y2 = ReLU(y1)^2 in V:N:M form (+ what the backward pass needs)
     if (L.packed8) {
       SF_TRY(launch_vnm(y1, d.T, d.F, d.F, d.V, d.M, 1, at(fwd_ctx, L.y2_vals), at(fwd_ctx, L.meta), nullptr,
                         at(fwd_ctx, L.colidx), at(fwd_ctx, L.relu_vals),
-                        L.expand ? nullptr : (void*)at(fwd_ctx, L.y2_dense), nullptr, at(fwd_ctx, L.vals24),
+                        L.expand ? nullptr : (void*)at(fwd_ctx, L.y2_dense), at(fwd_ctx, L.vals24),
                         at(fwd_ctx, L.meta24), at(fwd_ctx, L.meta24_hw), at(fwd_ctx, L.relu24), s));
     } else {
       SF_TRY(launch_vnm(y1, d.T, d.F, d.F, d.V, d.M, 1, at(fwd_ctx, L.y2_vals), at(fwd_ctx, L.meta),
                         at(fwd_ctx, L.meta_hw), at(fwd_ctx, L.colidx), at(fwd_ctx, L.relu_vals),
-                        at(fwd_ctx, L.y2_dense), at(fwd_ctx, L.relu_dense), nullptr, nullptr, nullptr, nullptr, s));
+                        at(fwd_ctx, L.y2_dense), nullptr, nullptr, nullptr, nullptr, s));
     }
     trace_mark(s);
   }
@@ -395,7 +370,7 @@ int sf_sparse_ffn_fwd(const sf_ffn_desc* desc, const void* X, const void* W1, co
     trace_mark(s);
     // (W2 given as [F, D]: the same product with W2 as the MN-major operand)
     SF_TRY(gemm_sparse24(at(fwd_ctx, L.vals24), at(fwd_ctx, L.meta24_hw), W2, !w2_fd, d.T, d.D, d.F, EPI_STORE, Y, d.D,
-                         nullptr, 0, status, s));
+                         status, s));
   } else {
     // condensed V:N:M operand; rows of W2^T are gathered by the kept columns (W2 given as [F, D] is that matrix)
     if (!w2_fd) SF_TRY(launch_transpose(W2, at(fwd_ctx, L.w2t), d.D, d.F, s));
@@ -444,14 +419,14 @@ int sf_sparse_ffn_bwd(const sf_ffn_desc* desc, const void* dY, const void* X, co
   if (L.packed8) {
     // M = 8: ReLU(y1) comes in the 2:4 layout of y2's mask and dy1 leaves in the same layout (plus, unless
     // the weight-gradient products expand their operands themselves, as a masked [T, F] matrix)
-    SF_TRY(gemm_sparse24(at(workspace, L.w2_vals), at(workspace, L.w2_meta_hw), dY, true, d.F, d.T, d.D,
-                         EPI_DRELU24_T, L.expand ? nullptr : (void*)at(workspace, L.dy1_dense), d.F,
-                         at(fwd_ctx, L.relu24), 0, status, s, at(fwd_ctx, L.meta24), at(workspace, L.dy1_vals24)));
+    SF_TRY(gemm_sparse24_drelu(at(workspace, L.w2_vals), at(workspace, L.w2_meta_hw), dY, d.F, d.T, d.D,
+                               ActMask{at(fwd_ctx, L.relu24), at(fwd_ctx, L.meta24), nullptr, d.V, d.M},
+                               at(workspace, L.dy1_vals24), L.expand ? nullptr : (void*)at(workspace, L.dy1_dense), status, s));
     trace_mark(s);
     trace_mark(s);
     // line 5: dX = dy1 W1 with W1 dense; W1 [F, D] is the MN-major operand
     SF_TRY(gemm_sparse24(at(workspace, L.dy1_vals24), at(fwd_ctx, L.meta24_hw), W1, false, d.T, d.D, d.F, EPI_STORE,
-                         dX, d.D, nullptr, 0, status, s));
+                         dX, d.D, status, s));
     trace_mark(s);
     hook_dx_done(s);
     // line 3: dW2 = dY^T y2 [D, F];  line 6: dW1 = dy1^T X [F, D]: dense tensor-core products (the reduction
@@ -475,19 +450,18 @@ int sf_sparse_ffn_bwd(const sf_ffn_desc* desc, const void* dY, const void* X, co
     trace_mark(s);
     return SF_OK;
   }
-  // (M = 4: the same epilogue also packs dy1 with y2's 2:4 metadata, the operand of the dX product)
-  SF_TRY(gemm_sparse24(at(workspace, L.w2_vals), at(workspace, L.w2_meta_hw), dY, true, d.F, d.T, d.D, EPI_DRELU_T,
-                       at(workspace, L.dy1_dense), d.F, at(fwd_ctx, L.relu_dense), d.F, status, s,
-                       L.plain24 ? at(fwd_ctx, L.meta24) : nullptr, L.plain24 ? at(workspace, L.dy1_vals24) : nullptr));
+  // M = 4: the packed activation is the 2:4 layout; M >= 16: the mask stays in V:N:M form. dy1 leaves packed like it
+  SF_TRY(gemm_sparse24_drelu(at(workspace, L.w2_vals), at(workspace, L.w2_meta_hw), dY, d.F, d.T, d.D,
+                             ActMask{at(fwd_ctx, L.relu_vals), at(fwd_ctx, L.meta),
+                                     L.plain24 ? nullptr : at(fwd_ctx, L.colidx), d.V, d.M},
+                             at(workspace, L.dy1_vals), at(workspace, L.dy1_dense), status, s));
   trace_mark(s);
   // line 5: dX = dy1 W1 with W1 dense
   if (L.plain24) {
     trace_mark(s);
     SF_TRY(gemm_sparse24(at(workspace, L.dy1_vals24), at(fwd_ctx, L.meta24_hw), W1, false, d.T, d.D, d.F, EPI_STORE,
-                         dX, d.D, nullptr, 0, status, s));
+                         dX, d.D, status, s));
   } else {
-    SF_TRY(launch_pack_like(at(workspace, L.dy1_dense), at(fwd_ctx, L.meta), at(fwd_ctx, L.colidx),
-                            at(workspace, L.dy1_vals), d.T, d.F, d.V, d.M, s));
     trace_mark(s);
     // rows of W1 gathered by the kept columns
     SF_TRY(gemm_venom(at(workspace, L.dy1_vals), at(fwd_ctx, L.meta_hw), at(fwd_ctx, L.colidx), W1, d.T, d.F, d.D,

@@ -36,8 +36,8 @@ __host__ __device__ constexpr int stage_bytes(bool sparse) {
   return a_stage_bytes(sparse) + kBStageBytes + (sparse ? kMetaStageBytes : 0);
 }
 __host__ __device__ constexpr int num_stages(bool sparse) { return sparse ? 5 : 4; }
-constexpr int kEpiStageRow = 80;                                                      // bytes: 32 bf16 + 16 pad
-constexpr int kEpiStageBytes = 4 * 32 * kEpiStageRow;                                 // 4 warps
+constexpr int kEpiWarpBytes = 16 * 32 * 4;                                            // 16 token pairs x 32 features
+constexpr int kEpiStageBytes = 4 * kEpiWarpBytes;                                     // 4 warps
 __host__ __device__ constexpr int smem_bytes(bool sparse) {
   return 1024 /*align slack*/ + num_stages(sparse) * stage_bytes(sparse) + kEpiStageBytes + 256 /*barriers*/;
 }
@@ -73,49 +73,39 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 }
 
 
+// Which epilogues run on two sets of four warps (one set per accumulator) on CTA pairs.
+__host__ __device__ constexpr bool is_drelu_t(int epi) { return epi == EPI_DRELU24_T || epi == EPI_DRELUV_T; }
+__host__ __device__ constexpr bool two_sets(int epi) { return epi == EPI_VNM8 || epi == EPI_ACT24_T || is_drelu_t(epi); }
+
+// This warp has read its part of an accumulator for the last time: hand it back to the MMA warp.
+__device__ __forceinline__ void release_accumulator(int lane, uint64_t* tmem_empty_bar) {
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) mbar_arrive_leader(tmem_empty_bar);
+}
+
+// A tile of accumulator columns (tokens) is transposed through shared memory as words of two neighbouring
+// tokens, [token pair][32 features]. This thread takes the eight features at `sp` of one pair back as two
+// rows of packed features: r0 = even token, r1 = odd token. Pairs alternate which 16-byte half they fetch
+// first, so that each of the two loads of a quarter-warp touches every bank exactly once.
+__device__ __forceinline__ void pair_rows(const uint32_t* sp, int lane, uint32_t (&r0)[4], uint32_t (&r1)[4]) {
+  const int swap = (lane >> 2) & 1;
+  const uint4 q0 = *reinterpret_cast<const uint4*>(sp + 4 * swap), q1 = *reinterpret_cast<const uint4*>(sp + 4 - 4 * swap);
+  const uint4 qa = swap ? q1 : q0, qb = swap ? q0 : q1;
+  r0[0] = __byte_perm(qa.x, qa.y, 0x5410); r0[1] = __byte_perm(qa.z, qa.w, 0x5410);
+  r0[2] = __byte_perm(qb.x, qb.y, 0x5410); r0[3] = __byte_perm(qb.z, qb.w, 0x5410);
+  r1[0] = __byte_perm(qa.x, qa.y, 0x7632); r1[1] = __byte_perm(qa.z, qa.w, 0x7632);
+  r1[2] = __byte_perm(qb.x, qb.y, 0x7632); r1[3] = __byte_perm(qb.z, qb.w, 0x7632);
+}
+
 // ---- epilogue (shared by the one-CTA and the two-CTA kernels) ---------------------------------------
 // One epilogue warp owns TMEM lanes [32q, 32q+32) of a 128 x 256 accumulator tile whose first row is
 // m0 and first column n0; `taddr` is the TMEM address of (lane 32q, column 0) of that accumulator.
 // kTileN: accumulator columns of the tile (a multiple of 32). Columns at or beyond args.N (a ragged last
 // tile, whole 32-column chunks only since N % 32 == 0) are neither prefetched nor stored.
-__host__ __device__ constexpr bool is_drelu_t(int epi) { return epi == EPI_DRELU_T || epi == EPI_DRELU24_T; }
-
-template <int kEpi, int kTileN = BN>
-__device__ __forceinline__ void epi_prefetch(const GemmArgs& args, int64_t m0, int64_t n0, int64_t n_limit, int q, int lane,
-                                             uint4 (&ax)[is_drelu_t(kEpi) ? kTileN / 32 : 1][4]) {
-  if (kEpi == EPI_DRELU24_T) {
-    // ReLU(y1) in the 2:4 layout of the activation mask: four stored values and two position nibbles per
-    // eight features; (x, y) = values, z = nibbles
-#pragma unroll
-    for (int ch = 0; ch < kTileN / 32; ++ch) {
-      if (n0 + ch * 32 >= n_limit) break;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int64_t token = n0 + ch * 32 + i * 8 + (lane >> 2), f = m0 + q * 32 + (lane & 3) * 8;
-        const uint2 r = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const uint16_t*>(args.aux) +
-                                                             token * (args.M >> 1) + (f >> 1)));
-        const uint32_t mb = __ldg(reinterpret_cast<const uint8_t*>(args.pack_meta) + token * (args.M >> 3) + (f >> 3));
-        ax[is_drelu_t(kEpi) ? ch : 0][i] = make_uint4(r.x, r.y, mb, 0u);
-      }
-    }
-  }
-  if (kEpi == EPI_DRELU_T) {
-#pragma unroll
-    for (int ch = 0; ch < kTileN / 32; ++ch) {
-      if (n0 + ch * 32 >= n_limit) break;
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        ax[kEpi == EPI_DRELU_T ? ch : 0][i] = __ldg(reinterpret_cast<const uint4*>(
-            reinterpret_cast<const uint16_t*>(args.aux) + (n0 + ch * 32 + i * 8 + (lane >> 2)) * args.ldaux + m0 +
-            q * 32 + (lane & 3) * 8));
-    }
-  }
-}
-
 template <int kEpi, int kTileN = BN>
 __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit,
-                                         int q, int lane, uint8_t* my_stage,
-                                         const uint4 (&ax)[is_drelu_t(kEpi) ? kTileN / 32 : 1][4]) {
+                                         int q, int lane, uint8_t* my_stage) {
   int64_t row = m0 + q * 32 + lane;                                        // this thread's D row
   if constexpr (kEpi == EPI_ROUTE) {
     // the row is a token, the first route_E columns its logits
@@ -144,7 +134,7 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
     row_live = r >= 0;
     row = r;
   }
-  auto chunk = [&](int ch, const uint4 (&a4)[4], const uint32_t (&v)[32]) {
+  auto chunk = [&](int ch, const uint32_t (&v)[32]) {
     const int64_t col0 = n0 + ch * 32;
     if (col0 >= n_limit) return;                                           // ragged last tile (warp-uniform)
     if (kEpi == EPI_STORE || kEpi == EPI_SQRELU || kEpi == EPI_DRELU) {
@@ -196,121 +186,48 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
         }
       }
     } else {
-      // Transposed output: D row = feature (lane), D column = token. C is [N, M] row-major.
-      float r[32];
-      // optional packed copy: the metadata words of this chunk's 32 tokens (features m0 + 32q .. + 31)
-      const bool pack = kEpi == EPI_DRELU24_T || (kEpi == EPI_DRELU_T && args.pack_vals != nullptr);
-      uint32_t mw[4] = {0, 0, 0, 0};
-      if (pack && kEpi == EPI_DRELU_T) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          mw[i] = __ldg(reinterpret_cast<const uint32_t*>(reinterpret_cast<const uint8_t*>(args.pack_meta) +
-                                                         (col0 + i * 8 + (lane >> 2)) * (args.M >> 3) +
-                                                         ((m0 + q * 32) >> 3)));
-      }
-      if (is_drelu_t(kEpi)) {
-        // aux[token, feature] chunk -> staging -> one column per lane
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          *reinterpret_cast<uint4*>(my_stage + (i * 8 + (lane >> 2)) * kEpiStageRow + (lane & 3) * 16) =
-              kEpi == EPI_DRELU24_T ? expand24_x8(make_uint2(a4[i].x, a4[i].y), a4[i].z) : a4[i];
-        __syncwarp();
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          r[j] = bf16_bits_to_float(*reinterpret_cast<const uint16_t*>(my_stage + j * kEpiStageRow + lane * 2));
-      }
+      // Transposed output: D row = feature (lane), D column = token. C is [N, M] row-major. Two tokens travel
+      // as one word: half the staging stores of a 16-bit transpose.
+      uint32_t* st = reinterpret_cast<uint32_t*>(my_stage);
       __syncwarp();
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        float x = __uint_as_float(v[j]);
-        uint32_t b;
-        if (is_drelu_t(kEpi)) {
-          // aux holds ReLU(y1) on the activation mask and +0 elsewhere: off-mask entries become +0
-          b = (r[j] == 0.f) ? 0u : float_to_bf16_bits(__fmul_rn(__fmul_rn(2.f, x), r[j]));
-        } else {
-          b = float_to_bf16_bits(x);
-        }
-        *reinterpret_cast<uint16_t*>(my_stage + j * kEpiStageRow + lane * 2) = (uint16_t)b;
-      }
+      for (int j = 0; j < 16; ++j)
+        st[j * 32 + lane] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
       __syncwarp();
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int t = i * 8 + (lane >> 2), seg = lane & 3;
-        const uint4 o = *reinterpret_cast<const uint4*>(my_stage + t * kEpiStageRow + seg * 16);
-        if (kEpi == EPI_ACT24_T) {
-          // o = y1 of eight neighbouring features of one token: SquaredReLU, then the two larger of every four
-          const int64_t token = col0 + t, fl = m0 + q * 32 + seg * 8, Fe = args.M;
-          const uint32_t r0w = bf2_relu(o.x), r1w = bf2_relu(o.y), r2w = bf2_relu(o.z), r3w = bf2_relu(o.w);
-          uint32_t pa, pb;
-          const uint32_t na = top2of4_packed(bf2_sq(r0w), bf2_sq(r1w), &pa), nb = top2of4_packed(bf2_sq(r2w), bf2_sq(r3w), &pb);
-          const uint32_t ra = __byte_perm(r0w, r1w, 0x1010u + (na & 3u) * 0x22u + (na >> 2) * 0x2200u);
-          const uint32_t rb = __byte_perm(r2w, r3w, 0x1010u + (nb & 3u) * 0x22u + (nb >> 2) * 0x2200u);
-          const int64_t pv = (token * (Fe >> 1) + (fl >> 1)) >> 2;             // 8-byte units
-          reinterpret_cast<uint2*>(args.vn_vals24)[pv] = make_uint2(pa, pb);
-          reinterpret_cast<uint2*>(args.vn_relu24)[pv] = make_uint2(ra, rb);
-          uint32_t mb = na | (nb << 4);
-          reinterpret_cast<uint4*>(args.vn_dense)[(token * Fe + fl) >> 3] = expand24_x8(make_uint2(pa, pb), mb);
-          if (args.vn_y1) reinterpret_cast<uint4*>(args.vn_y1)[(token * Fe + fl) >> 3] = o;
-          // metadata: one byte per lane, four neighbouring lanes hold the warp's 32 features of this token
-          mb |= __shfl_down_sync(0xFFFFFFFFu, mb, 1) << 8;
-          const uint32_t mb32 = (mb & 0xFFFFu) | (__shfl_down_sync(0xFFFFFFFFu, mb, 2) << 16);
-          const int64_t kw = (m0 + q * 32) >> 4;
-          if (seg == 0) reinterpret_cast<uint32_t*>(args.vn_meta24)[(token * (Fe >> 4) + kw) >> 1] = mb32;
-          if ((seg & 1) == 0)
-            *reinterpret_cast<uint16_t*>(reinterpret_cast<uint8_t*>(args.vn_meta24_hw) +
-                                         meta_hw_offset(token, kw + (seg >> 1), Fe)) = (uint16_t)mb;
-          continue;
-        }
-        if (kEpi != EPI_DRELU24_T || args.C != nullptr)
-          *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(args.C) + (col0 + t) * args.ldc + m0 + q * 32 + seg * 8) = o;
-        if (pack) {
-          // this lane's eight features are two groups of four: keep the two recorded positions of each
-          const uint32_t mb = kEpi == EPI_DRELU24_T ? (a4[i].z & 0xFFu) : ((mw[i] >> (8 * seg)) & 0xFFu);
-          const uint32_t p0 = __byte_perm(o.x, o.y, 0x1010u + (mb & 3u) * 0x22u + ((mb >> 2) & 3u) * 0x2200u);
-          const uint32_t p1 = __byte_perm(o.z, o.w, 0x1010u + ((mb >> 4) & 3u) * 0x22u + (mb >> 6) * 0x2200u);
-          *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(args.pack_vals) + (col0 + t) * (args.M >> 1) +
-                                    ((m0 + q * 32 + seg * 8) >> 1)) = make_uint2(p0, p1);
-        }
+      for (int i = 0; i < 2; ++i) {
+        uint32_t r0[4], r1[4];
+        pair_rows(st + (i * 8 + (lane >> 2)) * 32 + (lane & 3) * 8, lane, r0, r1);
+        uint16_t* c = reinterpret_cast<uint16_t*>(args.C) + (col0 + i * 16 + (lane >> 2) * 2) * args.ldc + m0 + q * 32 + (lane & 3) * 8;
+        *reinterpret_cast<uint4*>(c) = make_uint4(r0[0], r0[1], r0[2], r0[3]);
+        *reinterpret_cast<uint4*>(c + args.ldc) = make_uint4(r1[0], r1[1], r1[2], r1[3]);
       }
     }
-        };
+  };
   // Two register buffers: the TMEM load of the next 32 columns is in flight while this one is converted.
   uint32_t va[32], vb[32];
   tmem_ld_32x32b_x32(taddr, va);
   constexpr int kChunks = kTileN / 32;
-  if (is_drelu_t(kEpi)) {
-#pragma unroll
-    for (int ch = 0; ch < kChunks; ch += 2) {
-      tmem_ld_wait_on(va);
-      if (ch + 1 < kChunks) tmem_ld_32x32b_x32(taddr + (ch + 1) * 32, vb);
-      chunk(ch, ax[is_drelu_t(kEpi) ? ch : 0], va);
-      if (ch + 1 < kChunks) {
-        tmem_ld_wait_on(vb);
-        if (ch + 2 < kChunks) tmem_ld_32x32b_x32(taddr + (ch + 2) * 32, va);
-        chunk(ch + 1, ax[is_drelu_t(kEpi) ? (ch + 1 < kChunks ? ch + 1 : ch) : 0], vb);
-      }
-    }
-  } else if (kChunks % 2 == 0) {
+  if (kChunks % 2 == 0) {
 #pragma unroll 1
     for (int ch = 0; ch < kChunks; ch += 2) {
       tmem_ld_wait_on(va);
       tmem_ld_32x32b_x32(taddr + (ch + 1) * 32, vb);
-      chunk(ch, ax[0], va);
+      chunk(ch, va);
       tmem_ld_wait_on(vb);
       if (ch + 2 < kChunks) tmem_ld_32x32b_x32(taddr + (ch + 2) * 32, va);
-      chunk(ch + 1, ax[0], vb);
+      chunk(ch + 1, vb);
     }
   } else {
 #pragma unroll
     for (int ch = 0; ch < kChunks; ch += 2) {
       tmem_ld_wait_on(va);
       if (ch + 1 < kChunks) tmem_ld_32x32b_x32(taddr + (ch + 1) * 32, vb);
-      chunk(ch, ax[0], va);
+      chunk(ch, va);
       if (ch + 1 < kChunks) {
         tmem_ld_wait_on(vb);
         if (ch + 2 < kChunks) tmem_ld_32x32b_x32(taddr + (ch + 2) * 32, va);
-        chunk(ch + 1, ax[0], vb);
+        chunk(ch + 1, vb);
       }
     }
   }
@@ -334,8 +251,8 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
 // token), then colidx, the selector table and the nibble table of the block.
 __host__ __device__ constexpr int vnm_stage_bytes(int V) { return V * 64; }
 __host__ __device__ constexpr int vnm_warp_bytes(int V) { return vnm_stage_bytes(V) + 16 + 4 * 7 * 16 + 48; }
-constexpr int kVnmEpiWarps = 8;                                  // two sets of four: one set per accumulator buffer
-__host__ __device__ constexpr int vnm_epi_bytes(int V) { return kVnmEpiWarps * vnm_warp_bytes(V); }
+constexpr int kSetWarps = 8;                                     // two sets of four: one set per accumulator buffer
+__host__ __device__ constexpr int vnm_epi_bytes(int V) { return kSetWarps * vnm_warp_bytes(V); }
 
 template <int kTileN, int kV>
 __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0,
@@ -351,9 +268,7 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
   int nblk = kBlocks;
   while (nblk > 0 && n0 + (int64_t)(nblk - 1) * kV >= n_limit) --nblk;     // ragged last tile: whole blocks only
   if (nblk == 0) {
-    tc_fence_before();
-    __syncwarp();
-    if (lane == 0) mbar_arrive_leader(tmem_empty_bar);
+    release_accumulator(lane, tmem_empty_bar);
     return;
   }
   // strides per token of the outputs this thread writes (in the units of its pointers)
@@ -380,11 +295,7 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
         score = __fadd_rn(score, __uint_as_float(hp & 0xFFFF0000u));
       }
     }
-    if (b == nblk - 1) {
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_leader(tmem_empty_bar);
-    }
+    if (b == nblk - 1) release_accumulator(lane, tmem_empty_bar);
     // ---- rank the eight columns of each group
     const uint32_t sb = __float_as_uint(score);                            // scores are >= 0: the pattern orders them
     int rank = 0;
@@ -476,18 +387,10 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
         *reinterpret_cast<uint16_t*>(hw_atom + (mi >> 4) * 256u + (mi & 7u) * 16u + ((mi >> 3) & 1u) * 2u) = (uint16_t)mb;
       }
     };
-    // A quarter-warp reads two token pairs x four groups; pairs alternate which 16-byte half they fetch
-    // first, so each of the two loads touches every bank exactly once.
-    const int swap = (lane >> 2) & 1;
 #pragma unroll 1
     for (int it = 0; it < kV / 16; ++it) {
-      const uint4 q0 = *reinterpret_cast<const uint4*>(sp + 4 * swap), q1 = *reinterpret_cast<const uint4*>(sp + 4 - 4 * swap);
-      const uint4 qa = swap ? q1 : q0, qb = swap ? q0 : q1;
-      // de-interleave the token pair: low halves = even token, high halves = odd token
-      const uint32_t r0[4] = {__byte_perm(qa.x, qa.y, 0x5410), __byte_perm(qa.z, qa.w, 0x5410),
-                              __byte_perm(qb.x, qb.y, 0x5410), __byte_perm(qb.z, qb.w, 0x5410)};
-      const uint32_t r1[4] = {__byte_perm(qa.x, qa.y, 0x7632), __byte_perm(qa.z, qa.w, 0x7632),
-                              __byte_perm(qb.x, qb.y, 0x7632), __byte_perm(qb.z, qb.w, 0x7632)};
+      uint32_t r0[4], r1[4];
+      pair_rows(sp, lane, r0, r1);
       const uint32_t trow = (uint32_t)(tf & 127) + 16u * (uint32_t)it;
       emit(r0, 0, trow);
       emit(r1, 1, trow + 1u);
@@ -496,6 +399,184 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
       if (p_y1) p_y1 += 16 * s24;
       if (p_dense) p_dense += 16 * s24;
       p_meta += 16 * sm; p_m24 += 16 * sm24;
+    }
+  }
+}
+
+// ---- dy1 = 2 dy2 ReLU(y1) on the activation's mask (Eq. 6) -----------------------------------------------
+// Epilogue of the dy2 product: TMEM lane = feature, column = token. A chunk of 32 tokens x 32 features goes
+// through shared memory as float32, [token][feature] with rows 33 words apart (conflict-free column stores);
+// a lane then serves eight features of a token and fetches the accumulator values of the KEPT features only
+// (EPI_DRELU24_T: two per four, positions from the metadata byte; EPI_DRELUV_T: the two of a wide V:N:M group,
+// where they fall into its eight features). ReLU(y1) of the next chunk is requested while this one is worked on.
+// The transposed-mask form that this replaces (every feature multiplied, 16-bit transposes both ways, one set
+// of warps) issued twice the instructions and bound the product at small d_model: T 4096, D 2048, F 8192 (M = 8)
+// 102 -> 82 us, T 8192, D 4096, F 16384 555 -> 523 us.
+constexpr int kDreluRow = 33;
+constexpr int kDreluWarpBytes = 32 * kDreluRow * 4;
+
+// One 2:4 group back to its four dense columns through the 16-entry selector table.
+__device__ __forceinline__ void expand24_lut(const uint2* lut, uint32_t pair, uint32_t nib, uint32_t& w0, uint32_t& w1) {
+  const uint2 s = lut[nib];
+  w0 = __byte_perm(pair, 0u, s.x);
+  w1 = __byte_perm(pair, 0u, s.y);
+}
+
+template <int kEpi, int kTileN>
+__device__ __forceinline__ bool epi_drelu_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit,
+                                               bool live, int q, int lane, float* stage, const uint2* lut,
+                                               uint64_t* tmem_full_bar, uint32_t phase, volatile int* abort_flag,
+                                               uint64_t* tmem_empty_bar) {
+  constexpr bool kVenomMask = kEpi == EPI_DRELUV_T;
+  const int t8 = lane >> 2, seg = lane & 3;
+  const int64_t f = m0 + q * 32 + seg * 8;                                 // this lane's first feature
+  const int nch = live ? (int)min((int64_t)(kTileN / 32), (n_limit - n0) >> 5) : 0;
+  const int64_t tok = n0 + t8;                                             // this lane's first token
+  // per token: EPI_DRELU24_T four stored values + one metadata byte; EPI_DRELUV_T the group's pair + its nibble
+  const int64_t g = kVenomMask ? f / args.Mv : 0;
+  const int64_t s_relu = kVenomMask ? 2 * args.G : args.M >> 1, s_meta = kVenomMask ? args.G >> 1 : args.M >> 3;
+  const uint8_t* p_relu = reinterpret_cast<const uint8_t*>(args.aux) + 2 * (tok * s_relu + (kVenomMask ? 2 * g : f >> 1));
+  const uint8_t* p_meta = reinterpret_cast<const uint8_t*>(args.pack_meta) + tok * s_meta + (kVenomMask ? g >> 1 : f >> 3);
+  uint2 r[4];
+  uint32_t mb[4], c4 = 0, c4n = 0;
+  auto fetch = [&](int ch) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int64_t t = ch * 32 + i * 8;
+      if (kVenomMask) r[i].x = __ldg(reinterpret_cast<const uint32_t*>(p_relu + 2 * t * s_relu));
+      else            r[i] = __ldg(reinterpret_cast<const uint2*>(p_relu + 2 * t * s_relu));
+      mb[i] = __ldg(p_meta + t * s_meta);
+    }
+    if (kVenomMask)      // a chunk lies inside one V-block (V is a multiple of 32)
+      c4n = __ldg(reinterpret_cast<const uint32_t*>(args.colidx + ((n0 + ch * 32) / args.V * args.G + g) * 4));
+  };
+  if (nch > 0) fetch(0);
+  if (!mbar_wait(tmem_full_bar, phase, abort_flag)) return false;
+  tc_fence_after();
+  if (nch == 0) {
+    release_accumulator(lane, tmem_empty_bar);
+    return true;
+  }
+  uint32_t v[32];
+  tmem_ld_32x32b_x32(taddr, v);
+  const float* row0 = stage + t8 * kDreluRow + seg * 8;
+  uint16_t* p_dense = args.C ? reinterpret_cast<uint16_t*>(args.C) + tok * args.ldc + f : nullptr;
+  const int off = kVenomMask ? (int)(f & (args.Mv - 1)) : 0;               // this lane's first column inside its group
+#pragma unroll 1
+  for (int ch = 0; ch < nch; ++ch) {
+    tmem_ld_wait_on(v);
+    __syncwarp();                                                          // the previous chunk has been read
+#pragma unroll
+    for (int j = 0; j < 32; ++j) stage[j * kDreluRow + lane] = __uint_as_float(v[j]);
+    __syncwarp();
+    uint2 rc[4];
+    uint32_t mc[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { rc[i] = r[i]; mc[i] = mb[i]; }
+    c4 = c4n;
+    if (ch + 1 < nch) {
+      tmem_ld_32x32b_x32(taddr + (ch + 1) * 32, v);
+      fetch(ch + 1);
+    } else {
+      release_accumulator(lane, tmem_empty_bar);
+    }
+    // an off-mask entry is +0, also where the saved ReLU is zero
+    auto prod = [](float x, uint32_t rb) {
+      const float rv = bf16_bits_to_float(rb & 0xFFFFu);
+      return rv == 0.f ? 0.f : __fmul_rn(__fmul_rn(2.f, x), rv);
+    };
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float* row = row0 + i * 8 * kDreluRow;
+      const int64_t t = tok + ch * 32 + i * 8;
+      uint4 o;
+      if (!kVenomMask) {
+        const uint32_t m = mc[i];
+        const uint32_t pa = pack_bf16x2(prod(row[m & 3u], rc[i].x), prod(row[(m >> 2) & 3u], rc[i].x >> 16));
+        const uint32_t pb = pack_bf16x2(prod(row[4u + ((m >> 4) & 3u)], rc[i].y), prod(row[4u + (m >> 6)], rc[i].y >> 16));
+        *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(args.pack_vals) + t * (args.M >> 1) + (f >> 1)) = make_uint2(pa, pb);
+        expand24_lut(lut, pa, m & 15u, o.x, o.y);
+        expand24_lut(lut, pb, m >> 4, o.z, o.w);
+      } else {
+        const uint32_t nib = (mc[i] >> (4 * (g & 1))) & 15u;
+        const uint32_t da = ((c4 >> (8 * (nib & 3u))) & 0xFFu) - (uint32_t)off, db = ((c4 >> (8 * (nib >> 2))) & 0xFFu) - (uint32_t)off;
+        uint16_t* pv = reinterpret_cast<uint16_t*>(args.pack_vals) + t * (2 * args.G) + 2 * g;
+        uint32_t va = 0, vb = 0;
+        if (da < 8u) { va = float_to_bf16_bits(prod(row[da], rc[i].x)); pv[0] = (uint16_t)va; }
+        if (db < 8u) { vb = float_to_bf16_bits(prod(row[db], rc[i].x >> 16)); pv[1] = (uint16_t)vb; }
+        va <<= 16 * (da & 1u);
+        vb <<= 16 * (db & 1u);
+        const uint32_t wa = da >> 1, wb = db >> 1;                         // word of the kept column (beyond 3: not in this lane)
+        o.x = (wa == 0u ? va : 0u) | (wb == 0u ? vb : 0u);
+        o.y = (wa == 1u ? va : 0u) | (wb == 1u ? vb : 0u);
+        o.z = (wa == 2u ? va : 0u) | (wb == 2u ? vb : 0u);
+        o.w = (wa == 3u ? va : 0u) | (wb == 3u ? vb : 0u);
+      }
+      if (p_dense) *reinterpret_cast<uint4*>(p_dense + (int64_t)(ch * 32 + i * 8) * args.ldc) = o;
+    }
+  }
+  return true;
+}
+
+// ---- fused SquaredReLU + 2:4 selection inside every four features of a token ------------------------------
+// Epilogue of the routed y1 product and of the M = 4 step (a V x 4 block keeps all of its columns, so nothing
+// but the row-wise choice is left): y1 goes through shared memory as token pairs; a lane serves eight features
+// of two tokens and writes values, ReLU values, both metadata orders, the masked copy, and y1 if asked for.
+// The M = 4 step ran this as a second kernel on a stored y1 before: T 1920, D 1408, F 5504, whole step 224 -> 194 us.
+template <int kTileN>
+__device__ __forceinline__ void epi_act24_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit,
+                                               int q, int lane, uint32_t* stage, const uint2* lut, const Top2Entry* top2,
+                                               uint64_t* tmem_empty_bar) {
+  const int seg = lane & 3;
+  const int64_t Fe = args.M, f = m0 + q * 32 + seg * 8, kw = (m0 + q * 32) >> 4;
+  const int nch = (int)min((int64_t)(kTileN / 32), (n_limit - n0) >> 5);
+  uint32_t v[32];
+  tmem_ld_32x32b_x32(taddr, v);
+#pragma unroll 1
+  for (int ch = 0; ch < nch; ++ch) {
+    tmem_ld_wait_on(v);
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 16; ++j) stage[j * 32 + lane] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+    __syncwarp();
+    if (ch + 1 < nch) tmem_ld_32x32b_x32(taddr + (ch + 1) * 32, v);
+    else              release_accumulator(lane, tmem_empty_bar);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      uint32_t y[2][4];
+      pair_rows(stage + (i * 8 + (lane >> 2)) * 32 + seg * 8, lane, y[0], y[1]);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int64_t token = n0 + ch * 32 + i * 16 + (lane >> 2) * 2 + k;
+        uint32_t rw[4], hw[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { rw[j] = bf2_relu(y[k][j]); hw[j] = bf2_sq(rw[j]); }
+        Top2Entry ea, eb;
+        top2of4_x2(__byte_perm(hw[0], hw[2], 0x5410u), __byte_perm(hw[0], hw[2], 0x7632u), __byte_perm(hw[1], hw[3], 0x5410u),
+                   __byte_perm(hw[1], hw[3], 0x7632u), top2, ea, eb);
+        const uint32_t pa = __byte_perm(hw[0], hw[1], ea.kept), pb = __byte_perm(hw[2], hw[3], eb.kept);
+        const uint32_t na = (ea.kept >> 16) & 15u, nb = (eb.kept >> 16) & 15u;
+        const int64_t pv = (token * (Fe >> 1) + (f >> 1)) >> 2;              // 8-byte units
+        reinterpret_cast<uint2*>(args.vn_vals24)[pv] = make_uint2(pa, pb);
+        reinterpret_cast<uint2*>(args.vn_relu24)[pv] = make_uint2(__byte_perm(rw[0], rw[1], ea.kept), __byte_perm(rw[2], rw[3], eb.kept));
+        uint4 d;
+        expand24_lut(lut, pa, na, d.x, d.y);
+        expand24_lut(lut, pb, nb, d.z, d.w);
+        reinterpret_cast<uint4*>(args.vn_dense)[(token * Fe + f) >> 3] = d;
+        if (args.vn_y1) reinterpret_cast<uint4*>(args.vn_y1)[(token * Fe + f) >> 3] = make_uint4(y[k][0], y[k][1], y[k][2], y[k][3]);
+        // metadata: one byte per lane, four neighbouring lanes hold the warp's 32 features of this token
+        uint32_t mb = na | (nb << 4);
+        mb |= __shfl_down_sync(0xFFFFFFFFu, mb, 1) << 8;
+        const uint32_t mb32 = (mb & 0xFFFFu) | (__shfl_down_sync(0xFFFFFFFFu, mb, 2) << 16);
+        if (seg == 0) reinterpret_cast<uint32_t*>(args.vn_meta24)[(token * (Fe >> 4) + kw) >> 1] = mb32;
+        if ((seg & 1) == 0)
+          *reinterpret_cast<uint16_t*>(reinterpret_cast<uint8_t*>(args.vn_meta24_hw) + meta_hw_offset(token, kw + (seg >> 1), Fe)) =
+              (uint16_t)mb;
+        // V:N:M with groups of four: every block keeps columns 0..3 of its two groups here
+        if (args.vn_colidx && token % args.V == 0)
+          *reinterpret_cast<uint2*>(reinterpret_cast<uint8_t*>(args.vn_colidx) + (token / args.V) * Fe + f) =
+              make_uint2(0x03020100u, 0x03020100u);
+      }
     }
   }
 }
@@ -729,21 +810,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant_
   } else {
     // =========================== epilogue (warps 2..5) ===========================
     const int q = warp & 3;                                                    // TMEM lane quadrant
-    uint8_t* my_stage = epi_stage + q * 32 * kEpiStageRow;
+    uint8_t* my_stage = epi_stage + q * kEpiWarpBytes;
     uint32_t acc = 0, acc_phase = 0;
     bool ok = true;
     for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
       int mt, nt;
       tile_coords(tile, num_m_tiles, num_n_tiles_, mt, nt);
       const int64_t m0 = (int64_t)mt * BM, n0 = (int64_t)nt * BN;
-      // The dy1 epilogue multiplies by a [token, feature] tile of the saved activations; its loads do
-      // not depend on the accumulator, so they are issued before the wait and land during the main loop.
-      uint4 ax[is_drelu_t(kEpi) ? BN / 32 : 1][4];
-      epi_prefetch<kEpi>(args, m0, n0, args.N, q, lane, ax);
       if (!mbar_wait(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + acc * BN + ((uint32_t)(q * 32) << 16);
-      epi_tile<kEpi>(args, taddr, m0, n0, args.N, q, lane, my_stage, ax);
+      epi_tile<kEpi>(args, taddr, m0, n0, args.N, q, lane, my_stage);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctl->tmem_empty[acc]);
@@ -772,9 +849,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant_
 // four MMAs per barrier round trip keep the single issuing thread ahead of the tensor pipe.
 constexpr int kThreads2 = 192;
 constexpr int kThreads2Expand = 448;                     // + eight warps that expand a packed operand into its stage
-constexpr int kThreads2Vnm = 320;                        // + a second set of four epilogue warps (one set per accumulator)
+constexpr int kThreads2Sets = 320;                       // + a second set of four epilogue warps (one set per accumulator)
 __host__ __device__ constexpr int threads2(int epi, int expand) {
-  return expand ? kThreads2Expand : (epi == EPI_VNM8 ? kThreads2Vnm : kThreads2);
+  return expand ? kThreads2Expand : (two_sets(epi) ? kThreads2Sets : kThreads2);
 }
 constexpr int kPkStageBytes = 8192 + 1024;               // packed values [64 tokens][64] + metadata bytes [64][16]
 // 8-bit operands (fp8 = true) keep the byte geometry of a stage (128-byte rows now hold 128 elements, so a
@@ -789,7 +866,9 @@ __host__ __device__ constexpr int num_stages2(bool sparse, int bn = BN, bool exp
 // the fused activation epilogue holds whole V-blocks per tile: 192 columns = three blocks of 64, 128 = one of 128
 __host__ __device__ constexpr int vnm_block(int bn) { return bn == 192 ? 64 : 128; }
 __host__ __device__ constexpr int epi_bytes2(int epi, int bn = BN) {
-  return epi == EPI_VNM8 ? vnm_epi_bytes(vnm_block(bn)) : kEpiStageBytes;
+  return epi == EPI_VNM8 ? vnm_epi_bytes(vnm_block(bn))
+         : is_drelu_t(epi) ? kSetWarps * kDreluWarpBytes
+         : epi == EPI_ACT24_T ? kSetWarps * kEpiWarpBytes : 4 * kEpiWarpBytes;
 }
 __host__ __device__ constexpr int smem_bytes2(bool sparse, int bn = BN, int epi = EPI_STORE, bool expand = false,
                                               bool fp8 = false) {
@@ -803,7 +882,8 @@ struct SmemCtl2 {
   uint64_t pk_full[8];
   uint64_t tmem_full[2];
   uint64_t tmem_empty[2];
-  uint2 expand_lut[16];      // byte-permute selectors of a 2:4 nibble (see the operand expander)
+  uint2 expand_lut[16];      // byte-permute selectors of a 2:4 nibble (see expand24_lut)
+  Top2Entry top2_lut[16];    // EPI_ACT24_T
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -885,13 +965,14 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     ctl->abort_flag = 0;
     fence_mbar_init();
   }
-  if (kExpand && threadIdx.x >= 64 && threadIdx.x < 80) {
+  if ((kExpand || is_drelu_t(kEpi) || kEpi == EPI_ACT24_T) && threadIdx.x >= 64 && threadIdx.x < 80) {
     // nibble n = p0 | p1 << 2: output byte pair of column c takes stored value 0 (bytes 1,0) if c == p0,
     // value 1 (bytes 3,2) if c == p1, else the zero operand (byte 4)
     const uint32_t n = threadIdx.x - 64;
     const uint32_t sel = 0x44444444u ^ (0x54u << (8u * (n & 3u))) ^ (0x76u << (8u * (n >> 2)));
     ctl->expand_lut[n] = make_uint2(sel & 0xFFFFu, sel >> 16);
   }
+  if (kEpi == EPI_ACT24_T && threadIdx.x >= 96) top2_lut_init(ctl->top2_lut, (int)threadIdx.x - 96);
   if (warp == 1) {
     tmem_alloc_2cta(&ctl->tmem_base, kTmemCols);
     tmem_relinquish_2cta();
@@ -1068,50 +1149,53 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
         if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
     }
-  } else if constexpr (kEpi == EPI_VNM8) {
-    // =========================== fused activation epilogue (warps 2..9, both CTAs) ===========================
+  } else if constexpr (two_sets(kEpi)) {
+    // =========================== epilogue in two sets (warps 2..9, both CTAs) ===========================
     // Two sets of four warps, one per accumulator buffer: set 0 takes this pair's even tiles, set 1 the odd
     // ones, so each set has two main loops' time for one tile.
     const int q = warp & 3, set = (warp - 2) >> 2;
-    constexpr int kV = vnm_block(kBN);
-    uint8_t* wsm = epi_stage + (set * 4 + q) * vnm_warp_bytes(kV);
+    uint8_t* wsm = epi_stage + (set * 4 + q) * (epi_bytes2(kEpi, kBN) / kSetWarps);
+    const uint32_t taddr = tmem_base + set * kBN + ((uint32_t)(q * 32) << 16);
     uint32_t acc_phase = 0;
     for (int tile = pair + set * num_pairs; tile < num_tiles; tile += 2 * num_pairs) {
-      int mt, nt;
-      tile_coords(tile, num_m_tiles, num_n_tiles_, mt, nt);
-      const int64_t m0 = (int64_t)mt * 256 + (int64_t)rank * 128, n0 = (int64_t)nt * kBN;
-      const uint32_t taddr = tmem_base + set * kBN + ((uint32_t)(q * 32) << 16);
-      if (!mbar_wait(&ctl->tmem_full[set], acc_phase, abort_flag)) break;
-      tc_fence_after();
-      if (m0 >= args.M) {
-        // M % 256 == 128: the second CTA of the last row of pairs holds no rows (its operand loads were
-        // zero-filled); it only hands the accumulator back
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_leader(&ctl->tmem_empty[set]);
+      const GemmTile tc = get_tile<kBN>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
+      const int64_t m0 = (int64_t)tc.out_m + (int64_t)rank * 128, n0 = tc.out_n, n_limit = tc.n_limit;
+      // M % 256 == 128 (regular raster only): the second CTA of the last row of pairs holds no rows (its operand
+      // loads were zero-filled); it only hands the accumulator back
+      const bool live = args.tile_table != nullptr || m0 < args.M;
+      if constexpr (is_drelu_t(kEpi)) {
+        if (!epi_drelu_tile<kEpi, kBN>(args, taddr, m0, n0, n_limit, live, q, lane, reinterpret_cast<float*>(wsm), ctl->expand_lut,
+                                       &ctl->tmem_full[set], acc_phase, abort_flag, &ctl->tmem_empty[set]))
+          break;
       } else {
-        // releases the accumulator itself, as soon as its last column has been read
-        epi_vnm8_tile<kBN, kV>(args, taddr, m0, n0, args.N, q, lane, wsm, &ctl->tmem_empty[set]);
+        if (!mbar_wait(&ctl->tmem_full[set], acc_phase, abort_flag)) break;
+        tc_fence_after();
+        if (!live) {
+          release_accumulator(lane, &ctl->tmem_empty[set]);
+        } else if constexpr (kEpi == EPI_VNM8) {
+          epi_vnm8_tile<kBN, vnm_block(kBN)>(args, taddr, m0, n0, n_limit, q, lane, wsm, &ctl->tmem_empty[set]);
+        } else {
+          epi_act24_tile<kBN>(args, taddr, m0, n0, n_limit, q, lane, reinterpret_cast<uint32_t*>(wsm), ctl->expand_lut,
+                              ctl->top2_lut, &ctl->tmem_empty[set]);
+        }
       }
       acc_phase ^= 1;
     }
   } else {
     // =========================== epilogue (warps 2..5, both CTAs) ===========================
     const int q = warp & 3;
-    uint8_t* my_stage = epi_stage + q * 32 * kEpiStageRow;
+    uint8_t* my_stage = epi_stage + q * kEpiWarpBytes;
     uint32_t acc = 0, acc_phase = 0;
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
       const GemmTile tc = get_tile<kBN>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
       const int64_t m0 = (int64_t)tc.out_m + (int64_t)rank * 128, n0 = tc.out_n, n_limit = tc.n_limit;
       const uint32_t taddr = tmem_base + acc * kBN + ((uint32_t)(q * 32) << 16);
-      uint4 ax[is_drelu_t(kEpi) ? kBN / 32 : 1][4];
       // M % 256 == 128 (regular raster only): the second CTA of the last row of pairs holds no rows
       const bool live = args.tile_table != nullptr || m0 < args.M;
-      if (live) epi_prefetch<kEpi, kBN>(args, m0, n0, n_limit, q, lane, ax);
       if (!mbar_wait(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      if (live) epi_tile<kEpi, kBN>(args, taddr, m0, n0, n_limit, q, lane, my_stage, ax);
+      if (live) epi_tile<kEpi, kBN>(args, taddr, m0, n0, n_limit, q, lane, my_stage);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_leader(&ctl->tmem_empty[acc]);
@@ -1281,11 +1365,8 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
 }
 
 int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, bool b_kmajor, int64_t M, int64_t N,
-                  int64_t K, int epi, void* C, int64_t ldc, const void* aux, int64_t ldaux, int* status,
-                  cudaStream_t s, const void* pack_meta, void* pack_vals) {
-  if ((pack_meta != nullptr) != (pack_vals != nullptr) || (pack_vals && !is_drelu_t(epi))) return SF_ERR_UNSUPPORTED;
+                  int64_t K, int epi, void* C, int64_t ldc, int* status, cudaStream_t s) {
   const bool two = use_two_cta(M);
-  if (epi == EPI_DRELU24_T && (!pack_vals || !aux || !two)) return SF_ERR_UNSUPPORTED;   // C (dense copy) optional
   if (M % BM || N % (two ? 128 : BN) || K % 128) return SF_ERR_SHAPE;
   if (M == 0 || N == 0) return SF_OK;
   const bool plain = (epi == EPI_STORE);                 // row-major output, either B layout: two-CTA kernel only
@@ -1308,8 +1389,7 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   }
   GemmArgs a{};
   a.M = M; a.N = N; a.K = K;
-  a.C = C; a.ldc = ldc; a.aux = aux; a.ldaux = ldaux; a.meta_hw = meta_hw; a.status = status;
-  a.pack_meta = pack_meta; a.pack_vals = pack_vals;
+  a.C = C; a.ldc = ldc; a.meta_hw = meta_hw; a.status = status;
   a.num_m_tiles = (int)(M / BM); a.num_n_tiles = (int)(N / BN); a.num_k_blocks = (int)(K / 64);
   if (epi == EPI_STORE) {
     if (b_kmajor) return launch_two<MODE_SPARSE24, false, false, EPI_STORE>(ta, tb, tm, a, s);
@@ -1318,11 +1398,48 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   if (epi == EPI_STORE_T)
     return two ? launch_two<MODE_SPARSE24, false, false, EPI_STORE_T, kNarrowBN>(ta, tb, tm, a, s)
                : launch_one<MODE_SPARSE24, false, false, EPI_STORE_T>(ta, tb, a, s);
-  if (epi == EPI_DRELU_T)
-    return two ? launch_two<MODE_SPARSE24, false, false, EPI_DRELU_T, kNarrowBN>(ta, tb, tm, a, s)
-               : launch_one<MODE_SPARSE24, false, false, EPI_DRELU_T>(ta, tb, a, s);
-  if (epi == EPI_DRELU24_T) return launch_two<MODE_SPARSE24, false, false, EPI_DRELU24_T, kNarrowBN>(ta, tb, tm, a, s);
   return SF_ERR_UNSUPPORTED;
+}
+
+namespace {
+// The 2:4 weight-times-token products whose epilogue works on the activation: W [F, D] packed, tokens [T, D],
+// 224-column token tiles with two accumulators.
+int weight_token_maps(const void* w_vals, const uint8_t* meta_hw, const void* tokens, int64_t F, int64_t T, int64_t D, int bn,
+                      CUtensorMap* ta, CUtensorMap* tb, CUtensorMap* tm) {
+  int st = make_tmap(ta, w_vals, F, D / 2, D / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B);
+  if (st == SF_OK) st = make_tmap(tb, tokens, T, D, D, 64, bn / 2, CU_TENSOR_MAP_SWIZZLE_128B);
+  // hardware-ordered metadata: 2 KB atoms viewed as two rows of 256 uint32
+  if (st == SF_OK) st = make_tmap(tm, meta_hw, 2 * (F / 128) * (D / 128), 256, 256, 256, 2, CU_TENSOR_MAP_SWIZZLE_NONE, 1);
+  return st;
+}
+}  // namespace
+
+int gemm_sparse24_drelu(const void* w_vals, const uint8_t* meta_hw, const void* dY, int64_t F, int64_t T, int64_t D,
+                        const ActMask& mask, void* dy1_vals, void* dy1_dense, int* status, cudaStream_t s) {
+  if (F < 256 || F % 128 || T % 128 || D % 128) return SF_ERR_SHAPE;
+  CUtensorMap ta, tb, tm;
+  const int st = weight_token_maps(w_vals, meta_hw, dY, F, T, D, kNarrowBN, &ta, &tb, &tm);
+  if (st != SF_OK) return st;
+  GemmArgs a{};
+  a.M = F; a.N = T; a.K = D;
+  a.C = dy1_dense; a.ldc = F; a.aux = mask.relu; a.pack_meta = mask.meta; a.pack_vals = dy1_vals; a.status = status;
+  if (!mask.colidx) return launch_two<MODE_SPARSE24, false, false, EPI_DRELU24_T, kNarrowBN>(ta, tb, tm, a, s);
+  a.colidx = mask.colidx; a.V = mask.V; a.Mv = mask.Mv; a.G = F / mask.Mv;
+  return launch_two<MODE_SPARSE24, false, false, EPI_DRELUV_T, kNarrowBN>(ta, tb, tm, a, s);
+}
+
+int gemm_sparse24_act4(const void* w_vals, const uint8_t* meta_hw, const void* X, int64_t F, int64_t T, int64_t D, int V,
+                       const Act24Out& out, void* colidx, int* status, cudaStream_t s) {
+  if (F < 256 || F % 128 || T % 128 || D % 128) return SF_ERR_SHAPE;
+  CUtensorMap ta, tb, tm;
+  const int st = weight_token_maps(w_vals, meta_hw, X, F, T, D, kNarrowBN, &ta, &tb, &tm);
+  if (st != SF_OK) return st;
+  GemmArgs a{};
+  a.M = F; a.N = T; a.K = D; a.V = V;
+  a.status = status;
+  a.vn_vals24 = out.vals; a.vn_relu24 = out.relu; a.vn_meta24 = out.meta; a.vn_meta24_hw = out.meta_hw;
+  a.vn_dense = out.dense; a.vn_y1 = out.y1; a.vn_colidx = colidx;
+  return launch_two<MODE_SPARSE24, false, false, EPI_ACT24_T, kNarrowBN>(ta, tb, tm, a, s);
 }
 
 int gemm_route(const void* X, const void* means, int64_t T, int64_t D, int E, int* expert, float* logits, int* status,
@@ -1379,12 +1496,7 @@ int gemm_sparse24_vnm8(const void* a_vals, const uint8_t* meta_hw, const void* X
   // Token tiles hold whole V-blocks: three blocks of 64 (192 columns) or one block of 128.
   const int bn = V == 64 ? 192 : 128;
   CUtensorMap ta, tb, tm;
-  int st = make_tmap(&ta, a_vals, F, D / 2, D / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B);
-  if (st != SF_OK) return st;
-  st = make_tmap(&tb, X, T, D, D, 64, bn / 2, CU_TENSOR_MAP_SWIZZLE_128B);
-  if (st != SF_OK) return st;
-  const int64_t atoms = (F / 128) * (D / 128);
-  st = make_tmap(&tm, meta_hw, 2 * atoms, 256, 256, 256, 2, CU_TENSOR_MAP_SWIZZLE_NONE, 1);
+  const int st = weight_token_maps(a_vals, meta_hw, X, F, T, D, bn, &ta, &tb, &tm);
   if (st != SF_OK) return st;
   GemmArgs a{};
   a.M = F; a.N = T; a.K = D; a.V = V;
@@ -1405,11 +1517,7 @@ int gemm_grouped_act24(const void* a_vals, const uint8_t* meta_hw, const void* X
                        int* status, cudaStream_t s) {
   if (F % 256 || Fe % 256 || D % 128 || rows % 32 || max_tiles <= 0) return SF_ERR_SHAPE;
   CUtensorMap ta, tb, tm;
-  int st = make_tmap(&ta, a_vals, F, D / 2, D / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B);
-  if (st != SF_OK) return st;
-  st = make_tmap(&tb, Xp, rows, D, D, 64, kNarrowBN / 2, CU_TENSOR_MAP_SWIZZLE_128B);
-  if (st != SF_OK) return st;
-  st = make_tmap(&tm, meta_hw, 2 * (F / 128) * (D / 128), 256, 256, 256, 2, CU_TENSOR_MAP_SWIZZLE_NONE, 1);
+  const int st = weight_token_maps(a_vals, meta_hw, Xp, F, rows, D, kNarrowBN, &ta, &tb, &tm);
   if (st != SF_OK) return st;
   GemmArgs a{};
   a.M = Fe; a.N = rows; a.K = D;                           // M: width of the outputs (features per expert)
@@ -1425,11 +1533,7 @@ int gemm_grouped_drelu24(const void* a_vals, const uint8_t* meta_hw, const void*
                          const GemmTile* tiles, const int* num_tiles, int max_tiles, int* status, cudaStream_t s) {
   if (F % 256 || Fe % 256 || D % 128 || rows % 32 || max_tiles <= 0) return SF_ERR_SHAPE;
   CUtensorMap ta, tb, tm;
-  int st = make_tmap(&ta, a_vals, F, D / 2, D / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B);
-  if (st != SF_OK) return st;
-  st = make_tmap(&tb, dYp, rows, D, D, 64, kNarrowBN / 2, CU_TENSOR_MAP_SWIZZLE_128B);
-  if (st != SF_OK) return st;
-  st = make_tmap(&tm, meta_hw, 2 * (F / 128) * (D / 128), 256, 256, 256, 2, CU_TENSOR_MAP_SWIZZLE_NONE, 1);
+  const int st = weight_token_maps(a_vals, meta_hw, dYp, F, rows, D, kNarrowBN, &ta, &tb, &tm);
   if (st != SF_OK) return st;
   GemmArgs a{};
   a.M = Fe; a.N = rows; a.K = D;

@@ -13,13 +13,13 @@ enum GemmEpilogue {
   EPI_SQRELU = 1,   // C = y = bf16(acc);  C2 = bf16(max(y, 0)^2)                     (Eq. 2)
   EPI_DRELU = 2,    // C = bf16(2 * acc * max(aux[m, n], 0))                           (Eq. 6)
   EPI_STORE_T = 3,  // C[n, m] = bf16(acc)          (accumulator rows are output columns)
-  EPI_DRELU_T = 4,  // C[n, m] = bf16(2 * acc * aux[n, m]), +0 where aux is zero       (Eq. 6 on the mask)
+  EPI_DRELUV_T = 4, // dy1 = 2 * acc * ReLU(y1) on the mask of a V:N:M activation with groups wider than eight, given as
+                    // the packed ReLU values, metadata and colidx; writes dy1 packed and as a masked matrix    (Eq. 6)
   EPI_VNM8 = 5,     // SquaredReLU + V:N:M selection (groups of eight) on the accumulator tile itself: rows are
                     // features, columns are tokens; writes the packed activation, never the dense y1  (Eq. 2, Section 2.3)
-  EPI_DRELU24_T = 6,// as EPI_DRELU_T with aux given in the 2:4 layout of the mask (values [n, m/2] + pack_meta) and
-                    // only the packed output written
+  EPI_DRELU24_T = 6,// the same with the mask in the 2:4 layout (aux = values [n, m/2], pack_meta = metadata)
   EPI_ACT24_T = 7,  // transposed output with SquaredReLU and a 2:4 selection inside every four features of a token
-                    // (the routed step's activation, Section 3.1 step 3): packed values, packed ReLU values, both
+                    // (the activation of the routed step, Section 3.1 step 3, and of M = 4): packed values, packed ReLU values, both
                     // metadata orders and the masked dense copy; never the pre-activation unless asked for
   EPI_ROUTE = 8     // accumulator rows are tokens, its first route_E columns the experts' logits: each row writes its
                     // arg-max (ties to the lower expert) and, optionally, the float32 logits   (Section 3.1 step 1)
@@ -44,15 +44,15 @@ struct GemmArgs {
   const void* aux;
   int64_t ldaux;
   const uint8_t* meta_hw;   // sparse modes: hardware-ordered metadata atoms
-  const uint8_t* colidx;    // Venom: [T/V, G, 4]
-  int64_t G;                // Venom: groups per row (F / Mv)
+  const uint8_t* colidx;    // Venom, EPI_DRELUV_T: [T/V, G, 4]
+  int64_t G;                // the same: groups per row (F / Mv)
   int V, Mv;                // Venom block height and group width
   int* status;              // device status word (set to 1 when a bounded wait expires)
   int num_m_tiles, num_n_tiles, num_k_blocks;
   int gather_tma_groups;    // Venom: groups (of 16 per stage) fetched by TMA row gather; the rest by cp.async
-  // EPI_DRELU_T only, optional: also emit the output packed as a 2:4 operand at given positions
-  const void* pack_meta;    // canonical 2:4 metadata [N, M/16] uint16 (rows = output rows of Ct)
-  void* pack_vals;          // bf16 [N, M/2]
+  // EPI_DRELU24_T / EPI_DRELUV_T: metadata of the activation's mask and the packed output (see ActMask)
+  const void* pack_meta;
+  void* pack_vals;
   // EPI_VNM8 outputs (T = N tokens, F = M features, G = F / 8 groups per token)
   void* vn_vals;            // bf16 [T, 2G]   kept activation values (V:N:M packed)
   void* vn_relu;            // bf16 [T, 2G]   ReLU(y1) at the same positions
@@ -105,6 +105,10 @@ bool gemm_sparse24_vnm8_supported(int64_t F, int64_t T, int64_t D, int V);
 struct Act24Out {
   void *vals, *relu, *meta, *meta_hw, *dense, *y1;
 };
+// The y1 product of a step with M = 4 (blocks keep all their columns: only the row-wise 2:4 choice is left) with the
+// same epilogue over all F features, writing the constant colidx as well.
+int gemm_sparse24_act4(const void* w_vals, const uint8_t* meta_hw, const void* X, int64_t F, int64_t T, int64_t D, int V,
+                       const Act24Out& out, void* colidx, int* status, cudaStream_t s);
 // y1c = Xp W1s[expert block]^T with the epilogue above. a_vals/meta_hw: W1s [F, D] packed; Xp [rows, D].
 int gemm_grouped_act24(const void* a_vals, const uint8_t* meta_hw, const void* Xp, int64_t rows, int64_t F, int64_t Fe,
                        int64_t D, const Act24Out& out, const GemmTile* tiles, const int* num_tiles, int max_tiles,
@@ -125,18 +129,27 @@ int gemm_grouped_sparse24_rm(const void* a_vals, const uint8_t* meta_hw, const v
 int gemm_grouped_dense_tn(const void* A, int64_t Ma, const void* B, int64_t Nb, int64_t rows, void* C, int64_t ldc,
                           const GemmTile* tiles, const int* num_tiles, int max_tiles, int* status, cudaStream_t s);
 // A_s[M,K] 2:4-packed times B (b_kmajor: [N,K] row-major, else [K,N] row-major).
-// epi EPI_STORE_T / EPI_DRELU_T: transposed output Ct[N,M] (b_kmajor only); EPI_STORE: C[M,N]
+// epi EPI_STORE_T: transposed output Ct[N,M] (b_kmajor only); EPI_STORE: C[M,N]
 // (two-CTA kernel, M % 256 == 0).
-// pack_meta / pack_vals (EPI_DRELU_T, optional): additionally write Ct gathered at the positions of the
-// canonical 2:4 metadata pack_meta [N, M/16] into pack_vals [N, M/2].
 int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, bool b_kmajor, int64_t M, int64_t N,
-                  int64_t K, int epi, void* C, int64_t ldc, const void* aux, int64_t ldaux, int* status,
-                  cudaStream_t s, const void* pack_meta = nullptr, void* pack_vals = nullptr);
+                  int64_t K, int epi, void* C, int64_t ldc, int* status, cudaStream_t s);
+// The dy2 product dY[T, D] W2s[F, D]^T with Eq. 6 in its epilogue: dy1 = 2 dy2 ReLU(y1) on the activation's mask,
+// written packed like the mask's ReLU values (dy1_vals) and, unless dy1_dense is null, as a masked [T, F] matrix.
+struct ActMask {
+  const void *relu, *meta;    // colidx null: 2:4 layout over all F columns (values [T, F/2], metadata [T, F/16]);
+  const uint8_t* colidx;      // else V:N:M groups of Mv > 8 columns (values [T, 2F/Mv], metadata [T, F/(4 Mv)], colidx)
+  int V, Mv;
+};
+int gemm_sparse24_drelu(const void* w_vals, const uint8_t* meta_hw, const void* dY, int64_t F, int64_t T, int64_t D,
+                        const ActMask& mask, void* dy1_vals, void* dy1_dense, int* status, cudaStream_t s);
 // Routing on the tensor cores: logits[T, E] = X[T, D] means[E, D]^T in float32 accumulators, the arg-max per token
 // taken in the epilogue (ties to the lower expert). T % 256 == 0, D % 64 == 0, 1 <= E <= 16; the means need no
 // padding (rows beyond E are read as zeros by the tensor map).
 int gemm_route(const void* X, const void* means, int64_t T, int64_t D, int E, int* expert, float* logits, int* status,
                cudaStream_t s);
+// canonical [R, K/16] metadata words -> hardware-ordered atoms (R % 128 == 0, K % 128 == 0)
+int launch_meta_reorder(const void* meta, void* meta_hw, int64_t R, int64_t K, cudaStream_t s);
+
 // E4M3 operands, both K-major: C[M, N] = bf16(alpha * A B^T). sparse: A = 2:4 values [M, K/2] (codes) with
 // metadata in the 8-bit instruction's order (see meta_hw8_offset); else A [M, K]. B [N, K].
 // M % 256 == 0, N % 32 == 0, K % 256 == 0 (2:4) or K % 128 == 0 (dense).
@@ -150,11 +163,5 @@ int gemm_venom(const void* a_vals, const uint8_t* meta_hw, const uint8_t* colidx
 // elements with leading dimension ld; box = {box_cols, box_rows}.
 int make_tmap_2d(void* map, const void* base, int64_t rows, int64_t cols, int64_t ld, uint32_t box_cols,
                  uint32_t box_rows, bool swizzle128);
-
-// canonical [R, K/16] metadata words -> hardware-ordered atoms (R % 128 == 0, K % 128 == 0)
-int launch_meta_reorder(const void* meta, void* meta_hw, int64_t R, int64_t K, cudaStream_t s);
-// dy1 packing: gather a dense [T, F] matrix at the positions recorded by (colidx, meta)
-int launch_pack_like(const void* dense, const void* meta, const void* colidx, void* vals, int64_t T, int64_t F,
-                     int V, int Mv, cudaStream_t s);
 
 }  // namespace sf

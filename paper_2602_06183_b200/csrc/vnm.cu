@@ -56,8 +56,7 @@ template <int kW>
 __global__ void __launch_bounds__(kThreads)
 vnm_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, int V, int M, int apply,
            uint16_t* __restrict__ vals, uint16_t* __restrict__ meta, uint8_t* __restrict__ meta_hw,
-           uint8_t* __restrict__ colidx, uint16_t* __restrict__ relu_vals, uint16_t* __restrict__ dense_out,
-           uint16_t* __restrict__ relu_dense_out) {
+           uint8_t* __restrict__ colidx, uint16_t* __restrict__ relu_vals, uint16_t* __restrict__ dense_out) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   uint16_t* tile = reinterpret_cast<uint16_t*>(smem_raw);                        // [V][kW + kPad]
   uint32_t* score = reinterpret_cast<uint32_t*>(tile + (size_t)V * (kW + kPad)); // [kW] float bits
@@ -162,7 +161,6 @@ vnm_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, int
     uint16_t* p_vals = vals + trow * (2 * G) + 2 * (g0 + g);
     uint16_t* p_relu = want_relu ? relu_vals + trow * (2 * G) + 2 * (g0 + g) : nullptr;
     uint16_t* p_dense = dense_out ? dense_out + trow * F + c0 + g * M : nullptr;
-    uint16_t* p_rdense = relu_dense_out ? relu_dense_out + trow * F + c0 + g * M : nullptr;
     uint16_t* p_meta = meta + trow * (G >> 2) + ((g0 + g) >> 2);
     const int64_t kw = (g0 + g) >> 2;
     const int64_t s_vals = (int64_t)rstep * (2 * G), s_dense = (int64_t)rstep * F, s_meta = (int64_t)rstep * (G >> 2);
@@ -176,30 +174,25 @@ vnm_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, int
       *reinterpret_cast<uint32_t*>(p_vals) = packed;
       const uint32_t rpair = __byte_perm(rl_lo, rl_hi, 0x1010u + p0 * 0x22u + p1 * 0x2200u);
       if (want_relu) *reinterpret_cast<uint32_t*>(p_relu) = rpair;
-      if (dense_out || relu_dense_out) {
+      if (dense_out) {
         // whole 16-byte stores only: word j of the group holds the value kept at column 2j or 2j + 1
         const uint32_t ca = (c4 >> (8 * p0)) & 0xFFu, cb = (c4 >> (8 * p1)) & 0xFFu;       // kept columns, ca < cb
         const uint32_t wa = ca >> 1, wb = cb >> 1, sa = 16u * (ca & 1u), sb = 16u * (cb & 1u);
         const uint32_t ha = (packed & 0xFFFFu) << sa, hb = (packed >> 16) << sb;
-        const uint32_t ra = (rpair & 0xFFFFu) << sa, rb = (rpair >> 16) << sb;
         if (M >= 8) {
           for (int m8 = 0; m8 < M; m8 += 8) {
-            uint32_t dw[4], rw4[4];
+            uint32_t dw[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               const uint32_t wj = (uint32_t)(m8 >> 1) + j;
               const bool ia = wa == wj, ib = wb == wj;
               dw[j] = (ia ? ha : 0u) | (ib ? hb : 0u);
-              rw4[j] = (ia ? ra : 0u) | (ib ? rb : 0u);
             }
-            if (dense_out) *reinterpret_cast<uint4*>(p_dense + m8) = make_uint4(dw[0], dw[1], dw[2], dw[3]);
-            if (relu_dense_out) *reinterpret_cast<uint4*>(p_rdense + m8) = make_uint4(rw4[0], rw4[1], rw4[2], rw4[3]);
+            *reinterpret_cast<uint4*>(p_dense + m8) = make_uint4(dw[0], dw[1], dw[2], dw[3]);
           }
         } else {                                            // M == 4: one 8-byte group
           const uint32_t d0 = (wa == 0u ? ha : 0u) | (wb == 0u ? hb : 0u), d1 = (wa == 1u ? ha : 0u) | (wb == 1u ? hb : 0u);
-          const uint32_t q0 = (wa == 0u ? ra : 0u) | (wb == 0u ? rb : 0u), q1 = (wa == 1u ? ra : 0u) | (wb == 1u ? rb : 0u);
-          if (dense_out) *reinterpret_cast<uint2*>(p_dense) = make_uint2(d0, d1);
-          if (relu_dense_out) *reinterpret_cast<uint2*>(p_rdense) = make_uint2(q0, q1);
+          *reinterpret_cast<uint2*>(p_dense) = make_uint2(d0, d1);
         }
       }
       uint32_t word = nib;
@@ -213,7 +206,6 @@ vnm_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, int
       p_vals += s_vals;
       if (want_relu) p_relu += s_vals;
       if (dense_out) p_dense += s_dense;
-      if (relu_dense_out) p_rdense += s_dense;
       p_meta += s_meta;
     }
     return;
@@ -241,7 +233,6 @@ vnm_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, int
       if (relu_vals && apply) *reinterpret_cast<uint32_t*>(relu_vals + t * (2 * G) + 2 * (g0 + g)) = r0 | (r1 << 16);
       const uint32_t ca = (c4 >> (8 * p0)) & 0xFFu, cb = (c4 >> (8 * p1)) & 0xFFu;
       if (dense_out) write_group_dense(dense_out + t * F + c0 + g * M, M, ca, cb, v0, v1);
-      if (relu_dense_out) write_group_dense(relu_dense_out + t * F + c0 + g * M, M, ca, cb, r0, r1);
     }
     // four neighbouring groups of a row -> one metadata word (ng is a multiple of 4)
     uint32_t word = valid ? nib : 0u;
@@ -267,7 +258,7 @@ __global__ void __launch_bounds__(kThreads)
 vnm8_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, int V, int apply,
             uint16_t* __restrict__ vals, uint16_t* __restrict__ meta, uint8_t* __restrict__ meta_hw,
             uint8_t* __restrict__ colidx, uint16_t* __restrict__ relu_vals, uint16_t* __restrict__ dense_out,
-            uint16_t* __restrict__ relu_dense_out, uint16_t* __restrict__ vals24, uint16_t* __restrict__ meta24,
+            uint16_t* __restrict__ vals24, uint16_t* __restrict__ meta24,
             uint8_t* __restrict__ meta24_hw, uint16_t* __restrict__ relu24) {
   constexpr int M = 8;
   extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -384,7 +375,7 @@ vnm8_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, in
   }
   const bool lead4 = (g & 3) == 0, lead2 = (g & 1) == 0;
   const bool want_relu = relu_vals && apply, want24 = vals24 != nullptr;
-  const bool need_relu_pair = want_relu || (relu_dense_out != nullptr) || (relu24 != nullptr && apply);
+  const bool need_relu_pair = want_relu || (relu24 != nullptr && apply);
   const int64_t trow = t0 + r0;
   const uint16_t* tp = tile + r0 * kRow + g * M;
   const uint4* my_sel = sel_tab + g * 7;
@@ -392,7 +383,6 @@ vnm8_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, in
   uint16_t* p_vals = vals + trow * (2 * G) + 2 * (g0 + g);
   uint16_t* p_relu = want_relu ? relu_vals + trow * (2 * G) + 2 * (g0 + g) : nullptr;
   uint16_t* p_dense = dense_out ? dense_out + trow * F + c0 + g * M : nullptr;
-  uint16_t* p_rdense = relu_dense_out ? relu_dense_out + trow * F + c0 + g * M : nullptr;
   uint16_t* p_v24 = want24 ? vals24 + trow * (F >> 1) + (g0 + g) * 4 : nullptr;
   uint16_t* p_r24 = (want24 && relu24 && apply) ? relu24 + trow * (F >> 1) + (g0 + g) * 4 : nullptr;
   uint16_t* p_meta = meta + trow * (G >> 2) + ((g0 + g) >> 2);
@@ -433,9 +423,6 @@ vnm8_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, in
         *reinterpret_cast<uint2*>(p_r24) = make_uint2(__byte_perm(rpair, 0u, sel.w), __byte_perm(rpair, 0u, sel.w >> 16));
         p_r24 += s_v24;
       }
-      if (relu_dense_out)
-        *reinterpret_cast<uint4*>(p_rdense) = make_uint4(__byte_perm(rpair, 0u, sel.x), __byte_perm(rpair, 0u, sel.x >> 16),
-                                                         __byte_perm(rpair, 0u, sel.y), __byte_perm(rpair, 0u, sel.y >> 16));
     }
     if (dense_out)
       *reinterpret_cast<uint4*>(p_dense) = make_uint4(__byte_perm(packed, 0u, sel.x), __byte_perm(packed, 0u, sel.x >> 16),
@@ -469,7 +456,6 @@ vnm8_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, in
     p_vals += s_vals;
     if (want_relu) p_relu += s_vals;
     if (dense_out) p_dense += s_dense;
-    if (relu_dense_out) p_rdense += s_dense;
     p_meta += s_meta;
   }
 }
@@ -478,7 +464,7 @@ vnm8_kernel(const uint16_t* __restrict__ P, int64_t T, int64_t F, int64_t ld, in
 
 int launch_vnm(const void* P, int64_t T, int64_t F, int64_t ld, int V, int M, int apply_sqrelu,
                void* vals, void* meta, void* meta_hw, void* colidx, void* relu_vals, void* dense_out,
-               void* relu_dense_out, void* vals24, void* meta24, void* meta24_hw, void* relu24, cudaStream_t s) {
+               void* vals24, void* meta24, void* meta24_hw, void* relu24, cudaStream_t s) {
   if (T == 0 || F == 0) return SF_OK;
   const size_t smem = (size_t)V * (kCW + kPad) * 2 + kCW * 4 + kCW + kCW;
   static bool attr_set[64] = {false};                         // per device
@@ -510,7 +496,7 @@ int launch_vnm(const void* P, int64_t T, int64_t F, int64_t ld, int V, int M, in
     return launch_pdl(vnm8_kernel<kW8>, grid8, kThreads, smem8, s, (const uint16_t*)P, T, F, ld, V, apply_sqrelu, (uint16_t*)vals,
                                                     (uint16_t*)meta, (uint8_t*)meta_hw, (uint8_t*)colidx,
                                                     (uint16_t*)relu_vals, (uint16_t*)dense_out,
-                                                    (uint16_t*)relu_dense_out, (uint16_t*)vals24, (uint16_t*)meta24,
+                                                    (uint16_t*)vals24, (uint16_t*)meta24,
                                                     (uint8_t*)meta24_hw, (uint16_t*)relu24);
   }
   if (vals24) return SF_ERR_UNSUPPORTED;                 // the plain-2:4 view is produced by the fast path only
@@ -520,13 +506,11 @@ int launch_vnm(const void* P, int64_t T, int64_t F, int64_t ld, int V, int M, in
     dim3 grid_n((unsigned)((F + 127) / 128), (unsigned)(T / V));
     return launch_pdl(vnm_kernel<128>, grid_n, kThreads, smem_n, s, (const uint16_t*)P, T, F, ld, V, M, apply_sqrelu, (uint16_t*)vals,
                                                       (uint16_t*)meta, (uint8_t*)meta_hw, (uint8_t*)colidx,
-                                                      (uint16_t*)relu_vals, (uint16_t*)dense_out,
-                                                      (uint16_t*)relu_dense_out);
+                                                      (uint16_t*)relu_vals, (uint16_t*)dense_out);
   }
   return launch_pdl(vnm_kernel<256>, grid, kThreads, smem, s, (const uint16_t*)P, T, F, ld, V, M, apply_sqrelu, (uint16_t*)vals,
                                                   (uint16_t*)meta, (uint8_t*)meta_hw, (uint8_t*)colidx,
-                                                  (uint16_t*)relu_vals, (uint16_t*)dense_out,
-                                                  (uint16_t*)relu_dense_out);
+                                                  (uint16_t*)relu_vals, (uint16_t*)dense_out);
 }
 
 // True when launch_vnm can also emit the plain-2:4 view (vals24 / meta24) for this shape.
