@@ -76,6 +76,9 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // Which epilogues run on two sets of four warps (one set per accumulator) on CTA pairs.
 __host__ __device__ constexpr bool is_drelu_t(int epi) { return epi == EPI_DRELU24_T || epi == EPI_DRELUV_T; }
 __host__ __device__ constexpr bool two_sets(int epi) { return epi == EPI_VNM8 || epi == EPI_ACT24_T || is_drelu_t(epi); }
+// Dense products: two sets share every tile, each takes half of its columns (the last tile's epilogue is exposed:
+// 1024 x 256 x 1024 17.3 -> 14.3 us; the 2:4 products gained nothing from it).
+__host__ __device__ constexpr bool split_sets(int mode, int epi, int expand) { return mode == MODE_DENSE && epi != EPI_ROUTE && !expand; }
 
 // This warp has read its part of an accumulator for the last time: hand it back to the MMA warp.
 __device__ __forceinline__ void release_accumulator(int lane, uint64_t* tmem_empty_bar) {
@@ -101,13 +104,18 @@ __device__ __forceinline__ void pair_rows(const uint32_t* sp, int lane, uint32_t
 // ---- epilogue (shared by the one-CTA and the two-CTA kernels) ---------------------------------------
 // One epilogue warp owns TMEM lanes [32q, 32q+32) of a 128 x 256 accumulator tile whose first row is
 // m0 and first column n0; `taddr` is the TMEM address of (lane 32q, column 0) of that accumulator.
-// kTileN: accumulator columns of the tile (a multiple of 32). Columns at or beyond args.N (a ragged last
-// tile, whole 32-column chunks only since N % 32 == 0) are neither prefetched nor stored.
+// kTileN: accumulator columns of the tile (a multiple of 32). Columns at or beyond n_limit (a ragged last
+// tile, whole 32-column chunks only since N % 32 == 0) are not stored. `part` of `parts`: the share of the tile's
+// columns that this warp takes.
+// A thread holds one row. EPI_STORE stores from there (16 bytes of 32 rows per instruction): the shortest way out, and
+// the 2:4 product's epilogue is on its critical path (through shared memory as below that product took 2 % more at
+// K = 8192). The two-operand epilogues of the dense step move a chunk through shared memory, 64 contiguous bytes of
+// eight rows per instruction: y1 + SquaredReLU at T 4096, D 2048, F 8192 129 -> 96 us.
 template <int kEpi, int kTileN = BN>
 __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit,
-                                         int q, int lane, uint8_t* my_stage) {
-  int64_t row = m0 + q * 32 + lane;                                        // this thread's D row
+                                         int q, int lane, uint8_t* my_stage, int part = 0, int parts = 1) {
   if constexpr (kEpi == EPI_ROUTE) {
+    const int64_t row = m0 + q * 32 + lane;                                // this thread's D row
     // the row is a token, the first route_E columns its logits
     uint32_t v[32];
     tmem_ld_32x32b_x32(taddr, v);
@@ -128,62 +136,86 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
     }
     return;
   }
+  // chunks of 32 columns (warp-uniform): this warp's part of the live ones
+  const int live = (int)min((int64_t)(kTileN / 32), (n_limit - n0) >> 5);
+  const int ch0 = live * part / parts, nch = live * (part + 1) / parts;
+  if (ch0 >= nch) return;
+  int64_t row = m0 + q * 32 + lane;                                        // this thread's D row
   bool row_live = true;
   if (kEpi == EPI_STORE && args.row_map) {                                 // scattered output rows
     const int r = __ldg(args.row_map + row);
     row_live = r >= 0;
     row = r;
   }
-  auto chunk = [&](int ch, const uint32_t (&v)[32]) {
+  // EPI_SQRELU, EPI_DRELU: this thread moves 16-byte unit `u` of the rows `t8 + 8 i` of a chunk.
+  const int t8 = lane >> 2, u = lane & 3;
+  const int64_t out = m0 + q * 32 + t8;
+  // 32 x 32 bf16 in shared memory, 64 bytes a row, the four units of a row XOR-ed with bits of the row: conflict-free
+  // both for a thread per row and for four threads per row.
+  auto unit = [&](int r, int k) { return reinterpret_cast<uint4*>(my_stage + r * 64 + ((k ^ ((r >> 1) & 3)) << 4)); };
+  auto store_rows = [&](const uint32_t (&w)[16], void* C, int64_t ldc, int64_t col0) {
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) *unit(lane, j) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(C) + (out + 8 * i) * ldc + col0 + u * 8) = *unit(t8 + 8 * i, u);
+  };
+  uint4 a4[4];                                                             // EPI_DRELU: y1 of the next chunk
+  auto fetch = [&](int ch) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      a4[i] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(args.aux) + (out + 8 * i) * args.ldaux + n0 + ch * 32 + u * 8));
+  };
+  if (kEpi == EPI_DRELU) fetch(ch0);
+  // `v` holds (once its load is complete) the chunk's accumulator columns; `next` starts the load of the chunk after
+  auto chunk = [&](int ch, uint32_t (&v)[32], uint32_t (&next)[32]) {
     const int64_t col0 = n0 + ch * 32;
-    if (col0 >= n_limit) return;                                           // ragged last tile (warp-uniform)
-    if (kEpi == EPI_STORE || kEpi == EPI_SQRELU || kEpi == EPI_DRELU) {
-      uint16_t* crow = reinterpret_cast<uint16_t*>(args.C) + row * args.ldc + col0;
-      if (kEpi == EPI_STORE) {
-        if (!row_live) return;
-        const float al = args.out_scale != 0.f ? args.out_scale : 1.f;      // x 1 is exact: bf16 products unchanged
+    uint32_t w[16];
+    if (kEpi == EPI_DRELU) {                                               // y1 to a thread per row
+      __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint4 o;
-          o.x = pack_bf16x2(__fmul_rn(__uint_as_float(v[8 * j + 0]), al), __fmul_rn(__uint_as_float(v[8 * j + 1]), al));
-          o.y = pack_bf16x2(__fmul_rn(__uint_as_float(v[8 * j + 2]), al), __fmul_rn(__uint_as_float(v[8 * j + 3]), al));
-          o.z = pack_bf16x2(__fmul_rn(__uint_as_float(v[8 * j + 4]), al), __fmul_rn(__uint_as_float(v[8 * j + 5]), al));
-          o.w = pack_bf16x2(__fmul_rn(__uint_as_float(v[8 * j + 6]), al), __fmul_rn(__uint_as_float(v[8 * j + 7]), al));
-          reinterpret_cast<uint4*>(crow)[j] = o;
+      for (int i = 0; i < 4; ++i) *unit(t8 + 8 * i, u) = a4[i];
+      __syncwarp();
+      if (ch + 1 < nch) fetch(ch + 1);
+    }
+    tmem_ld_wait_on(v);
+    if (ch + 1 < nch) tmem_ld_32x32b_x32(taddr + (ch + 1) * 32, next);
+    if (kEpi == EPI_DRELU) {                                               // C = bf16(2 * acc * relu(aux))
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint4 a = *unit(lane, j);
+        const uint32_t aw[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float r0 = fmaxf(bf16_bits_to_float(aw[e] & 0xFFFFu), 0.f);
+          const float r1 = fmaxf(bf16_bits_to_float(aw[e] >> 16), 0.f);
+          w[4 * j + e] = pack_bf16x2(__fmul_rn(__fmul_rn(2.f, __uint_as_float(v[8 * j + 2 * e])), r0),
+                                     __fmul_rn(__fmul_rn(2.f, __uint_as_float(v[8 * j + 2 * e + 1])), r1));
         }
-      } else if (kEpi == EPI_SQRELU) {
-        uint16_t* hrow = reinterpret_cast<uint16_t*>(args.C2) + row * args.ldc2 + col0;
+      }
+    } else if (kEpi == EPI_STORE) {
+      const float al = args.out_scale != 0.f ? args.out_scale : 1.f;        // x 1 is exact: bf16 products unchanged
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint32_t y[4], h[4];
+      for (int j = 0; j < 16; ++j)
+        w[j] = pack_bf16x2(__fmul_rn(__uint_as_float(v[2 * j]), al), __fmul_rn(__uint_as_float(v[2 * j + 1]), al));
+    } else {
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const uint32_t y0 = float_to_bf16_bits(__uint_as_float(v[8 * j + 2 * e]));
-            const uint32_t y1 = float_to_bf16_bits(__uint_as_float(v[8 * j + 2 * e + 1]));
-            const float f0 = fmaxf(bf16_bits_to_float(y0), 0.f), f1 = fmaxf(bf16_bits_to_float(y1), 0.f);
-            y[e] = y0 | (y1 << 16);
-            h[e] = pack_bf16x2(__fmul_rn(f0, f0), __fmul_rn(f1, f1));
-          }
-          reinterpret_cast<uint4*>(crow)[j] = make_uint4(y[0], y[1], y[2], y[3]);
-          reinterpret_cast<uint4*>(hrow)[j] = make_uint4(h[0], h[1], h[2], h[3]);
-        }
-      } else {  // EPI_DRELU: C = bf16(2 * acc * relu(aux))
-        const uint16_t* arow = reinterpret_cast<const uint16_t*>(args.aux) + row * args.ldaux + col0;
+      for (int j = 0; j < 16; ++j) w[j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+    }
+    if (kEpi == EPI_STORE) {
+      if (row_live) {
+        uint4* c = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(args.C) + row * args.ldc + col0);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint4 a = __ldg(reinterpret_cast<const uint4*>(arow) + j);
-          const uint32_t aw[4] = {a.x, a.y, a.z, a.w};
-          uint32_t o[4];
+        for (int j = 0; j < 4; ++j) c[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+      }
+    } else if (kEpi != EPI_STORE_T) {
+      store_rows(w, args.C, args.ldc, col0);
+      if (kEpi == EPI_SQRELU) {
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float r0 = fmaxf(bf16_bits_to_float(aw[e] & 0xFFFFu), 0.f);
-            const float r1 = fmaxf(bf16_bits_to_float(aw[e] >> 16), 0.f);
-            const float d0 = __fmul_rn(__fmul_rn(2.f, __uint_as_float(v[8 * j + 2 * e])), r0);
-            const float d1 = __fmul_rn(__fmul_rn(2.f, __uint_as_float(v[8 * j + 2 * e + 1])), r1);
-            o[e] = pack_bf16x2(d0, d1);
-          }
-          reinterpret_cast<uint4*>(crow)[j] = make_uint4(o[0], o[1], o[2], o[3]);
-        }
+        for (int j = 0; j < 16; ++j) w[j] = bf2_sq(bf2_relu(w[j]));
+        store_rows(w, args.C2, args.ldc2, col0);
       }
     } else {
       // Transposed output: D row = feature (lane), D column = token. C is [N, M] row-major. Two tokens travel
@@ -191,45 +223,25 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
       uint32_t* st = reinterpret_cast<uint32_t*>(my_stage);
       __syncwarp();
 #pragma unroll
-      for (int j = 0; j < 16; ++j)
-        st[j * 32 + lane] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+      for (int j = 0; j < 16; ++j) st[j * 32 + lane] = w[j];
       __syncwarp();
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         uint32_t r0[4], r1[4];
-        pair_rows(st + (i * 8 + (lane >> 2)) * 32 + (lane & 3) * 8, lane, r0, r1);
-        uint16_t* c = reinterpret_cast<uint16_t*>(args.C) + (col0 + i * 16 + (lane >> 2) * 2) * args.ldc + m0 + q * 32 + (lane & 3) * 8;
+        pair_rows(st + (i * 8 + t8) * 32 + u * 8, lane, r0, r1);
+        uint16_t* c = reinterpret_cast<uint16_t*>(args.C) + (col0 + i * 16 + t8 * 2) * args.ldc + m0 + q * 32 + u * 8;
         *reinterpret_cast<uint4*>(c) = make_uint4(r0[0], r0[1], r0[2], r0[3]);
         *reinterpret_cast<uint4*>(c + args.ldc) = make_uint4(r1[0], r1[1], r1[2], r1[3]);
       }
     }
   };
-  // Two register buffers: the TMEM load of the next 32 columns is in flight while this one is converted.
+  // two register buffers: the TMEM load of the next 32 columns is in flight while this chunk is converted
   uint32_t va[32], vb[32];
-  tmem_ld_32x32b_x32(taddr, va);
-  constexpr int kChunks = kTileN / 32;
-  if (kChunks % 2 == 0) {
+  tmem_ld_32x32b_x32(taddr + ch0 * 32, va);
 #pragma unroll 1
-    for (int ch = 0; ch < kChunks; ch += 2) {
-      tmem_ld_wait_on(va);
-      tmem_ld_32x32b_x32(taddr + (ch + 1) * 32, vb);
-      chunk(ch, va);
-      tmem_ld_wait_on(vb);
-      if (ch + 2 < kChunks) tmem_ld_32x32b_x32(taddr + (ch + 2) * 32, va);
-      chunk(ch + 1, vb);
-    }
-  } else {
-#pragma unroll
-    for (int ch = 0; ch < kChunks; ch += 2) {
-      tmem_ld_wait_on(va);
-      if (ch + 1 < kChunks) tmem_ld_32x32b_x32(taddr + (ch + 1) * 32, vb);
-      chunk(ch, va);
-      if (ch + 1 < kChunks) {
-        tmem_ld_wait_on(vb);
-        if (ch + 2 < kChunks) tmem_ld_32x32b_x32(taddr + (ch + 2) * 32, va);
-        chunk(ch + 1, vb);
-      }
-    }
+  for (int ch = ch0; ch < nch; ch += 2) {
+    chunk(ch, va, vb);
+    if (ch + 1 < nch) chunk(ch + 1, vb, va);
   }
 }
 
@@ -849,9 +861,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant_
 // four MMAs per barrier round trip keep the single issuing thread ahead of the tensor pipe.
 constexpr int kThreads2 = 192;
 constexpr int kThreads2Expand = 448;                     // + eight warps that expand a packed operand into its stage
-constexpr int kThreads2Sets = 320;                       // + a second set of four epilogue warps (one set per accumulator)
-__host__ __device__ constexpr int threads2(int epi, int expand) {
-  return expand ? kThreads2Expand : (two_sets(epi) ? kThreads2Sets : kThreads2);
+constexpr int kThreads2Sets = 320;                       // + a second set of four epilogue warps
+__host__ __device__ constexpr int threads2(int mode, int epi, int expand) {
+  return expand ? kThreads2Expand : (two_sets(epi) || split_sets(mode, epi, expand) ? kThreads2Sets : kThreads2);
 }
 constexpr int kPkStageBytes = 8192 + 1024;               // packed values [64 tokens][64] + metadata bytes [64][16]
 // 8-bit operands (fp8 = true) keep the byte geometry of a stage (128-byte rows now hold 128 elements, so a
@@ -868,7 +880,7 @@ __host__ __device__ constexpr int vnm_block(int bn) { return bn == 192 ? 64 : 12
 __host__ __device__ constexpr int epi_bytes2(int epi, int bn = BN) {
   return epi == EPI_VNM8 ? vnm_epi_bytes(vnm_block(bn))
          : is_drelu_t(epi) ? kSetWarps * kDreluWarpBytes
-         : epi == EPI_ACT24_T ? kSetWarps * kEpiWarpBytes : 4 * kEpiWarpBytes;
+         : epi == EPI_STORE || epi == EPI_ROUTE ? 0 : kSetWarps * kEpiWarpBytes;
 }
 __host__ __device__ constexpr int smem_bytes2(bool sparse, int bn = BN, int epi = EPI_STORE, bool expand = false,
                                               bool fp8 = false) {
@@ -912,7 +924,7 @@ __device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) {
 // coordinates are given in 2-byte units (two codes each); only the instruction kind, the descriptor's formats
 // and the amount of metadata per stage differ.
 template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kEpi, kExpand), 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kMode, kEpi, kExpand), 1)
 gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB,
                 const __grid_constant__ CUtensorMap tmapMeta, const __grid_constant__ CUtensorMap tmapPk,
                 const GemmArgs args) {
@@ -960,7 +972,8 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&ctl->tmem_full[b], 1);
-      mbar_init(&ctl->tmem_empty[b], 8);                 // 4 epilogue warps in each CTA of the pair
+      // the epilogue warps of both CTAs that read the accumulator
+      mbar_init(&ctl->tmem_empty[b], split_sets(kMode, kEpi, kExpand) ? 16 : 8);
     }
     ctl->abort_flag = 0;
     fence_mbar_init();
@@ -1182,9 +1195,10 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
       acc_phase ^= 1;
     }
   } else {
-    // =========================== epilogue (warps 2..5, both CTAs) ===========================
-    const int q = warp & 3;
-    uint8_t* my_stage = epi_stage + q * kEpiWarpBytes;
+    // =========================== epilogue (warps 2..5 or 2..9, both CTAs) ===========================
+    const int q = warp & 3, set = (warp - 2) >> 2;
+    constexpr int kParts = split_sets(kMode, kEpi, kExpand) ? 2 : 1;
+    uint8_t* my_stage = epi_stage + (set * 4 + q) * kEpiWarpBytes;
     uint32_t acc = 0, acc_phase = 0;
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
@@ -1195,7 +1209,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
       const bool live = args.tile_table != nullptr || m0 < args.M;
       if (!mbar_wait(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      if (live) epi_tile<kEpi, kBN>(args, taddr, m0, n0, n_limit, q, lane, my_stage);
+      if (live) epi_tile<kEpi, kBN>(args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_leader(&ctl->tmem_empty[acc]);
@@ -1304,7 +1318,7 @@ int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
                                  : a.num_m_tiles * a.num_n_tiles;
   const int max_pairs = sm_count() / 2;
   const int pairs = tiles < max_pairs ? tiles : max_pairs;
-  return launch_pdl(kern, dim3(2 * pairs), threads2(kEpi, kExpand), smem, s, ta, tb, tm, tpk ? *tpk : ta, a);
+  return launch_pdl(kern, dim3(2 * pairs), threads2(kMode, kEpi, kExpand), smem, s, ta, tb, tm, tpk ? *tpk : ta, a);
 }
 
 // Tile width of the two-accumulator 2:4 variant (transposed-output products): 2 x 224 accumulator
