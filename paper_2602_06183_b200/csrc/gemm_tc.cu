@@ -427,6 +427,12 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
 constexpr int kDreluRow = 33;
 constexpr int kDreluWarpBytes = 32 * kDreluRow * 4;
 
+// Byte-permute selectors of nibble n = p0 | p1 << 2: output byte pair of column c takes stored value 0 (bytes 1,0) if
+// c == p0, value 1 (bytes 3,2) if c == p1, else the zero operand (byte 4).
+__device__ __forceinline__ uint2 expand_lut_entry(uint32_t n) {
+  const uint32_t sel = 0x44444444u ^ (0x54u << (8u * (n & 3u))) ^ (0x76u << (8u * (n >> 2)));
+  return make_uint2(sel & 0xFFFFu, sel >> 16);
+}
 // One 2:4 group back to its four dense columns through the 16-entry selector table.
 __device__ __forceinline__ void expand24_lut(const uint2* lut, uint32_t pair, uint32_t nib, uint32_t& w0, uint32_t& w1) {
   const uint2 s = lut[nib];
@@ -979,11 +985,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     fence_mbar_init();
   }
   if ((kExpand || is_drelu_t(kEpi) || kEpi == EPI_ACT24_T) && threadIdx.x >= 64 && threadIdx.x < 80) {
-    // nibble n = p0 | p1 << 2: output byte pair of column c takes stored value 0 (bytes 1,0) if c == p0,
-    // value 1 (bytes 3,2) if c == p1, else the zero operand (byte 4)
-    const uint32_t n = threadIdx.x - 64;
-    const uint32_t sel = 0x44444444u ^ (0x54u << (8u * (n & 3u))) ^ (0x76u << (8u * (n >> 2)));
-    ctl->expand_lut[n] = make_uint2(sel & 0xFFFFu, sel >> 16);
+    ctl->expand_lut[threadIdx.x - 64] = expand_lut_entry(threadIdx.x - 64);
   }
   if (kEpi == EPI_ACT24_T && threadIdx.x >= 96) top2_lut_init(ctl->top2_lut, (int)threadIdx.x - 96);
   if (warp == 1) {
@@ -1229,6 +1231,244 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   }
 }
 
+// ---- 512-row tiles of the 2:4 products ---------------------------------------------------------------
+// A CTA pair computes a 512 x 224 tile: two halves of 256 rows that share every stage's B columns, each with its own
+// accumulator (448 TMEM columns + 16 of metadata) and its own set of four epilogue warps.
+// Why: what bounds the 2:4 product is shared-memory bandwidth (128 B/clk). Per 128 logical K and SM a 256 x 256 tile
+// writes 50 KB (TMA) and its MMAs read 48 KB: 768 clocks against 512 of the tensor pipe (735 measured, with the ring
+// always full of data). Here B is written once for two halves: 64 KB written, 88 KB read, 1197 clocks against 896
+// (1190 measured), 10 % less per column than 256 x 256 and 15 % less than 256 x 224. The price: one accumulator per
+// half, so an epilogue overlaps the next main loop only as far as the halves are apart.
+// Against 256-row tiles, same box: y3 at T 16384, D 8192, F 28672 3540 -> 3090 us, dX 3550 -> 3110, dy1 4030 -> 3680;
+// 4096 x 16384 x 4096 296 -> 243 us, with E4M3 operands 196 -> 176.
+constexpr int kTallBN = 224, kTallStages = 3;
+constexpr int kTallThreads = 320;                         // producer, MMA issuer, two sets of four epilogue warps
+__host__ __device__ constexpr int tall_b_bytes(bool bmn) { return bmn ? 32768 : 28672; }
+__host__ __device__ constexpr int tall_stage_bytes(bool bmn, bool fp8) { return tall_b_bytes(bmn) + 2 * (16384 + meta_stage_bytes2(fp8)); }
+__host__ __device__ constexpr int tall_epi_bytes(int epi) {
+  return is_drelu_t(epi) ? kSetWarps * kDreluWarpBytes : epi == EPI_STORE ? 0 : kSetWarps * kEpiWarpBytes;
+}
+__host__ __device__ constexpr int tall_smem(int epi, bool bmn, bool fp8) {
+  return 1024 + kTallStages * tall_stage_bytes(bmn, fp8) + tall_epi_bytes(epi) + 1024;
+}
+
+struct SmemCtlTall {
+  uint64_t full[kTallStages], empty[kTallStages], tmem_full[2], tmem_empty[2];
+  uint2 expand_lut[16];
+  uint32_t tmem_base;
+  int abort_flag;
+};
+static_assert(sizeof(SmemCtlTall) <= 1024, "control block");
+
+// The l-th tile of CTA pair p (of P): -1 = no more. Full-width tiles are numbered first, the narrow ones of a ragged last
+// column (one per tile row) after them. Full tiles go round robin; narrow ones fill up the pairs whose last round is
+// empty, two each, where that takes all of them, else round robin too.
+__device__ __forceinline__ int tall_nth(const GemmArgs& args, int l, int p, int P) {
+  const int t = p + l * P, nfull = args.num_m_tiles * args.num_n_tiles;
+  if (t < nfull) return t;
+  const int nn = args.N % kTallBN ? args.num_m_tiles : 0;
+  if (nn == 0) return -1;
+  const int q = nfull / P, r = nfull - q * P, spare = P - r;
+  const int k = l - (q + (p < r));
+  int j;
+  if (r != 0 && nn <= 2 * spare) j = p < r ? nn : (p - r) + k * spare;
+  else                           j = (p < r ? p + spare : p - r) + k * P;
+  return j < nn ? nfull + j : -1;
+}
+
+struct TallTile {
+  int m0, n0, width, halves;   // first row and column, columns (a multiple of 32), 256-row halves that hold rows
+};
+__device__ __forceinline__ TallTile tall_tile(const GemmArgs& args, int tile) {
+  const int nfull = args.num_m_tiles * args.num_n_tiles;
+  int mt, nt;
+  if (tile < nfull) {
+    tile_coords(tile, args.num_m_tiles, args.num_n_tiles, mt, nt);
+  } else {
+    mt = tile - nfull;
+    nt = args.num_n_tiles;
+  }
+  const int m0 = mt * 512, n0 = nt * kTallBN;
+  return TallTile{m0, n0, min(kTallBN, (int)args.N - n0), m0 + 256 < (int)args.M ? 2 : 1};
+}
+
+// tmapB: B with boxes of 112 columns (K-major) or {64 n, 128 k} chunks (MN-major); tmapBn: K-major, boxes of half the
+// narrow last column.
+template <bool kBMN, int kEpi, bool kFp8>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTallThreads, 1)
+gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB,
+                 const __grid_constant__ CUtensorMap tmapBn, const __grid_constant__ CUtensorMap tmapMeta, const GemmArgs args) {
+  extern __shared__ uint8_t smem_dyn[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
+  constexpr int kBBytes = tall_b_bytes(kBMN), kMetaBytes = meta_stage_bytes2(kFp8), kStageBytes = tall_stage_bytes(kBMN, kFp8);
+  constexpr int kMetaAt = kBBytes + 2 * 16384;            // stage: B columns, A of either half, metadata of either half
+  constexpr int kSlab = (kTallBN / 2) * 128;              // K-major: this CTA's half of B for one 64-wide K slab
+  constexpr uint32_t kMetaCol = 2 * kTallBN, kMetaCols = kFp8 ? 8u : 4u;
+  static_assert(kMetaCol + 4 * kMetaCols <= kTmemCols, "TMEM columns");
+  static_assert(!kFp8 || (!kBMN && kEpi == EPI_STORE), "8-bit operands are K-major");
+  uint8_t* epi_stage = smem + kTallStages * kStageBytes;
+  SmemCtlTall* ctl = reinterpret_cast<SmemCtlTall*>(epi_stage + tall_epi_bytes(kEpi));
+  volatile int* abort_flag = &ctl->abort_flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
+  const int nkb = (int)(args.K / 128);
+
+  if (threadIdx.x == 0) {
+    prefetch_tmap(&tmapA);
+    prefetch_tmap(&tmapB);
+    prefetch_tmap(&tmapMeta);
+    for (int i = 0; i < kTallStages; ++i) { mbar_init(&ctl->full[i], 1); mbar_init(&ctl->empty[i], 1); }
+    for (int h = 0; h < 2; ++h) { mbar_init(&ctl->tmem_full[h], 1); mbar_init(&ctl->tmem_empty[h], 8); }
+    ctl->abort_flag = 0;
+    fence_mbar_init();
+  }
+  if (is_drelu_t(kEpi) && threadIdx.x >= 64 && threadIdx.x < 80) ctl->expand_lut[threadIdx.x - 64] = expand_lut_entry(threadIdx.x - 64);
+  if (warp == 1) {
+    tmem_alloc_2cta(&ctl->tmem_base, kTmemCols);
+    tmem_relinquish_2cta();
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();
+  tc_fence_after();
+  pdl_wait();
+  pdl_trigger();
+  const uint32_t tmem_base = ctl->tmem_base;
+
+  if (warp == 0) {
+    // =========================== TMA producer (both CTAs) ===========================
+    uint32_t stage = 0, phase = 0;
+    bool ok = true;
+    for (int l = 0, tile; ok && (tile = tall_nth(args, l, pair, num_pairs)) >= 0; ++l) {
+      const TallTile t = tall_tile(args, tile);
+      const int half_n = t.width / 2, m0 = t.m0 + (int)rank * 128, nb0 = t.n0 + (int)rank * half_n;
+      const int chunks = (half_n + 63) >> 6, atom0 = (m0 >> 7) * nkb;
+      const uint32_t tx = 2u * (t.halves * (16384u + (uint32_t)kMetaBytes) + (kBMN ? (uint32_t)chunks * 16384u : 256u * (uint32_t)half_n));
+      auto load_a = [&](int kb, int h, uint8_t* st, uint64_t* bar) {
+        tma_load_2d_2cta(st + kBBytes + h * 16384, &tmapA, bar, kb * 64, m0 + h * 256);           // stored values: box {64, 128}
+        // metadata atoms are rows of 2 x 1 KB in a [2 * atoms, 256] uint32 view (8-bit operands: pairs of atoms)
+        tma_load_2d_2cta(st + kMetaAt + h * kMetaBytes, &tmapMeta, bar, 0, (kFp8 ? 4 : 2) * (atom0 + 2 * h * nkb + kb));
+      };
+      for (int kb = 0; kb < nkb; ++kb) {
+        if (!mbar_wait(&ctl->empty[stage], phase ^ 1, abort_flag)) { ok = false; break; }
+        if (lane == 0) {
+          uint8_t* st = smem + stage * kStageBytes;
+          uint64_t* bar = &ctl->full[stage];
+          if (rank == 0) mbar_arrive_expect_tx(bar, tx);   // the leader's barrier collects the bytes of both CTAs
+          load_a(kb, 0, st, bar);
+          if (t.halves == 2) load_a(kb, 1, st, bar);
+          if (kBMN) {
+            tma_load_2d_2cta(st, &tmapB, bar, nb0, kb * 128);                                     // chunks {64 n, 128 k}
+            if (chunks == 2) tma_load_2d_2cta(st + 16384, &tmapB, bar, nb0 + 64, kb * 128);
+          } else if (t.width == kTallBN) {
+            tma_load_2d_2cta(st, &tmapB, bar, kb * 128, nb0);                                     // two 64-wide K slabs
+            tma_load_2d_2cta(st + kSlab, &tmapB, bar, kb * 128 + 64, nb0);
+          } else {
+            tma_load_2d_2cta(st, &tmapBn, bar, kb * 128, nb0);
+            tma_load_2d_2cta(st + kSlab, &tmapBn, bar, kb * 128 + 64, nb0);
+          }
+        }
+        if (++stage == kTallStages) { stage = 0; phase ^= 1; }
+      }
+    }
+  } else if (warp == 1) {
+    // =========================== MMA issuer (leader CTA only) ===========================
+    if (rank == 0 && lane == 0) {
+      constexpr uint32_t idesc0 = kFp8 ? idesc_e4m3(256, 0, true) : idesc_bf16(256, 0, false, kBMN, true);
+      const uint32_t idesc_wide = idesc0 | ((uint32_t)(kTallBN >> 3) << 17);
+      const uint32_t idesc_narrow = idesc0 | ((uint32_t)((int)args.N % kTallBN >> 3) << 17);
+      const uint32_t s0 = smem_u32(smem) >> 4;
+      const uint64_t a_proto = smem_desc(0, 16, 1024, kSwizzle128B), m_proto = smem_desc(0, 128, 128, kSwizzleNone);
+      const uint64_t b_proto = kBMN ? smem_desc(0, 16384, 1024, kSwizzle128B) : smem_desc(0, 16, 1024, kSwizzle128B);
+      const uint32_t a_hi = (uint32_t)(a_proto >> 32), b_hi = (uint32_t)(b_proto >> 32), m_hi = (uint32_t)(m_proto >> 32);
+      const int nfull = args.num_m_tiles * args.num_n_tiles;
+      uint32_t stage = 0, phase = 0, acc_phase0 = 1, acc_phase1 = 1;
+      bool ok = true;
+      for (int l = 0, tile; ok && (tile = tall_nth(args, l, pair, num_pairs)) >= 0; ++l) {
+        const int halves = tall_tile(args, tile).halves;
+        const uint32_t idesc = tile < nfull ? idesc_wide : idesc_narrow;
+        if (!mbar_wait(&ctl->tmem_empty[0], acc_phase0, abort_flag)) { ok = false; break; }
+        for (int kb = 0; kb < nkb; ++kb) {
+          if (!mbar_wait(&ctl->full[stage], phase, abort_flag)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t at = s0 + stage * (uint32_t)(kStageBytes >> 4), b_lo = (uint32_t)b_proto + at;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (h >= halves) break;
+            if (h == 1 && kb == 0) {
+              if (!mbar_wait(&ctl->tmem_empty[1], acc_phase1, abort_flag)) { ok = false; break; }
+              tc_fence_after();
+            }
+            const uint32_t a_lo = (uint32_t)a_proto + at + (uint32_t)((kBBytes + h * 16384) >> 4);
+            const uint32_t m_lo = (uint32_t)m_proto + at + (uint32_t)((kMetaAt + h * kMetaBytes) >> 4);
+            const uint32_t mbuf = tmem_base + kMetaCol + kMetaCols * (uint32_t)(2 * (kb & 1) + h);   // metadata double buffer
+            tmem_cp_128x128b_2cta(mbuf, desc64(m_lo, m_hi));
+            if (kFp8) tmem_cp_128x128b_2cta(mbuf + 4u, desc64(m_lo + (2048u >> 4), m_hi));
+            const uint32_t tmem_d = tmem_base + (uint32_t)(h * kTallBN);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const uint32_t accum = (kb > 0 || k > 0) ? 1u : 0u;
+              // K = 32 per instruction: 32 B of stored A, 64 B of B inside a 64-wide K slab, or 32 k rows of 128 B
+              const uint32_t bk = kBMN ? (uint32_t)k * (4096 >> 4) : (uint32_t)((k >> 1) * (kSlab >> 4) + (k & 1) * (64 >> 4));
+              if (kFp8)      // 64 logical K per instruction: two metadata columns each
+                mma_sp_f8_2cta(tmem_d, desc64(a_lo + k * 2, a_hi), desc64(b_lo + bk, b_hi), mbuf + 2u * (uint32_t)k, idesc, accum);
+              else
+                mma_sp_f16_2cta(tmem_d, desc64(a_lo + k * 2, a_hi), desc64(b_lo + bk, b_hi), mbuf + (uint32_t)(k & ~1),
+                                idesc | (uint32_t)(k & 1), accum);
+            }
+            if (h == 0 && kb == nkb - 1) mma_commit_2cta(&ctl->tmem_full[0]);
+          }
+          if (!ok) break;
+          mma_commit_2cta(&ctl->empty[stage]);             // frees the stage in both CTAs
+          if (++stage == kTallStages) { stage = 0; phase ^= 1; }
+        }
+        if (!ok) break;
+        acc_phase0 ^= 1;
+        if (halves == 2) {
+          mma_commit_2cta(&ctl->tmem_full[1]);
+          acc_phase1 ^= 1;
+        }
+      }
+    }
+  } else {
+    // =========================== epilogue (warps 2..9, both CTAs): a set of four warps per half ===========================
+    const int q = warp & 3, h = (warp - 2) >> 2;
+    uint8_t* wsm = epi_stage + (h * 4 + q) * (tall_epi_bytes(kEpi) / kSetWarps);
+    const uint32_t taddr = tmem_base + (uint32_t)(h * kTallBN) + ((uint32_t)(q * 32) << 16);
+    uint32_t phase = 0;
+    for (int l = 0, tile; (tile = tall_nth(args, l, pair, num_pairs)) >= 0; ++l) {
+      const TallTile t = tall_tile(args, tile);
+      if (h >= t.halves) continue;
+      const int64_t m0 = (int64_t)t.m0 + h * 256 + (int64_t)rank * 128, n0 = t.n0, n_limit = t.n0 + t.width;
+      // M % 256 == 128: the second CTA of the last half holds no rows; it only hands the accumulator back
+      const bool live = m0 < args.M;
+      if constexpr (is_drelu_t(kEpi)) {
+        if (!epi_drelu_tile<kEpi, kTallBN>(args, taddr, m0, n0, n_limit, live, q, lane, reinterpret_cast<float*>(wsm),
+                                           ctl->expand_lut, &ctl->tmem_full[h], phase, abort_flag, &ctl->tmem_empty[h]))
+          break;
+      } else {
+        if (!mbar_wait(&ctl->tmem_full[h], phase, abort_flag)) break;
+        tc_fence_after();
+        if (live) epi_tile<kEpi, kTallBN>(args, taddr, m0, n0, n_limit, q, lane, wsm);
+        release_accumulator(lane, &ctl->tmem_empty[h]);
+      }
+      phase ^= 1;
+    }
+  }
+
+  // =========================== teardown ===========================
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && ctl->abort_flag) atomicExch(args.status, 1);
+  cluster_sync_all();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc_2cta(tmem_base, kTmemCols);
+  }
+}
+
 // ---- host side -----------------------------------------------------------------------------------
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -1328,6 +1568,68 @@ int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
 #endif
 constexpr int kNarrowBN = SF_NARROW_BN;
 
+template <bool kBMN, int kEpi, bool kFp8 = false>
+int launch_tall(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tbn, const CUtensorMap& tm, GemmArgs a,
+                cudaStream_t s) {
+  auto kern = gemm_tall_kernel<kBMN, kEpi, kFp8>;
+  constexpr int smem = tall_smem(kEpi, kBMN, kFp8);
+  static_assert(smem <= 232448, "shared memory per CTA");
+  static bool attr_done[64] = {false};
+  int dev = 0;
+  SF_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64 || !attr_done[dev]) {
+    SF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    if (dev >= 0 && dev < 64) attr_done[dev] = true;
+  }
+  a.num_m_tiles = (int)((a.M + 511) / 512);
+  a.num_n_tiles = (int)(a.N / kTallBN);                                       // full-width columns
+  const int tiles = a.num_m_tiles * (a.num_n_tiles + (a.N % kTallBN ? 1 : 0)), max_pairs = sm_count() / 2;
+  return launch_pdl(kern, dim3(2 * (tiles < max_pairs ? tiles : max_pairs)), kTallThreads, smem, s, ta, tb, tbn, tm, a);
+}
+
+// Tensor maps of a tall product, lengths in 2-byte words (8-bit operands: two codes): vals [M, kw / 2] packed A, B [N, kw]
+// K-major or [kw, N] MN-major. kind: 0 bf16, 2 words; meta_rows: 1 KB metadata rows per 128 operand rows and stage.
+int tall_maps(const void* vals, const void* meta_hw, const void* B, bool b_kmajor, int64_t M, int64_t N, int64_t kw,
+              int kind, int meta_rows, CUtensorMap* ta, CUtensorMap* tb, CUtensorMap* tbn, CUtensorMap* tm) {
+  int st = make_tmap(ta, vals, M, kw / 2, kw / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, kind);
+  if (st == SF_OK)
+    st = b_kmajor ? make_tmap(tb, B, N, kw, kw, 64, kTallBN / 2, CU_TENSOR_MAP_SWIZZLE_128B, kind)
+                  : make_tmap(tb, B, kw, N, N, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, kind);
+  *tbn = *tb;
+  if (st == SF_OK && b_kmajor && N % kTallBN)
+    st = make_tmap(tbn, B, N, kw, kw, 64, (uint32_t)(N % kTallBN / 2), CU_TENSOR_MAP_SWIZZLE_128B, kind);
+  if (st == SF_OK)
+    st = make_tmap(tm, meta_hw, meta_rows * (M / 128) * (kw / 128), 256, 256, 256, (uint32_t)meta_rows, CU_TENSOR_MAP_SWIZZLE_NONE, 1);
+  return st;
+}
+
+// 512 x 224 tiles, or 256-row tiles of `bn` columns (bn = 256: one accumulator, its epilogue exposed)? Estimated clocks
+// of the busiest CTA pair: rounds of tiles x (k-stages x clocks per stage + the epilogue that nothing hides). A stage's
+// clocks measured with clock stamps on all SMs: 735 (256 wide), 680 (224 wide), 1190 (512 x 224). A narrow tile of the
+// last column takes nearly as long as a full one (three stages do not cover the load latency when there is so little
+// to multiply: 64 columns 95 us against 97 at K = 16384), which is why 8192 x 4096 stays on 256-row tiles (434 us
+// against 482 at K = 16384) while 16384 x 8192 does not.
+bool use_tall(int64_t M, int64_t N, int64_t stages, int bn, double flat_epi, double tall_epi) {
+  if (M < 512) return false;
+  const int64_t P = sm_count() / 2;
+  const int64_t flat_tiles = ((M + 255) / 256) * ((N + bn - 1) / bn);
+  const double flat = (double)((flat_tiles + P - 1) / P) * (stages * (bn == 256 ? 735.0 : 680.0) + flat_epi);
+  const int64_t nm = (M + 511) / 512, nfull = nm * (N / kTallBN), nn = N % kTallBN ? nm : 0, q = nfull / P, r = nfull % P, spare = P - r;
+  const double full = stages * 1190.0 + tall_epi, narrow = 0.95 * full, last = r ? full : 0.0;
+  double rest = last;
+  if (nn) {
+    if (r && nn <= 2 * spare) {
+      const double on_spare = (double)((nn + spare - 1) / spare) * narrow;
+      rest = on_spare > last ? on_spare : last;
+    } else {
+      const int64_t over = nn > spare ? (nn - spare + P - 1) / P : 0;
+      const double a = last + over * narrow, b = (double)((nn + P - 1) / P) * narrow;
+      rest = a > b ? a : b;
+    }
+  }
+  return q * full + rest < 0.99 * flat;
+}
+
 // CTA pairs work on 256-row tiles; with M % 256 == 128 the second CTA of the last row of pairs runs on
 // zero-filled operand rows and stores nothing. A single 128-row block runs the one-CTA kernels.
 bool use_two_cta(int64_t M) { return M >= 256; }
@@ -1386,6 +1688,16 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   const bool plain = (epi == EPI_STORE);                 // row-major output, either B layout: two-CTA kernel only
   if ((plain || !b_kmajor) && !two) return SF_ERR_UNSUPPORTED;
   CUtensorMap ta, tb, tm;
+  if (two && use_tall(M, N, K / 128, plain ? BN : kNarrowBN, plain ? 2500.0 : 0.0, 2500.0)) {
+    CUtensorMap tbn;
+    const int st = tall_maps(a_vals, meta_hw, B, b_kmajor, M, N, K, 0, 2, &ta, &tb, &tbn, &tm);
+    if (st != SF_OK) return st;
+    GemmArgs a{};
+    a.M = M; a.N = N; a.K = K;
+    a.C = C; a.ldc = ldc; a.status = status;
+    if (!plain) return launch_tall<false, EPI_STORE_T>(ta, tb, tbn, tm, a, s);
+    return b_kmajor ? launch_tall<false, EPI_STORE>(ta, tb, tbn, tm, a, s) : launch_tall<true, EPI_STORE>(ta, tb, tbn, tm, a, s);
+  }
   int st = two ? make_tmap(&ta, a_vals, M, K / 2, K / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B)
                : make_tmap(&ta, a_vals, M, K / 2, K / 2, 32, 128, CU_TENSOR_MAP_SWIZZLE_64B);
   if (st != SF_OK) return st;
@@ -1431,15 +1743,22 @@ int weight_token_maps(const void* w_vals, const uint8_t* meta_hw, const void* to
 int gemm_sparse24_drelu(const void* w_vals, const uint8_t* meta_hw, const void* dY, int64_t F, int64_t T, int64_t D,
                         const ActMask& mask, void* dy1_vals, void* dy1_dense, int* status, cudaStream_t s) {
   if (F < 256 || F % 128 || T % 128 || D % 128) return SF_ERR_SHAPE;
-  CUtensorMap ta, tb, tm;
-  const int st = weight_token_maps(w_vals, meta_hw, dY, F, T, D, kNarrowBN, &ta, &tb, &tm);
-  if (st != SF_OK) return st;
   GemmArgs a{};
   a.M = F; a.N = T; a.K = D;
   a.C = dy1_dense; a.ldc = F; a.aux = mask.relu; a.pack_meta = mask.meta; a.pack_vals = dy1_vals; a.status = status;
-  if (!mask.colidx) return launch_two<MODE_SPARSE24, false, false, EPI_DRELU24_T, kNarrowBN>(ta, tb, tm, a, s);
-  a.colidx = mask.colidx; a.V = mask.V; a.Mv = mask.Mv; a.G = F / mask.Mv;
-  return launch_two<MODE_SPARSE24, false, false, EPI_DRELUV_T, kNarrowBN>(ta, tb, tm, a, s);
+  if (mask.colidx) {
+    a.colidx = mask.colidx; a.V = mask.V; a.Mv = mask.Mv; a.G = F / mask.Mv;
+  }
+  CUtensorMap ta, tb, tbn, tm;
+  if (use_tall(F, T, D / 128, kNarrowBN, 0.0, 4000.0)) {
+    const int st = tall_maps(w_vals, meta_hw, dY, true, F, T, D, 0, 2, &ta, &tb, &tbn, &tm);
+    if (st != SF_OK) return st;
+    return mask.colidx ? launch_tall<false, EPI_DRELUV_T>(ta, tb, tbn, tm, a, s) : launch_tall<false, EPI_DRELU24_T>(ta, tb, tbn, tm, a, s);
+  }
+  const int st = weight_token_maps(w_vals, meta_hw, dY, F, T, D, kNarrowBN, &ta, &tb, &tm);
+  if (st != SF_OK) return st;
+  return mask.colidx ? launch_two<MODE_SPARSE24, false, false, EPI_DRELUV_T, kNarrowBN>(ta, tb, tm, a, s)
+                     : launch_two<MODE_SPARSE24, false, false, EPI_DRELU24_T, kNarrowBN>(ta, tb, tm, a, s);
 }
 
 int gemm_sparse24_act4(const void* w_vals, const uint8_t* meta_hw, const void* X, int64_t F, int64_t T, int64_t D, int V,
@@ -1480,6 +1799,15 @@ int gemm_fp8(bool sparse, const void* A, const uint8_t* meta_hw, const void* B, 
   // the operands in 2-byte units: [M, K/2] (dense) or [M, K/4] (2:4 values), [N, K/2]
   const int64_t K2 = K / 2;
   CUtensorMap ta, tb, tm;
+  if (sparse && use_tall(M, N, K / 256, BN, 2500.0, 2500.0)) {
+    CUtensorMap tbn;
+    const int st = tall_maps(A, meta_hw, B, true, M, N, K2, 2, 4, &ta, &tb, &tbn, &tm);
+    if (st != SF_OK) return st;
+    GemmArgs a{};
+    a.M = M; a.N = N; a.K = K2;
+    a.C = C; a.ldc = ldc; a.status = status; a.out_scale = alpha;
+    return launch_tall<false, EPI_STORE, true>(ta, tb, tbn, tm, a, s);
+  }
   int st = sparse ? make_tmap(&ta, A, M, K2 / 2, K2 / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2)
                   : make_tmap(&ta, A, M, K2, K2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2);
   if (st != SF_OK) return st;

@@ -70,6 +70,35 @@ def test_sparse24_gemm_row_major_output(b_k, Mr, Nc, K):
     assert_close_elementwise(f32(C), _f64(p.dense) @ Bf.T, K, "2:4 product, row-major output")
 
 
+def _integer_24_product(Mr, Nc, K, b_k, run):
+    """Small integers: every partial sum is exact in float32, so only the bf16 rounding of the result is left."""
+    rng = np.random.default_rng(Mr + Nc)
+    W = rng.integers(-3, 4, size=(Mr, K)).astype(np.float32)
+    B = rng.integers(-3, 4, size=(Nc, K)).astype(np.float32)
+    p = oracle.prune24(synth.f32_to_bf16_bits(W), group_dim=1, mode=0)
+    meta = torch.from_numpy(p.meta.view(np.int16)).cuda()
+    C, ws = run(to_dev(p.vals), meta, to_dev(synth.f32_to_bf16_bits(B if b_k else np.ascontiguousarray(B.T))))
+    assert binding.sf_check_status(ws) == binding.SF_OK
+    return bits(C), synth.f32_to_bf16_bits(oracle.bf16_to_f32(p.dense) @ B.T)
+
+
+@pytest.mark.parametrize("b_k", [True, False])
+@pytest.mark.parametrize("Mr,Nc,K", [(8192, 8192, 512),    # 512-row tiles, a narrow last column of 128
+                                     (8448, 4352, 512),    # the same, last tile row half empty, narrow column of 96
+                                     (8192, 7168, 384),    # whole columns only
+                                     (512, 256, 1024)])    # fewer tiles than CTA pairs
+def test_sparse24_gemm_tile_shapes(b_k, Mr, Nc, K):
+    got, ref = _integer_24_product(Mr, Nc, K, b_k, lambda v, m, b: binding.sf_gemm_sparse24_rm(v, m, b, b_k))
+    assert np.array_equal(got, ref)
+
+
+@pytest.mark.parametrize("Mr,Nc,K", [(37632, 256, 128),    # more narrow tiles than two per idle pair: round robin
+                                     (256, 7680, 128), (8576, 4864, 512)])
+def test_sparse24_gemm_tile_shapes_transposed_output(Mr, Nc, K):
+    got, ref = _integer_24_product(Mr, Nc, K, True, binding.sf_gemm_sparse24)
+    assert np.array_equal(got, np.ascontiguousarray(ref.T))
+
+
 def test_sparse24_gemm_one_hot_metadata_probe():
     """Each kept value is a distinct power of two in an otherwise zero row and B is an identity
     slice, so the output says which K position every stored value was multiplied with."""
