@@ -907,7 +907,7 @@ struct SmemCtl2 {
 };
 
 // The tile a CTA pair works on: from the regular raster, or from a device-built table (grouped products).
-template <int kBN>
+template <int kBN, bool kVar>
 __device__ __forceinline__ GemmTile get_tile(const GemmArgs& args, int tile, int num_m, int num_n, int nkb_full) {
   if (args.tile_table) {
     const int4* p = reinterpret_cast<const int4*>(args.tile_table + tile);
@@ -916,7 +916,8 @@ __device__ __forceinline__ GemmTile get_tile(const GemmArgs& args, int tile, int
   }
   int mt, nt;
   tile_coords(tile, num_m, num_n, mt, nt);
-  return GemmTile{mt * 256, 0, nt * kBN, 0, nkb_full, mt * 256, nt * kBN, (int)args.N};
+  const int n0 = nt * (kVar ? args.bn : kBN);
+  return GemmTile{mt * 256, 0, n0, 0, nkb_full, mt * 256, n0, kVar ? min((int)args.N, n0 + args.bn) : (int)args.N};
 }
 
 __device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) {
@@ -929,7 +930,11 @@ __device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) {
 // kFp8: E4M3 operands (both K-major). The kernel is unchanged in bytes: K, k-block counts and operand
 // coordinates are given in 2-byte units (two codes each); only the instruction kind, the descriptor's formats
 // and the amount of metadata per stage differ.
-template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false>
+// kVar: the tile is args.bn (a multiple of 32, at most kBN) columns wide. Where there are few tiles, narrower ones put
+// more SMs to work and shorten what one of them does: the eight kernels of a step at T 1024, D 256, F 1024 take 50 us
+// instead of 61 (graph replay). A kernel of its own, because the run-time width costs the issuing threads instructions
+// that the large products do not have (dense, 256 wide: 1.5 % and more).
+template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kMode, kEpi, kExpand), 1)
 gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB,
                 const __grid_constant__ CUtensorMap tmapMeta, const __grid_constant__ CUtensorMap tmapPk,
@@ -964,6 +969,9 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   const uint32_t rank = cluster_ctarank();               // 0 = leader
   const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
   const int num_m_tiles = args.num_m_tiles, num_n_tiles_ = args.num_n_tiles;   // 256-row tiles
+  const int half_n = kVar ? args.bn / 2 : kBN / 2;       // this CTA's columns of B
+  const int b_chunks = (half_n + 63) >> 6;               // MN-major B: chunks of 64 columns
+  const uint32_t b_bytes = kBMN ? (uint32_t)(b_chunks * (kSparse ? 16384 : 8192)) : (uint32_t)(half_n * (kSparse ? 256 : 128));
   const int nkb_full = (int)(args.K / kBK);
 
   if (threadIdx.x == 0) {
@@ -1006,9 +1014,9 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     uint32_t stage = 0, phase = 0;
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
-      const GemmTile tc = get_tile<kBN>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
+      const GemmTile tc = get_tile<kBN, kVar>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
       const int m0 = tc.a_row + (int)rank * 128;         // this CTA's rows of A / D
-      const int nb0 = tc.b_row + (int)rank * (kBN / 2);  // this CTA's columns of B
+      const int nb0 = tc.b_row + (int)rank * half_n;
       const int nkb = tc.nkb, ak0 = tc.a_k0, bk0 = tc.b_k0;
       for (int kb = 0; kb < nkb; ++kb) {
         if (!mbar_wait(&ctl->empty[stage], phase ^ 1, abort_flag)) { ok = false; break; }
@@ -1021,7 +1029,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
             // the leader's barrier collects the bytes of both CTAs (an expanded operand arrives by
             // shared-memory stores, not by TMA)
             mbar_arrive_expect_tx(bar, 2u * ((kExpand == 1 ? 0u : (uint32_t)kAStageBytes) +
-                                             (kExpand == 2 ? 0u : (uint32_t)kBHalfBytes) +
+                                             (kExpand == 2 ? 0u : b_bytes) +
                                              (kSparse ? (uint32_t)kMetaBytes : 0u)));
           }
           if (kMode == MODE_DENSE) {
@@ -1038,7 +1046,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
               tma_load_2d_2cta(sB, &tmapB, bar, bk0 + kb * 64, nb0);           // box {64 k, 128 n}
             } else {
               tma_load_2d_2cta(sB, &tmapB, bar, nb0, bk0 + kb * 64);           // box {64 n, 64 k}
-              tma_load_2d_2cta(sB + 8192, &tmapB, bar, nb0 + 64, bk0 + kb * 64);
+              if (!kVar || b_chunks == 2) tma_load_2d_2cta(sB + 8192, &tmapB, bar, nb0 + 64, bk0 + kb * 64);
             }
             if (kExpand) {
               const int f0 = kExpand == 1 ? m0 : nb0;                          // first feature of this CTA's half
@@ -1058,7 +1066,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
               tma_load_2d_2cta(sB + kBSlabBytes, &tmapB, bar, bk0 + kb * 128 + 64, nb0);
             } else {
               tma_load_2d_2cta(sB, &tmapB, bar, nb0, bk0 + kb * 128);          // two chunks {64 n, 128 k}
-              tma_load_2d_2cta(sB + 16384, &tmapB, bar, nb0 + 64, bk0 + kb * 128);
+              if (!kVar || b_chunks == 2) tma_load_2d_2cta(sB + 16384, &tmapB, bar, nb0 + 64, bk0 + kb * 128);
             }
           }
         }
@@ -1068,7 +1076,8 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   } else if (warp == 1) {
     // =========================== MMA issuer (leader CTA only) ===========================
     if (rank == 0 && lane == 0) {
-      constexpr uint32_t idesc = kFp8 ? idesc_e4m3(256, kBN, kSparse) : idesc_bf16(256, kBN, kAMN, kBMN, kSparse);
+      constexpr uint32_t idesc_full = kFp8 ? idesc_e4m3(256, kBN, kSparse) : idesc_bf16(256, kBN, kAMN, kBMN, kSparse);
+      const uint32_t idesc = kVar ? idesc_full - ((uint32_t)(kBN - args.bn) >> 3 << 17) : idesc_full;
       // Descriptor halves that never change: high word = stride offset, version, swizzle; the low
       // word is (address >> 4) | leading offset, advanced by plain 32-bit adds.
       const uint32_t smem0 = smem_u32(smem);
@@ -1173,7 +1182,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     const uint32_t taddr = tmem_base + set * kBN + ((uint32_t)(q * 32) << 16);
     uint32_t acc_phase = 0;
     for (int tile = pair + set * num_pairs; tile < num_tiles; tile += 2 * num_pairs) {
-      const GemmTile tc = get_tile<kBN>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
+      const GemmTile tc = get_tile<kBN, kVar>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
       const int64_t m0 = (int64_t)tc.out_m + (int64_t)rank * 128, n0 = tc.out_n, n_limit = tc.n_limit;
       // M % 256 == 128 (regular raster only): the second CTA of the last row of pairs holds no rows (its operand
       // loads were zero-filled); it only hands the accumulator back
@@ -1204,7 +1213,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     uint32_t acc = 0, acc_phase = 0;
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
-      const GemmTile tc = get_tile<kBN>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
+      const GemmTile tc = get_tile<kBN, kVar>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
       const int64_t m0 = (int64_t)tc.out_m + (int64_t)rank * 128, n0 = tc.out_n, n_limit = tc.n_limit;
       const uint32_t taddr = tmem_base + acc * kBN + ((uint32_t)(q * 32) << 16);
       // M % 256 == 128 (regular raster only): the second CTA of the last row of pairs holds no rows
@@ -1538,10 +1547,10 @@ int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const GemmArgs& a, 
                     ta, tb, a);
 }
 
-template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false>
+template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false>
 int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tm, GemmArgs a, cudaStream_t s,
                const CUtensorMap* tpk = nullptr) {
-  auto kern = gemm_tc2_kernel<kMode, kAMN, kBMN, kEpi, kBN, kExpand, kFp8>;
+  auto kern = gemm_tc2_kernel<kMode, kAMN, kBMN, kEpi, kBN, kExpand, kFp8, kVar>;
   constexpr int smem = smem_bytes2(kMode != MODE_DENSE, kBN, kEpi, kExpand != 0, kFp8);
   static_assert(smem <= 232448, "shared memory per CTA");
   static bool attr_done[64] = {false};
@@ -1552,7 +1561,8 @@ int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
     if (dev >= 0 && dev < 64) attr_done[dev] = true;
   }
   a.num_m_tiles = (int)((a.M + 255) / 256);
-  a.num_n_tiles = (int)((a.N + kBN - 1) / kBN);
+  const int bn = kVar ? a.bn : kBN;
+  a.num_n_tiles = (int)((a.N + bn - 1) / bn);
   // table-driven products: the table's length is on the device; launch for its upper bound
   const int tiles = a.tile_table ? a.num_k_blocks /* upper bound, see the grouped launchers */
                                  : a.num_m_tiles * a.num_n_tiles;
@@ -1603,6 +1613,27 @@ int tall_maps(const void* vals, const void* meta_hw, const void* B, bool b_kmajo
   return st;
 }
 
+// Tile width of a product on 256-row tiles: max_bn, or a narrower one where that ends sooner by the estimate: rounds of
+// tiles over the CTA pairs x (k-stages x clocks per stage + epilogue). A stage's clocks are its shared-memory traffic
+// (2:4: 0.93 x (272 + 2 w), measured 735 at w = 256 and 680 at 224; dense: 256 + w) or the tensor pipe's 2 w. chunk: epilogue
+// clocks per 32 columns; exposed: nothing hides the epilogue of a tile (one accumulator), else only the last one counts.
+// A narrower width has to gain 10 %: its kernel takes the width at run time (at 6 % the weight gradients of D 2048 took 224
+// columns, 0.94 by the estimate, and 1.02 of the time).
+int best_width(int64_t M, int64_t N, int64_t stages, bool sparse, int max_bn, int step, double chunk, bool exposed) {
+  const int64_t P = sm_count() / 2, nm = (M + 255) / 256;
+  auto cost = [&](int w) {
+    const int64_t tiles = nm * ((N + w - 1) / w);
+    const double smem = sparse ? 0.93 * (272 + 2 * w) : 256.0 + w, main = stages * (smem > 2.0 * w ? smem : 2.0 * w);
+    const double rounds = (double)((tiles + P - 1) / P), epi = chunk * (w / 32);
+    return exposed ? rounds * (main + epi) : rounds * (main > epi ? main : epi) + epi;
+  };
+  int best = max_bn;
+  double least = 0.90 * cost(max_bn);
+  for (int w = max_bn - step; w >= step; w -= step)
+    if (cost(w) < least) { least = cost(w); best = w; }
+  return best;
+}
+
 // 512 x 224 tiles, or 256-row tiles of `bn` columns (bn = 256: one accumulator, its epilogue exposed)? Estimated clocks
 // of the busiest CTA pair: rounds of tiles x (k-stages x clocks per stage + the epilogue that nothing hides). A stage's
 // clocks measured with clock stamps on all SMs: 735 (256 wide), 680 (224 wide), 1190 (512 x 224). A narrow tile of the
@@ -1646,6 +1677,7 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
                void* C, int64_t ldc, void* C2, int64_t ldc2, const void* aux, int64_t ldaux, int* status,
                cudaStream_t s) {
   const bool two = use_two_cta(M);
+  const int bn = two ? best_width(M, N, K / 64, false, BN, 32, epi == EPI_STORE ? 200.0 : 400.0, false) : BN;
   if (M % BM || N % (two ? 128 : BN) || K % 64) return SF_ERR_SHAPE;     // pairs: a ragged last tile of whole 32-column chunks
   if (M == 0 || N == 0) return SF_OK;
   CUtensorMap ta, tb;
@@ -1653,7 +1685,7 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
   if (a_kmajor) st = make_tmap(&ta, A, M, K, K, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B);
   else          st = make_tmap(&ta, A, K, M, M, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st != SF_OK) return st;
-  if (b_kmajor) st = make_tmap(&tb, B, N, K, K, 64, two ? 128 : 256, CU_TENSOR_MAP_SWIZZLE_128B);
+  if (b_kmajor) st = make_tmap(&tb, B, N, K, K, 64, two ? bn / 2 : 256, CU_TENSOR_MAP_SWIZZLE_128B);
   else          st = make_tmap(&tb, B, K, N, N, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st != SF_OK) return st;
   GemmArgs a{};
@@ -1661,9 +1693,11 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
   a.C = C; a.ldc = ldc; a.C2 = C2; a.ldc2 = ldc2; a.aux = aux; a.ldaux = ldaux;
   a.status = status;
   a.num_m_tiles = (int)(M / BM); a.num_n_tiles = (int)(N / BN); a.num_k_blocks = (int)(K / 64);
-#define SF_DENSE_CASE(AMN, BMN, EPI)                                              \
-  return two ? launch_two<MODE_DENSE, AMN, BMN, EPI>(ta, tb, ta, a, s)            \
-             : launch_one<MODE_DENSE, AMN, BMN, EPI>(ta, tb, a, s)
+  a.bn = bn;
+#define SF_DENSE_CASE(AMN, BMN, EPI)                                                                \
+  return !two       ? launch_one<MODE_DENSE, AMN, BMN, EPI>(ta, tb, a, s)                             \
+         : bn == BN ? launch_two<MODE_DENSE, AMN, BMN, EPI>(ta, tb, ta, a, s)                         \
+                    : launch_two<MODE_DENSE, AMN, BMN, EPI, BN, 0, false, true>(ta, tb, ta, a, s)
   const bool amn = !a_kmajor, bmn = !b_kmajor;
   if (epi == EPI_STORE) {
     if (!amn && !bmn) SF_DENSE_CASE(false, false, EPI_STORE);
@@ -1702,8 +1736,9 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
                : make_tmap(&ta, a_vals, M, K / 2, K / 2, 32, 128, CU_TENSOR_MAP_SWIZZLE_64B);
   if (st != SF_OK) return st;
   // transposed-output products on CTA pairs run 224-column tiles with two accumulators
-  const bool narrow = two && !plain;
-  if (b_kmajor) st = make_tmap(&tb, B, N, K, K, 64, two ? (narrow ? kNarrowBN / 2 : 128) : 256, CU_TENSOR_MAP_SWIZZLE_128B);
+  const int max_bn = plain ? BN : kNarrowBN;
+  const int bn = two ? best_width(M, N, K / 128, true, max_bn, 32, 400.0, plain) : BN;
+  if (b_kmajor) st = make_tmap(&tb, B, N, K, K, 64, two ? bn / 2 : 256, CU_TENSOR_MAP_SWIZZLE_128B);
   else          st = make_tmap(&tb, B, K, N, N, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st != SF_OK) return st;
   tm = ta;
@@ -1717,13 +1752,18 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   a.M = M; a.N = N; a.K = K;
   a.C = C; a.ldc = ldc; a.meta_hw = meta_hw; a.status = status;
   a.num_m_tiles = (int)(M / BM); a.num_n_tiles = (int)(N / BN); a.num_k_blocks = (int)(K / 64);
+  a.bn = bn;
+  const bool var = two && bn != max_bn;
   if (epi == EPI_STORE) {
-    if (b_kmajor) return launch_two<MODE_SPARSE24, false, false, EPI_STORE>(ta, tb, tm, a, s);
-    return launch_two<MODE_SPARSE24, false, true, EPI_STORE>(ta, tb, tm, a, s);
+    if (b_kmajor) return var ? launch_two<MODE_SPARSE24, false, false, EPI_STORE, BN, 0, false, true>(ta, tb, tm, a, s)
+                             : launch_two<MODE_SPARSE24, false, false, EPI_STORE>(ta, tb, tm, a, s);
+    return var ? launch_two<MODE_SPARSE24, false, true, EPI_STORE, BN, 0, false, true>(ta, tb, tm, a, s)
+               : launch_two<MODE_SPARSE24, false, true, EPI_STORE>(ta, tb, tm, a, s);
   }
   if (epi == EPI_STORE_T)
-    return two ? launch_two<MODE_SPARSE24, false, false, EPI_STORE_T, kNarrowBN>(ta, tb, tm, a, s)
-               : launch_one<MODE_SPARSE24, false, false, EPI_STORE_T>(ta, tb, a, s);
+    return !two ? launch_one<MODE_SPARSE24, false, false, EPI_STORE_T>(ta, tb, a, s)
+           : var ? launch_two<MODE_SPARSE24, false, false, EPI_STORE_T, kNarrowBN, 0, false, true>(ta, tb, tm, a, s)
+                 : launch_two<MODE_SPARSE24, false, false, EPI_STORE_T, kNarrowBN>(ta, tb, tm, a, s);
   return SF_ERR_UNSUPPORTED;
 }
 
@@ -1755,8 +1795,12 @@ int gemm_sparse24_drelu(const void* w_vals, const uint8_t* meta_hw, const void* 
     if (st != SF_OK) return st;
     return mask.colidx ? launch_tall<false, EPI_DRELUV_T>(ta, tb, tbn, tm, a, s) : launch_tall<false, EPI_DRELU24_T>(ta, tb, tbn, tm, a, s);
   }
-  const int st = weight_token_maps(w_vals, meta_hw, dY, F, T, D, kNarrowBN, &ta, &tb, &tm);
+  a.bn = best_width(F, T, D / 128, true, kNarrowBN, 32, 500.0, false);
+  const int st = weight_token_maps(w_vals, meta_hw, dY, F, T, D, a.bn, &ta, &tb, &tm);
   if (st != SF_OK) return st;
+  if (a.bn != kNarrowBN)
+    return mask.colidx ? launch_two<MODE_SPARSE24, false, false, EPI_DRELUV_T, kNarrowBN, 0, false, true>(ta, tb, tm, a, s)
+                       : launch_two<MODE_SPARSE24, false, false, EPI_DRELU24_T, kNarrowBN, 0, false, true>(ta, tb, tm, a, s);
   return mask.colidx ? launch_two<MODE_SPARSE24, false, false, EPI_DRELUV_T, kNarrowBN>(ta, tb, tm, a, s)
                      : launch_two<MODE_SPARSE24, false, false, EPI_DRELU24_T, kNarrowBN>(ta, tb, tm, a, s);
 }
@@ -1764,15 +1808,17 @@ int gemm_sparse24_drelu(const void* w_vals, const uint8_t* meta_hw, const void* 
 int gemm_sparse24_act4(const void* w_vals, const uint8_t* meta_hw, const void* X, int64_t F, int64_t T, int64_t D, int V,
                        const Act24Out& out, void* colidx, int* status, cudaStream_t s) {
   if (F < 256 || F % 128 || T % 128 || D % 128) return SF_ERR_SHAPE;
-  CUtensorMap ta, tb, tm;
-  const int st = weight_token_maps(w_vals, meta_hw, X, F, T, D, kNarrowBN, &ta, &tb, &tm);
-  if (st != SF_OK) return st;
   GemmArgs a{};
+  a.bn = best_width(F, T, D / 128, true, kNarrowBN, 32, 500.0, false);
+  CUtensorMap ta, tb, tm;
+  const int st = weight_token_maps(w_vals, meta_hw, X, F, T, D, a.bn, &ta, &tb, &tm);
+  if (st != SF_OK) return st;
   a.M = F; a.N = T; a.K = D; a.V = V;
   a.status = status;
   a.vn_vals24 = out.vals; a.vn_relu24 = out.relu; a.vn_meta24 = out.meta; a.vn_meta24_hw = out.meta_hw;
   a.vn_dense = out.dense; a.vn_y1 = out.y1; a.vn_colidx = colidx;
-  return launch_two<MODE_SPARSE24, false, false, EPI_ACT24_T, kNarrowBN>(ta, tb, tm, a, s);
+  return a.bn == kNarrowBN ? launch_two<MODE_SPARSE24, false, false, EPI_ACT24_T, kNarrowBN>(ta, tb, tm, a, s)
+                           : launch_two<MODE_SPARSE24, false, false, EPI_ACT24_T, kNarrowBN, 0, false, true>(ta, tb, tm, a, s);
 }
 
 int gemm_route(const void* X, const void* means, int64_t T, int64_t D, int E, int* expert, float* logits, int* status,
@@ -1811,7 +1857,8 @@ int gemm_fp8(bool sparse, const void* A, const uint8_t* meta_hw, const void* B, 
   int st = sparse ? make_tmap(&ta, A, M, K2 / 2, K2 / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2)
                   : make_tmap(&ta, A, M, K2, K2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2);
   if (st != SF_OK) return st;
-  st = make_tmap(&tb, B, N, K2, K2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2);
+  const int bn = best_width(M, N, K2 / (sparse ? 128 : 64), sparse, BN, 32, sparse ? 400.0 : 200.0, sparse);
+  st = make_tmap(&tb, B, N, K2, K2, 64, bn / 2, CU_TENSOR_MAP_SWIZZLE_128B, 2);
   if (st != SF_OK) return st;
   tm = ta;
   if (sparse) {
@@ -1824,8 +1871,12 @@ int gemm_fp8(bool sparse, const void* A, const uint8_t* meta_hw, const void* B, 
   a.M = M; a.N = N; a.K = K2;
   a.C = C; a.ldc = ldc; a.meta_hw = meta_hw; a.status = status; a.out_scale = alpha;
   a.num_k_blocks = (int)(K2 / 64);
-  if (sparse) return launch_two<MODE_SPARSE24, false, false, EPI_STORE, BN, 0, true>(ta, tb, tm, a, s);
-  return launch_two<MODE_DENSE, false, false, EPI_STORE, BN, 0, true>(ta, tb, tm, a, s);
+  a.bn = bn;
+  if (bn != BN)
+    return sparse ? launch_two<MODE_SPARSE24, false, false, EPI_STORE, BN, 0, true, true>(ta, tb, tm, a, s)
+                  : launch_two<MODE_DENSE, false, false, EPI_STORE, BN, 0, true, true>(ta, tb, tm, a, s);
+  return sparse ? launch_two<MODE_SPARSE24, false, false, EPI_STORE, BN, 0, true>(ta, tb, tm, a, s)
+                : launch_two<MODE_DENSE, false, false, EPI_STORE, BN, 0, true>(ta, tb, tm, a, s);
 }
 
 bool gemm_sparse24_vnm8_supported(int64_t F, int64_t T, int64_t D, int V) {
@@ -1835,18 +1886,20 @@ bool gemm_sparse24_vnm8_supported(int64_t F, int64_t T, int64_t D, int V) {
 int gemm_sparse24_vnm8(const void* a_vals, const uint8_t* meta_hw, const void* X, int64_t F, int64_t T, int64_t D,
                        int V, const Vnm8Out& out, int* status, cudaStream_t s) {
   if (!gemm_sparse24_vnm8_supported(F, T, D, V)) return SF_ERR_SHAPE;
-  // Token tiles hold whole V-blocks: three blocks of 64 (192 columns) or one block of 128.
-  const int bn = V == 64 ? 192 : 128;
-  CUtensorMap ta, tb, tm;
-  const int st = weight_token_maps(a_vals, meta_hw, X, F, T, D, bn, &ta, &tb, &tm);
-  if (st != SF_OK) return st;
+  // Token tiles hold whole V-blocks: up to three blocks of 64 (192 columns) or one block of 128.
   GemmArgs a{};
+  a.bn = V == 64 ? best_width(F, T, D / 128, true, 192, 64, 1500.0, false) : 128;
+  CUtensorMap ta, tb, tm;
+  const int st = weight_token_maps(a_vals, meta_hw, X, F, T, D, a.bn, &ta, &tb, &tm);
+  if (st != SF_OK) return st;
   a.M = F; a.N = T; a.K = D; a.V = V;
   a.meta_hw = meta_hw; a.status = status;
   a.vn_vals = out.vals; a.vn_relu = out.relu; a.vn_meta = out.meta; a.vn_colidx = out.colidx;
   a.vn_vals24 = out.vals24; a.vn_relu24 = out.relu24; a.vn_meta24 = out.meta24; a.vn_meta24_hw = out.meta24_hw;
   a.vn_y1 = out.y1; a.vn_dense = out.dense;
-  if (V == 64) return launch_two<MODE_SPARSE24, false, false, EPI_VNM8, 192>(ta, tb, tm, a, s);
+  if (V == 64)
+    return a.bn == 192 ? launch_two<MODE_SPARSE24, false, false, EPI_VNM8, 192>(ta, tb, tm, a, s)
+                       : launch_two<MODE_SPARSE24, false, false, EPI_VNM8, 192, 0, false, true>(ta, tb, tm, a, s);
   return launch_two<MODE_SPARSE24, false, false, EPI_VNM8, 128>(ta, tb, tm, a, s);
 }
 

@@ -49,6 +49,7 @@ struct GemmArgs {
   int V, Mv;                // Venom block height and group width
   int* status;              // device status word (set to 1 when a bounded wait expires)
   int num_m_tiles, num_n_tiles, num_k_blocks;
+  int bn;                   // CTA-pair kernels with a run-time tile width: that width
   int gather_tma_groups;    // Venom: groups (of 16 per stage) fetched by TMA row gather; the rest by cp.async
   // EPI_DRELU24_T / EPI_DRELUV_T: metadata of the activation's mask and the packed output (see ActMask)
   const void* pack_meta;
