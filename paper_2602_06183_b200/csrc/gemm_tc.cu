@@ -546,8 +546,22 @@ __device__ __forceinline__ void epi_act24_tile(const GemmArgs& args, uint32_t ta
                                                int q, int lane, uint32_t* stage, const uint2* lut, const Top2Entry* top2,
                                                uint64_t* tmem_empty_bar) {
   const int seg = lane & 3;
-  const int64_t Fe = args.M, f = m0 + q * 32 + seg * 8, kw = (m0 + q * 32) >> 4;
+  const int64_t Fe = args.M, f = m0 + q * 32 + seg * 8;
   const int nch = (int)min((int64_t)(kTileN / 32), (n_limit - n0) >> 5);
+  // Output addresses of this lane's first token; every store of the loop is a constant stride away from them. (Address
+  // arithmetic written per store, with a division by V among it, was most of this epilogue's instructions.)
+  const int64_t tok0 = n0 + (lane >> 2) * 2;
+  uint2* p_vals = reinterpret_cast<uint2*>(args.vn_vals24) + ((tok0 * Fe + f) >> 3);           // 8-byte units: F / 8 per token
+  uint2* p_relu = reinterpret_cast<uint2*>(args.vn_relu24) + ((tok0 * Fe + f) >> 3);
+  uint4* p_dense = reinterpret_cast<uint4*>(args.vn_dense) + ((tok0 * Fe + f) >> 3);
+  uint4* p_y1 = args.vn_y1 ? reinterpret_cast<uint4*>(args.vn_y1) + ((tok0 * Fe + f) >> 3) : nullptr;
+  uint32_t* p_meta = reinterpret_cast<uint32_t*>(args.vn_meta24) + ((tok0 * Fe + f) >> 5);
+  const int64_t s8 = Fe >> 3, s32 = Fe >> 5;
+  // tensor-core order: a 16-token group is 256 bytes of an atom (tiles start at multiples of 32 tokens); see meta_hw_offset
+  const int64_t kw = f >> 4;
+  uint8_t* hw0 = reinterpret_cast<uint8_t*>(args.vn_meta24_hw) + (kw >> 3) * 2048 + (kw & 1) * 128 + ((kw >> 1) & 3) * 4 +
+                 (((lane >> 2) * 2) & 7) * 16 + ((lane >> 2) >> 2) * 2;
+  const uint32_t vmask = args.vn_colidx ? (uint32_t)args.V - 1u : 0u;      // V is 64 or 128
   uint32_t v[32];
   tmem_ld_32x32b_x32(taddr, v);
 #pragma unroll 1
@@ -563,39 +577,41 @@ __device__ __forceinline__ void epi_act24_tile(const GemmArgs& args, uint32_t ta
     for (int i = 0; i < 2; ++i) {
       uint32_t y[2][4];
       pair_rows(stage + (i * 8 + (lane >> 2)) * 32 + seg * 8, lane, y[0], y[1]);
+      const uint32_t t16 = (uint32_t)n0 + (uint32_t)(ch * 32 + i * 16);    // first token of this 16-token group
+      uint8_t* hw = hw0 + (int64_t)(t16 >> 7) * (Fe >> 7) * 2048 + ((t16 >> 4) & 7u) * 256;
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        const int64_t token = n0 + ch * 32 + i * 16 + (lane >> 2) * 2 + k;
-        uint32_t rw[4], hw[4];
+        const int64_t o8 = (i * 16 + k) * s8;
+        uint32_t rw[4], hw4[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) { rw[j] = bf2_relu(y[k][j]); hw[j] = bf2_sq(rw[j]); }
+        for (int j = 0; j < 4; ++j) { rw[j] = bf2_relu(y[k][j]); hw4[j] = bf2_sq(rw[j]); }
         Top2Entry ea, eb;
-        top2of4_x2(__byte_perm(hw[0], hw[2], 0x5410u), __byte_perm(hw[0], hw[2], 0x7632u), __byte_perm(hw[1], hw[3], 0x5410u),
-                   __byte_perm(hw[1], hw[3], 0x7632u), top2, ea, eb);
-        const uint32_t pa = __byte_perm(hw[0], hw[1], ea.kept), pb = __byte_perm(hw[2], hw[3], eb.kept);
+        top2of4_x2(__byte_perm(hw4[0], hw4[2], 0x5410u), __byte_perm(hw4[0], hw4[2], 0x7632u), __byte_perm(hw4[1], hw4[3], 0x5410u),
+                   __byte_perm(hw4[1], hw4[3], 0x7632u), top2, ea, eb);
+        const uint32_t pa = __byte_perm(hw4[0], hw4[1], ea.kept), pb = __byte_perm(hw4[2], hw4[3], eb.kept);
         const uint32_t na = (ea.kept >> 16) & 15u, nb = (eb.kept >> 16) & 15u;
-        const int64_t pv = (token * (Fe >> 1) + (f >> 1)) >> 2;              // 8-byte units
-        reinterpret_cast<uint2*>(args.vn_vals24)[pv] = make_uint2(pa, pb);
-        reinterpret_cast<uint2*>(args.vn_relu24)[pv] = make_uint2(__byte_perm(rw[0], rw[1], ea.kept), __byte_perm(rw[2], rw[3], eb.kept));
+        p_vals[o8] = make_uint2(pa, pb);
+        p_relu[o8] = make_uint2(__byte_perm(rw[0], rw[1], ea.kept), __byte_perm(rw[2], rw[3], eb.kept));
         uint4 d;
         expand24_lut(lut, pa, na, d.x, d.y);
         expand24_lut(lut, pb, nb, d.z, d.w);
-        reinterpret_cast<uint4*>(args.vn_dense)[(token * Fe + f) >> 3] = d;
-        if (args.vn_y1) reinterpret_cast<uint4*>(args.vn_y1)[(token * Fe + f) >> 3] = make_uint4(y[k][0], y[k][1], y[k][2], y[k][3]);
+        p_dense[o8] = d;
+        if (p_y1) p_y1[o8] = make_uint4(y[k][0], y[k][1], y[k][2], y[k][3]);
         // metadata: one byte per lane, four neighbouring lanes hold the warp's 32 features of this token
         uint32_t mb = na | (nb << 4);
         mb |= __shfl_down_sync(0xFFFFFFFFu, mb, 1) << 8;
         const uint32_t mb32 = (mb & 0xFFFFu) | (__shfl_down_sync(0xFFFFFFFFu, mb, 2) << 16);
-        if (seg == 0) reinterpret_cast<uint32_t*>(args.vn_meta24)[(token * (Fe >> 4) + kw) >> 1] = mb32;
-        if ((seg & 1) == 0)
-          *reinterpret_cast<uint16_t*>(reinterpret_cast<uint8_t*>(args.vn_meta24_hw) + meta_hw_offset(token, kw + (seg >> 1), Fe)) =
-              (uint16_t)mb;
+        if (seg == 0) p_meta[(i * 16 + k) * s32] = mb32;
+        if ((seg & 1) == 0) *reinterpret_cast<uint16_t*>(hw + k * 16) = (uint16_t)mb;
         // V:N:M with groups of four: every block keeps columns 0..3 of its two groups here
-        if (args.vn_colidx && token % args.V == 0)
-          *reinterpret_cast<uint2*>(reinterpret_cast<uint8_t*>(args.vn_colidx) + (token / args.V) * Fe + f) =
+        const uint32_t token = t16 + (uint32_t)((lane >> 2) * 2 + k);
+        if (vmask && (token & vmask) == 0)
+          *reinterpret_cast<uint2*>(reinterpret_cast<uint8_t*>(args.vn_colidx) + (int64_t)(token >> (31 - __clz(vmask + 1u))) * Fe + f) =
               make_uint2(0x03020100u, 0x03020100u);
       }
     }
+    p_vals += 32 * s8; p_relu += 32 * s8; p_dense += 32 * s8; p_meta += 32 * s32;
+    if (p_y1) p_y1 += 32 * s8;
   }
 }
 
