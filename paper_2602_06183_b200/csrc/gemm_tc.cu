@@ -249,33 +249,54 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
 // ---- fused SquaredReLU + V:N:M selection (groups of eight) ---------------------------------------------
 // Epilogue of the y1 product: the accumulator tile is y1^T (TMEM lane = feature, column = token), so a
 // lane owns one feature column of every V x 8 block and eight neighbouring lanes own one block.
-// Per V-block of the tile, each epilogue warp (32 features = four groups):
-//   pass 1  reads its lanes' V accumulator columns, rounds them to bf16 (this is y1), parks them in
-//           shared memory as [token][feature], and accumulates the column score of Section 2.3 in
-//           float32, token by token in ascending order (the order is part of the format);
-//   rank    the eight lanes of a group exchange scores; the four best columns stay (ties to the lower
-//           column), their indices go to colidx and into per-group byte-permute selector tables;
+// A set of four warps works on a block of V tokens x the CTA's 128 features (16 groups):
+//   pass 1  a warp reads its lanes' V accumulator columns, rounds them to bf16 (this is y1), parks them in the set's
+//           shared memory as [token pair][feature], and accumulates the column score of Section 2.3 in float32,
+//           token by token in ascending order (the order is part of the format);
+//   rank    the eight lanes of a group exchange scores; the four best columns stay (ties to the lower column),
+//           their indices go to colidx and into per-group byte-permute selector tables;
 //   pass 2  one thread per (token, group) takes the group's eight values back from shared memory, applies
 //           SquaredReLU, keeps the two largest of the four kept columns and writes the packed activation,
 //           the packed ReLU values, both metadata forms and the 2:4 view.
+// In pass 2 a warp serves all 16 groups of two token pairs: its stores are whole rows of the CTA's features (64 to 256
+// contiguous bytes a token). With the warps' own 32 features it wrote 16 to 64 bytes of eight tokens, 64 lines an emit
+// against 20, and that traffic through the L1 slowed the main loop, which needs the same shared-memory cycles: y1 at T 8192,
+// D 4096, F 16384 607 -> 588 us.
 // The accumulator is released to the MMA warp as soon as the last block's pass 1 has read it.
-// Shared memory of one epilogue warp: y1 of one block as [token pair][feature] words (low half = even
-// token), then colidx, the selector table and the nibble table of the block.
-__host__ __device__ constexpr int vnm_stage_bytes(int V) { return V * 64; }
-__host__ __device__ constexpr int vnm_warp_bytes(int V) { return vnm_stage_bytes(V) + 16 + 4 * 7 * 16 + 48; }
+__host__ __device__ constexpr int vnm_stage_bytes(int V) { return V * 256; }
+__host__ __device__ constexpr int vnm_set_bytes(int V) { return vnm_stage_bytes(V) + 16 * 4 + 16 * 7 * 16 + 192; }
 constexpr int kSetWarps = 8;                                     // two sets of four: one set per accumulator buffer
-__host__ __device__ constexpr int vnm_epi_bytes(int V) { return kSetWarps * vnm_warp_bytes(V); }
+__host__ __device__ constexpr int vnm_epi_bytes(int V) { return 2 * vnm_set_bytes(V); }
+
+// Barrier of one set of four epilogue warps.
+__device__ __forceinline__ void set_sync(int set) { asm volatile("bar.sync %0, 128;" ::"r"(set + 1) : "memory"); }
+// The same with a vote: true when all four warps say so.
+__device__ __forceinline__ bool set_all(int set, bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t"
+      ".reg .pred P, Q;\n\t"
+      "setp.ne.b32 P, %1, 0;\n\t"
+      "barrier.cta.red.and.pred Q, %2, 128, P;\n\t"
+      "selp.b32 %0, 1, 0, Q;\n\t"
+      "}\n"
+      : "=r"(r)
+      : "r"((uint32_t)ok), "r"(set + 1)
+      : "memory");
+  return r != 0;
+}
 
 template <int kTileN, int kV>
 __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0,
-                                              int64_t n_limit, int q, int lane, uint8_t* wsm, uint64_t* tmem_empty_bar) {
-  uint32_t* stage = reinterpret_cast<uint32_t*>(wsm);                     // [kV / 2][32 features]
-  uint8_t* cidx = wsm + vnm_stage_bytes(kV);                              // [4 groups][4]
-  uint4* sel_tab = reinterpret_cast<uint4*>(wsm + vnm_stage_bytes(kV) + 16);   // [4 groups][7]
-  uint8_t* nib_tab = wsm + vnm_stage_bytes(kV) + 16 + 4 * 7 * 16;         // [4 groups][7]
+                                              int64_t n_limit, int q, int set, int lane, uint8_t* wsm, uint64_t* tmem_empty_bar) {
+  uint32_t* stage = reinterpret_cast<uint32_t*>(wsm);                     // [kV / 2][128 features]
+  uint8_t* cidx = wsm + vnm_stage_bytes(kV);                               // [16 groups][4]
+  uint4* sel_tab = reinterpret_cast<uint4*>(cidx + 16 * 4);               // [16 groups][7]
+  uint8_t* nib_tab = cidx + 16 * 4 + 16 * 7 * 16;                         // [16 groups][7]
   const int64_t F = args.M, G = F >> 3;
-  const int64_t f0 = m0 + q * 32, g0 = f0 >> 3;                           // this warp's first feature / group
-  const int jm = lane & 7, gl = lane & 3;
+  const int64_t g0 = m0 >> 3;                                             // the CTA's first group
+  const int jm = lane & 7;
+  const int gl = lane & 15, psub = lane >> 4;                             // pass 2: group, which of two token pairs
   constexpr int kBlocks = kTileN / kV;
   int nblk = kBlocks;
   while (nblk > 0 && n0 + (int64_t)(nblk - 1) * kV >= n_limit) --nblk;     // ragged last tile: whole blocks only
@@ -285,11 +306,11 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
   }
   // strides per token of the outputs this thread writes (in the units of its pointers)
   const int sv = (int)G, s24 = (int)(F >> 3), sm = (int)(G >> 2), sm24 = (int)(F >> 5);
-  const bool lead4 = gl == 0, lead2 = (gl & 1) == 0;
+  const bool lead4 = (gl & 3) == 0, lead2 = (gl & 1) == 0;
 #pragma unroll 1
   for (int b = 0; b < kBlocks; ++b) {
     if (b >= nblk) break;
-    __syncwarp();                                                          // the previous block's pass 2 has read the stage
+    if (b > 0) set_sync(set);                                              // the previous block's pass 2 has read the stage
     const int64_t t0 = n0 + (int64_t)b * kV;
     // ---- pass 1: two tokens per step on packed bf16 pairs
     float score = 0.f;
@@ -301,7 +322,7 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         const uint32_t yp = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
-        stage[(c * 16 + j) * 32 + lane] = yp;
+        stage[(c * 16 + j) * 128 + q * 32 + lane] = yp;
         const uint32_t hp = bf2_sq(bf2_relu(yp));
         score = __fadd_rn(score, __uint_as_float(hp << 16));
         score = __fadd_rn(score, __uint_as_float(hp & 0xFFFF0000u));
@@ -320,13 +341,13 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
     const bool keep = rank < 4;
     const uint32_t ball = __ballot_sync(0xFFFFFFFFu, keep);
     const uint32_t gbyte = (ball >> (lane & 24)) & 0xFFu;
-    if (keep) cidx[(lane >> 3) * 4 + __popc(gbyte & ((1u << jm) - 1u))] = (uint8_t)jm;
+    if (keep) cidx[(q * 4 + (lane >> 3)) * 4 + __popc(gbyte & ((1u << jm) - 1u))] = (uint8_t)jm;
     __syncwarp();
     if (lane < 4)
-      *reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(args.vn_colidx) + ((t0 / kV) * G + g0 + lane) * 4) =
-          *reinterpret_cast<const uint32_t*>(cidx + lane * 4);
+      *reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(args.vn_colidx) + ((t0 / kV) * G + g0 + q * 4 + lane) * 4) =
+          *reinterpret_cast<const uint32_t*>(cidx + (q * 4 + lane) * 4);
     if (lane < 24) {
-      const int ge = lane / 6, pe = lane - ge * 6;
+      const int ge = q * 4 + lane / 6, pe = lane % 6;
       const int pi = pe < 3 ? 0 : (pe < 5 ? 1 : 2), pj = pe < 3 ? pe + 1 : (pe < 5 ? pe - 1 : 3);
       uint4 selv;
       uint32_t nib24;
@@ -335,8 +356,8 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
       sel_tab[slot] = selv;
       nib_tab[slot] = (uint8_t)nib24;
     }
-    __syncwarp();
-    // ---- pass 2: this thread serves group gl of the token pairs (lane >> 2) + 8 * it
+    set_sync(set);                                                         // all 128 features of the block are in
+    // ---- pass 2: this thread serves group gl of the token pairs 2 q + psub + 8 * it
     const uint32_t c4 = *reinterpret_cast<const uint32_t*>(cidx + gl * 4);
     uint32_t selp[2], mhi[2];
 #pragma unroll
@@ -349,19 +370,20 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
     const uint4* my_sel = sel_tab + gl * 7;
     const uint8_t* my_nib = nib_tab + gl * 7;
     // output pointers of this thread's first token; every pointer advances by a constant per token
-    const int64_t tf = t0 + 2 * (lane >> 2);
+    const int pair0 = 2 * q + psub;
+    const int64_t tf = t0 + 2 * pair0;
     uint32_t* p_vals = reinterpret_cast<uint32_t*>(args.vn_vals) + tf * G + g0 + gl;
     uint32_t* p_relu = reinterpret_cast<uint32_t*>(args.vn_relu) + tf * G + g0 + gl;
     uint2* p_v24 = reinterpret_cast<uint2*>(args.vn_vals24) + tf * (F >> 3) + g0 + gl;
     uint2* p_r24 = reinterpret_cast<uint2*>(args.vn_relu24) + tf * (F >> 3) + g0 + gl;
     uint4* p_y1 = args.vn_y1 ? reinterpret_cast<uint4*>(args.vn_y1) + tf * (F >> 3) + g0 + gl : nullptr;
     uint4* p_dense = args.vn_dense ? reinterpret_cast<uint4*>(args.vn_dense) + tf * (F >> 3) + g0 + gl : nullptr;
-    uint16_t* p_meta = reinterpret_cast<uint16_t*>(args.vn_meta) + tf * (G >> 2) + (g0 >> 2);
-    uint32_t* p_m24 = reinterpret_cast<uint32_t*>(args.vn_meta24) + tf * (F >> 5) + (f0 >> 5);
+    uint16_t* p_meta = reinterpret_cast<uint16_t*>(args.vn_meta) + tf * (G >> 2) + ((g0 + gl) >> 2);
+    uint32_t* p_m24 = reinterpret_cast<uint32_t*>(args.vn_meta24) + tf * (F >> 5) + ((g0 + gl) >> 2);
     // tensor-core-ordered copy: the block lies inside one 128-row band, so the atom is fixed
-    const int64_t kw24 = (f0 >> 4) + (gl >> 1);
+    const int64_t kw24 = (m0 >> 4) + (gl >> 1);
     uint8_t* hw_atom = reinterpret_cast<uint8_t*>(args.vn_meta24_hw) + meta_hw_offset(t0 & ~int64_t(127), kw24, F);
-    const uint32_t* sp = stage + (lane >> 2) * 32 + gl * 8;
+    const uint32_t* sp = stage + pair0 * 128 + gl * 8;
 
     auto emit = [&](const uint32_t (&yw)[4], int dt, uint32_t trow) {
       uint32_t rw[4], hw[4];
@@ -406,7 +428,7 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
       const uint32_t trow = (uint32_t)(tf & 127) + 16u * (uint32_t)it;
       emit(r0, 0, trow);
       emit(r1, 1, trow + 1u);
-      sp += 8 * 32;
+      sp += 8 * 128;
       p_vals += 16 * sv; p_relu += 16 * sv; p_v24 += 16 * s24; p_r24 += 16 * s24;
       if (p_y1) p_y1 += 16 * s24;
       if (p_dense) p_dense += 16 * s24;
@@ -1208,12 +1230,16 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
                                        &ctl->tmem_full[set], acc_phase, abort_flag, &ctl->tmem_empty[set]))
           break;
       } else {
-        if (!mbar_wait(&ctl->tmem_full[set], acc_phase, abort_flag)) break;
+        bool ok = mbar_wait(&ctl->tmem_full[set], acc_phase, abort_flag);
+        // the set's warps meet at barriers inside the tile: they go on, or leave, together
+        if (kEpi == EPI_VNM8) ok = set_all(set, ok);
+        if (!ok) break;
         tc_fence_after();
         if (!live) {
           release_accumulator(lane, &ctl->tmem_empty[set]);
         } else if constexpr (kEpi == EPI_VNM8) {
-          epi_vnm8_tile<kBN, vnm_block(kBN)>(args, taddr, m0, n0, n_limit, q, lane, wsm, &ctl->tmem_empty[set]);
+          epi_vnm8_tile<kBN, vnm_block(kBN)>(args, taddr, m0, n0, n_limit, q, set, lane, epi_stage + set * vnm_set_bytes(vnm_block(kBN)),
+                                             &ctl->tmem_empty[set]);
         } else {
           epi_act24_tile<kBN>(args, taddr, m0, n0, n_limit, q, lane, reinterpret_cast<uint32_t*>(wsm), ctl->expand_lut,
                               ctl->top2_lut, &ctl->tmem_empty[set]);
