@@ -5,8 +5,8 @@
 // renumbering of the FFN's hidden units, done once offline together with the clustering). Per step:
 //   step 1  route_kernel        logits = x . ExpertMeans, top-1 expert per token (ties to the lower expert)
 //   step 2  group_kernel        tokens grouped by expert, stable, every segment padded to 256 rows of zeros;
-//           tile_tables_kernel  one table entry per output tile of each grouped product (no host round trip)
-//           gather_rows_kernel  gathers X (and dY) into that order (Y and dX go back to token order through
+//           gather_rows_kernel  one table entry per output tile of each grouped product (no host round trip), and
+//                               X (and dY) gathered into that order (Y and dX go back to token order through
 //                               the row map of the product's own epilogue)
 //   step 3  grouped tensor-core products over the tables: every product touches only the expert's Fe features
 //           of a token, so each costs 1 / E of its dense counterpart (and the 2:4 ones half of that again).
@@ -154,15 +154,26 @@ group_kernel(const int* __restrict__ expert, int T, int E, int rows_max, int* __
     if (e < E) cnt[e * 1024 + tid] = local[e];
   for (int r = tid; r < rows_max; r += 1024) src_of_row[r] = -1;
   __syncthreads();
-  if (tid < E) {                           // exclusive scan of this expert's counts over the threads
+  // exclusive scan of an expert's counts over the threads: one warp per expert, 32 counts a pass (the serial scan by one
+  // thread per expert took 11 of this kernel's 17 us)
+  const int warp = tid >> 5, lane = tid & 31;
+  if (warp < E) {
     int run = 0;
-    for (int i = 0; i < 1024; ++i) {
-      const int c = cnt[tid * 1024 + i];
-      cnt[tid * 1024 + i] = run;
-      run += c;
+    for (int i = 0; i < 1024; i += 32) {
+      const int c = cnt[warp * 1024 + i + lane];
+      int x = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x += y;
+      }
+      cnt[warp * 1024 + i + lane] = run + x - c;
+      run += __shfl_sync(0xFFFFFFFFu, x, 31);
     }
-    seg[E + 1 + tid] = run;
-    sseg[tid + 1] = run;                   // totals, turned into boundaries below
+    if (lane == 0) {
+      seg[E + 1 + warp] = run;
+      sseg[warp + 1] = run;                // totals, turned into boundaries below
+    }
   }
   __syncthreads();
   if (tid == 0) {
@@ -191,62 +202,64 @@ group_kernel(const int* __restrict__ expert, int T, int E, int rows_max, int* __
   }
 }
 
-// Tile tables of the grouped products (one CTA; entries are written by a thread-strided loop per table).
+// Tile tables of the grouped products, written by `parts` CTAs (this is one of them).
 //   tabA  features-on-rows products (y1, dy1): A rows = the expert's feature tile, B rows = a token tile
 //   tabB  tokens-on-rows products (y3, dX): A rows = a token tile, reduction over the expert's features
 //   tabC  dW2 [D, F]: rows = d_model tile, columns = the expert's feature tile, reduction over its tokens
 //   tabD  dW1 [F, D]: rows = the expert's feature tile, columns = d_model tile, reduction over its tokens
 // counts[0..3] receive the table lengths.
-__global__ void __launch_bounds__(256)
-tile_tables_kernel(const int* __restrict__ seg, int E, int D, int F, GemmTile* __restrict__ tabA,
-                   GemmTile* __restrict__ tabB, GemmTile* __restrict__ tabC, GemmTile* __restrict__ tabD,
-                   int* __restrict__ counts) {
-  __shared__ int baseA[kMaxExperts + 1], baseB[kMaxExperts + 1], baseC[kMaxExperts + 1];
-  const int Fe = F / E, fm = Fe / 256, dm = D / 256;
-  pdl_wait();
-  pdl_trigger();
-  if (threadIdx.x == 0) {
-    baseA[0] = baseB[0] = baseC[0] = 0;
-    for (int e = 0; e < E; ++e) {
-      const int rows = seg[e + 1] - seg[e];
-      baseA[e + 1] = baseA[e] + fm * ((rows + kActTileN - 1) / kActTileN);
-      baseB[e + 1] = baseB[e] + (rows / 256) * dm;
-      baseC[e + 1] = baseC[e] + fm * dm;
-    }
-    counts[0] = baseA[E]; counts[1] = baseB[E]; counts[2] = baseC[E]; counts[3] = baseC[E];
-  }
-  __syncthreads();
+struct TableArgs {
+  GemmTile *tabA, *tabB, *tabC, *tabD;
+  int* counts;
+  int E, D, F;
+};
+constexpr int kTableCtas = 32;
+
+__device__ void build_tables(const int* __restrict__ seg, const TableArgs& t, int part, int parts) {
+  const int E = t.E, D = t.D, Fe = t.F / E, fm = Fe / 256, dm = D / 256;
+  const int first = part * (int)blockDim.x + (int)threadIdx.x, step = parts * (int)blockDim.x;
+  int baseA = 0, baseB = 0, baseC = 0;
   for (int e = 0; e < E; ++e) {
-    const int s0 = seg[e], rows = seg[e + 1] - seg[e];
-    const int nA = baseA[e + 1] - baseA[e];
-    for (int i = threadIdx.x; i < nA; i += blockDim.x) {
+    const int s0 = __ldg(seg + e), rows = __ldg(seg + e + 1) - s0;
+    const int nA = fm * ((rows + kActTileN - 1) / kActTileN);
+    for (int i = first; i < nA; i += step) {
       const int nt = i / fm, mt = i - nt * fm;                       // feature tiles fastest: they share the token tile
-      tabA[baseA[e] + i] = GemmTile{e * Fe + mt * 256, 0, s0 + nt * kActTileN, 0, D / 128, mt * 256, s0 + nt * kActTileN,
-                                    s0 + rows};
+      t.tabA[baseA + i] = GemmTile{e * Fe + mt * 256, 0, s0 + nt * kActTileN, 0, D / 128, mt * 256, s0 + nt * kActTileN, s0 + rows};
     }
-    const int nB = baseB[e + 1] - baseB[e];
-    for (int i = threadIdx.x; i < nB; i += blockDim.x) {
+    const int nB = (rows / 256) * dm;
+    for (int i = first; i < nB; i += step) {
       const int nt = i / (rows / 256), rt = i - nt * (rows / 256);   // token tiles fastest: they share the weight tile
-      tabB[baseB[e] + i] = GemmTile{s0 + rt * 256, 0, nt * 256, e * Fe, Fe / 128, s0 + rt * 256, nt * 256, D};
+      t.tabB[baseB + i] = GemmTile{s0 + rt * 256, 0, nt * 256, e * Fe, Fe / 128, s0 + rt * 256, nt * 256, D};
     }
     const int nC = fm * dm;
-    for (int i = threadIdx.x; i < nC; i += blockDim.x) {
+    for (int i = first; i < nC; i += step) {
       const int nt = i / dm, mt = i - nt * dm;
-      tabC[baseC[e] + i] = GemmTile{mt * 256, s0, nt * 256, s0, rows / 64, mt * 256, e * Fe + nt * 256, F};
+      t.tabC[baseC + i] = GemmTile{mt * 256, s0, nt * 256, s0, rows / 64, mt * 256, e * Fe + nt * 256, t.F};
       const int nt2 = i / fm, mt2 = i - nt2 * fm;
-      tabD[baseC[e] + i] = GemmTile{mt2 * 256, s0, nt2 * 256, s0, rows / 64, e * Fe + mt2 * 256, nt2 * 256, D};
+      t.tabD[baseC + i] = GemmTile{mt2 * 256, s0, nt2 * 256, s0, rows / 64, e * Fe + mt2 * 256, nt2 * 256, D};
     }
+    baseA += nA; baseB += nB; baseC += nC;
+  }
+  if (first == 0) {
+    t.counts[0] = baseA; t.counts[1] = baseB; t.counts[2] = baseC; t.counts[3] = baseC;
   }
 }
 
 // out[r, :] = src[r] >= 0 ? in[src[r], :] : 0. One warp per output row; a lane keeps four 16-byte loads in
 // flight, every instruction of the warp covers 512 contiguous bytes.
+// kTables: the first kTableCtas CTAs build the tile tables instead (the forward pass; a launch of its own on one CTA took
+// 9 us and a gap).
+template <bool kTables>
 __global__ void __launch_bounds__(256)
 gather_rows_kernel(const uint4* __restrict__ in, const int* __restrict__ src, uint4* __restrict__ out, int rows,
-                   int row_u4) {
+                   int row_u4, const int* __restrict__ seg, const TableArgs tables) {
   pdl_wait();
   pdl_trigger();
-  const int r = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (kTables && blockIdx.x < kTableCtas) {
+    build_tables(seg, tables, (int)blockIdx.x, kTableCtas);
+    return;
+  }
+  const int r = ((int)blockIdx.x - (kTables ? kTableCtas : 0)) * 8 + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= rows) return;
   const int s = __ldg(src + r);
   const uint4* ip = in + (int64_t)(s >= 0 ? s : 0) * row_u4;
@@ -344,10 +357,12 @@ int launch_route(const void* X, const void* means, int64_t T, int64_t D, int E, 
                     (const uint16_t*)X, (const uint16_t*)means, (int)T, (int)D, E, (int*)expert, (float*)logits);
 }
 
-int launch_gather_rows(const void* in, const int* src, void* out, int64_t rows, int64_t cols, cudaStream_t s) {
+int launch_gather_rows(const void* in, const int* src, void* out, int64_t rows, int64_t cols, cudaStream_t s,
+                       const int* seg = nullptr, const TableArgs* tables = nullptr) {
   if (rows == 0 || cols == 0) return SF_OK;
-  return launch_pdl(gather_rows_kernel, dim3((unsigned)((rows + 7) / 8)), 256, 0, s, (const uint4*)in, src, (uint4*)out,
-                    (int)rows, (int)(cols / 8));
+  return launch_pdl(tables ? gather_rows_kernel<true> : gather_rows_kernel<false>,
+                    dim3((unsigned)((rows + 7) / 8) + (tables ? kTableCtas : 0)), 256, 0, s, (const uint4*)in, src, (uint4*)out,
+                    (int)rows, (int)(cols / 8), seg, tables ? *tables : TableArgs{});
 }
 
 }  // namespace
@@ -423,9 +438,9 @@ int sf_routed_ffn_fwd(const sf_router_desc* desc, const void* X, const void* W1,
   }
   SF_TRY(launch_pdl(group_kernel, dim3(1), 1024, gsm, s, expert, (int)d.T, d.E, (int)L.rows_max,
                     (int*)at(fwd_ctx, L.row_of_token), src, seg));
-  SF_TRY(launch_pdl(tile_tables_kernel, dim3(1), 256, 0, s, seg, d.E, (int)d.D, (int)d.F, (GemmTile*)at(fwd_ctx, L.tabA),
-                    (GemmTile*)at(fwd_ctx, L.tabB), (GemmTile*)at(fwd_ctx, L.tabC), (GemmTile*)at(fwd_ctx, L.tabD), counts));
-  SF_TRY(launch_gather_rows(X, src, at(fwd_ctx, L.xp), L.rows_max, d.D, s));
+  const TableArgs tables{(GemmTile*)at(fwd_ctx, L.tabA), (GemmTile*)at(fwd_ctx, L.tabB), (GemmTile*)at(fwd_ctx, L.tabC),
+                         (GemmTile*)at(fwd_ctx, L.tabD), counts, d.E, (int)d.D, (int)d.F};
+  SF_TRY(launch_gather_rows(X, src, at(fwd_ctx, L.xp), L.rows_max, d.D, s, seg, &tables));
   trace_mark(s);
   // step 3: y1 = Xp W1s[expert]^T with SquaredReLU and the 2:4 selection in the epilogue
   Act24Out out{at(fwd_ctx, L.y2_vals), at(fwd_ctx, L.relu_vals), at(fwd_ctx, L.meta), at(fwd_ctx, L.meta_hw),
