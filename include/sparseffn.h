@@ -420,10 +420,12 @@ SF_API int sf_selftest_wait_expiry(void* workspace, int64_t budget_clocks, void*
  * tracing is switched off with capacity 0. While set, every FFN step call records one event
  * before its first kernel and one after each kernel, in launch order, on the call's stream:
  *   sparse fwd: 6 events (prune W1 | y1 product | V:N:M | W2 transpose | y3 product); intervals of
- *               kernels a path does not launch are empty (M <= 8: no W2 transpose; M == 8 with the
- *               selection fused into the y1 product: no V:N:M kernel)
+ *               kernels a path does not launch are empty (M <= 8: no W2 transpose; M == 4, or M == 8
+ *               with the selection fused into the y1 product: no V:N:M kernel)
  *   sparse bwd: 7 events (prune W2 | dy1 product | pack | dX product | dW2 product | dW1 product);
- *               for M <= 8 the dy1 product packs its own output and the pack interval is empty
+ *               dy1 leaves its product packed, so the pack interval is empty; where the two weight gradients
+ *               share one launch (it saves rounds of tiles on small and middle sizes), the dW2 interval
+ *               holds both and the dW1 interval is empty (dense bwd: the same)
  *   dense fwd: 3 events, dense bwd: 5 events.
  *   routed fwd: 6 events (prune W1 | route | group + tile tables + gather X | y1 product | y3 product)
  *   routed bwd: 7 events (prune W2 | gather dY | dy1 product | dX product | dW2 product | dW1 product).

@@ -187,6 +187,28 @@ int check_desc(const sf_ffn_desc* d) {
 inline uint8_t* at(void* base, size_t off) { return reinterpret_cast<uint8_t*>(base) + off; }
 inline const uint8_t* at(const void* base, size_t off) { return reinterpret_cast<const uint8_t*>(base) + off; }
 
+// dW2 = dY^T h in the layout of W2 ([D, F], or [F, D] = h^T dY with w2_fd) and dW1 = dy1^T X [F, D]: in one launch where
+// that saves rounds of tiles. The host-buffer step keeps them apart: it downloads dW2 while dW1 is computed.
+int weight_grads(const sf_ffn_desc& d, const void* dY, const void* h, const void* dy1, const void* X, void* dW2, void* dW1,
+                 int* status, cudaStream_t s) {
+  const bool w2_fd = (d.flags & SF_FFN_W2_FD) != 0;
+  const void *a2 = w2_fd ? h : dY, *b2 = w2_fd ? dY : h;
+  const int64_t m2 = w2_fd ? d.F : d.D, n2 = w2_fd ? d.D : d.F;
+  if (!g_hooks && gemm_dual_tn_pays(m2, n2, d.F, d.D)) {
+    const int st = gemm_dual_tn(a2, b2, m2, n2, dW2, dy1, X, d.F, d.D, dW1, d.T, status, s);
+    trace_mark(s);
+    trace_mark(s);      // (one launch: the dW1 interval is empty)
+    return st;
+  }
+  int st = gemm_dense(a2, false, b2, false, m2, n2, d.T, EPI_STORE, dW2, n2, nullptr, 0, nullptr, 0, status, s);
+  if (st != SF_OK) return st;
+  trace_mark(s);
+  hook_dw2_done(s);
+  st = gemm_dense(dy1, false, X, false, d.F, d.D, d.T, EPI_STORE, dW1, d.D, nullptr, 0, nullptr, 0, status, s);
+  trace_mark(s);
+  return st;
+}
+
 }  // namespace
 
 void trace_mark(cudaStream_t s) {
@@ -394,12 +416,6 @@ int sf_sparse_ffn_bwd(const sf_ffn_desc* desc, const void* dY, const void* X, co
   cudaStream_t s = (cudaStream_t)stream;
   int* status = (int*)workspace;
   const bool w2_fd = (d.flags & SF_FFN_W2_FD) != 0;
-  // dW2 = dY^T y2 in the layout of W2: [D, F], or [F, D] = y2^T dY when W2 is stored that way
-  auto grad_w2 = [&](const void* y2_dense) -> int {
-    return w2_fd ? gemm_dense(y2_dense, false, dY, false, d.F, d.D, d.T, EPI_STORE, dW2, d.D, nullptr, 0, nullptr, 0, status, s)
-                 : gemm_dense(dY, false, y2_dense, false, d.D, d.F, d.T, EPI_STORE, dW2, d.F, nullptr, 0, nullptr, 0, status, s);
-  };
-
   // Algorithm 2 line 2: W2s = sparsify24(W2^T) along d_model (contiguous in the saved W2^T copy),
   // dy2 = dY W2s;  line 4: dy1 = 2 dy2 ReLU(y1) on y2's mask (fused into the product's epilogue)
   trace_mark(s);
@@ -432,21 +448,13 @@ int sf_sparse_ffn_bwd(const sf_ffn_desc* desc, const void* dY, const void* X, co
     // line 3: dW2 = dY^T y2 [D, F];  line 6: dW1 = dy1^T X [F, D]: dense tensor-core products (the reduction
     // runs over tokens); their masked operand is a stored [T, F] matrix or is expanded from its packed form
     // inside the kernel
-    if (L.expand) {
-      if (w2_fd) SF_TRY(gemm_dense_expand(dY, 1, at(fwd_ctx, L.vals24), at(fwd_ctx, L.meta24), d.F, d.D, d.T, dW2, d.D, status, s));
-      else       SF_TRY(gemm_dense_expand(dY, 2, at(fwd_ctx, L.vals24), at(fwd_ctx, L.meta24), d.D, d.F, d.T, dW2, d.F, status, s));
-    } else {
-      SF_TRY(grad_w2(at(fwd_ctx, L.y2_dense)));
-    }
+    if (!L.expand)
+      return weight_grads(d, dY, at(fwd_ctx, L.y2_dense), at(workspace, L.dy1_dense), X, dW2, dW1, status, s);
+    if (w2_fd) SF_TRY(gemm_dense_expand(dY, 1, at(fwd_ctx, L.vals24), at(fwd_ctx, L.meta24), d.F, d.D, d.T, dW2, d.D, status, s));
+    else       SF_TRY(gemm_dense_expand(dY, 2, at(fwd_ctx, L.vals24), at(fwd_ctx, L.meta24), d.D, d.F, d.T, dW2, d.F, status, s));
     trace_mark(s);
     hook_dw2_done(s);
-    if (L.expand) {
-      SF_TRY(gemm_dense_expand(X, 1, at(workspace, L.dy1_vals24), at(fwd_ctx, L.meta24), d.F, d.D, d.T, dW1, d.D,
-                               status, s));
-    } else {
-      SF_TRY(gemm_dense(at(workspace, L.dy1_dense), false, X, false, d.F, d.D, d.T, EPI_STORE, dW1, d.D, nullptr, 0,
-                        nullptr, 0, status, s));
-    }
+    SF_TRY(gemm_dense_expand(X, 1, at(workspace, L.dy1_vals24), at(fwd_ctx, L.meta24), d.F, d.D, d.T, dW1, d.D, status, s));
     trace_mark(s);
     return SF_OK;
   }
@@ -470,13 +478,7 @@ int sf_sparse_ffn_bwd(const sf_ffn_desc* desc, const void* dY, const void* X, co
   trace_mark(s);
   hook_dx_done(s);
   // line 3: dW2 = dY^T y2 [D, F];  line 6: dW1 = dy1^T X [F, D]  (reduction over tokens)
-  SF_TRY(grad_w2(at(fwd_ctx, L.y2_dense)));
-  trace_mark(s);
-  hook_dw2_done(s);
-  SF_TRY(gemm_dense(at(workspace, L.dy1_dense), false, X, false, d.F, d.D, d.T, EPI_STORE, dW1, d.D, nullptr, 0,
-                    nullptr, 0, status, s));
-  trace_mark(s);
-  return SF_OK;
+  return weight_grads(d, dY, at(fwd_ctx, L.y2_dense), at(workspace, L.dy1_dense), X, dW2, dW1, status, s);
 }
 
 int sf_dense_ffn_fwd(const sf_ffn_desc* desc, const void* X, const void* W1, const void* W2, void* Y, void* fwd_ctx,
@@ -524,17 +526,7 @@ int sf_dense_ffn_bwd(const sf_ffn_desc* desc, const void* dY, const void* X, con
   trace_mark(s);
   hook_dx_done(s);
   // Eq. 5: dW2 = dY^T h [D, F];  Eq. 8: dW1 = dy1^T X [F, D]
-  if (w2_fd)
-    SF_TRY(gemm_dense(at(fwd_ctx, L.h), false, dY, false, d.F, d.D, d.T, EPI_STORE, dW2, d.D, nullptr, 0, nullptr, 0,
-                      status, s));
-  else
-    SF_TRY(gemm_dense(dY, false, at(fwd_ctx, L.h), false, d.D, d.F, d.T, EPI_STORE, dW2, d.F, nullptr, 0, nullptr, 0,
-                      status, s));
-  trace_mark(s);
-  hook_dw2_done(s);
-  SF_TRY(gemm_dense(dy1, false, X, false, d.F, d.D, d.T, EPI_STORE, dW1, d.D, nullptr, 0, nullptr, 0, status, s));
-  trace_mark(s);
-  return SF_OK;
+  return weight_grads(d, dY, at(fwd_ctx, L.h), dy1, X, dW2, dW1, status, s);
 }
 
 int sf_ctx_view(const sf_ffn_desc* desc, const void* buf, int field, const void** ptr, size_t* bytes) {

@@ -113,7 +113,7 @@ __device__ __forceinline__ void pair_rows(const uint32_t* sp, int lane, uint32_t
 // eight rows per instruction: y1 + SquaredReLU at T 4096, D 2048, F 8192 129 -> 96 us.
 template <int kEpi, int kTileN = BN>
 __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit,
-                                         int q, int lane, uint8_t* my_stage, int part = 0, int parts = 1) {
+                                         int q, int lane, uint8_t* my_stage, int part = 0, int parts = 1, bool second = false) {
   if constexpr (kEpi == EPI_ROUTE) {
     const int64_t row = m0 + q * 32 + lane;                                // this thread's D row
     // the row is a token, the first route_E columns its logits
@@ -206,7 +206,7 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
     }
     if (kEpi == EPI_STORE) {
       if (row_live) {
-        uint4* c = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(args.C) + row * args.ldc + col0);
+        uint4* c = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(second ? args.C2 : args.C) + row * (second ? args.ldc2 : args.ldc) + col0);
 #pragma unroll
         for (int j = 0; j < 4; ++j) c[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
       }
@@ -945,17 +945,21 @@ struct SmemCtl2 {
 };
 
 // The tile a CTA pair works on: from the regular raster, or from a device-built table (grouped products).
-template <int kBN, bool kVar>
+template <int kBN, bool kVar, bool kDual>
 __device__ __forceinline__ GemmTile get_tile(const GemmArgs& args, int tile, int num_m, int num_n, int nkb_full) {
   if (args.tile_table) {
     const int4* p = reinterpret_cast<const int4*>(args.tile_table + tile);
     const int4 a = __ldg(p), b = __ldg(p + 1);
     return GemmTile{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
   }
-  int mt, nt;
+  int mt, nt, N = (int)args.N;
+  if (kDual && tile >= num_m * num_n) {                    // the second product's tiles follow the first one's
+    tile -= num_m * num_n;
+    num_m = args.num_m_tiles2; num_n = args.num_n_tiles2; N = (int)args.N2;
+  }
   tile_coords(tile, num_m, num_n, mt, nt);
   const int n0 = nt * (kVar ? args.bn : kBN);
-  return GemmTile{mt * 256, 0, n0, 0, nkb_full, mt * 256, n0, kVar ? min((int)args.N, n0 + args.bn) : (int)args.N};
+  return GemmTile{mt * 256, 0, n0, 0, nkb_full, mt * 256, n0, kVar ? min(N, n0 + args.bn) : N};
 }
 
 __device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) {
@@ -972,7 +976,9 @@ __device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) {
 // more SMs to work and shorten what one of them does: the eight kernels of a step at T 1024, D 256, F 1024 take 50 us
 // instead of 61 (graph replay). A kernel of its own, because the run-time width costs the issuing threads instructions
 // that the large products do not have (dense, 256 wide: 1.5 % and more).
-template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false>
+// kDual: two independent products with the same reduction length in one launch (the weight gradients). The second one's
+// operands are tmapMeta (A) and tmapPk (B), its output args.C2.
+template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false, bool kDual = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kMode, kEpi, kExpand), 1)
 gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB,
                 const __grid_constant__ CUtensorMap tmapMeta, const __grid_constant__ CUtensorMap tmapPk,
@@ -983,6 +989,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   constexpr int kStages = num_stages2(kSparse, kBN, kExpand != 0);
   constexpr int kBK = kSparse ? 128 : 64;                // logical K per stage
   static_assert(kExpand == 0 || (kMode == MODE_DENSE && kAMN && kBMN), "packed operands: weight-gradient products only");
+  static_assert(!kDual || (kMode == MODE_DENSE && kExpand == 0 && kEpi == EPI_STORE), "pairs of plain dense products");
   static_assert(!kFp8 || (!kAMN && !kBMN && kExpand == 0 && kMode != MODE_VENOM), "8-bit operands are K-major");
   constexpr int kMetaBytes = meta_stage_bytes2(kFp8);
   constexpr uint32_t kMetaCols = kFp8 ? 8u : 4u;          // TMEM columns of one stage's metadata
@@ -1044,7 +1051,8 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   tc_fence_after();
   pdl_wait();                                            // everything above overlaps the previous kernel's tail
   pdl_trigger();
-  const int num_tiles = args.tile_table ? __ldg(args.num_tiles_dev) : num_m_tiles * num_n_tiles_;
+  const int num_tiles = args.tile_table ? __ldg(args.num_tiles_dev)
+                                        : num_m_tiles * num_n_tiles_ + (kDual ? args.num_m_tiles2 * args.num_n_tiles2 : 0);
   const uint32_t tmem_base = ctl->tmem_base;
 
   if (warp == 0) {
@@ -1052,8 +1060,10 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     uint32_t stage = 0, phase = 0;
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
-      const GemmTile tc = get_tile<kBN, kVar>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
+      const GemmTile tc = get_tile<kBN, kVar, kDual>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
       const int m0 = tc.a_row + (int)rank * 128;         // this CTA's rows of A / D
+      const bool second = kDual && tile >= num_m_tiles * num_n_tiles_;
+      const CUtensorMap *mapA = second ? &tmapMeta : &tmapA, *mapB = second ? &tmapPk : &tmapB;
       const int nb0 = tc.b_row + (int)rank * half_n;
       const int nkb = tc.nkb, ak0 = tc.a_k0, bk0 = tc.b_k0;
       for (int kb = 0; kb < nkb; ++kb) {
@@ -1074,17 +1084,17 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
             if (kExpand == 1) {
               // packed A: this CTA's 128 features of 64 tokens, into the staging ring (own barrier)
             } else if (!kAMN) {
-              tma_load_2d_2cta(sA, &tmapA, bar, ak0 + kb * 64, m0);
+              tma_load_2d_2cta(sA, mapA, bar, ak0 + kb * 64, m0);
             } else {
-              tma_load_2d_2cta(sA, &tmapA, bar, m0, ak0 + kb * 64);
-              tma_load_2d_2cta(sA + 8192, &tmapA, bar, m0 + 64, ak0 + kb * 64);
+              tma_load_2d_2cta(sA, mapA, bar, m0, ak0 + kb * 64);
+              tma_load_2d_2cta(sA + 8192, mapA, bar, m0 + 64, ak0 + kb * 64);
             }
             if (kExpand == 2) {
             } else if (!kBMN) {
-              tma_load_2d_2cta(sB, &tmapB, bar, bk0 + kb * 64, nb0);           // box {64 k, 128 n}
+              tma_load_2d_2cta(sB, mapB, bar, bk0 + kb * 64, nb0);           // box {64 k, 128 n}
             } else {
-              tma_load_2d_2cta(sB, &tmapB, bar, nb0, bk0 + kb * 64);           // box {64 n, 64 k}
-              if (!kVar || b_chunks == 2) tma_load_2d_2cta(sB + 8192, &tmapB, bar, nb0 + 64, bk0 + kb * 64);
+              tma_load_2d_2cta(sB, mapB, bar, nb0, bk0 + kb * 64);           // box {64 n, 64 k}
+              if (!kVar || b_chunks == 2) tma_load_2d_2cta(sB + 8192, mapB, bar, nb0 + 64, bk0 + kb * 64);
             }
             if (kExpand) {
               const int f0 = kExpand == 1 ? m0 : nb0;                          // first feature of this CTA's half
@@ -1220,7 +1230,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     const uint32_t taddr = tmem_base + set * kBN + ((uint32_t)(q * 32) << 16);
     uint32_t acc_phase = 0;
     for (int tile = pair + set * num_pairs; tile < num_tiles; tile += 2 * num_pairs) {
-      const GemmTile tc = get_tile<kBN, kVar>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
+      const GemmTile tc = get_tile<kBN, kVar, kDual>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
       const int64_t m0 = (int64_t)tc.out_m + (int64_t)rank * 128, n0 = tc.out_n, n_limit = tc.n_limit;
       // M % 256 == 128 (regular raster only): the second CTA of the last row of pairs holds no rows (its operand
       // loads were zero-filled); it only hands the accumulator back
@@ -1255,14 +1265,15 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     uint32_t acc = 0, acc_phase = 0;
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
-      const GemmTile tc = get_tile<kBN, kVar>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
+      const GemmTile tc = get_tile<kBN, kVar, kDual>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
       const int64_t m0 = (int64_t)tc.out_m + (int64_t)rank * 128, n0 = tc.out_n, n_limit = tc.n_limit;
       const uint32_t taddr = tmem_base + acc * kBN + ((uint32_t)(q * 32) << 16);
       // M % 256 == 128 (regular raster only): the second CTA of the last row of pairs holds no rows
-      const bool live = args.tile_table != nullptr || m0 < args.M;
+      const bool second = kDual && tile >= num_m_tiles * num_n_tiles_;
+      const bool live = args.tile_table != nullptr || m0 < (second ? args.M2 : args.M);
       if (!mbar_wait(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      if (live) epi_tile<kEpi, kBN>(args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts);
+      if (live) epi_tile<kEpi, kBN>(args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts, second);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_leader(&ctl->tmem_empty[acc]);
@@ -1589,10 +1600,10 @@ int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const GemmArgs& a, 
                     ta, tb, a);
 }
 
-template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false>
+template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false, bool kDual = false>
 int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tm, GemmArgs a, cudaStream_t s,
                const CUtensorMap* tpk = nullptr) {
-  auto kern = gemm_tc2_kernel<kMode, kAMN, kBMN, kEpi, kBN, kExpand, kFp8, kVar>;
+  auto kern = gemm_tc2_kernel<kMode, kAMN, kBMN, kEpi, kBN, kExpand, kFp8, kVar, kDual>;
   constexpr int smem = smem_bytes2(kMode != MODE_DENSE, kBN, kEpi, kExpand != 0, kFp8);
   static_assert(smem <= 232448, "shared memory per CTA");
   static bool attr_done[64] = {false};
@@ -1607,7 +1618,7 @@ int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
   a.num_n_tiles = (int)((a.N + bn - 1) / bn);
   // table-driven products: the table's length is on the device; launch for its upper bound
   const int tiles = a.tile_table ? a.num_k_blocks /* upper bound, see the grouped launchers */
-                                 : a.num_m_tiles * a.num_n_tiles;
+                                 : a.num_m_tiles * a.num_n_tiles + (kDual ? a.num_m_tiles2 * a.num_n_tiles2 : 0);
   const int max_pairs = sm_count() / 2;
   const int pairs = tiles < max_pairs ? tiles : max_pairs;
   return launch_pdl(kern, dim3(2 * pairs), threads2(kMode, kEpi, kExpand), smem, s, ta, tb, tm, tpk ? *tpk : ta, a);
@@ -1661,10 +1672,11 @@ int tall_maps(const void* vals, const void* meta_hw, const void* B, bool b_kmajo
 // clocks per 32 columns; exposed: nothing hides the epilogue of a tile (one accumulator), else only the last one counts.
 // A narrower width has to gain 10 %: its kernel takes the width at run time (at 6 % the weight gradients of D 2048 took 224
 // columns, 0.94 by the estimate, and 1.02 of the time).
-int best_width(int64_t M, int64_t N, int64_t stages, bool sparse, int max_bn, int step, double chunk, bool exposed) {
-  const int64_t P = sm_count() / 2, nm = (M + 255) / 256;
+int best_width(int64_t M, int64_t N, int64_t stages, bool sparse, int max_bn, int step, double chunk, bool exposed,
+               int64_t M2 = 0, int64_t N2 = 0) {
+  const int64_t P = sm_count() / 2, nm = (M + 255) / 256, nm2 = (M2 + 255) / 256;
   auto cost = [&](int w) {
-    const int64_t tiles = nm * ((N + w - 1) / w);
+    const int64_t tiles = nm * ((N + w - 1) / w) + nm2 * ((N2 + w - 1) / w);
     const double smem = sparse ? 0.93 * (272 + 2 * w) : 256.0 + w, main = stages * (smem > 2.0 * w ? smem : 2.0 * w);
     const double rounds = (double)((tiles + P - 1) / P), epi = chunk * (w / 32);
     return exposed ? rounds * (main + epi) : rounds * (main > epi ? main : epi) + epi;
@@ -1754,6 +1766,34 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
   }
 #undef SF_DENSE_CASE
   return SF_ERR_UNSUPPORTED;
+}
+
+bool gemm_dual_tn_pays(int64_t M1, int64_t N1, int64_t M2, int64_t N2) {
+  if (M1 < 256 || M2 < 256) return false;
+  const int64_t P = sm_count() / 2;
+  const int64_t t1 = ((M1 + 255) / 256) * ((N1 + 255) / 256), t2 = ((M2 + 255) / 256) * ((N2 + 255) / 256);
+  const int64_t apart = (t1 + P - 1) / P + (t2 + P - 1) / P, together = (t1 + t2 + P - 1) / P;
+  return (double)together <= 0.97 * (double)apart;
+}
+
+int gemm_dual_tn(const void* A1, const void* B1, int64_t M1, int64_t N1, void* C1, const void* A2, const void* B2, int64_t M2,
+                 int64_t N2, void* C2, int64_t K, int* status, cudaStream_t s) {
+  if (M1 < 256 || M2 < 256 || M1 % 128 || N1 % 128 || M2 % 128 || N2 % 128 || K % 64) return SF_ERR_SHAPE;
+  GemmArgs a{};
+  a.bn = best_width(M1, N1, K / 64, false, BN, 32, 200.0, false, M2, N2);
+  CUtensorMap ta, tb, ta2, tb2;
+  int st = make_tmap(&ta, A1, K, M1, M1, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
+  if (st == SF_OK) st = make_tmap(&tb, B1, K, N1, N1, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
+  if (st == SF_OK) st = make_tmap(&ta2, A2, K, M2, M2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
+  if (st == SF_OK) st = make_tmap(&tb2, B2, K, N2, N2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
+  if (st != SF_OK) return st;
+  a.M = M1; a.N = N1; a.K = K; a.C = C1; a.ldc = N1;
+  a.M2 = M2; a.N2 = N2; a.C2 = C2; a.ldc2 = N2;
+  a.num_m_tiles2 = (int)((M2 + 255) / 256);
+  a.num_n_tiles2 = (int)((N2 + a.bn - 1) / a.bn);
+  a.status = status;
+  return a.bn == BN ? launch_two<MODE_DENSE, true, true, EPI_STORE, BN, 0, false, false, true>(ta, tb, ta2, a, s, &tb2)
+                    : launch_two<MODE_DENSE, true, true, EPI_STORE, BN, 0, false, true, true>(ta, tb, ta2, a, s, &tb2);
 }
 
 int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, bool b_kmajor, int64_t M, int64_t N,

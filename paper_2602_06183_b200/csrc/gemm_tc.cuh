@@ -50,6 +50,8 @@ struct GemmArgs {
   int* status;              // device status word (set to 1 when a bounded wait expires)
   int num_m_tiles, num_n_tiles, num_k_blocks;
   int bn;                   // CTA-pair kernels with a run-time tile width: that width
+  int64_t M2, N2;           // second product of a launch of two (output C2)
+  int num_m_tiles2, num_n_tiles2;
   int gather_tma_groups;    // Venom: groups (of 16 per stage) fetched by TMA row gather; the rest by cp.async
   // EPI_DRELU24_T / EPI_DRELUV_T: metadata of the activation's mask and the packed output (see ActMask)
   const void* pack_meta;
@@ -87,6 +89,12 @@ struct Vnm8Out {
 int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64_t M, int64_t N, int64_t K, int epi,
                void* C, int64_t ldc, void* C2, int64_t ldc2, const void* aux, int64_t ldaux, int* status,
                cudaStream_t s);
+// Two products C1[M1,N1] = A1[K,M1]^T B1[K,N1] and C2[M2,N2] = A2[K,M2]^T B2[K,N2] in one launch. _pays: whether that saves
+// rounds of tiles (a launch of its own leaves its last round part empty): D 2048, F 8192: 4 + 4 rounds against 7; a
+// small layer: one kernel less. M >= 256, all sizes multiples of 128.
+bool gemm_dual_tn_pays(int64_t M1, int64_t N1, int64_t M2, int64_t N2);
+int gemm_dual_tn(const void* A1, const void* B1, int64_t M1, int64_t N1, void* C1, const void* A2, const void* B2, int64_t M2,
+                 int64_t N2, void* C2, int64_t K, int* status, cudaStream_t s);
 // The weight-gradient products with one operand given packed: D[M,N] = A^T B with A [K, M] and B [K, N]
 // row-major (reduction over the rows), where operand `packed_operand` (1 = A, 2 = B) is not read as a
 // dense matrix but expanded on the fly from its 2:4 layout: values [K, X/2] + canonical metadata
