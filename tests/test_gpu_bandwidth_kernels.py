@@ -108,6 +108,22 @@ def test_vnm_streaming_kernel_bit_exact(T, F, V, M, apply):
             assert np.array_equal(bits(relu), ref.relu_vals)
 
 
+@pytest.mark.parametrize("T,F,V,apply", [
+    (5120, 2368, 128, True),      # 19 half-strips wide, many per CTA: both scoring turns across the ring's wrap; ragged
+    (1120, 448, 112, True), (400, 320, 80, False),
+    (1600, 6464, 16, True),       # eight slots, many strips per CTA
+    (16, 64, 16, True)])          # one strip, a quarter of it
+def test_vnm8_streaming_strip_heights(T, F, V, apply):
+    p = synth.act_sweep_matrix(T, F, seed=7100 + T + V)
+    ref = oracle.vnm_sparsify(p, V=V, M=8, apply_sqrelu=apply)
+    vals, meta, colidx, relu, _ = binding.sf_vnm_sparsify_act(to_dev(p), V, 8, apply_sqrelu=apply)
+    torch.cuda.synchronize()
+    assert np.array_equal(colidx.cpu().numpy(), ref.colidx)
+    assert np.array_equal(bits(meta), ref.meta) and np.array_equal(bits(vals), ref.vals)
+    if apply:
+        assert np.array_equal(bits(relu), ref.relu_vals)
+
+
 def test_vnm_no_activation_and_ties():
     # raw magnitudes with many exact ties, negative values, apply_sqrelu = 0
     p = synth.prune_sweep_matrix(128, 512, seed=9, tie_frac=0.5)
