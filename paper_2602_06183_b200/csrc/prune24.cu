@@ -178,7 +178,7 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64
         for (int j = 0; j < 4; ++j) rw[j] = *reinterpret_cast<const uint32_t*>(&tile[kr + j][c]);
         // the two columns of the pair share one pass of the 16-bit-halves selection
         Top2Entry ent[2];
-        top2of4_x2<kSoft>(rw[0], rw[1], rw[2], rw[3], lut, ent[0], ent[1]);
+        top2of4_x2<kSoft, true>(rw[0], rw[1], rw[2], rw[3], lut, ent[0], ent[1]);
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const uint32_t sel = e ? 0x7632u : 0x5410u;
