@@ -250,23 +250,48 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
 // Epilogue of the y1 product: the accumulator tile is y1^T (TMEM lane = feature, column = token), so a
 // lane owns one feature column of every V x 8 block and eight neighbouring lanes own one block.
 // A set of four warps works on a block of V tokens x the CTA's 128 features (16 groups):
-//   pass 1  a warp reads its lanes' V accumulator columns, rounds them to bf16 (this is y1), parks them in the set's
-//           shared memory as [token pair][feature], and accumulates the column score of Section 2.3 in float32,
-//           token by token in ascending order (the order is part of the format);
-//   rank    the eight lanes of a group exchange scores; the four best columns stay (ties to the lower column),
-//           their indices go to colidx and into per-group byte-permute selector tables;
-//   pass 2  one thread per (token, group) takes the group's eight values back from shared memory, applies
-//           SquaredReLU, keeps the two largest of the four kept columns and writes the packed activation,
-//           the packed ReLU values, both metadata forms and the 2:4 view.
-// In pass 2 a warp serves all 16 groups of two token pairs: its stores are whole rows of the CTA's features (64 to 256
-// contiguous bytes a token). With the warps' own 32 features it wrote 16 to 64 bytes of eight tokens, 64 lines an emit
-// against 20, and that traffic through the L1 slowed the main loop, which needs the same shared-memory cycles: y1 at T 8192,
-// D 4096, F 16384 607 -> 588 us.
-// The accumulator is released to the MMA warp as soon as the last block's pass 1 has read it.
-__host__ __device__ constexpr int vnm_stage_bytes(int V) { return V * 256; }
-__host__ __device__ constexpr int vnm_set_bytes(int V) { return vnm_stage_bytes(V) + 16 * 4 + 16 * 7 * 16 + 192; }
+//   pass 1  a warp reads its lanes' V accumulator columns into registers, rounded to bf16 (this is y1) as token pairs, and
+//           sums the column score of Section 2.3 in float32, token by token in ascending order (the order is part of the
+//           format);
+//   rank    the eight lanes of a group exchange scores; the four best columns stay (ties to the lower column). Only they
+//           go to shared memory, ReLU applied, four token pairs to a 16-byte store;
+//   pass 2  one thread per (eight tokens, group): with the kept columns of two tokens in the halves of four words, one
+//           selection serves both tokens; values, ReLU values, both metadata forms, the 2:4 view and the masked copy follow
+//           by byte permutes. The masked copy's selectors belong to the group (a dropped column takes the sign byte of a
+//           value that is not negative), the 2:4 view's come from a table over the pairs of columns.
+// In pass 2 a warp serves all 16 groups of two tokens at a time: its stores are whole rows of the CTA's features (64 to
+// 256 contiguous bytes a token).
+// What bounds it: a set has two main loops' time for a tile, and what it moves through shared memory and the L1 is taken
+// from theirs. With all columns parked in shared memory as [token][feature], selected token by token and the selectors
+// worked out per block, a block took 7300 clocks of its set; this takes 4000. y1 at T 4096, D 2048, F 8192 102 -> 92 us,
+// T 8192, D 4096, F 16384 608 -> 583 us, T 4096, D 512, F 8192 95 -> 78 us.
+__host__ __device__ constexpr int vnm_stage_bytes(int V) { return V * 128; }             // [V / 8][64 kept columns][4 token pairs]
+__host__ __device__ constexpr int vnm_set_bytes(int V) { return 2 * (vnm_stage_bytes(V) + 16 * 4 + 16 * 8); }
+struct VnmTables {
+  uint4 top2[16];            // of a keep mask: {Top2Entry::kept, selector of the two columns' numbers, half masks of the four}
+  uint2 pair[64];            // of columns (a, b), at a + 8 b: {selectors of the 2:4 view's halves, its metadata byte}
+};
+__device__ __forceinline__ void vnm_tables_init(VnmTables* t, int tid) {               // 64 threads
+  uint4 sel;
+  uint32_t nib24;
+  vnm8_pair_selectors((uint32_t)tid & 7u, (uint32_t)tid >> 3, sel, nib24);
+  t->pair[tid] = make_uint2(sel.w, nib24);
+  if (tid < 16) {
+    const uint32_t m = (uint32_t)tid, p0 = __ffs(m) - 1u, p1 = 31u - __clz(m);
+    t->top2[tid] = __popc(m) != 2 ? make_uint4(0u, 0u, 0u, 0u)
+                                  : make_uint4(top2_lut_entry(m).kept, 0x4400u | p0 | (p1 << 4),
+                                               (m & 1u) * 0xFFFFu | (m >> 1 & 1u) * 0xFFFF0000u,
+                                               (m >> 2 & 1u) * 0xFFFFu | (m >> 3 & 1u) * 0xFFFF0000u);
+  }
+}
 constexpr int kSetWarps = 8;                                     // two sets of four: one set per accumulator buffer
-__host__ __device__ constexpr int vnm_epi_bytes(int V) { return 2 * vnm_set_bytes(V); }
+__host__ __device__ constexpr int vnm_epi_bytes(int V) { return 2 * vnm_set_bytes(V) + (int)sizeof(VnmTables); }
+// Byte permute with the sign mode: selector nibble 8 + i gives the sign of byte i in all eight bits.
+__device__ __forceinline__ uint32_t prmt_signed(uint32_t a, uint32_t b, uint32_t sel) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+  return r;
+}
 
 // Barrier of one set of four epilogue warps.
 __device__ __forceinline__ void set_sync(int set) { asm volatile("bar.sync %0, 128;" ::"r"(set + 1) : "memory"); }
@@ -286,17 +311,17 @@ __device__ __forceinline__ bool set_all(int set, bool ok) {
   return r != 0;
 }
 
+// buf: which of the set's two stages this block takes; a warp that has passed the barrier of block n - 1 knows that all have
+// read block n - 2, so one barrier a block is enough.
 template <int kTileN, int kV>
-__device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0,
-                                              int64_t n_limit, int q, int set, int lane, uint8_t* wsm, uint64_t* tmem_empty_bar) {
-  uint32_t* stage = reinterpret_cast<uint32_t*>(wsm);                     // [kV / 2][128 features]
-  uint8_t* cidx = wsm + vnm_stage_bytes(kV);                               // [16 groups][4]
-  uint4* sel_tab = reinterpret_cast<uint4*>(cidx + 16 * 4);               // [16 groups][7]
-  uint8_t* nib_tab = cidx + 16 * 4 + 16 * 7 * 16;                         // [16 groups][7]
-  const int64_t F = args.M, G = F >> 3;
+__device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit, int q,
+                                              int set, int lane, uint8_t* epi_stage, uint32_t& buf, uint64_t* tmem_empty_bar) {
+  const VnmTables* tables = reinterpret_cast<const VnmTables*>(epi_stage + 2 * vnm_set_bytes(kV));
+  const int64_t F = args.M;
+  const int G = (int)(F >> 3);
   const int64_t g0 = m0 >> 3;                                             // the CTA's first group
-  const int jm = lane & 7;
-  const int gl = lane & 15, psub = lane >> 4;                             // pass 2: group, which of two token pairs
+  const int jm = lane & 7, gw = q * 4 + (lane >> 3);                      // pass 1: column of its group, group
+  const int gl = lane & 15, psub = lane >> 4, odd = gl & 1;               // pass 2: group, which of two quads of token pairs
   constexpr int kBlocks = kTileN / kV;
   int nblk = kBlocks;
   while (nblk > 0 && n0 + (int64_t)(nblk - 1) * kV >= n_limit) --nblk;     // ragged last tile: whole blocks only
@@ -304,31 +329,59 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
     release_accumulator(lane, tmem_empty_bar);
     return;
   }
-  // strides per token of the outputs this thread writes (in the units of its pointers)
-  const int sv = (int)G, s24 = (int)(F >> 3), sm = (int)(G >> 2), sm24 = (int)(F >> 5);
-  const bool lead4 = (gl & 3) == 0, lead2 = (gl & 1) == 0;
+  const uint32_t nib_mask = 0xF0000u << (4 * (gl & 3));                  // this group's nibble of its metadata word (high half)
 #pragma unroll 1
-  for (int b = 0; b < kBlocks; ++b) {
-    if (b >= nblk) break;
-    if (b > 0) set_sync(set);                                              // the previous block's pass 2 has read the stage
+  for (int b = 0; b < nblk; ++b, buf ^= 1) {
     const int64_t t0 = n0 + (int64_t)b * kV;
-    // ---- pass 1: two tokens per step on packed bf16 pairs
+    uint8_t* stage = epi_stage + set * vnm_set_bytes(kV) + buf * (vnm_set_bytes(kV) / 2);
+    uint8_t* cidx = stage + vnm_stage_bytes(kV);                           // [16 groups][4] kept columns
+    uint8_t* dsel = cidx + 16 * 4;                                         // [16 groups][8] selector byte of each column
+    // ---- pass 1: the next 32 columns are on their way while these are worked on
     float score = 0.f;
-    uint32_t v[32];
-#pragma unroll 1
-    for (int c = 0; c < kV / 32; ++c) {
-      tmem_ld_32x32b_x32(taddr + (uint32_t)(b * kV + c * 32), v);
-      tmem_ld_wait_on(v);
+    uint32_t yp[kV / 2], va[32], vb[32];
+    auto take = [&](const uint32_t (&v)[32], int c) {
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const uint32_t yp = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
-        stage[(c * 16 + j) * 128 + q * 32 + lane] = yp;
-        const uint32_t hp = bf2_sq(bf2_relu(yp));
-        score = __fadd_rn(score, __uint_as_float(hp << 16));
-        score = __fadd_rn(score, __uint_as_float(hp & 0xFFFF0000u));
-      }
+      for (int j = 0; j < 16; ++j) yp[c * 16 + j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+    };
+    tmem_ld_32x32b_x32(taddr + (uint32_t)(b * kV), va);
+#pragma unroll
+    for (int c = 0; c < kV / 32; c += 2) {
+      tmem_ld_wait_on(va);
+      tmem_ld_32x32b_x32(taddr + (uint32_t)(b * kV + c * 32 + 32), vb);
+      take(va, c);
+      tmem_ld_wait_on(vb);
+      if (c + 2 < kV / 32) tmem_ld_32x32b_x32(taddr + (uint32_t)(b * kV + c * 32 + 64), va);
+      take(vb, c + 1);
     }
     if (b == nblk - 1) release_accumulator(lane, tmem_empty_bar);
+    if (args.vn_y1) {
+      // y1 itself, through this warp's quarter of the stage, 32 tokens at a time
+      uint32_t* st = reinterpret_cast<uint32_t*>(stage + q * (vnm_stage_bytes(kV) / 4));
+#pragma unroll
+      for (int c = 0; c < kV / 32; ++c) {
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 16; ++j) st[j * 32 + lane] = yp[c * 16 + j];
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          uint32_t r0[4], r1[4];
+          const int pr = i * 8 + (lane >> 2);
+          pair_rows(st + pr * 32 + (lane & 3) * 8, lane, r0, r1);
+          uint16_t* y = reinterpret_cast<uint16_t*>(args.vn_y1) + (t0 + c * 32 + 2 * pr) * F + m0 + q * 32 + (lane & 3) * 8;
+          *reinterpret_cast<uint4*>(y) = make_uint4(r0[0], r0[1], r0[2], r0[3]);
+          *reinterpret_cast<uint4*>(y + F) = make_uint4(r1[0], r1[1], r1[2], r1[3]);
+        }
+      }
+      set_sync(set);                                                       // the quarters have been read
+    }
+#pragma unroll
+    for (int j = 0; j < kV / 2; ++j) {
+      yp[j] = bf2_relu(yp[j]);
+      const uint32_t hp = bf2_sq(yp[j]);
+      score = __fadd_rn(score, __uint_as_float(hp << 16));
+      score = __fadd_rn(score, __uint_as_float(hp & 0xFFFF0000u));
+    }
     // ---- rank the eight columns of each group
     const uint32_t sb = __float_as_uint(score);                            // scores are >= 0: the pattern orders them
     int rank = 0;
@@ -339,100 +392,89 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
       rank += (o > sb) || (o == sb && oj < jm);
     }
     const bool keep = rank < 4;
-    const uint32_t ball = __ballot_sync(0xFFFFFFFFu, keep);
-    const uint32_t gbyte = (ball >> (lane & 24)) & 0xFFu;
-    if (keep) cidx[(q * 4 + (lane >> 3)) * 4 + __popc(gbyte & ((1u << jm) - 1u))] = (uint8_t)jm;
-    __syncwarp();
-    if (lane < 4)
-      *reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(args.vn_colidx) + ((t0 / kV) * G + g0 + q * 4 + lane) * 4) =
-          *reinterpret_cast<const uint32_t*>(cidx + (q * 4 + lane) * 4);
-    if (lane < 24) {
-      const int ge = q * 4 + lane / 6, pe = lane % 6;
-      const int pi = pe < 3 ? 0 : (pe < 5 ? 1 : 2), pj = pe < 3 ? pe + 1 : (pe < 5 ? pe - 1 : 3);
-      uint4 selv;
-      uint32_t nib24;
-      vnm8_pair_selectors(cidx[ge * 4 + pi], cidx[ge * 4 + pj], selv, nib24);
-      const int slot = ge * 7 + (int)nib_slot((uint32_t)pi | ((uint32_t)pj << 2));
-      sel_tab[slot] = selv;
-      nib_tab[slot] = (uint8_t)nib24;
+    const uint32_t gbyte = (__ballot_sync(0xFFFFFFFFu, keep) >> (lane & 24)) & 0xFFu;
+    const int pos = __popc(gbyte & ((1u << jm) - 1u));
+    // bytes 2 pos and 2 pos + 1 of the four kept values, or the sign (zero) of byte 1
+    dsel[gw * 8 + jm] = keep ? (uint8_t)(0x10 + 0x22 * pos) : (uint8_t)0x99;
+    if (keep) {
+      cidx[gw * 4 + pos] = (uint8_t)jm;
+      // unit of column pos: XOR-ed so that eight neighbouring groups' units of one column lie in different banks
+      uint4* dst = reinterpret_cast<uint4*>(stage) + gw * 4 + (pos ^ ((gw >> 1) & 3));
+#pragma unroll
+      for (int u = 0; u < kV / 8; ++u) dst[u * 64] = make_uint4(yp[4 * u], yp[4 * u + 1], yp[4 * u + 2], yp[4 * u + 3]);
     }
-    set_sync(set);                                                         // all 128 features of the block are in
-    // ---- pass 2: this thread serves group gl of the token pairs 2 q + psub + 8 * it
+    set_sync(set);                                                         // the kept columns of all 128 features are in
+    // ---- pass 2
     const uint32_t c4 = *reinterpret_cast<const uint32_t*>(cidx + gl * 4);
-    uint32_t selp[2], mhi[2];
-#pragma unroll
-    for (int pr = 0; pr < 2; ++pr) {
-      const uint32_t ca = (c4 >> (16 * pr)) & 0xFFu, cb = (c4 >> (16 * pr + 8)) & 0xFFu;
-      const uint32_t sa = 2u * (ca & 3u), sbb = 2u * (cb & 3u);
-      selp[pr] = sa | ((sa + 1u) << 4) | (sbb << 8) | ((sbb + 1u) << 12);
-      mhi[pr] = ((ca & 4u) ? 0x0000FFFFu : 0u) | ((cb & 4u) ? 0xFFFF0000u : 0u);
-    }
-    const uint4* my_sel = sel_tab + gl * 7;
-    const uint8_t* my_nib = nib_tab + gl * 7;
-    // output pointers of this thread's first token; every pointer advances by a constant per token
-    const int pair0 = 2 * q + psub;
-    const int64_t tf = t0 + 2 * pair0;
-    uint32_t* p_vals = reinterpret_cast<uint32_t*>(args.vn_vals) + tf * G + g0 + gl;
-    uint32_t* p_relu = reinterpret_cast<uint32_t*>(args.vn_relu) + tf * G + g0 + gl;
-    uint2* p_v24 = reinterpret_cast<uint2*>(args.vn_vals24) + tf * (F >> 3) + g0 + gl;
-    uint2* p_r24 = reinterpret_cast<uint2*>(args.vn_relu24) + tf * (F >> 3) + g0 + gl;
-    uint4* p_y1 = args.vn_y1 ? reinterpret_cast<uint4*>(args.vn_y1) + tf * (F >> 3) + g0 + gl : nullptr;
-    uint4* p_dense = args.vn_dense ? reinterpret_cast<uint4*>(args.vn_dense) + tf * (F >> 3) + g0 + gl : nullptr;
-    uint16_t* p_meta = reinterpret_cast<uint16_t*>(args.vn_meta) + tf * (G >> 2) + ((g0 + gl) >> 2);
-    uint32_t* p_m24 = reinterpret_cast<uint32_t*>(args.vn_meta24) + tf * (F >> 5) + ((g0 + gl) >> 2);
-    // tensor-core-ordered copy: the block lies inside one 128-row band, so the atom is fixed
-    const int64_t kw24 = (m0 >> 4) + (gl >> 1);
-    uint8_t* hw_atom = reinterpret_cast<uint8_t*>(args.vn_meta24_hw) + meta_hw_offset(t0 & ~int64_t(127), kw24, F);
-    const uint32_t* sp = stage + pair0 * 128 + gl * 8;
-
-    auto emit = [&](const uint32_t (&yw)[4], int dt, uint32_t trow) {
-      uint32_t rw[4], hw[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) { rw[j] = bf2_relu(yw[j]); hw[j] = bf2_sq(rw[j]); }
-      const uint32_t a0 = __byte_perm(hw[0], hw[1], selp[0]), b0 = __byte_perm(hw[2], hw[3], selp[0]);
-      const uint32_t a1 = __byte_perm(hw[0], hw[1], selp[1]), b1 = __byte_perm(hw[2], hw[3], selp[1]);
-      const uint32_t hk0 = (a0 & ~mhi[0]) | (b0 & mhi[0]), hk1 = (a1 & ~mhi[1]) | (b1 & mhi[1]);
-      uint32_t packed;
-      const uint32_t nib = top2of4_packed(hk0, hk1, &packed);
-      const uint32_t slot = nib_slot(nib);
-      const uint4 sel = my_sel[slot];
-      const uint32_t x = __byte_perm(rw[0], rw[1], sel.z), y = __byte_perm(rw[2], rw[3], sel.z);
-      const uint32_t rpair = __byte_perm(x, y, sel.z >> 16);
-      p_vals[dt * sv] = packed;
-      p_relu[dt * sv] = rpair;
-      p_v24[dt * s24] = make_uint2(__byte_perm(packed, 0u, sel.w), __byte_perm(packed, 0u, sel.w >> 16));
-      p_r24[dt * s24] = make_uint2(__byte_perm(rpair, 0u, sel.w), __byte_perm(rpair, 0u, sel.w >> 16));
-      if (p_y1) p_y1[dt * s24] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
-      if (p_dense)
-        p_dense[dt * s24] = make_uint4(__byte_perm(packed, 0u, sel.x), __byte_perm(packed, 0u, sel.x >> 16),
-                                       __byte_perm(packed, 0u, sel.y), __byte_perm(packed, 0u, sel.y >> 16));
-      // canonical V:N:M metadata: the warp's four groups of a token form one word
-      uint32_t word = nib;
-      word |= __shfl_down_sync(0xFFFFFFFFu, word, 1) << 4;
-      word |= __shfl_down_sync(0xFFFFFFFFu, word, 2) << 8;
-      if (lead4) p_meta[dt * sm] = (uint16_t)word;
-      // metadata of the 2:4 view: one byte per group, one 16-bit word per pair of groups
-      uint32_t mb = my_nib[slot];
-      mb |= __shfl_down_sync(0xFFFFFFFFu, mb, 1) << 8;
-      const uint32_t mb32 = (mb & 0xFFFFu) | (__shfl_down_sync(0xFFFFFFFFu, mb, 2) << 16);
-      if (lead4) p_m24[dt * sm24] = mb32;
-      if (lead2) {
-        const uint32_t mi = trow & 127u;
-        *reinterpret_cast<uint16_t*>(hw_atom + (mi >> 4) * 256u + (mi & 7u) * 16u + ((mi >> 3) & 1u) * 2u) = (uint16_t)mb;
-      }
-    };
+    const uint2 ds = *reinterpret_cast<const uint2*>(dsel + gl * 8);
+    if (q == 0 && psub == 0)
+      *reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(args.vn_colidx) + ((t0 / kV) * G + g0 + gl) * 4) = c4;
 #pragma unroll 1
-    for (int it = 0; it < kV / 16; ++it) {
-      uint32_t r0[4], r1[4];
-      pair_rows(sp, lane, r0, r1);
-      const uint32_t trow = (uint32_t)(tf & 127) + 16u * (uint32_t)it;
-      emit(r0, 0, trow);
-      emit(r1, 1, trow + 1u);
-      sp += 8 * 128;
-      p_vals += 16 * sv; p_relu += 16 * sv; p_v24 += 16 * s24; p_r24 += 16 * s24;
-      if (p_y1) p_y1 += 16 * s24;
-      if (p_dense) p_dense += 16 * s24;
-      p_meta += 16 * sm; p_m24 += 16 * sm24;
+    for (int u = 2 * q + psub; u < kV / 8; u += 8) {
+      const int64_t t = t0 + 8 * u;                                        // this thread's first token
+      const int64_t at = t * G + g0 + gl;
+      uint32_t* p_vals = reinterpret_cast<uint32_t*>(args.vn_vals) + at;
+      uint32_t* p_relu = reinterpret_cast<uint32_t*>(args.vn_relu) + at;
+      uint2* p_v24 = reinterpret_cast<uint2*>(args.vn_vals24) + at;
+      uint2* p_r24 = reinterpret_cast<uint2*>(args.vn_relu24) + at;
+      uint4* p_dense = args.vn_dense ? reinterpret_cast<uint4*>(args.vn_dense) + at : nullptr;
+      // the metadata of four groups is one word: their first two lanes write a token each
+      const int64_t atm = (t + odd) * (G >> 2) + ((g0 + gl) >> 2);
+      uint16_t* p_meta = reinterpret_cast<uint16_t*>(args.vn_meta) + atm;
+      uint32_t* p_m24 = reinterpret_cast<uint32_t*>(args.vn_meta24) + atm;
+      // tensor-core-ordered copy: eight tokens are one column of 16-byte rows of an atom
+      uint8_t* p_hw = reinterpret_cast<uint8_t*>(args.vn_meta24_hw) + meta_hw_offset(t, (m0 >> 4) + (gl >> 1), F) + odd * 16;
+      const uint4* src = reinterpret_cast<const uint4*>(stage) + u * 64 + gl * 4;
+      const int sw = (gl >> 1) & 3;
+      const uint4 x0 = src[sw], x1 = src[1 ^ sw], x2 = src[2 ^ sw], x3 = src[3 ^ sw];
+      // two tokens: r_i holds kept column i of both
+      auto emit = [&](uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3, int k) {
+        const uint32_t e = 2u * top2_offsets_x2(bf2_sq(r0), bf2_sq(r1), bf2_sq(r2), bf2_sq(r3));
+        const uint8_t* base = reinterpret_cast<const uint8_t*>(tables->top2);
+        uint4 ent[2];
+        ent[0] = *reinterpret_cast<const uint4*>(base + (e & 0xFFFFu));
+        ent[1] = *reinterpret_cast<const uint4*>(base + (e >> 16));
+        uint32_t mb[2];
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+          const uint32_t half = d ? 0x7632u : 0x5410u;
+          const uint32_t ra = __byte_perm(r0, r1, half), rb = __byte_perm(r2, r3, half);
+          const uint32_t ha = bf2_sq(ra), hb = bf2_sq(rb);
+          const uint32_t packed = __byte_perm(ha, hb, ent[d].x), rpair = __byte_perm(ra, rb, ent[d].x);
+          const int off = (2 * k + d) * G;
+          p_vals[off] = packed;
+          p_relu[off] = rpair;
+          // {selectors, metadata byte} of the two columns: 8 a + 64 b
+          const uint2 pe = *reinterpret_cast<const uint2*>(reinterpret_cast<const uint8_t*>(tables->pair) +
+                                                           __dp4a(__byte_perm(c4, 0u, ent[d].y), 0x4008u, 0u));
+          const uint32_t sel = pe.x;
+          mb[d] = pe.y;
+          p_v24[off] = make_uint2(__byte_perm(packed, 0u, sel), __byte_perm(packed, 0u, sel >> 16));
+          p_r24[off] = make_uint2(__byte_perm(rpair, 0u, sel), __byte_perm(rpair, 0u, sel >> 16));
+          if (p_dense) {
+            const uint32_t za = ha & ent[d].z, zb = hb & ent[d].w;
+            p_dense[off] = make_uint4(prmt_signed(za, zb, ds.x), prmt_signed(za, zb, ds.x >> 16), prmt_signed(za, zb, ds.y),
+                                      prmt_signed(za, zb, ds.y >> 16));
+          }
+        }
+        // even token in the low half, odd token in the high half
+        uint32_t w = ((ent[0].x & nib_mask) >> 16) | (ent[1].x & nib_mask);
+        w |= __shfl_xor_sync(0xFFFFFFFFu, w, 1);
+        w |= __shfl_xor_sync(0xFFFFFFFFu, w, 2);
+        uint32_t m = (mb[0] | (mb[1] << 16)) << (8 * odd);
+        m |= __shfl_xor_sync(0xFFFFFFFFu, m, 1);
+        const uint32_t m2 = __shfl_xor_sync(0xFFFFFFFFu, m, 2);
+        *reinterpret_cast<uint16_t*>(p_hw + k * 32) = (uint16_t)(odd ? m >> 16 : m);
+        if ((gl & 2) == 0) {
+          const int off = 2 * k * (G >> 2);
+          p_meta[off] = (uint16_t)(odd ? w >> 16 : w);
+          p_m24[off] = __byte_perm(m, m2, odd ? 0x7632u : 0x5410u);
+        }
+      };
+      emit(x0.x, x1.x, x2.x, x3.x, 0);
+      emit(x0.y, x1.y, x2.y, x3.y, 1);
+      emit(x0.z, x1.z, x2.z, x3.z, 2);
+      emit(x0.w, x1.w, x2.w, x3.w, 3);
     }
   }
 }
@@ -642,7 +684,7 @@ __global__ void __launch_bounds__(kMode == MODE_VENOM ? kThreadsVenom : kThreads
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB,
                const GemmArgs args) {
   extern __shared__ uint8_t smem_dyn[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t1023);
   constexpr bool kSparse = kMode != MODE_DENSE;
   constexpr int kStages = num_stages(kSparse);
   constexpr int kAStageBytes = a_stage_bytes(kSparse);
@@ -984,7 +1026,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
                 const __grid_constant__ CUtensorMap tmapMeta, const __grid_constant__ CUtensorMap tmapPk,
                 const GemmArgs args) {
   extern __shared__ uint8_t smem_dyn[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t1023);
   constexpr bool kSparse = kMode == MODE_SPARSE24;
   constexpr int kStages = num_stages2(kSparse, kBN, kExpand != 0);
   constexpr int kBK = kSparse ? 128 : 64;                // logical K per stage
@@ -1040,6 +1082,8 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   if ((kExpand || is_drelu_t(kEpi) || kEpi == EPI_ACT24_T) && threadIdx.x >= 64 && threadIdx.x < 80) {
     ctl->expand_lut[threadIdx.x - 64] = expand_lut_entry(threadIdx.x - 64);
   }
+  if (kEpi == EPI_VNM8 && threadIdx.x >= 64 && threadIdx.x < 128)
+    vnm_tables_init(reinterpret_cast<VnmTables*>(epi_stage + 2 * vnm_set_bytes(vnm_block(kBN))), (int)threadIdx.x - 64);
   if (kEpi == EPI_ACT24_T && threadIdx.x >= 96) top2_lut_init(ctl->top2_lut, (int)threadIdx.x - 96);
   if (warp == 1) {
     tmem_alloc_2cta(&ctl->tmem_base, kTmemCols);
@@ -1228,7 +1272,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     const int q = warp & 3, set = (warp - 2) >> 2;
     uint8_t* wsm = epi_stage + (set * 4 + q) * (epi_bytes2(kEpi, kBN) / kSetWarps);
     const uint32_t taddr = tmem_base + set * kBN + ((uint32_t)(q * 32) << 16);
-    uint32_t acc_phase = 0;
+    uint32_t acc_phase = 0, vnm_buf = 0;
     for (int tile = pair + set * num_pairs; tile < num_tiles; tile += 2 * num_pairs) {
       const GemmTile tc = get_tile<kBN, kVar, kDual>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
       const int64_t m0 = (int64_t)tc.out_m + (int64_t)rank * 128, n0 = tc.out_n, n_limit = tc.n_limit;
@@ -1248,8 +1292,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
         if (!live) {
           release_accumulator(lane, &ctl->tmem_empty[set]);
         } else if constexpr (kEpi == EPI_VNM8) {
-          epi_vnm8_tile<kBN, vnm_block(kBN)>(args, taddr, m0, n0, n_limit, q, set, lane, epi_stage + set * vnm_set_bytes(vnm_block(kBN)),
-                                             &ctl->tmem_empty[set]);
+          epi_vnm8_tile<kBN, vnm_block(kBN)>(args, taddr, m0, n0, n_limit, q, set, lane, epi_stage, vnm_buf, &ctl->tmem_empty[set]);
         } else {
           epi_act24_tile<kBN>(args, taddr, m0, n0, n_limit, q, lane, reinterpret_cast<uint32_t*>(wsm), ctl->expand_lut,
                               ctl->top2_lut, &ctl->tmem_empty[set]);
@@ -1361,7 +1404,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTallThreads, 1)
 gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB,
                  const __grid_constant__ CUtensorMap tmapBn, const __grid_constant__ CUtensorMap tmapMeta, const GemmArgs args) {
   extern __shared__ uint8_t smem_dyn[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t1023);
   constexpr int kBBytes = tall_b_bytes(kBMN), kMetaBytes = meta_stage_bytes2(kFp8), kStageBytes = tall_stage_bytes(kBMN, kFp8);
   constexpr int kMetaAt = kBBytes + 2 * 16384;            // stage: B columns, A of either half, metadata of either half
   constexpr int kSlab = (kTallBN / 2) * 128;              // K-major: this CTA's half of B for one 64-wide K slab

@@ -145,9 +145,9 @@ __device__ __forceinline__ void top2_lut_init(Top2Entry* lut, int tid) {
 // kFma: the six subtractions are written as multiply-adds by -1 (blockDim.z is 1 in every launch here, which the compiler
 // does not know), so they issue on the FMA pipe. For the strided prune kernel, which runs out of the integer pipe (42.4 ->
 // 41.1 us at 4096 x 16384); the others are slower by half a percent with it.
-template <bool kDropped = false, bool kFma = false>
-__device__ __forceinline__ void top2of4_x2(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, const Top2Entry* lut,
-                                           Top2Entry& entry_a, Top2Entry& entry_b) {
+// top2_offsets_x2: the byte offsets of the two groups' entries in the table, in the halves of a word.
+template <bool kFma = false>
+__device__ __forceinline__ uint32_t top2_offsets_x2(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3) {
   constexpr uint32_t kMag = 0x7FFF7FFFu, kTop = 0x80008000u;
   const uint32_t m1 = x1 & kMag, m2 = x2 & kMag, m3 = x3 & kMag;
   const uint32_t o0 = x0 | kTop, o1 = x1 | kTop, o2 = x2 | kTop;
@@ -160,8 +160,13 @@ __device__ __forceinline__ void top2of4_x2(uint32_t x0, uint32_t x1, uint32_t x2
   const uint32_t k2 = (~g02 & ~g12) | (~g02 & g23) | (~g12 & g23);
   const uint32_t k3 = ~((g03 & g13) | (g03 & g23) | (g13 & g23));
   // flags (bits 15 and 31) -> byte offsets into the table (bits 3..6 of either half)
-  const uint32_t t = ((k0 >> 12) & 0x00080008u) | ((k1 >> 11) & 0x00100010u) | ((k2 >> 10) & 0x00200020u) |
-                     ((k3 >> 9) & 0x00400040u);
+  return ((k0 >> 12) & 0x00080008u) | ((k1 >> 11) & 0x00100010u) | ((k2 >> 10) & 0x00200020u) |
+         ((k3 >> 9) & 0x00400040u);
+}
+template <bool kDropped = false, bool kFma = false>
+__device__ __forceinline__ void top2of4_x2(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, const Top2Entry* lut,
+                                           Top2Entry& entry_a, Top2Entry& entry_b) {
+  const uint32_t t = top2_offsets_x2<kFma>(x0, x1, x2, x3);
   const uint8_t* base = reinterpret_cast<const uint8_t*>(lut);
   if (kDropped) {
     const uint2 a = *reinterpret_cast<const uint2*>(base + (t & 0xFFFFu)), b = *reinterpret_cast<const uint2*>(base + (t >> 16));
