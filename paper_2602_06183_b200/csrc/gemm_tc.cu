@@ -684,7 +684,7 @@ __global__ void __launch_bounds__(kMode == MODE_VENOM ? kThreadsVenom : kThreads
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB,
                const GemmArgs args) {
   extern __shared__ uint8_t smem_dyn[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t1023);
+  uint8_t* smem = smem_dyn + align_pad(smem_dyn, 1024);
   constexpr bool kSparse = kMode != MODE_DENSE;
   constexpr int kStages = num_stages(kSparse);
   constexpr int kAStageBytes = a_stage_bytes(kSparse);
@@ -1026,7 +1026,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
                 const __grid_constant__ CUtensorMap tmapMeta, const __grid_constant__ CUtensorMap tmapPk,
                 const GemmArgs args) {
   extern __shared__ uint8_t smem_dyn[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t1023);
+  uint8_t* smem = smem_dyn + align_pad(smem_dyn, 1024);
   constexpr bool kSparse = kMode == MODE_SPARSE24;
   constexpr int kStages = num_stages2(kSparse, kBN, kExpand != 0);
   constexpr int kBK = kSparse ? 128 : 64;                // logical K per stage
@@ -1404,7 +1404,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTallThreads, 1)
 gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB,
                  const __grid_constant__ CUtensorMap tmapBn, const __grid_constant__ CUtensorMap tmapMeta, const GemmArgs args) {
   extern __shared__ uint8_t smem_dyn[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t1023);
+  uint8_t* smem = smem_dyn + align_pad(smem_dyn, 1024);
   constexpr int kBBytes = tall_b_bytes(kBMN), kMetaBytes = meta_stage_bytes2(kFp8), kStageBytes = tall_stage_bytes(kBMN, kFp8);
   constexpr int kMetaAt = kBBytes + 2 * 16384;            // stage: B columns, A of either half, metadata of either half
   constexpr int kSlab = (kTallBN / 2) * 128;              // K-major: this CTA's half of B for one 64-wide K slab

@@ -14,6 +14,10 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// Bytes from `p` (dynamic shared memory) to the next multiple of `align`. Adding them to the pointer, instead of rounding its
+// address as an integer, lets the compiler see that what is derived from it is shared memory.
+__device__ __forceinline__ uint32_t align_pad(const void* p, uint32_t align) { return (0u - smem_u32(p)) & (align - 1u); }
+
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred = 0;
   asm volatile(

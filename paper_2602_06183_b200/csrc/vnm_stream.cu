@@ -45,7 +45,7 @@ vnm_stream_kernel(const __grid_constant__ CUtensorMap tmapP, int64_t T, int64_t 
                    uint16_t* __restrict__ vals, uint16_t* __restrict__ meta, uint8_t* __restrict__ colidx,
                    uint16_t* __restrict__ relu_vals) {
   extern __shared__ uint8_t smem_dyn[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 127) & ~uintptr_t(127));
+  uint8_t* smem = smem_dyn + align_pad(smem_dyn, 128);
   const int strip_bytes = V * kSW * 2;
   using Aux = StripAux<kSW>;
   Aux* aux = reinterpret_cast<Aux*>(smem + kSlots * strip_bytes);
@@ -272,7 +272,7 @@ vnm8_stream_kernel(const __grid_constant__ CUtensorMap tmapP, int64_t T, int64_t
                    uint4* __restrict__ vals, uint16_t* __restrict__ meta, uint32_t* __restrict__ colidx,
                    uint4* __restrict__ relu_vals) {
   extern __shared__ uint8_t smem_dyn[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = smem_dyn + align_pad(smem_dyn, 1024);
   const int strip_bytes = V * kSW * 2, seg_bytes = V * 128;
   constexpr int kGS = kSW / 8;                              // groups per strip
   Stream8Sel* sel = reinterpret_cast<Stream8Sel*>(smem + nslots * strip_bytes);     // [nslots][kGS]
