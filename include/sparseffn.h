@@ -60,10 +60,8 @@ typedef enum sf_ffn_flags {
   SF_FFN_SAVE_Y1 = 1,     /* also store the full bf16 pre-activation y1 in the context (SF_CTX_Y1) */
   SF_FFN_UNFUSED_ACT = 2, /* M == 8: run SquaredReLU + V:N:M as its own kernel on a stored y1, never inside the
                              y1 product's epilogue */
-  SF_FFN_FUSED_ACT = 4,   /* M == 8: run them inside the y1 product's epilogue whenever the shape allows. With
-                             neither bit the library fuses for V == 64 (token tiles of three blocks) and not for
-                             V == 128 (a one-block tile re-reads the weight operand too often). Same results
-                             either way, bit for bit. */
+  SF_FFN_FUSED_ACT = 4,   /* M == 8: run them inside the y1 product's epilogue whenever the shape allows, which is
+                             also what happens with neither bit. Same results either way, bit for bit. */
   SF_FFN_PACKED_GRAD_OPERANDS = 8 /* M == 8: keep no masked [T, F] copy of y2 and dy1; the two weight-gradient
                              products expand their operand from its packed form inside the kernel. Saves
                              4*T*F bytes of context + workspace, costs about a third more time in those two

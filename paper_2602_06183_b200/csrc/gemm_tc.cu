@@ -265,8 +265,8 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
 // from theirs. With all columns parked in shared memory as [token][feature], selected token by token and the selectors
 // worked out per block, a block took 7300 clocks of its set; this takes 4000. y1 at T 4096, D 2048, F 8192 102 -> 92 us,
 // T 8192, D 4096, F 16384 608 -> 583 us, T 4096, D 512, F 8192 95 -> 78 us.
-__host__ __device__ constexpr int vnm_stage_bytes(int V) { return V * 128; }             // [V / 8][64 kept columns][4 token pairs]
-__host__ __device__ constexpr int vnm_set_bytes(int V) { return 2 * (vnm_stage_bytes(V) + 16 * 4 + 16 * 8); }
+constexpr int kVnmStageBytes = 64 * 128;                                 // 64 tokens: [8][64 kept columns][4 token pairs]
+constexpr int kVnmSetBytes = kVnmStageBytes + 16 * 4 + 16 * 8;
 struct VnmTables {
   uint4 top2[16];            // of a keep mask: {Top2Entry::kept, selector of the two columns' numbers, half masks of the four}
   uint2 pair[64];            // of columns (a, b), at a + 8 b: {selectors of the 2:4 view's halves, its metadata byte}
@@ -285,7 +285,7 @@ __device__ __forceinline__ void vnm_tables_init(VnmTables* t, int tid) {        
   }
 }
 constexpr int kSetWarps = 8;                                     // two sets of four: one set per accumulator buffer
-__host__ __device__ constexpr int vnm_epi_bytes(int V) { return 2 * vnm_set_bytes(V) + (int)sizeof(VnmTables); }
+constexpr int kVnmEpiBytes = 2 * kVnmSetBytes + (int)sizeof(VnmTables);
 // Byte permute with the sign mode: selector nibble 8 + i gives the sign of byte i in all eight bits.
 __device__ __forceinline__ uint32_t prmt_signed(uint32_t a, uint32_t b, uint32_t sel) {
   uint32_t r;
@@ -311,54 +311,60 @@ __device__ __forceinline__ bool set_all(int set, bool ok) {
   return r != 0;
 }
 
-// buf: which of the set's two stages this block takes; a warp that has passed the barrier of block n - 1 knows that all have
-// read block n - 2, so one barrier a block is enough.
-template <int kTileN, int kV>
+// kCols: columns of the tile that this set takes at most; kStep: tokens in registers at a time (64: V = 64 only,
+// with less code and fewer registers).
+template <int kCols, int kStep>
 __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit, int q,
-                                              int set, int lane, uint8_t* epi_stage, uint32_t& buf, uint64_t* tmem_empty_bar) {
-  const VnmTables* tables = reinterpret_cast<const VnmTables*>(epi_stage + 2 * vnm_set_bytes(kV));
+                                              int set, int lane, uint8_t* epi_stage, uint64_t* tmem_empty_bar) {
+  const VnmTables* tables = reinterpret_cast<const VnmTables*>(epi_stage + 2 * kVnmSetBytes);
   const int64_t F = args.M;
   const int G = (int)(F >> 3);
   const int64_t g0 = m0 >> 3;                                             // the CTA's first group
   const int jm = lane & 7, gw = q * 4 + (lane >> 3);                      // pass 1: column of its group, group
   const int gl = lane & 15, psub = lane >> 4, odd = gl & 1;               // pass 2: group, which of two quads of token pairs
-  constexpr int kBlocks = kTileN / kV;
-  int nblk = kBlocks;
-  while (nblk > 0 && n0 + (int64_t)(nblk - 1) * kV >= n_limit) --nblk;     // ragged last tile: whole blocks only
-  if (nblk == 0) {
+  const int cols = (int)min((int64_t)kCols, n_limit - n0);                // ragged last tile: whole blocks only
+  if (cols <= 0) {
     release_accumulator(lane, tmem_empty_bar);
     return;
   }
+  const bool tall = kStep == 128 && args.V == 128;                        // (64 otherwise)
   const uint32_t nib_mask = 0xF0000u << (4 * (gl & 3));                  // this group's nibble of its metadata word (high half)
+  uint8_t* stage = epi_stage + set * kVnmSetBytes;
+  uint8_t* cidx = stage + kVnmStageBytes;                                  // [16 groups][4] kept columns
+  uint8_t* dsel = cidx + 16 * 4;                                           // [16 groups][8] selector byte of each column
 #pragma unroll 1
-  for (int b = 0; b < nblk; ++b, buf ^= 1) {
-    const int64_t t0 = n0 + (int64_t)b * kV;
-    uint8_t* stage = epi_stage + set * vnm_set_bytes(kV) + buf * (vnm_set_bytes(kV) / 2);
-    uint8_t* cidx = stage + vnm_stage_bytes(kV);                           // [16 groups][4] kept columns
-    uint8_t* dsel = cidx + 16 * 4;                                         // [16 groups][8] selector byte of each column
-    // ---- pass 1: the next 32 columns are on their way while these are worked on
-    float score = 0.f;
-    uint32_t yp[kV / 2], va[32], vb[32];
+  for (int c0 = 0; c0 < cols; c0 += kStep) {
+    // ---- pass 1, kStep tokens (or the tile's last 64): the next 32 columns are on their way while these are worked on
+    const bool both = kStep == 128 && cols - c0 > 64;
+    uint32_t yp[kStep / 2], va[32], vb[32];
     auto take = [&](const uint32_t (&v)[32], int c) {
 #pragma unroll
       for (int j = 0; j < 16; ++j) yp[c * 16 + j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
     };
-    tmem_ld_32x32b_x32(taddr + (uint32_t)(b * kV), va);
-#pragma unroll
-    for (int c = 0; c < kV / 32; c += 2) {
-      tmem_ld_wait_on(va);
-      tmem_ld_32x32b_x32(taddr + (uint32_t)(b * kV + c * 32 + 32), vb);
-      take(va, c);
-      tmem_ld_wait_on(vb);
-      if (c + 2 < kV / 32) tmem_ld_32x32b_x32(taddr + (uint32_t)(b * kV + c * 32 + 64), va);
-      take(vb, c + 1);
+    tmem_ld_32x32b_x32(taddr + (uint32_t)c0, va);
+    tmem_ld_wait_on(va);
+    tmem_ld_32x32b_x32(taddr + (uint32_t)(c0 + 32), vb);
+    take(va, 0);
+    tmem_ld_wait_on(vb);
+    if (both) tmem_ld_32x32b_x32(taddr + (uint32_t)(c0 + 64), va);
+    take(vb, 1);
+    if constexpr (kStep == 128) {
+      if (both) {
+        tmem_ld_wait_on(va);
+        tmem_ld_32x32b_x32(taddr + (uint32_t)(c0 + 96), vb);
+        take(va, 2);
+        tmem_ld_wait_on(vb);
+        take(vb, 3);
+      }
     }
-    if (b == nblk - 1) release_accumulator(lane, tmem_empty_bar);
+    if (c0 + kStep >= cols) release_accumulator(lane, tmem_empty_bar);
     if (args.vn_y1) {
+      if (c0 > 0) set_sync(set);
       // y1 itself, through this warp's quarter of the stage, 32 tokens at a time
-      uint32_t* st = reinterpret_cast<uint32_t*>(stage + q * (vnm_stage_bytes(kV) / 4));
+      uint32_t* st = reinterpret_cast<uint32_t*>(stage + q * (kVnmStageBytes / 4));
 #pragma unroll
-      for (int c = 0; c < kV / 32; ++c) {
+      for (int c = 0; c < kStep / 32; ++c) {
+        if (c >= 2 && !both) break;
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < 16; ++j) st[j * 32 + lane] = yp[c * 16 + j];
@@ -368,49 +374,69 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
           uint32_t r0[4], r1[4];
           const int pr = i * 8 + (lane >> 2);
           pair_rows(st + pr * 32 + (lane & 3) * 8, lane, r0, r1);
-          uint16_t* y = reinterpret_cast<uint16_t*>(args.vn_y1) + (t0 + c * 32 + 2 * pr) * F + m0 + q * 32 + (lane & 3) * 8;
+          uint16_t* y = reinterpret_cast<uint16_t*>(args.vn_y1) + (n0 + c0 + c * 32 + 2 * pr) * F + m0 + q * 32 + (lane & 3) * 8;
           *reinterpret_cast<uint4*>(y) = make_uint4(r0[0], r0[1], r0[2], r0[3]);
           *reinterpret_cast<uint4*>(y + F) = make_uint4(r1[0], r1[1], r1[2], r1[3]);
         }
       }
       set_sync(set);                                                       // the quarters have been read
     }
-#pragma unroll
-    for (int j = 0; j < kV / 2; ++j) {
-      yp[j] = bf2_relu(yp[j]);
-      const uint32_t hp = bf2_sq(yp[j]);
-      score = __fadd_rn(score, __uint_as_float(hp << 16));
-      score = __fadd_rn(score, __uint_as_float(hp & 0xFFFF0000u));
-    }
-    // ---- rank the eight columns of each group
-    const uint32_t sb = __float_as_uint(score);                            // scores are >= 0: the pattern orders them
-    int rank = 0;
-#pragma unroll
-    for (int i = 1; i < 8; ++i) {
-      const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, sb, i);
-      const int oj = jm ^ i;
-      rank += (o > sb) || (o == sb && oj < jm);
-    }
-    const bool keep = rank < 4;
-    const uint32_t gbyte = (__ballot_sync(0xFFFFFFFFu, keep) >> (lane & 24)) & 0xFFu;
-    const int pos = __popc(gbyte & ((1u << jm) - 1u));
-    // bytes 2 pos and 2 pos + 1 of the four kept values, or the sign (zero) of byte 1
-    dsel[gw * 8 + jm] = keep ? (uint8_t)(0x10 + 0x22 * pos) : (uint8_t)0x99;
-    if (keep) {
-      cidx[gw * 4 + pos] = (uint8_t)jm;
-      // unit of column pos: XOR-ed so that eight neighbouring groups' units of one column lie in different banks
-      uint4* dst = reinterpret_cast<uint4*>(stage) + gw * 4 + (pos ^ ((gw >> 1) & 3));
-#pragma unroll
-      for (int u = 0; u < kV / 8; ++u) dst[u * 64] = make_uint4(yp[4 * u], yp[4 * u + 1], yp[4 * u + 2], yp[4 * u + 3]);
-    }
-    set_sync(set);                                                         // the kept columns of all 128 features are in
-    // ---- pass 2
-    const uint32_t c4 = *reinterpret_cast<const uint32_t*>(cidx + gl * 4);
-    const uint2 ds = *reinterpret_cast<const uint2*>(dsel + gl * 8);
-    if (q == 0 && psub == 0)
-      *reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(args.vn_colidx) + ((t0 / kV) * G + g0 + gl) * 4) = c4;
+    bool keep = false;
+    int pos = 0;
 #pragma unroll 1
-    for (int u = 2 * q + psub; u < kV / 8; u += 8) {
+    for (int h = 0; h < (both ? 2 : 1); ++h) {
+      if (!tall || h == 0) {
+        float score = 0.f;
+        auto add = [&](int j0) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            yp[j0 + j] = bf2_relu(yp[j0 + j]);
+            const uint32_t hp = bf2_sq(yp[j0 + j]);
+            score = __fadd_rn(score, __uint_as_float(hp << 16));
+            score = __fadd_rn(score, __uint_as_float(hp & 0xFFFF0000u));
+          }
+        };
+        add(0);
+        if constexpr (kStep == 128) {
+          if (tall) add(32);
+        }
+        // ---- rank the eight columns of each group
+        const uint32_t sb = __float_as_uint(score);                            // scores are >= 0: the pattern orders them
+        int rank = 0;
+#pragma unroll
+        for (int i = 1; i < 8; ++i) {
+          const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, sb, i);
+          const int oj = jm ^ i;
+          rank += (o > sb) || (o == sb && oj < jm);
+        }
+        keep = rank < 4;
+        const uint32_t gbyte = (__ballot_sync(0xFFFFFFFFu, keep) >> (lane & 24)) & 0xFFu;
+        pos = __popc(gbyte & ((1u << jm) - 1u));
+      }
+      if (c0 + h > 0) set_sync(set);                                       // the stage has been read
+      if (!tall || h == 0) {
+        // bytes 2 pos and 2 pos + 1 of the four kept values, or the sign (zero) of byte 1
+        dsel[gw * 8 + jm] = keep ? (uint8_t)(0x10 + 0x22 * pos) : (uint8_t)0x99;
+        if (keep) cidx[gw * 4 + pos] = (uint8_t)jm;
+      }
+      if (keep) {
+        // unit of column pos: XOR-ed so that eight neighbouring groups' units of one column lie in different banks
+        uint4* dst = reinterpret_cast<uint4*>(stage) + gw * 4 + (pos ^ ((gw >> 1) & 3));
+#pragma unroll
+        for (int u = 0; u < 8; ++u) dst[u * 64] = make_uint4(yp[4 * u], yp[4 * u + 1], yp[4 * u + 2], yp[4 * u + 3]);
+      }
+      if constexpr (kStep == 128) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) yp[j] = yp[32 + j];
+      }
+      set_sync(set);                                                       // the kept columns of all 128 features are in
+      // ---- pass 2
+      const uint32_t c4 = *reinterpret_cast<const uint32_t*>(cidx + gl * 4);
+      const uint2 ds = *reinterpret_cast<const uint2*>(dsel + gl * 8);
+      const int64_t t0 = n0 + c0 + 64 * h;
+      if (q == 0 && psub == 0 && (!tall || h == 0))
+        *reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(args.vn_colidx) + ((t0 >> (tall ? 7 : 6)) * G + g0 + gl) * 4) = c4;
+      const int u = 2 * q + psub;                                            // eight tokens each
       const int64_t t = t0 + 8 * u;                                        // this thread's first token
       const int64_t at = t * G + g0 + gl;
       uint32_t* p_vals = reinterpret_cast<uint32_t*>(args.vn_vals) + at;
@@ -426,7 +452,7 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
       uint8_t* p_hw = reinterpret_cast<uint8_t*>(args.vn_meta24_hw) + meta_hw_offset(t, (m0 >> 4) + (gl >> 1), F) + odd * 16;
       const uint4* src = reinterpret_cast<const uint4*>(stage) + u * 64 + gl * 4;
       const int sw = (gl >> 1) & 3;
-      const uint4 x0 = src[sw], x1 = src[1 ^ sw], x2 = src[2 ^ sw], x3 = src[3 ^ sw];
+      uint4 x0 = src[sw], x1 = src[1 ^ sw], x2 = src[2 ^ sw], x3 = src[3 ^ sw];
       // two tokens: r_i holds kept column i of both
       auto emit = [&](uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3, int k) {
         const uint32_t e = 2u * top2_offsets_x2(bf2_sq(r0), bf2_sq(r1), bf2_sq(r2), bf2_sq(r3));
@@ -471,10 +497,14 @@ __device__ __forceinline__ void epi_vnm8_tile(const GemmArgs& args, uint32_t tad
           p_m24[off] = __byte_perm(m, m2, odd ? 0x7632u : 0x5410u);
         }
       };
-      emit(x0.x, x1.x, x2.x, x3.x, 0);
-      emit(x0.y, x1.y, x2.y, x3.y, 1);
-      emit(x0.z, x1.z, x2.z, x3.z, 2);
-      emit(x0.w, x1.w, x2.w, x3.w, 3);
+#pragma unroll(kStep == 128 ? 1 : 4)
+      for (int k = 0; k < 4; ++k) {
+        emit(x0.x, x1.x, x2.x, x3.x, k);
+        x0.x = x0.y; x0.y = x0.z; x0.z = x0.w;
+        x1.x = x1.y; x1.y = x1.z; x1.z = x1.w;
+        x2.x = x2.y; x2.y = x2.z; x2.z = x2.w;
+        x3.x = x3.y; x3.y = x3.z; x3.z = x3.w;
+      }
     }
   }
 }
@@ -961,10 +991,8 @@ __host__ __device__ constexpr int stage_bytes2(bool sparse, int bn = BN, bool fp
 __host__ __device__ constexpr int num_stages2(bool sparse, int bn = BN, bool expand = false) {
   return sparse ? 4 : (expand ? 5 : 6);
 }
-// the fused activation epilogue holds whole V-blocks per tile: 192 columns = three blocks of 64, 128 = one of 128
-__host__ __device__ constexpr int vnm_block(int bn) { return bn == 192 ? 64 : 128; }
 __host__ __device__ constexpr int epi_bytes2(int epi, int bn = BN) {
-  return epi == EPI_VNM8 ? vnm_epi_bytes(vnm_block(bn))
+  return epi == EPI_VNM8 ? kVnmEpiBytes
          : is_drelu_t(epi) ? kSetWarps * kDreluWarpBytes
          : epi == EPI_STORE || epi == EPI_ROUTE ? 0 : kSetWarps * kEpiWarpBytes;
 }
@@ -1074,7 +1102,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     for (int b = 0; b < 2; ++b) {
       mbar_init(&ctl->tmem_full[b], 1);
       // the epilogue warps of both CTAs that read the accumulator
-      mbar_init(&ctl->tmem_empty[b], split_sets(kMode, kEpi, kExpand) ? 16 : 8);
+      mbar_init(&ctl->tmem_empty[b], split_sets(kMode, kEpi, kExpand) || (two_sets(kEpi) && kAccBufs == 1) ? 16 : 8);
     }
     ctl->abort_flag = 0;
     fence_mbar_init();
@@ -1083,7 +1111,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     ctl->expand_lut[threadIdx.x - 64] = expand_lut_entry(threadIdx.x - 64);
   }
   if (kEpi == EPI_VNM8 && threadIdx.x >= 64 && threadIdx.x < 128)
-    vnm_tables_init(reinterpret_cast<VnmTables*>(epi_stage + 2 * vnm_set_bytes(vnm_block(kBN))), (int)threadIdx.x - 64);
+    vnm_tables_init(reinterpret_cast<VnmTables*>(epi_stage + 2 * kVnmSetBytes), (int)threadIdx.x - 64);
   if (kEpi == EPI_ACT24_T && threadIdx.x >= 96) top2_lut_init(ctl->top2_lut, (int)threadIdx.x - 96);
   if (warp == 1) {
     tmem_alloc_2cta(&ctl->tmem_base, kTmemCols);
@@ -1268,34 +1296,37 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   } else if constexpr (two_sets(kEpi)) {
     // =========================== epilogue in two sets (warps 2..9, both CTAs) ===========================
     // Two sets of four warps, one per accumulator buffer: set 0 takes this pair's even tiles, set 1 the odd
-    // ones, so each set has two main loops' time for one tile.
+    // ones, so each set has two main loops' time for one tile. With one accumulator they share every tile, 128 columns each.
     const int q = warp & 3, set = (warp - 2) >> 2;
     uint8_t* wsm = epi_stage + (set * 4 + q) * (epi_bytes2(kEpi, kBN) / kSetWarps);
-    const uint32_t taddr = tmem_base + set * kBN + ((uint32_t)(q * 32) << 16);
-    uint32_t acc_phase = 0, vnm_buf = 0;
-    for (int tile = pair + set * num_pairs; tile < num_tiles; tile += 2 * num_pairs) {
+    constexpr bool kShare = kAccBufs == 1;
+    static_assert(!kShare || kEpi == EPI_VNM8, "the other epilogues walk whole tiles");
+    const int acc = kShare ? 0 : set;
+    const uint32_t taddr = tmem_base + set * (kShare ? 128 : kBN) + ((uint32_t)(q * 32) << 16);
+    uint32_t acc_phase = 0;
+    for (int tile = kShare ? pair : pair + set * num_pairs; tile < num_tiles; tile += kShare ? num_pairs : 2 * num_pairs) {
       const GemmTile tc = get_tile<kBN, kVar, kDual>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
-      const int64_t m0 = (int64_t)tc.out_m + (int64_t)rank * 128, n0 = tc.out_n, n_limit = tc.n_limit;
+      const int64_t m0 = (int64_t)tc.out_m + (int64_t)rank * 128, n0 = tc.out_n + (kShare ? set * 128 : 0), n_limit = tc.n_limit;
       // M % 256 == 128 (regular raster only): the second CTA of the last row of pairs holds no rows (its operand
       // loads were zero-filled); it only hands the accumulator back
       const bool live = args.tile_table != nullptr || m0 < args.M;
       if constexpr (is_drelu_t(kEpi)) {
         if (!epi_drelu_tile<kEpi, kBN>(args, taddr, m0, n0, n_limit, live, q, lane, reinterpret_cast<float*>(wsm), ctl->expand_lut,
-                                       &ctl->tmem_full[set], acc_phase, abort_flag, &ctl->tmem_empty[set]))
+                                       &ctl->tmem_full[acc], acc_phase, abort_flag, &ctl->tmem_empty[acc]))
           break;
       } else {
-        bool ok = mbar_wait(&ctl->tmem_full[set], acc_phase, abort_flag);
+        bool ok = mbar_wait(&ctl->tmem_full[acc], acc_phase, abort_flag);
         // the set's warps meet at barriers inside the tile: they go on, or leave, together
         if (kEpi == EPI_VNM8) ok = set_all(set, ok);
         if (!ok) break;
         tc_fence_after();
         if (!live) {
-          release_accumulator(lane, &ctl->tmem_empty[set]);
+          release_accumulator(lane, &ctl->tmem_empty[acc]);
         } else if constexpr (kEpi == EPI_VNM8) {
-          epi_vnm8_tile<kBN, vnm_block(kBN)>(args, taddr, m0, n0, n_limit, q, set, lane, epi_stage, vnm_buf, &ctl->tmem_empty[set]);
+          epi_vnm8_tile<kShare ? 128 : kBN, kBN == 192 ? 64 : 128>(args, taddr, m0, n0, n_limit, q, set, lane, epi_stage, &ctl->tmem_empty[acc]);
         } else {
           epi_act24_tile<kBN>(args, taddr, m0, n0, n_limit, q, lane, reinterpret_cast<uint32_t*>(wsm), ctl->expand_lut,
-                              ctl->top2_lut, &ctl->tmem_empty[set]);
+                              ctl->top2_lut, &ctl->tmem_empty[acc]);
         }
       }
       acc_phase ^= 1;
@@ -2008,12 +2039,27 @@ bool gemm_sparse24_vnm8_supported(int64_t F, int64_t T, int64_t D, int V) {
   return F >= 256 && T > 0 && F % 128 == 0 && D % 128 == 0 && (V == 64 || V == 128) && T % V == 0;
 }
 
+// Token columns of a tile. 256 (one accumulator, shared by both sets of epilogue warps) costs 16 % less shared-memory traffic a
+// column than 192 (two accumulators): y1 at T 8192, D 4096, F 16384 578 -> 558 us, T 16384, D 8192, F 28672 4.41 -> 3.95 ms.
+// With few k-stages or few tiles the narrower ones end sooner: T 4096, D 2048, F 8192 90 us at 192 columns and 92 at 256,
+// D 512 79 and 89. Estimated clocks: rounds of tiles x the longer of main loop and epilogue, plus the last epilogue; per 64
+// tokens the epilogue takes 3000 where two tiles' overlap and 6500 where both sets work on one tile; reading a shared
+// accumulator, 2500, is exposed. Tiles hold whole V-blocks: the narrow width for V = 128 is 128.
+static int vnm8_width(int64_t F, int64_t T, int64_t stages, int V) {
+  const int64_t P = sm_count() / 2, nm = (F + 255) / 256;
+  auto rounds = [&](int w) { return (double)((nm * ((T + w - 1) / w) + P - 1) / P); };
+  const int narrow = V == 128 ? 128 : best_width(F, T, stages, true, 192, 64, 1500.0, false);
+  const double epi = 1500.0 * (narrow / 32), main = stages * 0.93 * (272 + 2 * narrow), wide = stages * 735.0 + 2500.0;
+  const double cost_narrow = rounds(narrow) * (main > epi ? main : epi) + epi;
+  const double cost_wide = rounds(256) * (wide > 13000.0 ? wide : 13000.0) + 9000.0;
+  return cost_wide < cost_narrow ? 256 : narrow;
+}
+
 int gemm_sparse24_vnm8(const void* a_vals, const uint8_t* meta_hw, const void* X, int64_t F, int64_t T, int64_t D,
                        int V, const Vnm8Out& out, int* status, cudaStream_t s) {
   if (!gemm_sparse24_vnm8_supported(F, T, D, V)) return SF_ERR_SHAPE;
-  // Token tiles hold whole V-blocks: up to three blocks of 64 (192 columns) or one block of 128.
   GemmArgs a{};
-  a.bn = V == 64 ? best_width(F, T, D / 128, true, 192, 64, 1500.0, false) : 128;
+  a.bn = vnm8_width(F, T, D / 128, V);
   CUtensorMap ta, tb, tm;
   const int st = weight_token_maps(a_vals, meta_hw, X, F, T, D, a.bn, &ta, &tb, &tm);
   if (st != SF_OK) return st;
@@ -2022,10 +2068,9 @@ int gemm_sparse24_vnm8(const void* a_vals, const uint8_t* meta_hw, const void* X
   a.vn_vals = out.vals; a.vn_relu = out.relu; a.vn_meta = out.meta; a.vn_colidx = out.colidx;
   a.vn_vals24 = out.vals24; a.vn_relu24 = out.relu24; a.vn_meta24 = out.meta24; a.vn_meta24_hw = out.meta24_hw;
   a.vn_y1 = out.y1; a.vn_dense = out.dense;
-  if (V == 64)
-    return a.bn == 192 ? launch_two<MODE_SPARSE24, false, false, EPI_VNM8, 192>(ta, tb, tm, a, s)
-                       : launch_two<MODE_SPARSE24, false, false, EPI_VNM8, 192, 0, false, true>(ta, tb, tm, a, s);
-  return launch_two<MODE_SPARSE24, false, false, EPI_VNM8, 128>(ta, tb, tm, a, s);
+  return a.bn == 256 ? launch_two<MODE_SPARSE24, false, false, EPI_VNM8, 256>(ta, tb, tm, a, s)
+         : V == 128  ? launch_two<MODE_SPARSE24, false, false, EPI_VNM8, 128>(ta, tb, tm, a, s)
+                     : launch_two<MODE_SPARSE24, false, false, EPI_VNM8, 192, 0, false, true>(ta, tb, tm, a, s);
 }
 
 // ---- grouped (table-driven) products of the routed step --------------------------------------------------
