@@ -111,9 +111,11 @@ __device__ __forceinline__ void pair_rows(const uint32_t* sp, int lane, uint32_t
 // the 2:4 product's epilogue is on its critical path (through shared memory as below that product took 2 % more at
 // K = 8192). The two-operand epilogues of the dense step move a chunk through shared memory, 64 contiguous bytes of
 // eight rows per instruction: y1 + SquaredReLU at T 4096, D 2048, F 8192 129 -> 96 us.
-template <int kEpi, int kTileN = BN>
+// kEarly: the accumulator is handed back when the first chunk has been read; `last_first` turns the order of the chunks round.
+template <int kEpi, int kTileN = BN, bool kEarly = false>
 __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit,
-                                         int q, int lane, uint8_t* my_stage, int part = 0, int parts = 1, bool second = false) {
+                                         int q, int lane, uint8_t* my_stage, int part = 0, int parts = 1, bool second = false,
+                                         bool last_first = false, uint64_t* tmem_empty_bar = nullptr) {
   if constexpr (kEpi == EPI_ROUTE) {
     const int64_t row = m0 + q * 32 + lane;                                // this thread's D row
     // the row is a token, the first route_E columns its logits
@@ -139,7 +141,10 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
   // chunks of 32 columns (warp-uniform): this warp's part of the live ones
   const int live = (int)min((int64_t)(kTileN / 32), (n_limit - n0) >> 5);
   const int ch0 = live * part / parts, nch = live * (part + 1) / parts;
-  if (ch0 >= nch) return;
+  if (ch0 >= nch) {
+    if (kEarly) release_accumulator(lane, tmem_empty_bar);
+    return;
+  }
   int64_t row = m0 + q * 32 + lane;                                        // this thread's D row
   bool row_live = true;
   if (kEpi == EPI_STORE && args.row_map) {                                 // scattered output rows
@@ -170,7 +175,9 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
   };
   if (kEpi == EPI_DRELU) fetch(ch0);
   // `v` holds (once its load is complete) the chunk's accumulator columns; `next` starts the load of the chunk after
-  auto chunk = [&](int ch, uint32_t (&v)[32], uint32_t (&next)[32]) {
+  auto at = [&](int i) { return kEarly && last_first ? nch - 1 - i : i; };   // (kEarly: ch0 = 0)
+  auto chunk = [&](int i, uint32_t (&v)[32], uint32_t (&next)[32]) {
+    const int ch = at(i);
     const int64_t col0 = n0 + ch * 32;
     uint32_t w[16];
     if (kEpi == EPI_DRELU) {                                               // y1 to a thread per row
@@ -181,7 +188,8 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
       if (ch + 1 < nch) fetch(ch + 1);
     }
     tmem_ld_wait_on(v);
-    if (ch + 1 < nch) tmem_ld_32x32b_x32(taddr + (ch + 1) * 32, next);
+    if (kEarly && i == 0) release_accumulator(lane, tmem_empty_bar);
+    if (i + 1 < nch) tmem_ld_32x32b_x32(taddr + at(i + 1) * 32, next);
     if (kEpi == EPI_DRELU) {                                               // C = bf16(2 * acc * relu(aux))
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -237,11 +245,11 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
   };
   // two register buffers: the TMEM load of the next 32 columns is in flight while this chunk is converted
   uint32_t va[32], vb[32];
-  tmem_ld_32x32b_x32(taddr + ch0 * 32, va);
+  tmem_ld_32x32b_x32(taddr + at(ch0) * 32, va);
 #pragma unroll 1
-  for (int ch = ch0; ch < nch; ch += 2) {
-    chunk(ch, va, vb);
-    if (ch + 1 < nch) chunk(ch + 1, vb, va);
+  for (int i = ch0; i < nch; i += 2) {
+    chunk(i, va, vb);
+    if (i + 1 < nch) chunk(i + 1, vb, va);
   }
 }
 
@@ -1067,11 +1075,16 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   constexpr int kBSlabBytes = (kBN / 2) * 128;            // this CTA's half of B for one 64-wide K slab
   constexpr int kBHalfBytes = kSparse ? 2 * kBSlabBytes : kBSlabBytes;
   constexpr int kStageBytes = stage_bytes2(kSparse, kBN, kFp8);
-  // 2:4 mode: TMEM holds the metadata next to the accumulators, so 256-column tiles leave room for one
-  // accumulator only; 224-column tiles fit two (448 columns + 8 of metadata) and the epilogue of a tile
-  // then overlaps the main loop of the next.
-  constexpr int kAccBufs = (kSparse && kBN > 248) ? 1 : 2;
-  constexpr uint32_t kMetaCol = kSparse ? (uint32_t)(kAccBufs * kBN) : 0u;
+  // 2:4 mode: TMEM holds the metadata next to the accumulators. 224-column tiles fit two (448 columns + 8 of metadata), and
+  // the epilogue of a tile overlaps the main loop of the next; 256-column tiles leave room for one. kOverlap: they alternate
+  // between columns 0..255 and 224..479, and the next main loop starts when the 32 columns that both use have been read,
+  // which the epilogue does first. One pair of barriers serves both positions: a warp hands tile n back when it has read
+  // those columns, and by then it has read all of tile n - 1. It counts where k is short: the routed step at T 8192, D 4096,
+  // F 16384 in four experts (32 k-stages a tile) 1309 -> 1293 us; with 64 stages and more, and in the fused activation
+  // epilogue (more registers), nothing was gained: what the main loop loses by waiting it makes up from the full ring.
+  constexpr bool kOneAcc = kSparse && kBN > 248, kOverlap = kOneAcc && kEpi == EPI_STORE && !kVar;
+  constexpr int kAccBufs = kOneAcc ? 1 : 2;
+  constexpr uint32_t kMetaCol = kSparse ? (kOverlap ? 480u : (uint32_t)(kAccBufs * kBN)) : 0u;
   static_assert(kBN % 32 == 0 && kBN <= 256, "tile width");
   static_assert(!(kMode == MODE_DENSE) || kBN == BN, "dense mode uses 256-column tiles");
   static_assert(!kBMN || kBN == BN, "MN-major B is loaded in 64-column chunks");
@@ -1213,13 +1226,13 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
       // per-instruction advances of the low words (in 16-byte units)
       constexpr uint32_t a_step = (kMode == MODE_DENSE && kAMN) ? (2048 >> 4) : (32 >> 4);
       uint32_t stage = 0, phase = 0;
-      uint32_t acc = 0, acc_phase = 0;
+      uint32_t acc = 0, acc_phase = 0, shift = 0;
       bool ok = true;
-      for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
+      for (int tile = pair; tile < num_tiles && ok; tile += num_pairs, shift ^= kOverlap ? 224u : 0u) {
         const int nkb = args.tile_table ? __ldg(&args.tile_table[tile].nkb) : nkb_full;
         if (!mbar_wait(&ctl->tmem_empty[acc], acc_phase ^ 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t tmem_d = tmem_base + acc * kBN;
+        const uint32_t tmem_d = tmem_base + acc * kBN + shift;
         for (int kb = 0; kb < nkb; ++kb) {
           if (!mbar_wait(&ctl->full[stage], phase, abort_flag)) { ok = false; break; }
           tc_fence_after();
@@ -1341,16 +1354,15 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
       const GemmTile tc = get_tile<kBN, kVar, kDual>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
       const int64_t m0 = (int64_t)tc.out_m + (int64_t)rank * 128, n0 = tc.out_n, n_limit = tc.n_limit;
-      const uint32_t taddr = tmem_base + acc * kBN + ((uint32_t)(q * 32) << 16);
+      const uint32_t taddr = tmem_base + acc * kBN + (kOverlap ? acc_phase * 224u : 0u) + ((uint32_t)(q * 32) << 16);
       // M % 256 == 128 (regular raster only): the second CTA of the last row of pairs holds no rows
       const bool second = kDual && tile >= num_m_tiles * num_n_tiles_;
       const bool live = args.tile_table != nullptr || m0 < (second ? args.M2 : args.M);
       if (!mbar_wait(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      if (live) epi_tile<kEpi, kBN>(args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts, second);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_leader(&ctl->tmem_empty[acc]);
+      if (live) epi_tile<kEpi, kBN, kOverlap>(args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts, second, acc_phase == 0,
+                                              &ctl->tmem_empty[0]);
+      if (!kOverlap || !live) release_accumulator(lane, &ctl->tmem_empty[acc]);
       if (++acc == (uint32_t)kAccBufs) { acc = 0; acc_phase ^= 1; }
     }
   }
