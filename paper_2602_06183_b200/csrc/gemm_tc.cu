@@ -542,15 +542,19 @@ __device__ __forceinline__ void expand24_lut(const uint2* lut, uint32_t pair, ui
   w1 = __byte_perm(pair, 0u, s.y);
 }
 
-template <int kEpi, int kTileN>
+// kShare: the two sets work on one tile of 256 columns, four chunks each; the accumulator is handed back when the first chunk has
+// been read, and the second set starts with its last one (see kOverlap in the kernel). The chunk is then staged in two halves.
+template <int kEpi, int kTileN, bool kShare>
 __device__ __forceinline__ bool epi_drelu_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit,
-                                               bool live, int q, int lane, float* stage, const uint2* lut,
+                                               bool live, int q, int set, int lane, float* stage, const uint2* lut,
                                                uint64_t* tmem_full_bar, uint32_t phase, volatile int* abort_flag,
                                                uint64_t* tmem_empty_bar) {
   constexpr bool kVenomMask = kEpi == EPI_DRELUV_T;
   const int t8 = lane >> 2, seg = lane & 3;
   const int64_t f = m0 + q * 32 + seg * 8;                                 // this lane's first feature
-  const int nch = live ? (int)min((int64_t)(kTileN / 32), (n_limit - n0) >> 5) : 0;
+  const int nch = live ? (int)min((int64_t)(kShare ? 4 : kTileN / 32), (n_limit - n0) >> 5) : 0;
+  auto at = [&](int i) { return kShare && set == 1 ? nch - 1 - i : i; };
+  constexpr int kRows = kShare ? 16 : 32;                                  // tokens staged at a time
   const int64_t tok = n0 + t8;                                             // this lane's first token
   // per token: EPI_DRELU24_T four stored values + one metadata byte; EPI_DRELUV_T the group's pair + its nibble
   const int64_t g = kVenomMask ? f / args.Mv : 0;
@@ -570,36 +574,29 @@ __device__ __forceinline__ bool epi_drelu_tile(const GemmArgs& args, uint32_t ta
     if (kVenomMask)      // a chunk lies inside one V-block (V is a multiple of 32)
       c4n = __ldg(reinterpret_cast<const uint32_t*>(args.colidx + ((n0 + ch * 32) / args.V * args.G + g) * 4));
   };
-  if (nch > 0) fetch(0);
+  if (nch > 0) fetch(at(0));
   if (!mbar_wait(tmem_full_bar, phase, abort_flag)) return false;
   tc_fence_after();
-  if (nch == 0) {
+  if (nch <= 0) {
     release_accumulator(lane, tmem_empty_bar);
     return true;
   }
   uint32_t v[32];
-  tmem_ld_32x32b_x32(taddr, v);
+  tmem_ld_32x32b_x32(taddr + at(0) * 32, v);
   const float* row0 = stage + t8 * kDreluRow + seg * 8;
   uint16_t* p_dense = args.C ? reinterpret_cast<uint16_t*>(args.C) + tok * args.ldc + f : nullptr;
   const int off = kVenomMask ? (int)(f & (args.Mv - 1)) : 0;               // this lane's first column inside its group
 #pragma unroll 1
-  for (int ch = 0; ch < nch; ++ch) {
+  for (int ci = 0; ci < nch; ++ci) {
+    const int ch = at(ci);
     tmem_ld_wait_on(v);
-    __syncwarp();                                                          // the previous chunk has been read
-#pragma unroll
-    for (int j = 0; j < 32; ++j) stage[j * kDreluRow + lane] = __uint_as_float(v[j]);
-    __syncwarp();
+    if (kShare && ci == 0) release_accumulator(lane, tmem_empty_bar);
     uint2 rc[4];
     uint32_t mc[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) { rc[i] = r[i]; mc[i] = mb[i]; }
     c4 = c4n;
-    if (ch + 1 < nch) {
-      tmem_ld_32x32b_x32(taddr + (ch + 1) * 32, v);
-      fetch(ch + 1);
-    } else {
-      release_accumulator(lane, tmem_empty_bar);
-    }
+    if (ci + 1 < nch) fetch(at(ci + 1));
     // an off-mask entry is +0, also where the saved ReLU is zero
     auto prod = [](float x, uint32_t rb) {
       const float rv = bf16_bits_to_float(rb & 0xFFFFu);
@@ -607,7 +604,17 @@ __device__ __forceinline__ bool epi_drelu_tile(const GemmArgs& args, uint32_t ta
     };
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const float* row = row0 + i * 8 * kDreluRow;
+      if (i % (kRows / 8) == 0) {                                          // the next kRows tokens
+        __syncwarp();                                                      // the previous ones have been read
+#pragma unroll
+        for (int j = 0; j < kRows; ++j) stage[j * kDreluRow + lane] = __uint_as_float(v[i * 8 + j]);
+        __syncwarp();
+        if (i + kRows / 8 == 4) {
+          if (ci + 1 < nch) tmem_ld_32x32b_x32(taddr + at(ci + 1) * 32, v);
+          else if (!kShare) release_accumulator(lane, tmem_empty_bar);
+        }
+      }
+      const float* row = row0 + (i % (kRows / 8)) * 8 * kDreluRow;
       const int64_t t = tok + ch * 32 + i * 8;
       uint4 o;
       if (!kVenomMask) {
@@ -1001,7 +1008,7 @@ __host__ __device__ constexpr int num_stages2(bool sparse, int bn = BN, bool exp
 }
 __host__ __device__ constexpr int epi_bytes2(int epi, int bn = BN) {
   return epi == EPI_VNM8 ? kVnmEpiBytes
-         : is_drelu_t(epi) ? kSetWarps * kDreluWarpBytes
+         : is_drelu_t(epi) ? kSetWarps * kDreluWarpBytes / (bn == 256 ? 2 : 1)
          : epi == EPI_STORE || epi == EPI_ROUTE ? 0 : kSetWarps * kEpiWarpBytes;
 }
 __host__ __device__ constexpr int smem_bytes2(bool sparse, int bn = BN, int epi = EPI_STORE, bool expand = false,
@@ -1082,7 +1089,8 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   // those columns, and by then it has read all of tile n - 1. It counts where k is short: the routed step at T 8192, D 4096,
   // F 16384 in four experts (32 k-stages a tile) 1309 -> 1293 us; with 64 stages and more, and in the fused activation
   // epilogue (more registers), nothing was gained: what the main loop loses by waiting it makes up from the full ring.
-  constexpr bool kOneAcc = kSparse && kBN > 248, kOverlap = kOneAcc && kEpi == EPI_STORE && !kVar;
+  // The dy1 epilogue holds on to its accumulator for long, so there it is what lets 256 columns be used.
+  constexpr bool kOneAcc = kSparse && kBN > 248, kOverlap = kOneAcc && (kEpi == EPI_STORE || is_drelu_t(kEpi)) && !kVar;
   constexpr int kAccBufs = kOneAcc ? 1 : 2;
   constexpr uint32_t kMetaCol = kSparse ? (kOverlap ? 480u : (uint32_t)(kAccBufs * kBN)) : 0u;
   static_assert(kBN % 32 == 0 && kBN <= 256, "tile width");
@@ -1313,7 +1321,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     const int q = warp & 3, set = (warp - 2) >> 2;
     uint8_t* wsm = epi_stage + (set * 4 + q) * (epi_bytes2(kEpi, kBN) / kSetWarps);
     constexpr bool kShare = kAccBufs == 1;
-    static_assert(!kShare || kEpi == EPI_VNM8, "the other epilogues walk whole tiles");
+    static_assert(!kShare || kEpi == EPI_VNM8 || is_drelu_t(kEpi), "the other epilogues walk whole tiles");
     const int acc = kShare ? 0 : set;
     const uint32_t taddr = tmem_base + set * (kShare ? 128 : kBN) + ((uint32_t)(q * 32) << 16);
     uint32_t acc_phase = 0;
@@ -1324,8 +1332,9 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
       // loads were zero-filled); it only hands the accumulator back
       const bool live = args.tile_table != nullptr || m0 < args.M;
       if constexpr (is_drelu_t(kEpi)) {
-        if (!epi_drelu_tile<kEpi, kBN>(args, taddr, m0, n0, n_limit, live, q, lane, reinterpret_cast<float*>(wsm), ctl->expand_lut,
-                                       &ctl->tmem_full[acc], acc_phase, abort_flag, &ctl->tmem_empty[acc]))
+        if (!epi_drelu_tile<kEpi, kBN, kShare>(args, taddr + (kOverlap ? acc_phase * 224u : 0u), m0, n0, n_limit, live, q, set, lane,
+                                               reinterpret_cast<float*>(wsm), ctl->expand_lut, &ctl->tmem_full[acc], acc_phase,
+                                               abort_flag, &ctl->tmem_empty[acc]))
           break;
       } else {
         bool ok = mbar_wait(&ctl->tmem_full[acc], acc_phase, abort_flag);
@@ -1592,7 +1601,7 @@ gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constan
       // M % 256 == 128: the second CTA of the last half holds no rows; it only hands the accumulator back
       const bool live = m0 < args.M;
       if constexpr (is_drelu_t(kEpi)) {
-        if (!epi_drelu_tile<kEpi, kTallBN>(args, taddr, m0, n0, n_limit, live, q, lane, reinterpret_cast<float*>(wsm),
+        if (!epi_drelu_tile<kEpi, kTallBN, false>(args, taddr, m0, n0, n_limit, live, q, 0, lane, reinterpret_cast<float*>(wsm),
                                            ctl->expand_lut, &ctl->tmem_full[h], phase, abort_flag, &ctl->tmem_empty[h]))
           break;
       } else {
@@ -1958,14 +1967,24 @@ int gemm_sparse24_drelu(const void* w_vals, const uint8_t* meta_hw, const void* 
     a.colidx = mask.colidx; a.V = mask.V; a.Mv = mask.Mv; a.G = F / mask.Mv;
   }
   CUtensorMap ta, tb, tbn, tm;
-  if (use_tall(F, T, D / 128, kNarrowBN, 0.0, 4000.0)) {
+  // 256-column tiles (one accumulator, 1000 clocks before the next main loop starts) or 224 and narrower (two), by estimated
+  // clocks: T 4096, D 2048, F 8192 is 7 rounds of 256-column tiles or 9 of 224: 71.6 us against 79.3.
+  // (At T 8192, D 4096, F 16384, 28 and 32 rounds, the two are equal: it has to gain 5 %.)
+  const int64_t stages = D / 128, P = sm_count() / 2, nm = (F + 255) / 256;
+  auto rounds = [&](int64_t w) { return (double)((nm * ((T + w - 1) / w) + P - 1) / P); };
+  a.bn = best_width(F, T, stages, true, kNarrowBN, 32, 500.0, false);
+  const bool wide = stages >= 8 && a.bn == kNarrowBN && rounds(256) * (stages * 735.0 + 1000.0) < 0.95 * rounds(kNarrowBN) * (stages * 680.0);
+  if (use_tall(F, T, stages, wide ? 256 : kNarrowBN, wide ? 1000.0 : 0.0, 4000.0)) {
     const int st = tall_maps(w_vals, meta_hw, dY, true, F, T, D, 0, 2, &ta, &tb, &tbn, &tm);
     if (st != SF_OK) return st;
     return mask.colidx ? launch_tall<false, EPI_DRELUV_T>(ta, tb, tbn, tm, a, s) : launch_tall<false, EPI_DRELU24_T>(ta, tb, tbn, tm, a, s);
   }
-  a.bn = best_width(F, T, D / 128, true, kNarrowBN, 32, 500.0, false);
+  if (wide) a.bn = 256;
   const int st = weight_token_maps(w_vals, meta_hw, dY, F, T, D, a.bn, &ta, &tb, &tm);
   if (st != SF_OK) return st;
+  if (wide)
+    return mask.colidx ? launch_two<MODE_SPARSE24, false, false, EPI_DRELUV_T, 256>(ta, tb, tm, a, s)
+                       : launch_two<MODE_SPARSE24, false, false, EPI_DRELU24_T, 256>(ta, tb, tm, a, s);
   if (a.bn != kNarrowBN)
     return mask.colidx ? launch_two<MODE_SPARSE24, false, false, EPI_DRELUV_T, kNarrowBN, 0, false, true>(ta, tb, tm, a, s)
                        : launch_two<MODE_SPARSE24, false, false, EPI_DRELU24_T, kNarrowBN, 0, false, true>(ta, tb, tm, a, s);
