@@ -422,3 +422,22 @@ def test_sparse_ffn_random_legal_shapes(T, D, F, V, M, prune_mode, act_shift, se
     cfg = dict(T=T, D=D, F=F, V=V, N=2, M=M, sigma_w=0.05, seed=seed)
     inputs, g = _run_sparse(cfg, prune_mode, act_shift)
     _check_against_oracle(inputs, g, cfg, prune_mode)
+
+
+@pytest.mark.parametrize("T,D,F,V", [(2432, 2048, 3456, 64), (2176, 2048, 3968, 64), (2176, 3072, 3968, 128)])
+def test_sparse_ffn_on_256_column_tiles(T, D, F, V):
+    """Shapes at which the fused y1 product and the dy1 product take 256-column tiles on one accumulator, more than one
+    tile to a CTA pair, the last token tile and the last row of tiles half empty. The activation is checked bit for bit
+    against the two-kernel path, dy1 against the float64 product of the pruned W2 times the saved ReLU."""
+    cfg = dict(T=T, D=D, F=F, V=V, N=2, M=8, sigma_w=0.05, seed=29)
+    inputs, fused = _run_sparse(cfg, flags=binding.SF_FFN_SAVE_Y1)
+    _, two = _run_sparse(cfg, flags=binding.SF_FFN_SAVE_Y1 | binding.SF_FFN_UNFUSED_ACT)
+    for k in fused:
+        assert np.array_equal(fused[k], two[k]), k
+    w2s = oracle.prune24(np.ascontiguousarray(inputs[2].T), 1, 0).dense
+    f64 = lambda a: torch.from_numpy(oracle.bf16_to_f32(a)).cuda().double()
+    dy2 = (f64(inputs[3]) @ f64(w2s).T).cpu().numpy()
+    ref = 2.0 * dy2 * oracle.bf16_to_f32(oracle.decompress24(fused["relu24"], fused["meta24"]))
+    got = oracle.bf16_to_f32(fused["dy1_dense"])
+    assert rel_fro(got, ref) < TOL
+    assert_close_elementwise(got, ref, D, "dy1")
