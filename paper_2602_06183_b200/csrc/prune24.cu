@@ -91,16 +91,26 @@ prune24_rows_kernel(const uint4* __restrict__ W, int64_t rows, int cols, int64_t
 // vals [Rc, Kd/2], meta [Rc, Kd/16]. Panel: 128 reduction rows x 64 columns.
 // Persistent CTAs walk the panels. One TMA load brings the next panel into a two-slot ring
 // (out-of-range rows and columns arrive as zeros), so no thread computes load addresses; selection runs
-// on column pairs; packed values, canonical metadata and the tensor-core-ordered metadata of a panel are
-// assembled in shared memory and leave as 128-bit stores.
+// on column pairs; packed values and metadata words of a panel are collected in shared memory and leave as
+// 128-bit stores, the metadata in either order.
+// What bounds it: shared memory (a panel is written once by TMA, read and written once by the selection, read by the
+// stores) and integer issue. Two barriers a panel: the one behind the wait for the load also says that the previous panel
+// is stored. With a third one before the wait, metadata placed by 16-bit stores and columns staged in order, 4096 x 16384
+// took 47.7 us soft / 40.8 hard, 8192 x 28672 hard 162, 2048 x 8192 soft 15.6; now 44.4 / 37.7, 150 and 14.1
+// (4.9 TB/s at 8192 x 28672). The changes to shared memory alone gave 46.2 / 39.1, 168 and 15.1: the barrier is what
+// the large size needs.
 constexpr int kPanelK = 128, kPanelC = 64;
 constexpr int kColsSlots = 2;                       // the next panel loads while this one is worked on
 constexpr int kStageRow = (kPanelK / 2) * 2 + 16;   // packed bytes per column + 16 B pad
 constexpr int kColsTileBytes = kPanelK * kPanelC * 2, kColsStageBytes = kPanelC * kStageRow;
-constexpr int kColsMetaBytes = kPanelC * (kPanelK / 16) * 2;       // canonical words [column][8]; the same again in hardware order
-constexpr int kColsSmemBytes = 128 + kColsSlots * kColsTileBytes + kColsStageBytes + 2 * kColsMetaBytes + 64;
-constexpr int kColsCtasPerSm = 5;                   // 44 KB each; measured best among 3..5 with two or three slots
+constexpr int kColsMetaBytes = kPanelC * (kPanelK / 16) * 2;       // metadata words [chunk][column]
+constexpr int kColsSmemBytes = 128 + kColsSlots * kColsTileBytes + kColsStageBytes + kColsMetaBytes + 64;
+constexpr int kColsCtasPerSm = 5;                   // 43 KB each; measured best among 3..5 with two or three slots
 static_assert(kPanelK / 16 == 8 && kPanelC == 64, "index shifts in prune24_cols_kernel assume a 128 x 64 panel");
+
+// Row of the stage buffer that holds a column: even columns first. A warp writes 32 columns of one parity, 144 bytes
+// apart in this order, so its 16-byte stores touch every bank once a quarter warp (288 bytes apart they met two by two).
+__device__ __forceinline__ int stage_row(int c) { return (c >> 1) + (c & 1) * (kPanelC / 2); }
 
 // kFp8: the kept values leave as E4M3 codes of float(value) * scale (vals = uint8 [Rc, Kd/2]); no masked copy.
 template <bool kSoft, bool kFp8 = false>
@@ -113,11 +123,10 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64
   uint8_t* cols_smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(cols_smem_raw) + 127) & ~uintptr_t(127));
   typedef uint16_t TileRow[kPanelC];
   typedef uint8_t StageRow[kStageRow];
-  typedef uint16_t MetaRow[kPanelK / 16];
+  typedef uint16_t MetaRow[kPanelC];
   StageRow* stage = reinterpret_cast<StageRow*>(cols_smem + kColsSlots * kColsTileBytes);              // [kPanelC]
-  MetaRow* mstage = reinterpret_cast<MetaRow*>(cols_smem + kColsSlots * kColsTileBytes + kColsStageBytes);   // [kPanelC]
-  uint8_t* mhw = reinterpret_cast<uint8_t*>(mstage) + kColsMetaBytes;                                   // four 256-byte row blocks
-  uint64_t* full = reinterpret_cast<uint64_t*>(mhw + kColsMetaBytes);                                   // [kColsSlots]
+  MetaRow* mstage = reinterpret_cast<MetaRow*>(cols_smem + kColsSlots * kColsTileBytes + kColsStageBytes);   // [kPanelK / 16]
+  uint64_t* full = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(mstage) + kColsMetaBytes);    // [kColsSlots]
   int* abort_flag = reinterpret_cast<int*>(full + kColsSlots);
   const int tid = threadIdx.x;
 
@@ -147,15 +156,15 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64
   int it = 0;
   for (int panel = blockIdx.x; panel < num_panels; panel += gridDim.x, ++it) {
     const int slot = it % kColsSlots;
-    __syncthreads();            // the previous panel is stored: its stage buffers and the slot of the panel before are free
-    if (tid == 0) {
-      fence_proxy_async_smem(); // earlier generic writes to that slot (masked copy) before the TMA write
-      issue(it + kColsSlots - 1);
-    }
     // one warp waits for the load (bounded), the block follows through the barrier
     bool ok = true;
     if (tid < 32) ok = mbar_wait(&full[slot], (uint32_t)(it / kColsSlots) & 1u, abort_flag);
     if (__syncthreads_or(!ok)) break;
+    // every warp has stored the previous panel: its stage buffers and its slot are free
+    if (tid == 0) {
+      fence_proxy_async_smem(); // earlier generic writes to that slot (masked copy) before the TMA write
+      issue(it + kColsSlots - 1);
+    }
 
     const int py = panel / panels_x, px = panel - py * panels_x;
     const int64_t c0 = (int64_t)px * kPanelC, k0 = (int64_t)py * kPanelK;
@@ -199,16 +208,12 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64
         if (kFp8) {
           const uint32_t q0 = quant2(packed[e][0], scale), q1 = quant2(packed[e][1], scale);
           const uint32_t q2 = quant2(packed[e][2], scale), q3 = quant2(packed[e][3], scale);
-          *reinterpret_cast<uint2*>(&stage[c + e][ch * 8]) = make_uint2(q0 | (q1 << 16), q2 | (q3 << 16));
+          *reinterpret_cast<uint2*>(&stage[stage_row(c + e)][ch * 8]) = make_uint2(q0 | (q1 << 16), q2 | (q3 << 16));
         } else {
-          *reinterpret_cast<uint4*>(&stage[c + e][ch * 16]) = make_uint4(packed[e][0], packed[e][1], packed[e][2], packed[e][3]);
+          *reinterpret_cast<uint4*>(&stage[stage_row(c + e)][ch * 16]) = make_uint4(packed[e][0], packed[e][1], packed[e][2], packed[e][3]);
         }
-        mstage[c + e][ch] = (uint16_t)m[e];
-        // tensor-core order (see meta_hw_offset): the panel's 64 output rows are four 16-row blocks of one atom
-        const int mi = c + e;
-        *reinterpret_cast<uint16_t*>(mhw + (mi >> 4) * 256 + (ch & 1) * 128 + (mi & 7) * 16 + (ch >> 1) * 4 +
-                                     ((mi >> 3) & 1) * 2) = (uint16_t)m[e];
       }
+      *reinterpret_cast<uint32_t*>(&mstage[ch][c]) = m[0] | (m[1] << 16);
     }
     __syncthreads();
 
@@ -221,29 +226,39 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64
       const int64_t orow = c0 + c;
       if (kFp8) {
         *reinterpret_cast<uint2*>(reinterpret_cast<uint8_t*>(vals) + orow * (Kd >> 1) + (k0 >> 1) + ch * 8) =
-            *reinterpret_cast<const uint2*>(&stage[c][ch * 8]);
+            *reinterpret_cast<const uint2*>(&stage[stage_row(c)][ch * 8]);
       } else {
-        *reinterpret_cast<uint4*>(vals + orow * (Kd >> 1) + (k0 >> 1) + ch * 8) = *reinterpret_cast<const uint4*>(&stage[c][ch * 16]);
+        *reinterpret_cast<uint4*>(vals + orow * (Kd >> 1) + (k0 >> 1) + ch * 8) = *reinterpret_cast<const uint4*>(&stage[stage_row(c)][ch * 16]);
       }
     }
     if (full_k && (Kd & 127) == 0) {
-      // whole panels: a column's eight metadata words are 16 contiguous, aligned bytes in either order
+      // whole panels: a column's eight metadata words are 16 contiguous, aligned bytes in either order. Each store's words
+      // are gathered here by the 64 threads that write it: with each selecting thread placing its four words in the two
+      // orders itself, those 16-bit stores met in four banks, 24 passes of shared memory per warp and panel instead of 1.
       if (tid < kPanelC) {
-        if (tid < cvalid)
-          *reinterpret_cast<uint4*>(meta + (c0 + tid) * (Kd >> 4) + (k0 >> 4)) = *reinterpret_cast<const uint4*>(&mstage[tid][0]);
+        if (tid < cvalid) {
+          uint32_t w[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) w[j] = mstage[2 * j][tid] | ((uint32_t)mstage[2 * j + 1][tid] << 16);
+          *reinterpret_cast<uint4*>(meta + (c0 + tid) * (Kd >> 4) + (k0 >> 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
       } else if (tid < 2 * kPanelC && meta_hw) {
-        const int t = tid - kPanelC;                                        // 16-byte piece of the panel's 1 KB
+        // tensor-core order (see meta_hw_offset): the panel's 64 output rows are four 16-row blocks of one atom; 16-byte
+        // piece t of the panel's 1 KB holds rows r and r + 8 of one block for every second chunk
         // (the hardware order exists for whole 128-row blocks only, so all 64 columns are valid here)
+        const int t = tid - kPanelC, r = (t >> 4) * 16 + (t & 7), odd = (t >> 3) & 1;
+        uint32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = mstage[2 * j + odd][r] | ((uint32_t)mstage[2 * j + odd][r + 8] << 16);
         const int64_t atom = (c0 >> 7) * (Kd >> 7) + (k0 >> 7);
-        *reinterpret_cast<uint4*>(meta_hw + atom * 2048 + ((c0 & 127) >> 4) * 256 + t * 16) =
-            *reinterpret_cast<const uint4*>(mhw + t * 16);
+        *reinterpret_cast<uint4*>(meta_hw + atom * 2048 + ((c0 & 127) >> 4) * 256 + t * 16) = make_uint4(w[0], w[1], w[2], w[3]);
       }
     } else {
       for (int i = tid; i < kPanelC * chunks; i += 256) {
         const int c = i / chunks, ch = i - c * chunks;
         if (c >= cvalid) continue;
         const int64_t orow = c0 + c, kw = (k0 >> 4) + ch;
-        const uint16_t mw = mstage[c][ch];
+        const uint16_t mw = mstage[ch][c];
         meta[orow * (Kd >> 4) + kw] = mw;
         if (meta_hw) *reinterpret_cast<uint16_t*>(meta_hw + meta_hw_offset(orow, kw, Kd)) = mw;
       }

@@ -35,6 +35,17 @@ def test_prune24_cols_bit_exact(rows, cols, mode):
     assert np.array_equal(bits(dense), ref.dense)
 
 
+@pytest.mark.parametrize("rows,cols,mode,want_dense", [(1040, 8200, 0, False), (1552, 8200, 1, True)])
+def test_prune24_cols_several_panels_per_cta(rows, cols, mode, want_dense):
+    # 1161 and 1677 panels of 128 x 64 for at most 740 resident CTAs: two and three turns of the two-slot load ring
+    w = synth.prune_sweep_matrix(rows, cols, seed=2300 + rows + mode, tie_frac=0.1, axis=0)
+    ref = oracle.prune24(w, group_dim=0, mode=mode)
+    vals, meta, dense = binding.sf_prune24_compress(to_dev(w), 0, mode, want_dense=want_dense)
+    assert np.array_equal(bits(meta), ref.meta)
+    assert np.array_equal(bits(vals), ref.vals)
+    assert not want_dense or np.array_equal(bits(dense), ref.dense)
+
+
 def test_prune24_strided_input_and_special_values():
     w = synth.prune_sweep_matrix(64, 512, seed=5, tie_frac=0.5)
     w[:, :16] = 0                       # all-zero groups
