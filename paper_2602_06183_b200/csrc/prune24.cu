@@ -96,9 +96,8 @@ prune24_rows_kernel(const uint4* __restrict__ W, int64_t rows, int cols, int64_t
 // What bounds it: shared memory (a panel is written once by TMA, read and written once by the selection, read by the
 // stores) and integer issue. Two barriers a panel: the one behind the wait for the load also says that the previous panel
 // is stored. With a third one before the wait, metadata placed by 16-bit stores and columns staged in order, 4096 x 16384
-// took 47.7 us soft / 40.8 hard, 8192 x 28672 hard 162, 2048 x 8192 soft 15.6; now 44.4 / 37.7, 150 and 14.1
-// (4.9 TB/s at 8192 x 28672). The changes to shared memory alone gave 46.2 / 39.1, 168 and 15.1: the barrier is what
-// the large size needs.
+// took 47.7 us soft / 40.8 hard, 8192 x 28672 hard 167, 2048 x 8192 soft 15.6; without them 44.4 / 37.7, 153 and 14.1, and
+// with the stores of whole panels unrolled 42.8 / 36.6, 151 and 13.7 (4.9 TB/s at 8192 x 28672).
 constexpr int kPanelK = 128, kPanelC = 64;
 constexpr int kColsSlots = 2;                       // the next panel loads while this one is worked on
 constexpr int kStageRow = (kPanelK / 2) * 2 + 16;   // packed bytes per column + 16 B pad
@@ -220,15 +219,24 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64
     // store packed values: per column kvalid/2 elements = kvalid bytes, 16 B per thread
     const int chunks = kvalid >> 4;
     const bool full_k = chunks == kPanelK / 16;
-    for (int i = tid; i < kPanelC * chunks; i += 256) {
-      const int c = full_k ? (i >> 3) : (i / chunks), ch = i - c * chunks;
-      if (c >= cvalid) continue;
-      const int64_t orow = c0 + c;
+    auto put = [&](int c, int ch) {
+      const int64_t at = (c0 + c) * (Kd >> 1) + (k0 >> 1) + ch * 8;
       if (kFp8) {
-        *reinterpret_cast<uint2*>(reinterpret_cast<uint8_t*>(vals) + orow * (Kd >> 1) + (k0 >> 1) + ch * 8) =
-            *reinterpret_cast<const uint2*>(&stage[stage_row(c)][ch * 8]);
+        *reinterpret_cast<uint2*>(reinterpret_cast<uint8_t*>(vals) + at) = *reinterpret_cast<const uint2*>(&stage[stage_row(c)][ch * 8]);
       } else {
-        *reinterpret_cast<uint4*>(vals + orow * (Kd >> 1) + (k0 >> 1) + ch * 8) = *reinterpret_cast<const uint4*>(&stage[stage_row(c)][ch * 16]);
+        *reinterpret_cast<uint4*>(vals + at) = *reinterpret_cast<const uint4*>(&stage[stage_row(c)][ch * 16]);
+      }
+    };
+    if (full_k) {
+#pragma unroll
+      for (int j = 0; j < kPanelC / 32; ++j) {
+        const int c = (tid >> 3) + 32 * j;
+        if (c < cvalid) put(c, tid & 7);
+      }
+    } else {
+      for (int i = tid; i < kPanelC * chunks; i += 256) {
+        const int c = i / chunks;
+        if (c < cvalid) put(c, i - c * chunks);
       }
     }
     if (full_k && (Kd & 127) == 0) {
