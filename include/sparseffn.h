@@ -406,9 +406,10 @@ SF_API int sf_routed_ctx_view(const sf_router_desc* desc, const void* fwd_ctx_or
 /* Bounded-wait self-test (the paper has no counterpart). Every device-side wait of the tensor-core
  * kernels gives up after a clock budget, raises the status word at the start of the workspace and
  * lets its CTA leave; sf_check_status then reports SF_ERR_TIMEOUT. This call runs that mechanism
- * in isolation: one CTA of one warp waits, with the same wait routine and a budget of
- * `budget_clocks` SM clocks (1 <= budget_clocks <= 2^31), on an mbarrier that nothing completes.
- * The wait runs out by construction, the kernel sets the status word and returns; nothing is
+ * in isolation: a warp waits, with the same wait routine and a budget of `budget_clocks` SM clocks
+ * (1 <= budget_clocks <= 2^31), on an mbarrier that is completed only after one of its lanes has given
+ * up, so that the lanes see different outcomes. The wait runs out by construction, the warp leaves as
+ * one (the status word is set only if every lane was told so) and the kernel returns; nothing is
  * left waiting and the context stays usable. `workspace`: device buffer whose first int is the
  * (zeroed) status word. Enqueues on `stream`. */
 SF_API int sf_selftest_wait_expiry(void* workspace, int64_t budget_clocks, void* stream);

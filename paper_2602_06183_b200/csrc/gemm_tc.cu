@@ -303,21 +303,6 @@ __device__ __forceinline__ uint32_t prmt_signed(uint32_t a, uint32_t b, uint32_t
 
 // Barrier of one set of four epilogue warps.
 __device__ __forceinline__ void set_sync(int set) { asm volatile("bar.sync %0, 128;" ::"r"(set + 1) : "memory"); }
-// The same with a vote: true when all four warps say so.
-__device__ __forceinline__ bool set_all(int set, bool ok) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t"
-      ".reg .pred P, Q;\n\t"
-      "setp.ne.b32 P, %1, 0;\n\t"
-      "barrier.cta.red.and.pred Q, %2, 128, P;\n\t"
-      "selp.b32 %0, 1, 0, Q;\n\t"
-      "}\n"
-      : "=r"(r)
-      : "r"((uint32_t)ok), "r"(set + 1)
-      : "memory");
-  return r != 0;
-}
 
 // kCols: columns of the tile that this set takes at most; kStep: tokens in registers at a time (64: V = 64 only,
 // with less code and fewer registers).
@@ -575,7 +560,7 @@ __device__ __forceinline__ bool epi_drelu_tile(const GemmArgs& args, uint32_t ta
       c4n = __ldg(reinterpret_cast<const uint32_t*>(args.colidx + ((n0 + ch * 32) / args.V * args.G + g) * 4));
   };
   if (nch > 0) fetch(at(0));
-  if (!mbar_wait(tmem_full_bar, phase, abort_flag)) return false;
+  if (!mbar_wait_warp(tmem_full_bar, phase, abort_flag)) return false;
   tc_fence_after();
   if (nch <= 0) {
     release_accumulator(lane, tmem_empty_bar);
@@ -960,7 +945,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant_
       int mt, nt;
       tile_coords(tile, num_m_tiles, num_n_tiles_, mt, nt);
       const int64_t m0 = (int64_t)mt * BM, n0 = (int64_t)nt * BN;
-      if (!mbar_wait(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
+      if (!mbar_wait_warp(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + acc * BN + ((uint32_t)(q * 32) << 16);
       epi_tile<kEpi>(args, taddr, m0, n0, args.N, q, lane, my_stage);
@@ -1288,7 +1273,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
       for (int kb = 0; kb < nkb_full; ++kb) {
-        if (!mbar_wait(&ctl->pk_full[stage], phase, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(&ctl->pk_full[stage], phase, abort_flag)) { ok = false; break; }
         const uint8_t* sP = pk_stage + stage * kPkStageBytes;
         uint8_t* dst = smem + stage * kStageBytes + (kExpand == 1 ? 0 : kAStageBytes) + (seg >> 3) * 8192;
         uint2 v[4];
@@ -1337,9 +1322,9 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
                                                abort_flag, &ctl->tmem_empty[acc]))
           break;
       } else {
-        bool ok = mbar_wait(&ctl->tmem_full[acc], acc_phase, abort_flag);
+        bool ok = mbar_wait_warp(&ctl->tmem_full[acc], acc_phase, abort_flag);
         // the set's warps meet at barriers inside the tile: they go on, or leave, together
-        if (kEpi == EPI_VNM8) ok = set_all(set, ok);
+        if (kEpi == EPI_VNM8) ok = named_all(set + 1, 128, ok);
         if (!ok) break;
         tc_fence_after();
         if (!live) {
@@ -1367,7 +1352,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
       // M % 256 == 128 (regular raster only): the second CTA of the last row of pairs holds no rows
       const bool second = kDual && tile >= num_m_tiles * num_n_tiles_;
       const bool live = args.tile_table != nullptr || m0 < (second ? args.M2 : args.M);
-      if (!mbar_wait(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
+      if (!mbar_wait_warp(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
       if (live) epi_tile<kEpi, kBN, kOverlap>(args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts, second, acc_phase == 0,
                                               &ctl->tmem_empty[0]);
@@ -1605,7 +1590,7 @@ gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constan
                                            ctl->expand_lut, &ctl->tmem_full[h], phase, abort_flag, &ctl->tmem_empty[h]))
           break;
       } else {
-        if (!mbar_wait(&ctl->tmem_full[h], phase, abort_flag)) break;
+        if (!mbar_wait_warp(&ctl->tmem_full[h], phase, abort_flag)) break;
         tc_fence_after();
         if (live) epi_tile<kEpi, kTallBN>(args, taddr, m0, n0, n_limit, q, lane, wsm);
         release_accumulator(lane, &ctl->tmem_empty[h]);

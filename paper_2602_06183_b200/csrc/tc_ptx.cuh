@@ -1,6 +1,6 @@
 // Thin inline-PTX wrappers for the Blackwell (sm_100a) tensor-core path: mbarrier, TMA
 // (cp.async.bulk[.tensor]), tcgen05 (TMEM alloc / mma / mma.sp / cp / ld / commit / fences).
-// Every wait is bounded: it gives up after a clock budget and reports failure to the caller.
+// Every mbarrier wait is bounded: it gives up after a clock budget and reports failure to the caller.
 #pragma once
 
 #include <cuda.h>
@@ -78,6 +78,30 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     }
   }
   return true;
+}
+// The same called by a whole warp, with one answer for all of it. mbar_wait answers each lane by itself: around an expiry one
+// lane can see the barrier complete and another the abort flag or its spent budget, and lanes that went different ways must
+// not meet warp-collective code (.sync.aligned TMEM loads, full-mask shuffles, named barriers). A role that runs such code
+// waits with this; the roles in which one lane works (TMA, MMA issue) use mbar_wait.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                               long long budget = kWaitBudgetClocks) {
+  return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag, budget));
+}
+// Named barrier of `threads` threads (whole warps) with a vote: true when all of them say so. Warps that meet at barriers of
+// their own go on, or leave, together: one that has given up does not leave the others waiting.
+__device__ __forceinline__ bool named_all(int id, int threads, bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t"
+      ".reg .pred P, Q;\n\t"
+      "setp.ne.b32 P, %1, 0;\n\t"
+      "barrier.cta.red.and.pred Q, %2, %3, P;\n\t"
+      "selp.b32 %0, 1, 0, Q;\n\t"
+      "}\n"
+      : "=r"(r)
+      : "r"((uint32_t)ok), "r"(id), "r"(threads)
+      : "memory");
+  return r != 0;
 }
 
 // ---- fences ------------------------------------------------------------------------------------

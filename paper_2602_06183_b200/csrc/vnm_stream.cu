@@ -90,9 +90,9 @@ vnm_stream_kernel(const __grid_constant__ CUtensorMap tmapP, int64_t T, int64_t 
       const int64_t blk = i / nsx, cx = i - blk * nsx;
       const int cvalid = (int)min((int64_t)kSW, F - cx * kSW);
       Aux& a = aux[slot];
-      if (!mbar_wait(&ctl->full[slot], phase, abort_flag)) break;
+      const bool ok = mbar_wait_warp(&ctl->full[slot], phase, abort_flag);
       // rows first to last, one float32 add per element: two columns per thread (256-column strips) or one
-      if constexpr (kSW == 256) {
+      if (ok && kSW == 256) {
         const uint32_t* col = reinterpret_cast<const uint32_t*>(smem + slot * strip_bytes) + ts;
         float s0 = 0.f, s1 = 0.f;
         for (int r = 0; r < V; r += 8) {
@@ -110,7 +110,7 @@ vnm_stream_kernel(const __grid_constant__ CUtensorMap tmapP, int64_t T, int64_t 
         }
         a.score[2 * ts] = __float_as_uint(s0);
         a.score[2 * ts + 1] = __float_as_uint(s1);
-      } else {
+      } else if (ok) {
         const uint16_t* col = reinterpret_cast<const uint16_t*>(smem + slot * strip_bytes) + ts;
         float s0 = 0.f;
         for (int r = 0; r < V; r += 16) {
@@ -125,7 +125,7 @@ vnm_stream_kernel(const __grid_constant__ CUtensorMap tmapP, int64_t T, int64_t 
         }
         a.score[ts] = __float_as_uint(s0);
       }
-      named_sync(1, 128);
+      if (!named_all(1, 128, ok)) break;                       // the four warps go on, or leave, together
       constexpr int kCPT = kSW / 128;                          // columns per scoring thread
 #pragma unroll
       for (int c = 0; c < kCPT; ++c) {
@@ -169,7 +169,7 @@ vnm_stream_kernel(const __grid_constant__ CUtensorMap tmapP, int64_t T, int64_t 
       const int cvalid = (int)min((int64_t)kSW, F - cx * kSW);
       const bool live = g < cvalid / kM;
       const Aux& a = aux[slot];
-      if (!mbar_wait(&ctl->scored[slot], phase, abort_flag)) break;
+      if (!mbar_wait_warp(&ctl->scored[slot], phase, abort_flag)) break;
       const uint32_t c4 = *reinterpret_cast<const uint32_t*>(a.cidx + g * 4);
       const int64_t gg = cx * (kSW / kM) + g, trow = blk * V + r0;
       const uint8_t* tp = smem + slot * strip_bytes + r0 * (kSW * 2) + g * (kM * 2);
@@ -330,7 +330,7 @@ vnm8_stream_kernel(const __grid_constant__ CUtensorMap tmapP, int64_t T, int64_t
         continue;
       }
       const int blk = i / nsx, cx = i - blk * nsx;
-      if (!mbar_wait(&ctl->full[slot], phase, abort_flag)) break;
+      if (!mbar_wait_warp(&ctl->full[slot], phase, abort_flag)) break;
       const uint8_t* base = smem + slot * strip_bytes;
       // rows first to last, one float32 addition per element
       float s0 = 0.f, s1 = 0.f;
@@ -381,7 +381,7 @@ vnm8_stream_kernel(const __grid_constant__ CUtensorMap tmapP, int64_t T, int64_t
     for (int i = blockIdx.x; i < nstrips; i += gridDim.x) {
       const int blk = i / nsx, cx = i - blk * nsx;
       const bool live = cx * kSW + quad * 32 < F;
-      if (!mbar_wait(&ctl->scored[slot], phase, abort_flag)) break;
+      if (!mbar_wait_warp(&ctl->scored[slot], phase, abort_flag)) break;
       Stream8Sel sl[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) sl[j] = sel[slot * kGS + quad * 4 + j];

@@ -1,0 +1,27 @@
+"""What the device-side waits have to keep to, read off the CUDA sources (no GPU needed): a time-out cannot be produced in
+the product kernels without holding up a GPU, so the rules that make it end are checked where they are written."""
+import glob
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2602_06183_b200", "csrc")
+
+
+def _sources():
+    return {os.path.basename(p): open(p).read() for p in sorted(glob.glob(os.path.join(CSRC, "*.cu")))}
+
+
+def test_roles_of_whole_warps_wait_as_a_warp():
+    """Accumulators, packed tiles and scored strips are consumed by whole warps (aligned TMEM loads, shuffles, named
+    barriers): these waits give one answer to the warp. A wait answered lane by lane would let lanes part at an expiry."""
+    collective = re.compile(r"\bmbar_wait\(\s*(?:&ctl->(?:tmem_full|pk_full|scored)\b|tmem_full_bar\b)")
+    for name, text in _sources().items():
+        assert not collective.search(text), name
+    stream = _sources()["vnm_stream.cu"]
+    assert not re.search(r"\bmbar_wait\(&ctl->full\b", stream)          # scoring warps: shuffles and named barriers
+
+
+def test_warps_that_meet_at_named_barriers_leave_together():
+    """A warp that gave up must not leave the others of its set waiting at a named barrier: the sets that use one vote."""
+    assert re.search(r"named_all\(set \+ 1, 128, ok\)", _sources()["gemm_tc.cu"])
+    assert re.search(r"if \(!named_all\(1, 128, ok\)\) break;", _sources()["vnm_stream.cu"])

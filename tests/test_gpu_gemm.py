@@ -165,3 +165,13 @@ def test_bounded_wait_runs_out_and_is_reported():
     Cm, ws2 = binding.sf_gemm_dense(to_dev(A), True, to_dev(B), True)
     assert binding.sf_check_status(ws2) == binding.SF_OK
     assert rel_fro(f32(Cm), _f64(A) @ _f64(B).T) < TOL
+
+
+@pytest.mark.parametrize("budget", [200_000, 1_000_000, 3_000_000])
+def test_an_expired_wait_is_one_answer_for_the_warp(budget):
+    """The self-test completes the barrier right after lane 0 has given up, so the other lanes of the warp see it complete;
+    the status word is set only if all of them were told that the wait failed."""
+    ws = torch.zeros((256,), dtype=torch.uint8, device="cuda")
+    for _ in range(3):
+        binding.sf_selftest_wait_expiry(ws, budget_clocks=budget)
+        assert binding.sf_check_status(ws) == binding.SF_ERR_TIMEOUT
