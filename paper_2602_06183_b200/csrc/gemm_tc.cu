@@ -962,6 +962,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant_
   __syncthreads();
   if (threadIdx.x == 0 && ctl->abort_flag) atomicExch(args.status, 1);
   if (warp == 1) {
+    if (ctl->abort_flag) drain_after_expiry();
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }
@@ -1365,7 +1366,10 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   __syncwarp();
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && ctl->abort_flag) atomicExch(args.status, 1);
+  if (threadIdx.x == 0 && ctl->abort_flag) {
+    atomicExch(args.status, 1);
+    drain_after_expiry();
+  }
   cluster_sync_all();                                    // the peer is done with our shared memory and barriers
   if (warp == 1) {
     tc_fence_after();
@@ -1603,7 +1607,10 @@ gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constan
   __syncwarp();
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && ctl->abort_flag) atomicExch(args.status, 1);
+  if (threadIdx.x == 0 && ctl->abort_flag) {
+    atomicExch(args.status, 1);
+    drain_after_expiry();
+  }
   cluster_sync_all();
   if (warp == 1) {
     tc_fence_after();

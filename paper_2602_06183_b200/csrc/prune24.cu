@@ -158,6 +158,7 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64
     // one warp waits for the load (bounded), the block follows through the barrier
     bool ok = true;
     if (tid < 32) ok = mbar_wait(&full[slot], (uint32_t)(it / kColsSlots) & 1u, abort_flag);
+    if (!ok) drain_after_expiry();      // (here and not behind the loop: there it cost eight registers and 2 % of the time)
     if (__syncthreads_or(!ok)) break;
     // every warp has stored the previous panel: its stage buffers and its slot are free
     if (tid == 0) {

@@ -104,6 +104,14 @@ __device__ __forceinline__ bool named_all(int id, int threads, bool ok) {
   return r != 0;
 }
 
+// After an expired wait a CTA may leave with copies into its shared memory, or products reading it, still under way; that
+// memory goes to the next CTA. They take microseconds: waiting 2^22 clocks (2 to 3 ms) lets them land. Every kernel that
+// issues such copies calls this before it leaves, when its abort flag is set.
+__device__ __forceinline__ void drain_after_expiry() {
+  const long long t0 = clock64();
+  while (clock64() - t0 < (1LL << 22)) {}
+}
+
 // ---- fences ------------------------------------------------------------------------------------
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

@@ -217,6 +217,7 @@ vnm_stream_kernel(const __grid_constant__ CUtensorMap tmapP, int64_t T, int64_t 
       if (++slot == kSlots) { slot = 0; phase ^= 1; }
     }
   }
+  if (*abort_flag) drain_after_expiry();
 }
 
 // ---- groups of eight ----------------------------------------------------------------------------------------------
@@ -423,6 +424,7 @@ vnm8_stream_kernel(const __grid_constant__ CUtensorMap tmapP, int64_t T, int64_t
       if (++slot == (uint32_t)nslots) { slot = 0; phase ^= 1; }
     }
   }
+  if (*abort_flag) drain_after_expiry();
 }
 
 }  // namespace

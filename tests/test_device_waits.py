@@ -25,3 +25,15 @@ def test_warps_that_meet_at_named_barriers_leave_together():
     """A warp that gave up must not leave the others of its set waiting at a named barrier: the sets that use one vote."""
     assert re.search(r"named_all\(set \+ 1, 128, ok\)", _sources()["gemm_tc.cu"])
     assert re.search(r"if \(!named_all\(1, 128, ok\)\) break;", _sources()["vnm_stream.cu"])
+
+
+def test_kernels_with_copies_in_flight_drain_them_after_an_expired_wait():
+    """A CTA that leaves early must not hand its shared memory on while copies into it are under way."""
+    kernels = 0
+    for name, text in _sources().items():
+        for body in re.split(r"\n__global__ ", text)[1:]:
+            body = body[:body.index("\n}\n")]
+            if re.search(r"\b(tma_load_2d|tma_load_2d_2cta|bulk_load|tma_gather4_2d)\(", body):
+                kernels += 1
+                assert "drain_after_expiry()" in body, (name, body[:200])
+    assert kernels == 6          # three products, two streaming sparsifiers, the strided prune
