@@ -14,8 +14,11 @@ namespace sf {
 // Most recent failing cudaError_t (process-wide, informational).
 extern int g_last_cuda_error;
 
+// Reports a failed call as a status. The runtime keeps a failed call's error until it is asked for it: it is taken out here, or
+// the next launch check of this host thread would report it as its own.
 inline int cuda_fail(cudaError_t e) {
   g_last_cuda_error = static_cast<int>(e);
+  cudaGetLastError();
   return SF_ERR_CUDA;
 }
 

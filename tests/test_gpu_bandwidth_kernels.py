@@ -244,3 +244,16 @@ def test_vnm_random_shapes(T, F, V, M, apply, pad, seed):
             assert np.array_equal(bits(relu), ref.relu_vals)
         if want_dense:
             assert np.array_equal(bits(dense), ref.dense)
+
+
+def test_a_refused_launch_is_reported_once():
+    """65537 blocks of one row are one more than the second dimension of a grid holds: the runtime refuses the launch on the
+    host. The call that made it reports it; the calls after it (the self-test checks its launch, torch its own) do not."""
+    p = torch.zeros((65537, 64), dtype=torch.bfloat16, device="cuda")
+    ws = torch.zeros((256,), dtype=torch.uint8, device="cuda")
+    with pytest.raises(binding.SparseFFNError) as e:
+        binding.sf_vnm_sparsify_act(p, 1, 4)
+    assert e.value.status == binding.SF_ERR_CUDA
+    binding.sf_selftest_wait_expiry(ws, budget_clocks=100_000)
+    assert binding.sf_check_status(ws) == binding.SF_ERR_TIMEOUT
+    assert float((torch.ones(4, device="cuda") + 1).sum()) == 8.0
