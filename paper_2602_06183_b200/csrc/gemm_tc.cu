@@ -16,6 +16,15 @@
 // Dense mode double-buffers the 256-column accumulator so the epilogue of tile i overlaps the main
 // loop of tile i+1; sparse modes keep one accumulator plus the metadata columns.
 // Every mbarrier wait is bounded; on expiry the CTA raises a flag in the status word and leaves.
+// The waits that carry no clock budget, and what ends each of them:
+//   TMEM allocation (before griddepcontrol.wait, so possibly while the predecessor still runs): two CTAs of these kernels do
+//     not fit one SM (kExclusiveSmem below), so the columns are free as soon as a CTA is placed; should another library's
+//     kernel hold some, it gives them back when it ends, and it does not wait for this one: a kernel behind this one in the
+//     stream is placed after every CTA here has triggered, which it does after its allocation
+//   cluster barriers: set-up, which every CTA of a placed cluster reaches without waiting for anything but the above; teardown,
+//     which every role reaches because its own waits are bounded
+//   named barriers of a set of epilogue warps: entered by all four or by none (the vote behind the accumulator wait)
+//   griddepcontrol.wait: the predecessor, whose CTAs are all placed by then (it triggers from each of them) and bounded likewise
 #include "sf_common.cuh"
 #include "tc_ptx.cuh"
 #include "gemm_tc.cuh"
@@ -45,6 +54,11 @@ constexpr int kThreads = 192;                 // dense / 2:4 modes: producer, MM
 constexpr int kThreadsVenom = 576;            // + 8 TMA-gather warps and 4 cp.async-gather warps
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kMetaTmemCol = 256;
+
+// More than half of an SM's 228 KB: a kernel that allocates all of TMEM takes this much, so that no two of its CTAs, nor one
+// of the kernel before it, share an SM (the second would sit in its TMEM allocation until the first ends).
+constexpr int kExclusiveSmem = 228 * 1024 / 2 + 1;
+static_assert(smem_bytes(false) >= kExclusiveSmem && smem_bytes(true) >= kExclusiveSmem, "one CTA per SM");
 
 struct SmemCtl {
   uint64_t full[kMaxStages];
@@ -1692,7 +1706,7 @@ int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
                const CUtensorMap* tpk = nullptr) {
   auto kern = gemm_tc2_kernel<kMode, kAMN, kBMN, kEpi, kBN, kExpand, kFp8, kVar, kDual>;
   constexpr int smem = smem_bytes2(kMode != MODE_DENSE, kBN, kEpi, kExpand != 0, kFp8);
-  static_assert(smem <= 232448, "shared memory per CTA");
+  static_assert(smem <= 232448 && smem >= kExclusiveSmem, "shared memory per CTA: fits, and one CTA per SM");
   static bool attr_done[64] = {false};
   int dev = 0;
   SF_CUDA_TRY(cudaGetDevice(&dev));
@@ -1723,7 +1737,7 @@ int launch_tall(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap&
                 cudaStream_t s) {
   auto kern = gemm_tall_kernel<kBMN, kEpi, kFp8>;
   constexpr int smem = tall_smem(kEpi, kBMN, kFp8);
-  static_assert(smem <= 232448, "shared memory per CTA");
+  static_assert(smem <= 232448 && smem >= kExclusiveSmem, "shared memory per CTA: fits, and one CTA per SM");
   static bool attr_done[64] = {false};
   int dev = 0;
   SF_CUDA_TRY(cudaGetDevice(&dev));

@@ -37,3 +37,12 @@ def test_kernels_with_copies_in_flight_drain_them_after_an_expired_wait():
                 kernels += 1
                 assert "drain_after_expiry()" in body, (name, body[:200])
     assert kernels == 6          # three products, two streaming sparsifiers, the strided prune
+
+
+def test_kernels_that_take_all_of_tmem_have_an_sm_to_themselves():
+    """Every launcher of a kernel that allocates tensor memory asserts at compile time that two such CTAs do not fit one SM:
+    a CTA placed beside its predecessor's would sit in the allocation, which has no time limit."""
+    text = _sources()["gemm_tc.cu"]
+    allocating = [b for b in re.split(r"\n__global__ ", text)[1:] if "tmem_alloc" in b[:b.index("\n}\n")]]
+    assert len(allocating) == 3
+    assert len(re.findall(r"static_assert\(.*kExclusiveSmem", text)) == 3          # one-CTA, CTA-pair and 512-row kernels
