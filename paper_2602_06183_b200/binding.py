@@ -142,10 +142,19 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 
 
+# The raw handle of the current stream, without a torch.cuda.Stream object where this torch offers it (a private name).
+try:
+    from torch._C import _cuda_getCurrentRawStream, _cuda_getDevice
+
+    def _current_stream() -> int:
+        return _cuda_getCurrentRawStream(_cuda_getDevice())
+except ImportError:
+    def _current_stream() -> int:
+        return torch.cuda.current_stream().cuda_stream
+
+
 def _stream(stream: Optional[torch.cuda.Stream] = None):
-    if stream is not None:
-        return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _current_stream() if stream is None else stream.cuda_stream
 
 
 def make_desc(T, D, F, V, M, N=2, prune_mode=0, flags=0) -> sf_ffn_desc:

@@ -183,3 +183,18 @@ def test_routed_step_argument_checks_on_the_host(lib):
     p, n = C.c_void_p(), C.c_size_t()
     assert lib.sf_routed_ctx_view(d, ok, binding.SF_RCTX_Y1, C.byref(p), C.byref(n)) == binding.SF_ERR_UNSUPPORTED
     assert lib.sf_routed_ctx_view(d, ok, 99, C.byref(p), C.byref(n)) == binding.SF_ERR_SHAPE
+
+
+def test_binding_works_without_the_private_torch_names():
+    """The current stream is read through private torch names where they exist; a torch without them has the public way."""
+    import subprocess
+    import sys
+    code = ("import torch\n"
+            "for n in ('_cuda_getCurrentRawStream', '_cuda_getDevice'):\n"
+            "    if hasattr(torch._C, n): delattr(torch._C, n)\n"
+            "class S: cuda_stream = 1234\n"
+            "torch.cuda.current_stream = lambda: S()\n"
+            "from paper_2602_06183_b200 import binding\n"
+            "assert binding._stream() == 1234 and binding._stream(S()) == 1234\n")
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
