@@ -243,6 +243,19 @@ SF_API int sf_gemm_fp8_sparse24(const void* a_vals, const void* a_meta, const vo
  * sf_dense_ffn_fwd/bwd: the same equations with no pruning; fwd_ctx holds y1 (bf16 [T,F]).
  */
 SF_API int sf_ffn_workspace_size(const sf_ffn_desc* desc, size_t* fwd_ctx_bytes, size_t* workspace_bytes);
+/* How the sparse step of `desc` runs on the current device (148 SMs are assumed where there is none): host
+ * arithmetic by the same rules as the step calls, for tests and for accounts of a step's launches. A product's
+ * output is cut into tiles of `rows` x `cols`, which at most `cta_pairs` CTA pairs work on. */
+typedef struct sf_ffn_plan {
+  int32_t cta_pairs;
+  int32_t y1_selects;            /* 1: SquaredReLU + selection inside the y1 product's epilogue; 0: a kernel of their own */
+  int32_t y1_rows, y1_cols;      /* features x tokens */
+  int32_t dy1_rows, dy1_cols;    /* features x tokens */
+  int32_t weight_grad_launches;  /* 1: dW2 and dW1 share a launch (never in sf_ffn_step_host), 2: one each */
+  int32_t weight_grad_cols;      /* tile columns of the shared launch (256 rows); 0 without one */
+} sf_ffn_plan;
+SF_API int sf_ffn_step_plan(const sf_ffn_desc* desc, sf_ffn_plan* plan);
+
 SF_API int sf_sparse_ffn_fwd(const sf_ffn_desc* desc, const void* X, const void* W1, const void* W2,
                       void* Y, void* fwd_ctx, size_t fwd_ctx_bytes, void* workspace, size_t workspace_bytes,
                       void* stream);

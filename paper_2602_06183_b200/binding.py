@@ -31,6 +31,11 @@ class sf_ffn_desc(C.Structure):
                 ("prune_mode", C.c_int32), ("flags", C.c_int32)]
 
 
+class sf_ffn_plan(C.Structure):
+    _fields_ = [(n, C.c_int32) for n in ("cta_pairs", "y1_selects", "y1_rows", "y1_cols", "dy1_rows", "dy1_cols",
+                                         "weight_grad_launches", "weight_grad_cols")]
+
+
 class sf_router_desc(C.Structure):
     _fields_ = [("T", C.c_int64), ("D", C.c_int64), ("F", C.c_int64), ("E", C.c_int32), ("prune_mode", C.c_int32),
                 ("flags", C.c_int32), ("reserved", C.c_int32)]
@@ -76,6 +81,7 @@ _SIGNATURES = {
     "sf_gemm_fp8_sparse24": (_i32, [_vp, _vp, _vp, _vp, _i64, _i64, _i64, C.c_float, _vp, _vp]),
     "sf_gemm_venom": (_i32, [_vp, _vp, _vp, _vp, _vp, _i64, _i64, _i64, _i32, _i32, _vp, _vp]),
     "sf_ffn_workspace_size": (_i32, [C.POINTER(sf_ffn_desc), C.POINTER(_sz), C.POINTER(_sz)]),
+    "sf_ffn_step_plan": (_i32, [C.POINTER(sf_ffn_desc), C.POINTER(sf_ffn_plan)]),
     "sf_sparse_ffn_fwd": (_i32, [C.POINTER(sf_ffn_desc), _vp, _vp, _vp, _vp, _vp, _sz, _vp, _sz, _vp]),
     "sf_sparse_ffn_bwd": (_i32, [C.POINTER(sf_ffn_desc), _vp, _vp, _vp, _vp, _vp, _sz, _vp, _vp, _vp, _vp, _sz, _vp]),
     "sf_dense_ffn_fwd": (_i32, [C.POINTER(sf_ffn_desc), _vp, _vp, _vp, _vp, _vp, _sz, _vp, _sz, _vp]),
@@ -364,6 +370,12 @@ def sf_ffn_workspace_size(desc: sf_ffn_desc):
     a, b = _sz(), _sz()
     _check(lib().sf_ffn_workspace_size(C.byref(desc), C.byref(a), C.byref(b)), "sf_ffn_workspace_size")
     return a.value, b.value
+
+
+def sf_ffn_step_plan(desc: sf_ffn_desc) -> sf_ffn_plan:
+    plan = sf_ffn_plan()
+    _check(lib().sf_ffn_step_plan(C.byref(desc), C.byref(plan)), "sf_ffn_step_plan")
+    return plan
 
 
 def alloc_ffn_buffers(desc: sf_ffn_desc, device="cuda"):

@@ -185,13 +185,21 @@ int check_desc(const sf_ffn_desc* d) {
 inline uint8_t* at(void* base, size_t off) { return reinterpret_cast<uint8_t*>(base) + off; }
 inline const uint8_t* at(const void* base, size_t off) { return reinterpret_cast<const uint8_t*>(base) + off; }
 
+// dW2 is [D, F], or [F, D] where W2 is held that way.
+struct WeightGradShapes {
+  int64_t m2, n2;
+  explicit WeightGradShapes(const sf_ffn_desc& d)
+      : m2((d.flags & SF_FFN_W2_FD) ? d.F : d.D), n2((d.flags & SF_FFN_W2_FD) ? d.D : d.F) {}
+};
+
 // dW2 = dY^T h in the layout of W2 ([D, F], or [F, D] = h^T dY with w2_fd) and dW1 = dy1^T X [F, D]: in one launch where
 // that saves rounds of tiles. The host-buffer step keeps them apart: it downloads dW2 while dW1 is computed.
 int weight_grads(const sf_ffn_desc& d, const void* dY, const void* h, const void* dy1, const void* X, void* dW2, void* dW1,
                  int* status, cudaStream_t s) {
   const bool w2_fd = (d.flags & SF_FFN_W2_FD) != 0;
   const void *a2 = w2_fd ? h : dY, *b2 = w2_fd ? dY : h;
-  const int64_t m2 = w2_fd ? d.F : d.D, n2 = w2_fd ? d.D : d.F;
+  const WeightGradShapes g(d);
+  const int64_t m2 = g.m2, n2 = g.n2;
   if (!g_hooks && gemm_dual_tn_pays(m2, n2, d.F, d.D)) {
     const int st = gemm_dual_tn(a2, b2, m2, n2, dW2, dy1, X, d.F, d.D, dW1, d.T, status, s);
     trace_mark(s);
@@ -306,6 +314,22 @@ int sf_ffn_workspace_size(const sf_ffn_desc* desc, size_t* fwd_ctx_bytes, size_t
   const DenseLayout Dn = dense_layout(*desc);
   *fwd_ctx_bytes = S.ctx_total > Dn.ctx_total ? S.ctx_total : Dn.ctx_total;
   *workspace_bytes = S.ws_total > Dn.ws_total ? S.ws_total : Dn.ws_total;
+  return SF_OK;
+}
+
+int sf_ffn_step_plan(const sf_ffn_desc* desc, sf_ffn_plan* plan) {
+  if (!plan) return SF_ERR_NULL;
+  SF_TRY(check_desc(desc));
+  const sf_ffn_desc& d = *desc;
+  const SparseLayout L = sparse_layout(d);
+  const TileShape y1 = L.fused    ? gemm_sparse24_vnm8_tile(d.F, d.T, d.D, d.V)
+                       : d.M == 4 ? gemm_sparse24_act4_tile(d.F, d.T, d.D)
+                                  : gemm_sparse24_tile(d.F, d.T, d.D, EPI_STORE_T);
+  const TileShape dy1 = gemm_sparse24_drelu_tile(d.F, d.T, d.D);
+  const WeightGradShapes g(d);
+  const bool shared = !L.expand && gemm_dual_tn_pays(g.m2, g.n2, d.F, d.D);
+  *plan = sf_ffn_plan{gemm_cta_pairs(), L.fused || d.M == 4, y1.rows, y1.cols, dy1.rows, dy1.cols, shared ? 1 : 2,
+                      shared ? gemm_dual_tn_tile(g.m2, g.n2, d.F, d.D, d.T).cols : 0};
   return SF_OK;
 }
 

@@ -1822,6 +1822,8 @@ bool use_two_cta(int64_t M) { return M >= 256; }
 
 }  // namespace
 
+int gemm_cta_pairs() { return sm_count() / 2; }
+
 int make_tmap_2d(void* map, const void* base, int64_t rows, int64_t cols, int64_t ld, uint32_t box_cols,
                  uint32_t box_rows, bool swizzle128) {
   return make_tmap(reinterpret_cast<CUtensorMap*>(map), base, rows, cols, ld, box_cols, box_rows,
@@ -1877,11 +1879,15 @@ bool gemm_dual_tn_pays(int64_t M1, int64_t N1, int64_t M2, int64_t N2) {
   return (double)together <= 0.97 * (double)apart;
 }
 
+TileShape gemm_dual_tn_tile(int64_t M1, int64_t N1, int64_t M2, int64_t N2, int64_t K) {
+  return TileShape{256, best_width(M1, N1, K / 64, false, BN, 32, 200.0, false, M2, N2)};
+}
+
 int gemm_dual_tn(const void* A1, const void* B1, int64_t M1, int64_t N1, void* C1, const void* A2, const void* B2, int64_t M2,
                  int64_t N2, void* C2, int64_t K, int* status, cudaStream_t s) {
   if (M1 < 256 || M2 < 256 || M1 % 128 || N1 % 128 || M2 % 128 || N2 % 128 || K % 64) return SF_ERR_SHAPE;
   GemmArgs a{};
-  a.bn = best_width(M1, N1, K / 64, false, BN, 32, 200.0, false, M2, N2);
+  a.bn = gemm_dual_tn_tile(M1, N1, M2, N2, K).cols;
   CUtensorMap ta, tb, ta2, tb2;
   int st = make_tmap(&ta, A1, K, M1, M1, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st == SF_OK) st = make_tmap(&tb, B1, K, N1, N1, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
@@ -1897,6 +1903,14 @@ int gemm_dual_tn(const void* A1, const void* B1, int64_t M1, int64_t N1, void* C
                     : launch_two<MODE_DENSE, true, true, EPI_STORE, BN, 0, false, true, true>(ta, tb, ta2, a, s, &tb2);
 }
 
+// Transposed-output products on CTA pairs run 224-column tiles with two accumulators.
+TileShape gemm_sparse24_tile(int64_t M, int64_t N, int64_t K, int epi) {
+  const bool plain = (epi == EPI_STORE);
+  const int max_bn = plain ? BN : kNarrowBN;
+  if (use_tall(M, N, K / 128, max_bn, plain ? 2500.0 : 0.0, 2500.0)) return TileShape{512, kTallBN};
+  return TileShape{256, best_width(M, N, K / 128, true, max_bn, 32, 400.0, plain)};
+}
+
 int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, bool b_kmajor, int64_t M, int64_t N,
                   int64_t K, int epi, void* C, int64_t ldc, int* status, cudaStream_t s) {
   const bool two = use_two_cta(M);
@@ -1905,7 +1919,8 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   const bool plain = (epi == EPI_STORE);                 // row-major output, either B layout: two-CTA kernel only
   if ((plain || !b_kmajor) && !two) return SF_ERR_UNSUPPORTED;
   CUtensorMap ta, tb, tm;
-  if (two && use_tall(M, N, K / 128, plain ? BN : kNarrowBN, plain ? 2500.0 : 0.0, 2500.0)) {
+  const TileShape tile = two ? gemm_sparse24_tile(M, N, K, epi) : TileShape{BM, BN};
+  if (tile.rows == 512) {
     CUtensorMap tbn;
     const int st = tall_maps(a_vals, meta_hw, B, b_kmajor, M, N, K, 0, 2, &ta, &tb, &tbn, &tm);
     if (st != SF_OK) return st;
@@ -1918,9 +1933,7 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   int st = two ? make_tmap(&ta, a_vals, M, K / 2, K / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B)
                : make_tmap(&ta, a_vals, M, K / 2, K / 2, 32, 128, CU_TENSOR_MAP_SWIZZLE_64B);
   if (st != SF_OK) return st;
-  // transposed-output products on CTA pairs run 224-column tiles with two accumulators
-  const int max_bn = plain ? BN : kNarrowBN;
-  const int bn = two ? best_width(M, N, K / 128, true, max_bn, 32, 400.0, plain) : BN;
+  const int bn = tile.cols;
   if (b_kmajor) st = make_tmap(&tb, B, N, K, K, 64, two ? bn / 2 : 256, CU_TENSOR_MAP_SWIZZLE_128B);
   else          st = make_tmap(&tb, B, K, N, N, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st != SF_OK) return st;
@@ -1936,7 +1949,7 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   a.C = C; a.ldc = ldc; a.meta_hw = meta_hw; a.status = status;
   a.num_m_tiles = (int)(M / BM); a.num_n_tiles = (int)(N / BN); a.num_k_blocks = (int)(K / 64);
   a.bn = bn;
-  const bool var = two && bn != max_bn;
+  const bool var = two && bn != (plain ? BN : kNarrowBN);
   if (epi == EPI_STORE) {
     if (b_kmajor) return var ? launch_two<MODE_SPARSE24, false, false, EPI_STORE, BN, 0, false, true>(ta, tb, tm, a, s)
                              : launch_two<MODE_SPARSE24, false, false, EPI_STORE>(ta, tb, tm, a, s);
@@ -1963,6 +1976,18 @@ int weight_token_maps(const void* w_vals, const uint8_t* meta_hw, const void* to
 }
 }  // namespace
 
+TileShape gemm_sparse24_drelu_tile(int64_t F, int64_t T, int64_t D) {
+  // 256-column tiles (one accumulator, 1000 clocks before the next main loop starts) or 224 and narrower (two), by estimated
+  // clocks: T 4096, D 2048, F 8192 is 7 rounds of 256-column tiles or 9 of 224: 71.6 us against 79.3.
+  // (At T 8192, D 4096, F 16384, 28 and 32 rounds, the two are equal: it has to gain 5 %.)
+  const int64_t stages = D / 128, P = sm_count() / 2, nm = (F + 255) / 256;
+  auto rounds = [&](int64_t w) { return (double)((nm * ((T + w - 1) / w) + P - 1) / P); };
+  const int bn = best_width(F, T, stages, true, kNarrowBN, 32, 500.0, false);
+  const bool wide = stages >= 8 && bn == kNarrowBN && rounds(256) * (stages * 735.0 + 1000.0) < 0.95 * rounds(kNarrowBN) * (stages * 680.0);
+  if (use_tall(F, T, stages, wide ? 256 : kNarrowBN, wide ? 1000.0 : 0.0, 4000.0)) return TileShape{512, kTallBN};
+  return TileShape{256, wide ? 256 : bn};
+}
+
 int gemm_sparse24_drelu(const void* w_vals, const uint8_t* meta_hw, const void* dY, int64_t F, int64_t T, int64_t D,
                         const ActMask& mask, void* dy1_vals, void* dy1_dense, int* status, cudaStream_t s) {
   if (F < 256 || F % 128 || T % 128 || D % 128) return SF_ERR_SHAPE;
@@ -1973,22 +1998,16 @@ int gemm_sparse24_drelu(const void* w_vals, const uint8_t* meta_hw, const void* 
     a.colidx = mask.colidx; a.V = mask.V; a.Mv = mask.Mv; a.G = F / mask.Mv;
   }
   CUtensorMap ta, tb, tbn, tm;
-  // 256-column tiles (one accumulator, 1000 clocks before the next main loop starts) or 224 and narrower (two), by estimated
-  // clocks: T 4096, D 2048, F 8192 is 7 rounds of 256-column tiles or 9 of 224: 71.6 us against 79.3.
-  // (At T 8192, D 4096, F 16384, 28 and 32 rounds, the two are equal: it has to gain 5 %.)
-  const int64_t stages = D / 128, P = sm_count() / 2, nm = (F + 255) / 256;
-  auto rounds = [&](int64_t w) { return (double)((nm * ((T + w - 1) / w) + P - 1) / P); };
-  a.bn = best_width(F, T, stages, true, kNarrowBN, 32, 500.0, false);
-  const bool wide = stages >= 8 && a.bn == kNarrowBN && rounds(256) * (stages * 735.0 + 1000.0) < 0.95 * rounds(kNarrowBN) * (stages * 680.0);
-  if (use_tall(F, T, stages, wide ? 256 : kNarrowBN, wide ? 1000.0 : 0.0, 4000.0)) {
+  const TileShape tile = gemm_sparse24_drelu_tile(F, T, D);
+  if (tile.rows == 512) {
     const int st = tall_maps(w_vals, meta_hw, dY, true, F, T, D, 0, 2, &ta, &tb, &tbn, &tm);
     if (st != SF_OK) return st;
     return mask.colidx ? launch_tall<false, EPI_DRELUV_T>(ta, tb, tbn, tm, a, s) : launch_tall<false, EPI_DRELU24_T>(ta, tb, tbn, tm, a, s);
   }
-  if (wide) a.bn = 256;
+  a.bn = tile.cols;
   const int st = weight_token_maps(w_vals, meta_hw, dY, F, T, D, a.bn, &ta, &tb, &tm);
   if (st != SF_OK) return st;
-  if (wide)
+  if (a.bn == 256)
     return mask.colidx ? launch_two<MODE_SPARSE24, false, false, EPI_DRELUV_T, 256>(ta, tb, tm, a, s)
                        : launch_two<MODE_SPARSE24, false, false, EPI_DRELU24_T, 256>(ta, tb, tm, a, s);
   if (a.bn != kNarrowBN)
@@ -1998,11 +2017,15 @@ int gemm_sparse24_drelu(const void* w_vals, const uint8_t* meta_hw, const void* 
                      : launch_two<MODE_SPARSE24, false, false, EPI_DRELU24_T, kNarrowBN>(ta, tb, tm, a, s);
 }
 
+TileShape gemm_sparse24_act4_tile(int64_t F, int64_t T, int64_t D) {
+  return TileShape{256, best_width(F, T, D / 128, true, kNarrowBN, 32, 500.0, false)};
+}
+
 int gemm_sparse24_act4(const void* w_vals, const uint8_t* meta_hw, const void* X, int64_t F, int64_t T, int64_t D, int V,
                        const Act24Out& out, void* colidx, int* status, cudaStream_t s) {
   if (F < 256 || F % 128 || T % 128 || D % 128) return SF_ERR_SHAPE;
   GemmArgs a{};
-  a.bn = best_width(F, T, D / 128, true, kNarrowBN, 32, 500.0, false);
+  a.bn = gemm_sparse24_act4_tile(F, T, D).cols;
   CUtensorMap ta, tb, tm;
   const int st = weight_token_maps(w_vals, meta_hw, X, F, T, D, a.bn, &ta, &tb, &tm);
   if (st != SF_OK) return st;
@@ -2082,21 +2105,21 @@ bool gemm_sparse24_vnm8_supported(int64_t F, int64_t T, int64_t D, int V) {
 // D 512 79 and 89. Estimated clocks: rounds of tiles x the longer of main loop and epilogue, plus the last epilogue; per 64
 // tokens the epilogue takes 3000 where two tiles' overlap and 6500 where both sets work on one tile; reading a shared
 // accumulator, 2500, is exposed. Tiles hold whole V-blocks: the narrow width for V = 128 is 128.
-static int vnm8_width(int64_t F, int64_t T, int64_t stages, int V) {
-  const int64_t P = sm_count() / 2, nm = (F + 255) / 256;
+TileShape gemm_sparse24_vnm8_tile(int64_t F, int64_t T, int64_t D, int V) {
+  const int64_t stages = D / 128, P = sm_count() / 2, nm = (F + 255) / 256;
   auto rounds = [&](int w) { return (double)((nm * ((T + w - 1) / w) + P - 1) / P); };
   const int narrow = V == 128 ? 128 : best_width(F, T, stages, true, 192, 64, 1500.0, false);
   const double epi = 1500.0 * (narrow / 32), main = stages * 0.93 * (272 + 2 * narrow), wide = stages * 735.0 + 2500.0;
   const double cost_narrow = rounds(narrow) * (main > epi ? main : epi) + epi;
   const double cost_wide = rounds(256) * (wide > 13000.0 ? wide : 13000.0) + 9000.0;
-  return cost_wide < cost_narrow ? 256 : narrow;
+  return TileShape{256, cost_wide < cost_narrow ? 256 : narrow};
 }
 
 int gemm_sparse24_vnm8(const void* a_vals, const uint8_t* meta_hw, const void* X, int64_t F, int64_t T, int64_t D,
                        int V, const Vnm8Out& out, int* status, cudaStream_t s) {
   if (!gemm_sparse24_vnm8_supported(F, T, D, V)) return SF_ERR_SHAPE;
   GemmArgs a{};
-  a.bn = vnm8_width(F, T, D / 128, V);
+  a.bn = gemm_sparse24_vnm8_tile(F, T, D, V).cols;
   CUtensorMap ta, tb, tm;
   const int st = weight_token_maps(a_vals, meta_hw, X, F, T, D, a.bn, &ta, &tb, &tm);
   if (st != SF_OK) return st;

@@ -85,6 +85,18 @@ struct Vnm8Out {
   void *vals, *relu, *meta, *colidx, *vals24, *relu24, *meta24, *meta24_hw, *y1, *dense;
 };
 
+// The tile that a product on CTA pairs takes for a problem, by the rules beside each (host arithmetic on the sizes and the
+// number of SMs; 148 are assumed where there is no device): rows x columns of the accumulator.
+struct TileShape {
+  int rows, cols;
+};
+TileShape gemm_sparse24_tile(int64_t M, int64_t N, int64_t K, int epi);
+TileShape gemm_sparse24_drelu_tile(int64_t F, int64_t T, int64_t D);
+TileShape gemm_sparse24_act4_tile(int64_t F, int64_t T, int64_t D);
+TileShape gemm_sparse24_vnm8_tile(int64_t F, int64_t T, int64_t D, int V);
+TileShape gemm_dual_tn_tile(int64_t M1, int64_t N1, int64_t M2, int64_t N2, int64_t K);
+int gemm_cta_pairs();
+
 // D[M,N] = op(A) op(B)^T, tiles 128 x 256, K % 64 == 0.
 int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64_t M, int64_t N, int64_t K, int epi,
                void* C, int64_t ldc, void* C2, int64_t ldc2, const void* aux, int64_t ldaux, int* status,

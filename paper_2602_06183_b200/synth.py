@@ -30,9 +30,9 @@ __all__ = [
 FFN_CONFIGS = {
     "c1_small": dict(T=1024, D=256, F=1024, V=64, N=2, M=8, sigma_w=0.02, seed=0),
     # the d_model = 4096 layer; the configuration says "V:2:8" and leaves V free: V = 64 is the block height of
-    # the paper's Table 5, and three such blocks fill one token tile of the fused y1 epilogue
+    # the paper's Table 5
     "c4_d4096": dict(T=8192, D=4096, F=16384, V=64, N=2, M=8, sigma_w=0.02, seed=4),
-    # the same layer with 128-token blocks (SquaredReLU + V:N:M then run as a second kernel by default)
+    # the same layer with 128-token blocks
     "c4_d4096_v128": dict(T=8192, D=4096, F=16384, V=128, N=2, M=8, sigma_w=0.02, seed=4),
     # one eighth of c4's tokens with the full-size layer: weights (134 MB each) still exceed the
     # L2, device footprint ~1.5 GB; used for profiler captures that must stay small

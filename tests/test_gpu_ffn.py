@@ -112,8 +112,8 @@ def test_sparse_ffn_c1_teacher_forced(prune_mode, act_shift):
 
 
 @pytest.mark.parametrize("cfg", [
-    dict(T=1024, D=256, F=1024, V=64, N=2, M=8, sigma_w=0.02, seed=0),      # fused epilogue, three 64-token blocks per tile
-    dict(T=512, D=256, F=512, V=128, N=2, M=8, sigma_w=0.05, seed=3),       # two-kernel path (the default for V = 128)
+    dict(T=1024, D=256, F=1024, V=64, N=2, M=8, sigma_w=0.02, seed=0),      # selection in the y1 epilogue, one 64-token block per tile
+    dict(T=512, D=256, F=512, V=128, N=2, M=8, sigma_w=0.05, seed=3),       # the same, one 128-token block per tile
     dict(T=512, D=256, F=2048, V=128, N=2, M=16, sigma_w=0.05, seed=17),    # condensed Venom products
 ], ids=["m8_v64", "m8_v128", "m16_v128"])
 def test_step_without_saved_y1_is_the_same_step(cfg):
@@ -132,8 +132,8 @@ def test_step_without_saved_y1_is_the_same_step(cfg):
 @pytest.mark.parametrize("V,act_shift", [(64, 0.0), (128, 0.0), (64, -1.3)])
 def test_fused_activation_epilogue_equals_the_two_kernel_path(V, act_shift):
     """SquaredReLU + V:N:M inside the y1 product's epilogue against the stand-alone kernel on a stored
-    y1: same accumulation, same selection rule, so every output must agree bit for bit. T is not a
-    multiple of the fused kernel's 192-token tile, so the last tile is ragged."""
+    y1: same accumulation, same selection rule, so every output must agree bit for bit. These sizes take tiles of one
+    V-block; wider ones, with a ragged last tile, are in test_step_tiles.py."""
     cfg = dict(T=1280, D=512, F=768, V=V, N=2, M=8, sigma_w=0.05, seed=41)
     Y1 = binding.SF_FFN_SAVE_Y1
     inputs, fused = _run_sparse(cfg, act_shift=act_shift, flags=Y1 | binding.SF_FFN_FUSED_ACT)
