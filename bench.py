@@ -167,9 +167,27 @@ TRACE_NAMES = ["prune24_W1", "gemm_y1", "vnm_sparsify", "transpose_W2", "gemm_y3
                None, "prune24_W2", "gemm_dy1", "pack_dy1", "gemm_dX", "gemm_dW2", "gemm_dW1"]
 
 
-def _step_path(V, M):
-    """Which kernels the library runs for this configuration (mirrors the rule in the step's layout)."""
-    return "fused" if M == 8 else "plain24" if M == 4 else "venom"
+def _step_kernels(plan, M, flags):
+    """(path, {kernel: trace intervals that hold it}) of one sparse step, from the library's own plan of it. Where both
+    weight gradients share a launch, the dW2 interval holds it and the dW1 interval is empty."""
+    from paper_2602_06183_b200 import binding
+    path = "plain24" if M == 4 else ("fused" if plan.y1_selects else "two_kernel") if M == 8 else "venom"
+    kernels = ["prune24_W1", "gemm_y1"] + ([] if plan.y1_selects else ["vnm_sparsify"])
+    kernels += ["transpose_W2"] if path == "venom" and not flags & binding.SF_FFN_W2_FD else []
+    kernels += ["gemm_y3", "prune24_W2", "gemm_dy1", "gemm_dX"]
+    held = {n: [n] for n in kernels}
+    if plan.weight_grad_launches == 1:
+        held["gemm_dW2_dW1"] = ["gemm_dW2", "gemm_dW1"]
+    else:
+        held.update(gemm_dW2=["gemm_dW2"], gemm_dW1=["gemm_dW1"])
+    return path, held
+
+
+def _step_products(kernels, M):
+    """{product: (algorithmic work in dense products, peak as a multiple of the dense peak)} of the launched products."""
+    work = {"gemm_y1": (1.0, 2.0), "gemm_dy1": (1.0, 2.0), "gemm_y3": (4.0 / M, 2.0), "gemm_dX": (4.0 / M, 2.0),
+            "gemm_dW2": (1.0, 1.0), "gemm_dW1": (1.0, 1.0), "gemm_dW2_dW1": (2.0, 1.0)}
+    return {n: w for n, w in work.items() if n in kernels}
 
 
 def run_ours(args, cfg):
@@ -259,11 +277,8 @@ def run_ours(args, cfg):
         for n, v in zip(TRACE_NAMES, d[13 * s: 13 * s + 12]):
             if n:
                 per.setdefault(n, []).append(v)
-    path = _step_path(V, M) if not (args.flags & (binding.SF_FFN_UNFUSED_ACT | binding.SF_FFN_FUSED_ACT)) else \
-        ("fused" if args.flags & binding.SF_FFN_FUSED_ACT else "two_kernel")
-    not_launched = {"fused": {"vnm_sparsify", "transpose_W2", "pack_dy1"}, "two_kernel": {"transpose_W2", "pack_dy1"},
-                    "plain24": {"vnm_sparsify", "transpose_W2", "pack_dy1"}, "venom": {"pack_dy1"}}[path]   # empty trace intervals
-    kern_ms = {n: float(np.mean(v)) for n, v in per.items() if n not in not_launched}
+    path, held = _step_kernels(binding.sf_ffn_step_plan(desc), M, args.flags)
+    kern_ms = {n: float(sum(np.mean(per[i]) for i in intervals)) for n, intervals in held.items()}
     kern_sum = float(sum(kern_ms.values()))
 
     def rested_warmup(fn):
@@ -344,8 +359,7 @@ def run_ours(args, cfg):
     # 2*T*D*F at the dense peak. The step loop runs for a long time at the power cap, so the peak is the SUSTAINED
     # measured bf16 GEMM figure (the burst figure is printed beside it).
     P = peaks["bf16_tflops_sustained"]
-    prod = {"gemm_y1": (1.0, 2.0), "gemm_dy1": (1.0, 2.0), "gemm_y3": (4.0 / M, 2.0), "gemm_dX": (4.0 / M, 2.0),
-            "gemm_dW2": (1.0, 1.0), "gemm_dW1": (1.0, 1.0)}
+    prod = _step_products(kern_ms, M)
     products = {}
     for n, (alg, ratio) in prod.items():
         t = kern_ms[n] / 1e3
@@ -355,7 +369,7 @@ def run_ours(args, cfg):
     if path == "fused":
         products["gemm_y1"]["includes"] = "SquaredReLU + V:N:M selection in the epilogue"
     groups = {"2:4 tensor kernels (y1, dy1, y3, dX)": (["gemm_y1", "gemm_dy1", "gemm_y3", "gemm_dX"], 2.0),
-              "dense tensor kernel (dW2, dW1)": (["gemm_dW2", "gemm_dW1"], 1.0)}
+              "dense tensor kernel (dW2, dW1)": ([n for n in prod if n.startswith("gemm_dW")], 1.0)}
     gstat = {}
     for g, (ks, ratio) in groups.items():
         t = sum(kern_ms[k] for k in ks) / 1e3
@@ -395,8 +409,7 @@ def run_ours(args, cfg):
     else:
         bw["vnm_sparsify"] = {"fused_into": "gemm_y1", "algorithmic_bytes": vnm_alg - 2.0 * T * F,
                               "note": "no separate kernel: y1 never leaves the chip"}
-    # (the weight gradients have the same work: where one launch takes both, the second interval is empty)
-    launches_per_step = len(kern_ms) - (kern_ms["gemm_dW1"] < 0.2 * kern_ms["gemm_dW2"])
+    launches_per_step = len(kern_ms)
 
     # ---- end to end through the host-buffer entry point (H2D of inputs and D2H of results timed)
     staging = torch.empty((binding.sf_ffn_host_staging_size(desc),), dtype=torch.uint8, device="cuda")
