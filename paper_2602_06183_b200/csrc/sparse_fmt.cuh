@@ -1,7 +1,6 @@
 // Device helpers for the two packed activation formats of the step: the V:N:M form with groups of
 // eight columns (Section 2.3) and its re-expression as a plain 2:4 operand over all columns.
-// Shared by the stand-alone sparsify kernel, the fused epilogue of the y1 product, the dy1 epilogue
-// and the operand expanders of the weight-gradient products.
+// Shared by the sparsify kernels and the activation epilogues of the products.
 #pragma once
 
 #include "sf_common.cuh"
@@ -50,29 +49,6 @@ __device__ __forceinline__ void vnm8_pair_selectors(uint32_t ca, uint32_t cb, ui
   const uint32_t nhi = both_hi ? pair_nib : (both_lo ? 4u : (pb == 0u ? 4u : (pb << 2)));
   sel = make_uint4(sd[0] | (sd[1] << 16), sd[2] | (sd[3] << 16), s1 | (s2 << 16), s_wlo | (s_whi << 16));
   nib24 = nlo | (nhi << 4);
-}
-
-// The six legal position pairs of a 2:4 nibble are distinct modulo 7: table slot of a nibble.
-__device__ __forceinline__ uint32_t nib_slot(uint32_t nib) { return nib - 7u * ((nib * 37u) >> 8); }
-
-// One 2:4 group back to its four dense columns: `pair` holds the two stored values (first in the
-// low half), `nib` = pos0 | pos1 << 2. w0 = columns 0, 1; w1 = columns 2, 3; dropped columns are +0.
-__device__ __forceinline__ void expand24(uint32_t pair, uint32_t nib, uint32_t& w0, uint32_t& w1) {
-  const uint32_t s0 = (nib & 3u) * 8u, s1 = (nib >> 2) * 8u;      // selector field of each kept column
-  uint32_t s = 0x44444444u;                                      // every byte from the zero operand
-  s = (s & ~(0xFFu << s0)) | (0x10u << s0);
-  s = (s & ~(0xFFu << s1)) | (0x32u << s1);
-  w0 = __byte_perm(pair, 0u, s & 0xFFFFu);
-  w1 = __byte_perm(pair, 0u, s >> 16);
-}
-
-// Eight dense columns (16 bytes) from the 2:4 layout: `v` = the four stored values of the two
-// groups, `mb` = their two nibbles (low nibble = first group).
-__device__ __forceinline__ uint4 expand24_x8(uint2 v, uint32_t mb) {
-  uint4 d;
-  expand24(v.x, mb & 0xFu, d.x, d.y);
-  expand24(v.y, (mb >> 4) & 0xFu, d.z, d.w);
-  return d;
 }
 
 }  // namespace sf

@@ -18,18 +18,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // address as an integer, lets the compiler see that what is derived from it is shared memory.
 __device__ __forceinline__ uint32_t align_pad(const void* p, uint32_t align) { return (0u - smem_u32(p)) & (align - 1u); }
 
-__device__ __forceinline__ bool elect_one() {
-  uint32_t pred = 0;
-  asm volatile(
-      "{\n\t"
-      ".reg .pred P;\n\t"
-      "elect.sync _|P, 0xFFFFFFFF;\n\t"
-      "selp.b32 %0, 1, 0, P;\n\t"
-      "}\n"
-      : "=r"(pred));
-  return pred != 0;
-}
-
 // ---- mbarrier --------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
@@ -210,9 +198,8 @@ __device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&v)
       : "r"(taddr)
       : "memory");
 }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// Same wait, with the loaded registers as in/out operands so that no use of them can be scheduled
-// before the wait (needed when another load is issued between this load and its wait).
+// Waits for the loads, with the loaded registers as in/out operands so that no use of them can be scheduled before the wait
+// (needed when another load is issued between this load and its wait).
 __device__ __forceinline__ void tmem_ld_wait_on(uint32_t (&v)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
