@@ -59,10 +59,13 @@ def _l2_note(operand_bytes: int, activation_bytes: int) -> str:
             "fit the 126 MB L2 and no flush is done: a parity-size workload, its timing is L2-resident and is not a benchmark figure")
 
 
-def _traffic():
-    """Per-launch DRAM traffic of the step's kernels from the committed single-pass ncu capture."""
+def _traffic(workload, prune_mode, flags):
+    """Per-launch DRAM traffic of the step's kernels from the committed single-pass ncu capture; nothing for a step other
+    than the captured one."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
-    return json.load(open(path)) if os.path.exists(path) else {}
+    t = json.load(open(path)) if os.path.exists(path) else {}
+    on = t.get("captured_on", {})
+    return t if (on.get("workload"), on.get("prune_mode"), on.get("flags")) == (workload, prune_mode, flags) else {}
 
 
 class ClockSampler:
@@ -377,7 +380,7 @@ def run_ours(args, cfg):
         gstat[g] = {"ms": t * 1e3, "launches_per_step": len(ks), "achieved": alg / t / 1e12, "peak": P * ratio,
                     "frac": alg / t / 1e12 / (P * ratio), "share_of_step": t * 1e3 / kern_sum}
     dom = max(gstat, key=lambda g: gstat[g]["ms"])
-    traffic = _traffic()
+    traffic = _traffic(args.workload, args.prune_mode, args.flags)
     roofline = {"bound": "tensor", "kernel": dom, "achieved": gstat[dom]["achieved"], "peak": gstat[dom]["peak"],
                 "unit": "TFLOP/s", "frac": gstat[dom]["frac"],
                 "traffic": traffic.get("kernels", {}).get(dom), "traffic_captured_on": traffic.get("captured_on"),

@@ -44,3 +44,11 @@ def test_launches_follow_the_flags():
     path, held, _ = _account(**m8, flags=binding.SF_FFN_UNFUSED_ACT)
     assert path == "two_kernel" and "vnm_sparsify" in held
     assert _account(T=1024, D=256, F=1024, V=64, M=4)[0] == "plain24"
+
+
+def test_measured_traffic_is_printed_for_the_captured_step_only():
+    """A capture says nothing about another workload, prune mode or flags."""
+    t = bench._traffic("c4_d4096", 0, 0)
+    assert set(t["kernels"]) >= {"prune24_W1", "gemm_y1", "gemm_y3", "prune24_W2", "gemm_dy1", "gemm_dX", "gemm_dW2", "gemm_dW1"}
+    for other in (("c5_d8192", 0, 0), ("c4_d4096", 1, 0), ("c4_d4096", 0, binding.SF_FFN_W2_FD)):
+        assert bench._traffic(*other) == {}
