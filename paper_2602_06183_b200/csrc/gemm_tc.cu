@@ -1789,6 +1789,10 @@ int best_width(int64_t M, int64_t N, int64_t stages, bool sparse, int max_bn, in
   return best;
 }
 
+// The comparison is with 256-row tiles of full width, not with the narrower ones that best_width would take: where those
+// end sooner by the estimate (4 % of drawn sizes, few tokens or few rows of tiles), less is lost than it says: dy1 at T 256,
+// D 3328, F 10752 takes 32.7 us on 512 x 224 tiles and 30.7 on 256 x 96, T 256, D 3456, F 12416 32.7 and 30.8. What the rule is
+// for: y3 at T 1024, D 4096, F 16384 70.5 us on 512-row tiles and 78.2 without, dX 67.9 and 74.1.
 // 512 x 224 tiles, or 256-row tiles of `bn` columns (bn = 256: one accumulator, its epilogue exposed)? Estimated clocks
 // of the busiest CTA pair: rounds of tiles x (k-stages x clocks per stage + the epilogue that nothing hides). A stage's
 // clocks measured with clock stamps on all SMs: 735 (256 wide), 680 (224 wide), 1190 (512 x 224). A narrow tile of the
@@ -1871,6 +1875,10 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
   return SF_ERR_UNSUPPORTED;
 }
 
+// By rounds of 256-column tiles, whatever width either side then runs, and without the launch that is saved: the shared
+// launch is never the slower one by the estimate where this takes it (165 000 drawn sizes), but it would also pay at sizes that
+// are left apart: whole step at T 1920, D 1408, F 5504 168.8 us apart and 160.6 together, T 512, D 1024, F 4096 77.6 and 72.4,
+// T 256, D 256, F 9728 99.4 and 92.1.
 bool gemm_dual_tn_pays(int64_t M1, int64_t N1, int64_t M2, int64_t N2) {
   if (M1 < 256 || M2 < 256) return false;
   const int64_t P = sm_count() / 2;
@@ -1980,6 +1988,9 @@ TileShape gemm_sparse24_drelu_tile(int64_t F, int64_t T, int64_t D) {
   // 256-column tiles (one accumulator, 1000 clocks before the next main loop starts) or 224 and narrower (two), by estimated
   // clocks: T 4096, D 2048, F 8192 is 7 rounds of 256-column tiles or 9 of 224: 71.6 us against 79.3.
   // (At T 8192, D 4096, F 16384, 28 and 32 rounds, the two are equal: it has to gain 5 %.)
+  // Fewer than eight k-stages (D < 1024) keep 224 columns. Sizes there for which the estimate prefers 256 are rare (11 of
+  // 165 000 drawn); 256 columns take T 768, D 896, F 24832 from 43.0 to 38.9 us, T 1024, D 768, F 23296 from 49.1 to 45.1, T 2048,
+  // D 896, F 11392 from 49.1 to 47.2 and T 768, D 768, F 23808 from 38.9 to 38.7, so the line could be lower.
   const int64_t stages = D / 128, P = sm_count() / 2, nm = (F + 255) / 256;
   auto rounds = [&](int64_t w) { return (double)((nm * ((T + w - 1) / w) + P - 1) / P); };
   const int bn = best_width(F, T, stages, true, kNarrowBN, 32, 500.0, false);

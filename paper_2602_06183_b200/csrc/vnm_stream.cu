@@ -7,7 +7,7 @@
 //   warps 1..4    column scores (sequential float32 sums, two columns per thread), ranking of the eight columns
 //                 of every group, colidx
 //   warps 5..12   emit: one thread per (row, group): 2:4 among the kept columns, packed stores
-// Persistent CTAs walk the strips; every wait is bounded (a role that gives up makes the others leave too).
+// Persistent CTAs walk the strips; every mbarrier wait is bounded (a role that gives up makes the others leave too).
 #include "sf_common.cuh"
 #include "sparse_fmt.cuh"
 #include "tc_ptx.cuh"
