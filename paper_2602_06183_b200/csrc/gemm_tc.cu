@@ -1789,16 +1789,16 @@ int best_width(int64_t M, int64_t N, int64_t stages, bool sparse, int max_bn, in
   return best;
 }
 
-// The comparison is with 256-row tiles of full width, not with the narrower ones that best_width would take: where those
-// end sooner by the estimate (4 % of drawn sizes, few tokens or few rows of tiles), less is lost than it says: dy1 at T 256,
-// D 3328, F 10752 takes 32.7 us on 512 x 224 tiles and 30.7 on 256 x 96, T 256, D 3456, F 12416 32.7 and 30.8. What the rule is
-// for: y3 at T 1024, D 4096, F 16384 70.5 us on 512-row tiles and 78.2 without, dX 67.9 and 74.1.
 // 512 x 224 tiles, or 256-row tiles of `bn` columns (bn = 256: one accumulator, its epilogue exposed)? Estimated clocks
 // of the busiest CTA pair: rounds of tiles x (k-stages x clocks per stage + the epilogue that nothing hides). A stage's
 // clocks measured with clock stamps on all SMs: 735 (256 wide), 680 (224 wide), 1190 (512 x 224). A narrow tile of the
 // last column takes nearly as long as a full one (three stages do not cover the load latency when there is so little
 // to multiply: 64 columns 95 us against 97 at K = 16384), which is why 8192 x 4096 stays on 256-row tiles (434 us
 // against 482 at K = 16384) while 16384 x 8192 does not.
+// The comparison is with 256-row tiles of full width, not with the narrower ones that best_width would take: where those
+// end sooner by the estimate (4 % of drawn sizes, few tokens or few rows of tiles), less is lost than it says: dy1 at T 256,
+// D 3328, F 10752 takes 32.7 us on 512 x 224 tiles and 30.7 on 256 x 96, T 256, D 3456, F 12416 32.7 and 30.8. What the rule is
+// for: y3 at T 1024, D 4096, F 16384 70.5 us on 512-row tiles and 78.2 without, dX 67.9 and 74.1.
 bool use_tall(int64_t M, int64_t N, int64_t stages, int bn, double flat_epi, double tall_epi) {
   if (M < 512) return false;
   const int64_t P = sm_count() / 2;
