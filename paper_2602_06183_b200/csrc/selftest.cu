@@ -2,9 +2,9 @@
 // A warp waits with ptx::mbar_wait_warp (the routine of every role that runs warp-collective code) on an mbarrier
 // that completes only after the wait has run out: lane 0 has the caller's budget and the other lanes that of the product
 // kernels beyond it, and a second warp completes the barrier as soon as lane 0 has given up (it waits for that in turn with
-// a limit). Lane by lane the outcomes then differ, expired in lane 0 and complete in the others; the warp has to leave
-// as one. If every lane was told that the wait failed, the kernel raises the status word exactly as the product kernels
-// do in their teardown, and returns.
+// a limit). Lane by lane the outcomes would then differ, expired in lane 0 and complete in the others; the warp has to
+// leave as one. If every lane was told that the wait failed, the kernel raises the status word exactly as the product
+// kernels do in their teardown, and returns.
 #include "sf_common.cuh"
 #include "tc_ptx.cuh"
 
