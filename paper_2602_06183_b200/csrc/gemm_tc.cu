@@ -1770,16 +1770,19 @@ int tall_maps(const void* vals, const void* meta_hw, const void* B, bool b_kmajo
 // Tile width of a product on 256-row tiles: max_bn, or a narrower one where that ends sooner by the estimate: rounds of
 // tiles over the CTA pairs x (k-stages x clocks per stage + epilogue). A stage's clocks are its shared-memory traffic
 // (2:4: 0.93 x (272 + 2 w), measured 735 at w = 256 and 680 at 224; dense: 256 + w) or the tensor pipe's 2 w. chunk: epilogue
-// clocks per 32 columns; exposed: nothing hides the epilogue of a tile (one accumulator), else only the last one counts.
+// clocks per 32 columns and `tile` per tile; exposed: nothing hides the epilogue of a tile (one accumulator), else only the
+// last one counts. `tile`: hand-overs between the warps and the latency of the first TMEM load. It is what a short reduction
+// is made of: transposed 2:4 product with K = 128, 28672 x 2048 48.8 us on 224 columns and 78.9 on the 32 that the estimate
+// took without it, 4096 x 4096 17.8 and 26.0, K = 256 18.7 and 21.6 (64 columns); row-major 2048 x 5632, K = 512 19.9 and 21.1.
 // A narrower width has to gain 10 %: its kernel takes the width at run time (at 6 % the weight gradients of D 2048 took 224
 // columns, 0.94 by the estimate, and 1.02 of the time).
 int best_width(int64_t M, int64_t N, int64_t stages, bool sparse, int max_bn, int step, double chunk, bool exposed,
-               int64_t M2 = 0, int64_t N2 = 0) {
+               double tile = 0.0, int64_t M2 = 0, int64_t N2 = 0) {
   const int64_t P = sm_count() / 2, nm = (M + 255) / 256, nm2 = (M2 + 255) / 256;
   auto cost = [&](int w) {
     const int64_t tiles = nm * ((N + w - 1) / w) + nm2 * ((N2 + w - 1) / w);
     const double smem = sparse ? 0.93 * (272 + 2 * w) : 256.0 + w, main = stages * (smem > 2.0 * w ? smem : 2.0 * w);
-    const double rounds = (double)((tiles + P - 1) / P), epi = chunk * (w / 32);
+    const double rounds = (double)((tiles + P - 1) / P), epi = chunk * (w / 32) + tile;
     return exposed ? rounds * (main + epi) : rounds * (main > epi ? main : epi) + epi;
   };
   int best = max_bn;
@@ -1888,7 +1891,7 @@ bool gemm_dual_tn_pays(int64_t M1, int64_t N1, int64_t M2, int64_t N2) {
 }
 
 TileShape gemm_dual_tn_tile(int64_t M1, int64_t N1, int64_t M2, int64_t N2, int64_t K) {
-  return TileShape{256, best_width(M1, N1, K / 64, false, BN, 32, 200.0, false, M2, N2)};
+  return TileShape{256, best_width(M1, N1, K / 64, false, BN, 32, 200.0, false, 0.0, M2, N2)};
 }
 
 int gemm_dual_tn(const void* A1, const void* B1, int64_t M1, int64_t N1, void* C1, const void* A2, const void* B2, int64_t M2,
@@ -1916,7 +1919,7 @@ TileShape gemm_sparse24_tile(int64_t M, int64_t N, int64_t K, int epi) {
   const bool plain = (epi == EPI_STORE);
   const int max_bn = plain ? BN : kNarrowBN;
   if (use_tall(M, N, K / 128, max_bn, plain ? 2500.0 : 0.0, 2500.0)) return TileShape{512, kTallBN};
-  return TileShape{256, best_width(M, N, K / 128, true, max_bn, 32, 400.0, plain)};
+  return TileShape{256, best_width(M, N, K / 128, true, max_bn, 32, 400.0, plain, 700.0)};
 }
 
 int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, bool b_kmajor, int64_t M, int64_t N,
@@ -2084,7 +2087,7 @@ int gemm_fp8(bool sparse, const void* A, const uint8_t* meta_hw, const void* B, 
   int st = sparse ? make_tmap(&ta, A, M, K2 / 2, K2 / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2)
                   : make_tmap(&ta, A, M, K2, K2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2);
   if (st != SF_OK) return st;
-  const int bn = best_width(M, N, K2 / (sparse ? 128 : 64), sparse, BN, 32, sparse ? 400.0 : 200.0, sparse);
+  const int bn = best_width(M, N, K2 / (sparse ? 128 : 64), sparse, BN, 32, sparse ? 400.0 : 200.0, sparse, sparse ? 700.0 : 0.0);
   st = make_tmap(&tb, B, N, K2, K2, 64, bn / 2, CU_TENSOR_MAP_SWIZZLE_128B, 2);
   if (st != SF_OK) return st;
   tm = ta;

@@ -76,6 +76,15 @@ def test_plan_of_a_step_on_the_host():
     assert binding.lib().sf_ffn_step_plan(None, None) == binding.SF_ERR_NULL
 
 
+@pytest.mark.parametrize("T,F", [(2048, 28672), (4096, 4096), (8192, 2048)])
+@pytest.mark.parametrize("D", [256, 512])
+def test_short_reductions_with_many_tiles_keep_wide_tiles(T, F, D):
+    """A tile costs its hand-overs however narrow it is: a product with two to four k-stages and enough tiles for every CTA
+    pair must not be cut into 32- or 64-column ones (measured 1.2 to 1.6 times the time)."""
+    plan = binding.sf_ffn_step_plan(binding.make_desc(T, D, F, 64, 8, flags=binding.SF_FFN_UNFUSED_ACT))
+    assert plan.y1_rows == 512 or plan.y1_cols >= 128
+
+
 def _integers(shape, limit, seed):
     return np.random.default_rng(seed).integers(-limit, limit + 1, size=shape).astype(np.float32)
 
