@@ -260,6 +260,17 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
   // two register buffers: the TMEM load of the next 32 columns is in flight while this chunk is converted
   uint32_t va[32], vb[32];
   tmem_ld_32x32b_x32(taddr + at(ch0) * 32, va);
+  if constexpr (kEpi == EPI_STORE_T) {
+    // Unrolled: with a short reduction this epilogue is the tile's time, and the staging of a chunk overlaps the stores of the
+    // one before. 8192 x 16384, K = 128 100.8 us rolled, 96.7 unrolled; 4096 x 16384, K = 256 56.9 and 54.5.
+#pragma unroll
+    for (int i = 0; i < kTileN / 32; i += 2) {
+      if (i >= nch) break;
+      chunk(i, va, vb);
+      if (i + 1 < kTileN / 32 && i + 1 < nch) chunk(i + 1, vb, va);
+    }
+    return;
+  }
 #pragma unroll 1
   for (int i = ch0; i < nch; i += 2) {
     chunk(i, va, vb);
