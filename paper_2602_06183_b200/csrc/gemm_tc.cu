@@ -92,7 +92,10 @@ __host__ __device__ constexpr bool is_drelu_t(int epi) { return epi == EPI_DRELU
 __host__ __device__ constexpr bool two_sets(int epi) { return epi == EPI_VNM8 || epi == EPI_ACT24_T || is_drelu_t(epi); }
 // Dense products: two sets share every tile, each takes half of its columns (the last tile's epilogue is exposed:
 // 1024 x 256 x 1024 17.3 -> 14.3 us; the 2:4 products gained nothing from it).
-__host__ __device__ constexpr bool split_sets(int mode, int epi, int expand) { return mode == MODE_DENSE && epi != EPI_ROUTE && !expand; }
+// (one: a single set, see one_epilogue_set)
+__host__ __device__ constexpr bool split_sets(int mode, int epi, int expand, bool one) {
+  return mode == MODE_DENSE && epi != EPI_ROUTE && !expand && !one;
+}
 
 // This warp has read its part of an accumulator for the last time: hand it back to the MMA warp.
 __device__ __forceinline__ void release_accumulator(int lane, uint64_t* tmem_empty_bar) {
@@ -1004,8 +1007,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant_
 constexpr int kThreads2 = 192;
 constexpr int kThreads2Expand = 448;                     // + eight warps that expand a packed operand into its stage
 constexpr int kThreads2Sets = 320;                       // + a second set of four epilogue warps
-__host__ __device__ constexpr int threads2(int mode, int epi, int expand) {
-  return expand ? kThreads2Expand : (two_sets(epi) || split_sets(mode, epi, expand) ? kThreads2Sets : kThreads2);
+__host__ __device__ constexpr int threads2(int mode, int epi, int expand, bool one) {
+  return expand ? kThreads2Expand : (two_sets(epi) || split_sets(mode, epi, expand, one) ? kThreads2Sets : kThreads2);
 }
 constexpr int kPkStageBytes = 8192 + 1024;               // packed values [64 tokens][64] + metadata bytes [64][16]
 // 8-bit operands (fp8 = true) keep the byte geometry of a stage (128-byte rows now hold 128 elements, so a
@@ -1072,10 +1075,11 @@ __device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) {
 // more SMs to work and shorten what one of them does: the eight kernels of a step at T 1024, D 256, F 1024 take 50 us
 // instead of 61 (graph replay). A kernel of its own, because the run-time width costs the issuing threads instructions
 // that the large products do not have (dense, 256 wide: 1.5 % and more).
+// kOneSet: dense products that store their tiles with one set of epilogue warps instead of two.
 // kDual: two independent products with the same reduction length in one launch (the weight gradients). The second one's
 // operands are tmapMeta (A) and tmapPk (B), its output args.C2.
-template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false, bool kDual = false>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kMode, kEpi, kExpand), 1)
+template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false, bool kDual = false, bool kOneSet = false>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kMode, kEpi, kExpand, kOneSet), 1)
 gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB,
                 const __grid_constant__ CUtensorMap tmapMeta, const __grid_constant__ CUtensorMap tmapPk,
                 const GemmArgs args) {
@@ -1134,7 +1138,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     for (int b = 0; b < 2; ++b) {
       mbar_init(&ctl->tmem_full[b], 1);
       // the epilogue warps of both CTAs that read the accumulator
-      mbar_init(&ctl->tmem_empty[b], split_sets(kMode, kEpi, kExpand) || (two_sets(kEpi) && kAccBufs == 1) ? 16 : 8);
+      mbar_init(&ctl->tmem_empty[b], split_sets(kMode, kEpi, kExpand, kOneSet) || (two_sets(kEpi) && kAccBufs == 1) ? 16 : 8);
     }
     ctl->abort_flag = 0;
     fence_mbar_init();
@@ -1367,7 +1371,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   } else {
     // =========================== epilogue (warps 2..5 or 2..9, both CTAs) ===========================
     const int q = warp & 3, set = (warp - 2) >> 2;
-    constexpr int kParts = split_sets(kMode, kEpi, kExpand) ? 2 : 1;
+    constexpr int kParts = split_sets(kMode, kEpi, kExpand, kOneSet) ? 2 : 1;
     uint8_t* my_stage = epi_stage + (set * 4 + q) * kEpiWarpBytes;
     uint32_t acc = 0, acc_phase = 0;
     bool ok = true;
@@ -1712,10 +1716,11 @@ int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const GemmArgs& a, 
                     ta, tb, a);
 }
 
-template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false, bool kDual = false>
+template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false, bool kDual = false,
+          bool kOneSet = false>
 int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tm, GemmArgs a, cudaStream_t s,
                const CUtensorMap* tpk = nullptr) {
-  auto kern = gemm_tc2_kernel<kMode, kAMN, kBMN, kEpi, kBN, kExpand, kFp8, kVar, kDual>;
+  auto kern = gemm_tc2_kernel<kMode, kAMN, kBMN, kEpi, kBN, kExpand, kFp8, kVar, kDual, kOneSet>;
   constexpr int smem = smem_bytes2(kMode != MODE_DENSE, kBN, kEpi, kExpand != 0, kFp8);
   static_assert(smem <= 232448 && smem >= kExclusiveSmem, "shared memory per CTA: fits, and one CTA per SM");
   static bool attr_done[64] = {false};
@@ -1733,8 +1738,28 @@ int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
                                  : a.num_m_tiles * a.num_n_tiles + (kDual ? a.num_m_tiles2 * a.num_n_tiles2 : 0);
   const int max_pairs = sm_count() / 2;
   const int pairs = tiles < max_pairs ? tiles : max_pairs;
-  return launch_pdl(kern, dim3(2 * pairs), threads2(kMode, kEpi, kExpand), smem, s, ta, tb, tm, tpk ? *tpk : ta, a);
+  return launch_pdl(kern, dim3(2 * pairs), threads2(kMode, kEpi, kExpand, kOneSet), smem, s, ta, tb, tm, tpk ? *tpk : ta, a);
 }
+
+int64_t l2_bytes() {
+  static int n[64] = {0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 126 << 20;
+  if (n[dev] == 0) {
+    int v = 0;
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, dev) != cudaSuccess || v <= 0) v = 126 << 20;
+    n[dev] = v;
+  }
+  return n[dev];
+}
+
+// Dense products: does one set of epilogue warps store a tile sooner than two that share it? Two halve an epilogue, and where
+// the output stays in the L2 they are the faster ones (12288 x 4096, K = 128 37.5 us, one set 39.9). Where it does not and the
+// reduction is short, the kernel lasts as long as its writes, and those of twice as many warps go slower: 8192 x 16384, K = 128
+// 132.9 us with two and 113.6 with one, K = 512 170.8 and 159.9, K = 1024 237.9 and 234.5, K = 2048 419 and 426; E4M3, K = 512
+// 146.3 and 125.6, K = 1024 176 and 165. (stages: 64 of K, E4M3 128; the dense step's two-operand epilogues keep two sets: y1 at
+// T 8192, D 256, F 16384 121 us with two and 135 with one, dy1 158 and 195)
+bool one_epilogue_set(int64_t out_elements, int64_t stages) { return stages <= 8 && 2 * out_elements > l2_bytes(); }
 
 // Tile width of the two-accumulator 2:4 variant (transposed-output products): 2 x 224 accumulator
 // columns + 8 metadata columns fit the 512 TMEM columns.
@@ -1873,18 +1898,23 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
   return !two       ? launch_one<MODE_DENSE, AMN, BMN, EPI>(ta, tb, a, s)                             \
          : bn == BN ? launch_two<MODE_DENSE, AMN, BMN, EPI>(ta, tb, ta, a, s)                         \
                     : launch_two<MODE_DENSE, AMN, BMN, EPI, BN, 0, false, true>(ta, tb, ta, a, s)
+#define SF_DENSE_STORE(AMN, BMN)                                                                                              \
+  if (two && bn == BN && one_epilogue_set(M * N, K / 64))                                                                     \
+    return launch_two<MODE_DENSE, AMN, BMN, EPI_STORE, BN, 0, false, false, false, true>(ta, tb, ta, a, s);                   \
+  SF_DENSE_CASE(AMN, BMN, EPI_STORE)
   const bool amn = !a_kmajor, bmn = !b_kmajor;
   if (epi == EPI_STORE) {
-    if (!amn && !bmn) SF_DENSE_CASE(false, false, EPI_STORE);
-    if (!amn && bmn) SF_DENSE_CASE(false, true, EPI_STORE);
-    if (amn && !bmn) SF_DENSE_CASE(true, false, EPI_STORE);
-    SF_DENSE_CASE(true, true, EPI_STORE);
+    if (!amn && !bmn) { SF_DENSE_STORE(false, false); }
+    if (!amn && bmn) { SF_DENSE_STORE(false, true); }
+    if (amn && !bmn) { SF_DENSE_STORE(true, false); }
+    SF_DENSE_STORE(true, true);
   } else if (epi == EPI_SQRELU) {
     if (!amn && !bmn) SF_DENSE_CASE(false, false, EPI_SQRELU);
   } else if (epi == EPI_DRELU) {
     if (!amn && bmn) SF_DENSE_CASE(false, true, EPI_DRELU);
     if (!amn && !bmn) SF_DENSE_CASE(false, false, EPI_DRELU);
   }
+#undef SF_DENSE_STORE
 #undef SF_DENSE_CASE
   return SF_ERR_UNSUPPORTED;
 }
@@ -1921,6 +1951,8 @@ int gemm_dual_tn(const void* A1, const void* B1, int64_t M1, int64_t N1, void* C
   a.num_m_tiles2 = (int)((M2 + 255) / 256);
   a.num_n_tiles2 = (int)((N2 + a.bn - 1) / a.bn);
   a.status = status;
+  if (a.bn == BN && one_epilogue_set(M1 * N1 + M2 * N2, K / 64))
+    return launch_two<MODE_DENSE, true, true, EPI_STORE, BN, 0, false, false, true, true>(ta, tb, ta2, a, s, &tb2);
   return a.bn == BN ? launch_two<MODE_DENSE, true, true, EPI_STORE, BN, 0, false, false, true>(ta, tb, ta2, a, s, &tb2)
                     : launch_two<MODE_DENSE, true, true, EPI_STORE, BN, 0, false, true, true>(ta, tb, ta2, a, s, &tb2);
 }
@@ -2113,6 +2145,8 @@ int gemm_fp8(bool sparse, const void* A, const uint8_t* meta_hw, const void* B, 
   a.C = C; a.ldc = ldc; a.meta_hw = meta_hw; a.status = status; a.out_scale = alpha;
   a.num_k_blocks = (int)(K2 / 64);
   a.bn = bn;
+  if (!sparse && bn == BN && one_epilogue_set(M * N, K2 / 64))
+    return launch_two<MODE_DENSE, false, false, EPI_STORE, BN, 0, true, false, false, true>(ta, tb, tm, a, s);
   if (bn != BN)
     return sparse ? launch_two<MODE_SPARSE24, false, false, EPI_STORE, BN, 0, true, true>(ta, tb, tm, a, s)
                   : launch_two<MODE_DENSE, false, false, EPI_STORE, BN, 0, true, true>(ta, tb, tm, a, s);

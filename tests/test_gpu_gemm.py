@@ -70,6 +70,24 @@ def test_sparse24_gemm_row_major_output(b_k, Mr, Nc, K):
     assert_close_elementwise(f32(C), _f64(p.dense) @ Bf.T, K, "2:4 product, row-major output")
 
 
+@pytest.mark.parametrize("a_k,b_k", [(True, True), (False, False)])
+@pytest.mark.parametrize("M,N,K", [(8320, 8192, 64),      # beyond the L2, one k-stage: one set of epilogue warps; half-empty last row
+                                   (4096, 16640, 512),    # the longest reduction of that kind
+                                   (8320, 8192, 576)])    # beyond the L2, two sets
+def test_dense_gemm_output_beyond_the_l2(a_k, b_k, M, N, K):
+    # small integers: every partial sum is exact in float32, only the bf16 rounding of the result is left
+    g = torch.Generator(device="cuda")
+    g.manual_seed(K)
+    ints = lambda *s: torch.randint(-3, 4, s, generator=g, device="cuda")
+    A, B = ints(M, K), ints(N, K)
+    dev = lambda t, kmajor: (t if kmajor else t.T).to(torch.bfloat16).contiguous()
+    out = Guarded((M, N), torch.bfloat16)
+    C, ws = binding.sf_gemm_dense(dev(A, a_k), a_k, dev(B, b_k), b_k, C_out=out.t)
+    assert binding.sf_check_status(ws) == binding.SF_OK
+    out.check("dense product")
+    assert torch.equal(C, (A.double() @ B.double().T).to(torch.bfloat16))
+
+
 def _integer_24_product(Mr, Nc, K, b_k, run):
     """Small integers: every partial sum is exact in float32, so only the bf16 rounding of the result is left."""
     rng = np.random.default_rng(Mr + Nc)
