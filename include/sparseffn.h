@@ -253,6 +253,7 @@ typedef struct sf_ffn_plan {
   int32_t dy1_rows, dy1_cols;    /* features x tokens */
   int32_t weight_grad_launches;  /* 1: dW2 and dW1 share a launch (never in sf_ffn_step_host), 2: one each */
   int32_t weight_grad_cols;      /* tile columns of the shared launch (256 rows); 0 without one */
+  int32_t y3_rows, y3_cols;      /* tokens x model width, also of dX; 0 where M >= 16 (the gathered V:N:M product) */
 } sf_ffn_plan;
 SF_API int sf_ffn_step_plan(const sf_ffn_desc* desc, sf_ffn_plan* plan);
 

@@ -33,7 +33,7 @@ class sf_ffn_desc(C.Structure):
 
 class sf_ffn_plan(C.Structure):
     _fields_ = [(n, C.c_int32) for n in ("cta_pairs", "y1_selects", "y1_rows", "y1_cols", "dy1_rows", "dy1_cols",
-                                         "weight_grad_launches", "weight_grad_cols")]
+                                         "weight_grad_launches", "weight_grad_cols", "y3_rows", "y3_cols")]
 
 
 class sf_router_desc(C.Structure):

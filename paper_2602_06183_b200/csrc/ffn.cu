@@ -326,10 +326,11 @@ int sf_ffn_step_plan(const sf_ffn_desc* desc, sf_ffn_plan* plan) {
                        : d.M == 4 ? gemm_sparse24_act4_tile(d.F, d.T, d.D)
                                   : gemm_sparse24_tile(d.F, d.T, d.D, EPI_STORE_T);
   const TileShape dy1 = gemm_sparse24_drelu_tile(d.F, d.T, d.D);
+  const TileShape y3 = L.plain24 ? gemm_sparse24_tile(d.T, d.D, d.F, EPI_STORE) : TileShape{0, 0};
   const WeightGradShapes g(d);
   const bool shared = !L.expand && gemm_dual_tn_pays(g.m2, g.n2, d.F, d.D);
   *plan = sf_ffn_plan{gemm_cta_pairs(), L.fused || d.M == 4, y1.rows, y1.cols, dy1.rows, dy1.cols, shared ? 1 : 2,
-                      shared ? gemm_dual_tn_tile(g.m2, g.n2, d.F, d.D, d.T).cols : 0};
+                      shared ? gemm_dual_tn_tile(g.m2, g.n2, d.F, d.D, d.T).cols : 0, y3.rows, y3.cols};
   return SF_OK;
 }
 

@@ -1859,6 +1859,18 @@ bool use_tall(int64_t M, int64_t N, int64_t stages, int bn, double flat_epi, dou
   return q * full + rest < 0.99 * flat;
 }
 
+// The same for the products that store row-major (y3, dX; E4M3). With a short reduction and an output beyond the L2 the kernel
+// lasts as long as its writes, which the clocks above do not hold, and the two sets of epilogue warps of a 512-row tile write
+// slower than the one of a 256-row tile: 8192 x 16384 K = 128 130 us on 512-row tiles and 117 on 256-row ones, K = 256 134 and
+// 123, K = 512 152 and 137; E4M3 K = 256 131 and 118, K = 512 138 and 123, K = 1024 168 and 147.
+// The line could lie higher: in bursts 256-row tiles also win at 8 to 16 stages (8192 x 16384, K = 1024 207 and 189 us, E4M3 K = 2048
+// 237 and 219), but not under the power cap: 4096 x 16384 x 4096 in E4M3, 16 stages, 175 and 167 us in a burst, and 213 and
+// 220 us for prune, quantise and product call after call.
+bool use_tall_plain(int64_t M, int64_t N, int64_t stages) {
+  const bool write_bound = stages < 7 && 2 * M * N > l2_bytes();
+  return !write_bound && use_tall(M, N, stages, BN, 2500.0, 2500.0);
+}
+
 // CTA pairs work on 256-row tiles; with M % 256 == 128 the second CTA of the last row of pairs runs on
 // zero-filled operand rows and stores nothing. A single 128-row block runs the one-CTA kernels.
 bool use_two_cta(int64_t M) { return M >= 256; }
@@ -1961,7 +1973,7 @@ int gemm_dual_tn(const void* A1, const void* B1, int64_t M1, int64_t N1, void* C
 TileShape gemm_sparse24_tile(int64_t M, int64_t N, int64_t K, int epi) {
   const bool plain = (epi == EPI_STORE);
   const int max_bn = plain ? BN : kNarrowBN;
-  if (use_tall(M, N, K / 128, max_bn, plain ? 2500.0 : 0.0, 2500.0)) return TileShape{512, kTallBN};
+  if (plain ? use_tall_plain(M, N, K / 128) : use_tall(M, N, K / 128, max_bn, 0.0, 2500.0)) return TileShape{512, kTallBN};
   return TileShape{256, best_width(M, N, K / 128, true, max_bn, 32, 400.0, plain, 700.0)};
 }
 
@@ -2118,7 +2130,7 @@ int gemm_fp8(bool sparse, const void* A, const uint8_t* meta_hw, const void* B, 
   // the operands in 2-byte units: [M, K/2] (dense) or [M, K/4] (2:4 values), [N, K/2]
   const int64_t K2 = K / 2;
   CUtensorMap ta, tb, tm;
-  if (sparse && use_tall(M, N, K / 256, BN, 2500.0, 2500.0)) {
+  if (sparse && use_tall_plain(M, N, K / 256)) {
     CUtensorMap tbn;
     const int st = tall_maps(A, meta_hw, B, true, M, N, K2, 2, 4, &ta, &tb, &tbn, &tm);
     if (st != SF_OK) return st;

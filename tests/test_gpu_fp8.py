@@ -131,6 +131,23 @@ def test_sparse24_fp8_gemm_against_oracle_packing(M, N, K):
     assert_close_elementwise(f32(C), ref, K, "fp8 2:4 product")
 
 
+@pytest.mark.parametrize("M,N,K", [(4352, 16640, 1024),    # output beyond the L2, four k-stages: 256-row tiles
+                                   (7680, 6400, 2048)])    # 512-row tiles, the last of 15 rows and a last column of 128
+def test_sparse24_fp8_gemm_of_many_tiles(M, N, K):
+    # small integers: E4M3 holds them, every partial sum is exact in float32, only the bf16 rounding of the result is left
+    rng = np.random.default_rng(M)
+    W = rng.integers(-3, 4, size=(M, K)).astype(np.float32)
+    B = rng.integers(-3, 4, size=(N, K)).astype(np.float32)
+    p = fp8.prune24_fp8(synth.f32_to_bf16_bits(W), 1.0)
+    Bq = binding.sf_fp8_quantize(to_dev(synth.f32_to_bf16_bits(B)), 1.0)
+    out = Guarded((M, N), torch.bfloat16)
+    C, ws = binding.sf_gemm_fp8_sparse24(_dev8(p.vals), torch.from_numpy(p.meta.view(np.int16)).cuda(), Bq, 1.0, C_out=out.t)
+    assert binding.sf_check_status(ws) == binding.SF_OK
+    out.check("fp8 2:4 product")
+    ref = fp8.e4m3_to_f32(p.dense).reshape(M, K) @ B.T
+    assert np.array_equal(bits(C), synth.f32_to_bf16_bits(ref))
+
+
 def test_sparse24_fp8_metadata_probe_one_hot():
     """One stored value per row at a time, B = identity: the output row shows where the tensor core put it.
     Every (row mod 128, 16-column word) position class of the metadata order is visited."""

@@ -110,6 +110,16 @@ def test_sparse24_gemm_tile_shapes(b_k, Mr, Nc, K):
     assert np.array_equal(got, ref)
 
 
+@pytest.mark.parametrize("b_k", [True, False])
+@pytest.mark.parametrize("Mr,Nc,K,rows", [(4352, 16640, 768, 256),   # beyond the L2, the longest reduction of that rule
+                                          (8192, 8192, 256, 256),    # the smallest square beyond it
+                                          (7680, 6400, 512, 512)])   # within it: a narrow last column of 128
+def test_sparse24_gemm_short_reductions_about_the_l2(b_k, Mr, Nc, K, rows):
+    assert binding.sf_ffn_step_plan(binding.make_desc(Mr, Nc, K, 64, 4)).y3_rows == rows     # y3 is this product
+    got, ref = _integer_24_product(Mr, Nc, K, b_k, lambda v, m, b: binding.sf_gemm_sparse24_rm(v, m, b, b_k))
+    assert np.array_equal(got, ref)
+
+
 @pytest.mark.parametrize("Mr,Nc,K", [(37632, 256, 128),    # more narrow tiles than two per idle pair: round robin
                                      (256, 7680, 128), (8576, 4864, 512)])
 def test_sparse24_gemm_tile_shapes_transposed_output(Mr, Nc, K):

@@ -85,6 +85,17 @@ def test_short_reductions_with_many_tiles_keep_wide_tiles(T, F, D):
     assert plan.y1_rows == 512 or plan.y1_cols >= 128
 
 
+@pytest.mark.parametrize("T,D", [(8192, 16384), (16384, 8192), (4096, 16640)])
+@pytest.mark.parametrize("F", [256, 512, 768])
+def test_short_reductions_beyond_the_l2_stay_on_256_row_tiles(T, D, F):
+    """y3 and dX with up to six k-stages and an output larger than the L2 last as long as their writes, and 512-row tiles write
+    slower (measured 1.08 to 1.1 times the time); longer reductions go to 512-row tiles, smaller outputs by the clocks."""
+    y3_rows = lambda *a: binding.sf_ffn_step_plan(binding.make_desc(*a, 64, 8)).y3_rows
+    assert y3_rows(T, D, F) == 256
+    assert y3_rows(T, D, 16 * F) == 512
+    assert y3_rows(8192, 7296, F) == 512
+
+
 def _integers(shape, limit, seed):
     return np.random.default_rng(seed).integers(-limit, limit + 1, size=shape).astype(np.float32)
 
