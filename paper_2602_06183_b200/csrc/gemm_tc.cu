@@ -45,7 +45,7 @@ __host__ __device__ constexpr int stage_bytes(bool sparse) {
   return a_stage_bytes(sparse) + kBStageBytes + (sparse ? kMetaStageBytes : 0);
 }
 __host__ __device__ constexpr int num_stages(bool sparse) { return sparse ? 5 : 4; }
-constexpr int kEpiWarpBytes = 16 * 32 * 4;                                            // 16 token pairs x 32 features
+constexpr int kEpiWarpBytes = 32 * 32 * 2;                                            // 32 x 32 bf16, or 16 token pairs x 32
 constexpr int kEpiStageBytes = 4 * kEpiWarpBytes;                                     // 4 warps
 __host__ __device__ constexpr int smem_bytes(bool sparse) {
   return 1024 /*align slack*/ + num_stages(sparse) * stage_bytes(sparse) + kEpiStageBytes + 256 /*barriers*/;
@@ -243,21 +243,18 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
         store_rows(w, args.C2, args.ldc2, col0);
       }
     } else {
-      // Transposed output: D row = feature (lane), D column = token. C is [N, M] row-major. Two tokens travel
-      // as one word: half the staging stores of a 16-bit transpose.
-      uint32_t* st = reinterpret_cast<uint32_t*>(my_stage);
+      // Transposed output: D row = feature (lane), D column = token. C is [N, M] row-major. Token by token, so that a store
+      // instruction writes 64 bytes of eight CONSECUTIVE tokens. As words of two neighbouring tokens (half the staging
+      // stores; an instruction then writes every second one of 16 tokens) 8192 x 16384 takes 96.5 us at K = 128 and 130.0 at
+      // K = 512 instead of 71.5 and 113.5, 28672 x 2048, K = 128 47.0 instead of 37.5, 4096 x 4096, K = 1024 23.9 instead of 23.7.
       __syncwarp();
 #pragma unroll
-      for (int j = 0; j < 16; ++j) st[j * 32 + lane] = w[j];
+      for (int t = 0; t < 32; ++t)
+        reinterpret_cast<uint16_t*>(unit(t, lane >> 3))[lane & 7] = (uint16_t)(w[t >> 1] >> (16 * (t & 1)));
       __syncwarp();
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        uint32_t r0[4], r1[4];
-        pair_rows(st + (i * 8 + t8) * 32 + u * 8, lane, r0, r1);
-        uint16_t* c = reinterpret_cast<uint16_t*>(args.C) + (col0 + i * 16 + t8 * 2) * args.ldc + m0 + q * 32 + u * 8;
-        *reinterpret_cast<uint4*>(c) = make_uint4(r0[0], r0[1], r0[2], r0[3]);
-        *reinterpret_cast<uint4*>(c + args.ldc) = make_uint4(r1[0], r1[1], r1[2], r1[3]);
-      }
+      for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(args.C) + (col0 + i * 8 + t8) * args.ldc + m0 + q * 32 + u * 8) = *unit(t8 + 8 * i, u);
     }
   };
   // two register buffers: the TMEM load of the next 32 columns is in flight while this chunk is converted
@@ -265,7 +262,7 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
   tmem_ld_32x32b_x32(taddr + at(ch0) * 32, va);
   if constexpr (kEpi == EPI_STORE_T) {
     // Unrolled: with a short reduction this epilogue is the tile's time, and the staging of a chunk overlaps the stores of the
-    // one before. 8192 x 16384, K = 128 100.8 us rolled, 96.7 unrolled; 4096 x 16384, K = 256 56.9 and 54.5.
+    // one before. 8192 x 16384, K = 128 73.5 us rolled, 71.5 unrolled; 4096 x 16384, K = 256 45.3 and 44.3.
 #pragma unroll
     for (int i = 0; i < kTileN / 32; i += 2) {
       if (i >= nch) break;
@@ -1808,8 +1805,8 @@ int tall_maps(const void* vals, const void* meta_hw, const void* B, bool b_kmajo
 // (2:4: 0.93 x (272 + 2 w), measured 735 at w = 256 and 680 at 224; dense: 256 + w) or the tensor pipe's 2 w. chunk: epilogue
 // clocks per 32 columns and `tile` per tile; exposed: nothing hides the epilogue of a tile (one accumulator), else only the
 // last one counts. `tile`: hand-overs between the warps and the latency of the first TMEM load. It is what a short reduction
-// is made of: transposed 2:4 product with K = 128, 28672 x 2048 48.8 us on 224 columns and 78.9 on the 32 that the estimate
-// took without it, 4096 x 4096 17.8 and 26.0, K = 256 18.7 and 21.6 (64 columns); row-major 2048 x 5632, K = 512 19.9 and 21.1.
+// is made of: transposed 2:4 product with K = 128, 28672 x 2048 37.6 us on 224 columns and 64.5 on the 32 that the estimate
+// took without it, 4096 x 4096 14.7 and 22.1, K = 256 15.9 and 19.1 (64 columns); row-major 2048 x 5632, K = 512 19.9 and 21.1.
 // A narrower width has to gain 10 %: its kernel takes the width at run time (at 6 % the weight gradients of D 2048 took 224
 // columns, 0.94 by the estimate, and 1.02 of the time).
 int best_width(int64_t M, int64_t N, int64_t stages, bool sparse, int max_bn, int step, double chunk, bool exposed,
