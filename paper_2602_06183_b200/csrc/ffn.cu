@@ -67,10 +67,12 @@ int host_step_resources(HostStepResources** out) {
 
 // ---- small helper kernels -------------------------------------------------------------------
 
+// kEarly: the product that follows may set itself up while this kernel runs (see launch_meta_reorder).
+template <bool kEarly>
 __global__ void meta_reorder_kernel(const uint16_t* __restrict__ meta, uint8_t* __restrict__ meta_hw, int64_t R,
                                     int64_t K) {
   pdl_wait();
-  pdl_trigger();
+  if (kEarly) pdl_trigger();
   const int64_t words = K >> 4;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= R * words) return;
@@ -221,11 +223,19 @@ void trace_mark(cudaStream_t s) {
   if (g_trace_events && g_trace_n < g_trace_cap) cudaEventRecord(g_trace_events[g_trace_n++], s);
 }
 
-int launch_meta_reorder(const void* meta, void* meta_hw, int64_t R, int64_t K, cudaStream_t s) {
+// A product that is set up early takes the SMs in the order in which this kernel's last blocks leave them. The transposing one,
+// bound by its stores, then runs slower throughout, which a long one feels more than the half microsecond that the overlap
+// saves: 16384 x 8192, K = 512 119.0 us with an early start and 99.7 without, K = 1024 183.3 and 165.6, 28672 x 2048, K = 1024
+// 91.1 and 80.8, 8192 x 16384, K = 256 (64 k-stages to a CTA pair) 86.1 and 82.2; but 4096 x 4096, K = 1024 (33) 23.3 and 23.0,
+// K = 256 16.5 and 16.6, 12288 x 4096, K = 128 (12) 32.2 and 33.0, 7168 x 3328, K = 128 17.8 and 18.8. The row-major product does
+// not mind: 4096 x 4096, K = 256 18.2 and 18.6.
+// transposed_cols: columns of the transposing product that follows, 0 for any other.
+int launch_meta_reorder(const void* meta, void* meta_hw, int64_t R, int64_t K, int64_t transposed_cols, cudaStream_t s) {
+  const bool early = R * transposed_cols * K < (int64_t)48 * 74 * 256 * 224 * 128;   // 48 k-stages of a tile to each of 74 pairs
   const int64_t n = R * (K >> 4);
   if (n == 0) return SF_OK;
-  return launch_pdl(meta_reorder_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, s, (const uint16_t*)meta,
-                    (uint8_t*)meta_hw, R, K);
+  return launch_pdl(early ? meta_reorder_kernel<true> : meta_reorder_kernel<false>, dim3((unsigned)((n + 255) / 256)), 256, 0, s,
+                    (const uint16_t*)meta, (uint8_t*)meta_hw, R, K);
 }
 
 }  // namespace sf
@@ -270,7 +280,7 @@ int sf_gemm_sparse24(const void* a_vals, const void* a_meta, const void* B, void
   SF_TRY(check_arch());
   cudaStream_t s = (cudaStream_t)stream;
   uint8_t* hw = at(workspace, kStatusBytes);
-  SF_TRY(launch_meta_reorder(a_meta, hw, Mr, K, s));
+  SF_TRY(launch_meta_reorder(a_meta, hw, Mr, K, Nc, s));
   return gemm_sparse24(a_vals, hw, B, true, Mr, Nc, K, EPI_STORE_T, Ct, Mr, (int*)workspace, s);
 }
 
@@ -284,7 +294,7 @@ int sf_gemm_sparse24_rm(const void* a_vals, const void* a_meta, const void* B, i
   SF_TRY(check_arch());
   cudaStream_t s = (cudaStream_t)stream;
   uint8_t* hw = at(workspace, kStatusBytes);
-  SF_TRY(launch_meta_reorder(a_meta, hw, Mr, K, s));
+  SF_TRY(launch_meta_reorder(a_meta, hw, Mr, K, 0, s));
   return gemm_sparse24(a_vals, hw, B, b_kmajor != 0, Mr, Nc, K, EPI_STORE, C, Nc, (int*)workspace, s);
 }
 
@@ -301,7 +311,7 @@ int sf_gemm_venom(const void* a_vals, const void* a_meta, const void* colidx, co
   SF_TRY(check_arch());
   cudaStream_t s = (cudaStream_t)stream;
   uint8_t* hw = at(workspace, kStatusBytes);
-  SF_TRY(launch_meta_reorder(a_meta, hw, T, 4 * F / M, s));
+  SF_TRY(launch_meta_reorder(a_meta, hw, T, 4 * F / M, 0, s));
   return gemm_venom(a_vals, hw, (const uint8_t*)colidx, Bt, T, F, Nc, V, M, C, Nc, (int*)workspace, s);
 }
 

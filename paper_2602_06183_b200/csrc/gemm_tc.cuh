@@ -168,8 +168,9 @@ int gemm_sparse24_drelu(const void* w_vals, const uint8_t* meta_hw, const void* 
 // padding (rows beyond E are read as zeros by the tensor map).
 int gemm_route(const void* X, const void* means, int64_t T, int64_t D, int E, int* expert, float* logits, int* status,
                cudaStream_t s);
-// canonical [R, K/16] metadata words -> hardware-ordered atoms (R % 128 == 0, K % 128 == 0)
-int launch_meta_reorder(const void* meta, void* meta_hw, int64_t R, int64_t K, cudaStream_t s);
+// canonical [R, K/16] metadata words -> hardware-ordered atoms (R % 128 == 0, K % 128 == 0); transposed_cols: columns of the
+// transposing product that follows, 0 for any other
+int launch_meta_reorder(const void* meta, void* meta_hw, int64_t R, int64_t K, int64_t transposed_cols, cudaStream_t s);
 
 // E4M3 operands, both K-major: C[M, N] = bf16(alpha * A B^T). sparse: A = 2:4 values [M, K/2] (codes) with
 // metadata in the 8-bit instruction's order (see meta_hw8_offset); else A [M, K]. B [N, K].

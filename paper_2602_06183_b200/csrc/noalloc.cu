@@ -65,7 +65,7 @@ extern "C" int sf_gemm_sparse24_noalloc(const void* a_vals, const void* a_meta, 
   // metadata region is rewritten in full for this call's shape before the product reads it.
   SF_CUDA_TRY(cudaMemsetAsync(scratch, 0, kNoAllocStatusBytes, s));
   unsigned char* hw = scratch + kNoAllocStatusBytes;
-  st = launch_meta_reorder(a_meta, hw, Mr, K, s);
+  st = launch_meta_reorder(a_meta, hw, Mr, K, Nc, s);
   if (st != SF_OK) return st;
   return gemm_sparse24(a_vals, hw, B, true, Mr, Nc, K, EPI_STORE_T, Ct, Mr, reinterpret_cast<int*>(scratch), s);
 }

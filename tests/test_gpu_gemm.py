@@ -127,6 +127,26 @@ def test_sparse24_gemm_tile_shapes_transposed_output(Mr, Nc, K):
     assert np.array_equal(got, np.ascontiguousarray(ref.T))
 
 
+@pytest.mark.parametrize("Mr,Nc,K", [(4096, 8192, 512), (8192, 8192, 512)])    # set up while the metadata is converted, and after it
+def test_sparse24_gemm_transposed_output_call_after_call(Mr, Nc, K):
+    """Two operands in turn through one workspace: each product has to read the metadata that its own call converted."""
+    rng = np.random.default_rng(K)
+    B = rng.integers(-3, 4, size=(Nc, K)).astype(np.float32)
+    packed = [oracle.prune24(synth.f32_to_bf16_bits(rng.integers(-3, 4, size=(Mr, K)).astype(np.float32)), group_dim=1, mode=0)
+              for _ in range(2)]
+    dev = [(to_dev(p.vals), torch.from_numpy(p.meta.view(np.int16)).cuda()) for p in packed]
+    x = to_dev(synth.f32_to_bf16_bits(B))
+    ws = torch.zeros(binding.sf_gemm_workspace_size(Mr, K), dtype=torch.uint8, device="cuda")
+    outs = [torch.empty((Nc, Mr), dtype=torch.bfloat16, device="cuda") for _ in range(6)]
+    for i, out in enumerate(outs):
+        binding.sf_gemm_sparse24(*dev[i % 2], x, Ct_out=out, workspace=ws)
+    assert binding.sf_check_status(ws) == binding.SF_OK
+    # integers: exact in float32, one rounding to bf16
+    refs = [synth.f32_to_bf16_bits(B @ oracle.bf16_to_f32(p.dense).T) for p in packed]
+    for i, out in enumerate(outs):
+        assert np.array_equal(bits(out), refs[i % 2])
+
+
 def test_sparse24_gemm_one_hot_metadata_probe():
     """Each kept value is a distinct power of two in an otherwise zero row and B is an identity
     slice, so the output says which K position every stored value was multiplied with."""
