@@ -129,7 +129,8 @@ __device__ __forceinline__ void pair_rows(const uint32_t* sp, int lane, uint32_t
 // K = 8192). The two-operand epilogues of the dense step move a chunk through shared memory, 64 contiguous bytes of
 // eight rows per instruction: y1 + SquaredReLU at T 4096, D 2048, F 8192 129 -> 96 us.
 // kEarly: the accumulator is handed back when the first chunk has been read; `last_first` turns the order of the chunks round.
-template <int kEpi, int kTileN = BN, bool kEarly = false>
+// kPairs: the transposed store goes through shared memory as words of two tokens (see there).
+template <int kEpi, int kTileN = BN, bool kEarly = false, bool kPairs = false>
 __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit,
                                          int q, int lane, uint8_t* my_stage, int part = 0, int parts = 1, bool second = false,
                                          bool last_first = false, uint64_t* tmem_empty_bar = nullptr) {
@@ -243,18 +244,37 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
         store_rows(w, args.C2, args.ldc2, col0);
       }
     } else {
-      // Transposed output: D row = feature (lane), D column = token. C is [N, M] row-major. Token by token, so that a store
-      // instruction writes 64 bytes of eight CONSECUTIVE tokens. As words of two neighbouring tokens (half the staging
-      // stores; an instruction then writes every second one of 16 tokens) 8192 x 16384 takes 96.5 us at K = 128 and 130.0 at
-      // K = 512 instead of 71.5 and 113.5, 28672 x 2048, K = 128 47.0 instead of 37.5, 4096 x 4096, K = 1024 23.9 instead of 23.7.
+      // Transposed output: D row = feature (lane), D column = token. C is [N, M] row-major. Through shared memory token by token
+      // (32 16-bit stores, four 16-byte loads), or as words of two neighbouring tokens: half the stores, but the rows have to be
+      // taken apart on the chain from a load to the global store. A warp walks its chunks one after another, so where the
+      // epilogue is the tile's time (256-row tiles with a short reduction) the first is the faster one: 8192 x 16384,
+      // K = 128 71.7 us and 96.5, 28672 x 2048, K = 128 37.7 and 47.0, 4096 x 4096, K = 1024 24.0 and 24.8. (The order of the global
+      // stores is the smaller part: the pairs' order, every second one of 16 tokens, 76.7; pairs read so that eight consecutive
+      // tokens leave at once, 98.4.) 512-row tiles, whose long main loop shares the shared memory with it, take the second
+      // (kPairs): 4096 x 16384, K = 2048 140.5 us and 144.6, K = 4096 245.2 and 249.0, 8192 x 16384, K = 2048 282 and 287.
       __syncwarp();
+      if constexpr (kPairs) {
+        uint32_t* st = reinterpret_cast<uint32_t*>(my_stage);
 #pragma unroll
-      for (int t = 0; t < 32; ++t)
-        reinterpret_cast<uint16_t*>(unit(t, lane >> 3))[lane & 7] = (uint16_t)(w[t >> 1] >> (16 * (t & 1)));
-      __syncwarp();
+        for (int j = 0; j < 16; ++j) st[j * 32 + lane] = w[j];
+        __syncwarp();
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(args.C) + (col0 + i * 8 + t8) * args.ldc + m0 + q * 32 + u * 8) = *unit(t8 + 8 * i, u);
+        for (int i = 0; i < 2; ++i) {
+          uint32_t r0[4], r1[4];
+          pair_rows(st + (i * 8 + t8) * 32 + u * 8, lane, r0, r1);
+          uint16_t* c = reinterpret_cast<uint16_t*>(args.C) + (col0 + i * 16 + t8 * 2) * args.ldc + m0 + q * 32 + u * 8;
+          *reinterpret_cast<uint4*>(c) = make_uint4(r0[0], r0[1], r0[2], r0[3]);
+          *reinterpret_cast<uint4*>(c + args.ldc) = make_uint4(r1[0], r1[1], r1[2], r1[3]);
+        }
+      } else {
+#pragma unroll
+        for (int t = 0; t < 32; ++t)
+          reinterpret_cast<uint16_t*>(unit(t, lane >> 3))[lane & 7] = (uint16_t)(w[t >> 1] >> (16 * (t & 1)));
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(args.C) + (col0 + i * 8 + t8) * args.ldc + m0 + q * 32 + u * 8) = *unit(t8 + 8 * i, u);
+      }
     }
   };
   // two register buffers: the TMEM load of the next 32 columns is in flight while this chunk is converted
@@ -1622,7 +1642,7 @@ gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constan
       } else {
         if (!mbar_wait_warp(&ctl->tmem_full[h], phase, abort_flag)) break;
         tc_fence_after();
-        if (live) epi_tile<kEpi, kTallBN>(args, taddr, m0, n0, n_limit, q, lane, wsm);
+        if (live) epi_tile<kEpi, kTallBN, false, true>(args, taddr, m0, n0, n_limit, q, lane, wsm);
         release_accumulator(lane, &ctl->tmem_empty[h]);
       }
       phase ^= 1;
