@@ -90,11 +90,12 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // Which epilogues run on two sets of four warps (one set per accumulator) on CTA pairs.
 __host__ __device__ constexpr bool is_drelu_t(int epi) { return epi == EPI_DRELU24_T || epi == EPI_DRELUV_T; }
 __host__ __device__ constexpr bool two_sets(int epi) { return epi == EPI_VNM8 || epi == EPI_ACT24_T || is_drelu_t(epi); }
-// Dense products: two sets share every tile, each takes half of its columns (the last tile's epilogue is exposed:
-// 1024 x 256 x 1024 17.3 -> 14.3 us; the 2:4 products gained nothing from it).
-// (one: a single set, see one_epilogue_set)
-__host__ __device__ constexpr bool split_sets(int mode, int epi, int expand, bool one) {
-  return mode == MODE_DENSE && epi != EPI_ROUTE && !expand && !one;
+// Dense products, and the row-major 2:4 products on tiles of full width: two sets share every tile, each takes half of its columns
+// (dense, where the last tile's epilogue is exposed: 1024 x 256 x 1024 17.3 -> 14.3 us; 2:4, with the store through TMA, 2048 x
+// 2048 x 2048 14.9 -> 13.8, 4096 x 2048 x 1024 16.5 -> 15.3, 8192 x 16384, K = 256 117 -> 85; narrow 2:4 tiles have too few columns
+// for two: 1024 x 256 x 1024 7.72 us with one set and 7.86 with two).
+__host__ __device__ constexpr bool split_sets(int mode, int epi, int expand, bool var) {
+  return (mode == MODE_DENSE && epi != EPI_ROUTE && !expand) || (mode == MODE_SPARSE24 && epi == EPI_STORE && !var);
 }
 
 // This warp has read its part of an accumulator for the last time: hand it back to the MMA warp.
@@ -118,22 +119,43 @@ __device__ __forceinline__ void pair_rows(const uint32_t* sp, int lane, uint32_t
   r1[2] = __byte_perm(qb.x, qb.y, 0x7632); r1[3] = __byte_perm(qb.z, qb.w, 0x7632);
 }
 
+// Four lanes hold a row of 64 bytes each, as four 16-byte units in registers; afterwards lane k of the four holds unit k of all four
+// rows, in the order of the rows. Two exchanges, each of the half that the other side needs.
+__device__ __forceinline__ void quad_transpose(uint32_t (&x)[16], int lane) {
+  const bool hi = lane & 2, odd = lane & 1;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint32_t got = __shfl_xor_sync(0xFFFFFFFFu, hi ? x[j] : x[8 + j], 2);
+    if (hi) x[j] = got; else x[8 + j] = got;
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t got = __shfl_xor_sync(0xFFFFFFFFu, odd ? x[8 * h + j] : x[8 * h + 4 + j], 1);
+      if (odd) x[8 * h + j] = got; else x[8 * h + 4 + j] = got;
+    }
+}
+
 // ---- epilogue (shared by the one-CTA and the two-CTA kernels) ---------------------------------------
 // One epilogue warp owns TMEM lanes [32q, 32q+32) of a 128 x 256 accumulator tile whose first row is
 // m0 and first column n0; `taddr` is the TMEM address of (lane 32q, column 0) of that accumulator.
 // kTileN: accumulator columns of the tile (a multiple of 32). Columns at or beyond n_limit (a ragged last
 // tile, whole 32-column chunks only since N % 32 == 0) are not stored. `part` of `parts`: the share of the tile's
 // columns that this warp takes.
-// A thread holds one row. EPI_STORE stores from there (16 bytes of 32 rows per instruction): the shortest way out, and
-// the 2:4 product's epilogue is on its critical path (through shared memory as below that product took 2 % more at
-// K = 8192). The two-operand epilogues of the dense step move a chunk through shared memory, 64 contiguous bytes of
+// A thread holds one row. EPI_STORE stores from there (16 bytes of 32 rows per instruction), or with kQuad 64 bytes of eight rows
+// after an exchange among four lanes; tiles of full width go out through TMA instead (epi_store_tile), except where the rows
+// are scattered (row_map). Narrow tiles (run-time width), where the latency of a chunk is what counts, keep the first: with the
+// exchange the step at T 1024, D 256, F 1024 took 40.4 us instead of 40.0. kQuad in the routed step at T 8192, D 4096, F 16384 in
+// four experts: 1277 -> 1257 us. The two-operand epilogues of the dense step move a chunk through shared memory, 64 contiguous bytes of
 // eight rows per instruction: y1 + SquaredReLU at T 4096, D 2048, F 8192 129 -> 96 us.
-// kEarly: the accumulator is handed back when the first chunk has been read; `last_first` turns the order of the chunks round.
+// kEarly: the accumulator is handed back when the first chunk has been read; the second part starts with its last chunk, so that
+// the columns at either end of the tile are the first to be read.
 // kPairs: the transposed store goes through shared memory as words of two tokens (see there).
-template <int kEpi, int kTileN = BN, bool kEarly = false, bool kPairs = false>
+template <int kEpi, int kTileN = BN, bool kEarly = false, bool kPairs = false, bool kQuad = false>
 __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit,
                                          int q, int lane, uint8_t* my_stage, int part = 0, int parts = 1, bool second = false,
-                                         bool last_first = false, uint64_t* tmem_empty_bar = nullptr) {
+                                         uint64_t* tmem_empty_bar = nullptr) {
   if constexpr (kEpi == EPI_ROUTE) {
     const int64_t row = m0 + q * 32 + lane;                                // this thread's D row
     // the row is a token, the first route_E columns its logits
@@ -170,6 +192,18 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
     row_live = r >= 0;
     row = r;
   }
+  // kQuad: this thread stores 16-byte unit `lane & 3` of the four rows of its four lanes
+  int rows4[4];
+  const int64_t ldq = second ? args.ldc2 : args.ldc;
+  uint16_t* cq = reinterpret_cast<uint16_t*>(second ? args.C2 : args.C) + (lane & 3) * 8;
+  if (kQuad) {
+    if (args.row_map) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) rows4[i] = __shfl_sync(0xFFFFFFFFu, (int)row, (lane & 28) + i);
+    } else {
+      cq += (m0 + q * 32 + (lane & 28)) * ldq;
+    }
+  }
   // EPI_SQRELU, EPI_DRELU: this thread moves 16-byte unit `u` of the rows `t8 + 8 i` of a chunk.
   const int t8 = lane >> 2, u = lane & 3;
   const int64_t out = m0 + q * 32 + t8;
@@ -193,7 +227,7 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
   };
   if (kEpi == EPI_DRELU) fetch(ch0);
   // `v` holds (once its load is complete) the chunk's accumulator columns; `next` starts the load of the chunk after
-  auto at = [&](int i) { return kEarly && last_first ? nch - 1 - i : i; };   // (kEarly: ch0 = 0)
+  auto at = [&](int i) { return kEarly && part == 1 ? nch - 1 - (i - ch0) : i; };
   auto chunk = [&](int i, uint32_t (&v)[32], uint32_t (&next)[32]) {
     const int ch = at(i);
     const int64_t col0 = n0 + ch * 32;
@@ -206,7 +240,7 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
       if (ch + 1 < nch) fetch(ch + 1);
     }
     tmem_ld_wait_on(v);
-    if (kEarly && i == 0) release_accumulator(lane, tmem_empty_bar);
+    if (kEarly && i == ch0) release_accumulator(lane, tmem_empty_bar);
     if (i + 1 < nch) tmem_ld_32x32b_x32(taddr + at(i + 1) * 32, next);
     if (kEpi == EPI_DRELU) {                                               // C = bf16(2 * acc * relu(aux))
 #pragma unroll
@@ -231,7 +265,13 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
       for (int j = 0; j < 16; ++j) w[j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
     }
     if (kEpi == EPI_STORE) {
-      if (row_live) {
+      if constexpr (kQuad) {
+        quad_transpose(w, lane);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (!args.row_map || rows4[i] >= 0)
+            *reinterpret_cast<uint4*>(cq + (args.row_map ? rows4[i] : i) * ldq + col0) = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+      } else if (row_live) {
         uint4* c = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(second ? args.C2 : args.C) + row * (second ? args.ldc2 : args.ldc) + col0);
 #pragma unroll
         for (int j = 0; j < 4; ++j) c[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
@@ -298,6 +338,67 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
   }
 }
 
+
+// ---- the plain store through TMA -----------------------------------------------------------------------
+// What bounded the plain store: an epilogue thread holds a row, so a 16-byte store of a warp went to 32 rows, 32 cycles of the
+// load/store unit each (7000 clocks for the 256 x 224 outputs of an SM in a 512-row tile), on the chain from one main loop to the
+// next and in the way of the MMAs' shared-memory reads. Here a warp puts 32 x 32 results into shared memory, 64 bytes a row, and one
+// thread hands them to TMA. Same box, call after call: 2:4 row-major 8192 x 16384, K = 128 115 -> 67 us, K = 1024 215 -> 167,
+// K = 4096 535 -> 503; E4M3 2:4 4096 x 16384 x 4096 170 -> 150; dense 8192 x 16384, K = 128 119 -> 79, 16384 x 8192, K = 512 168 -> 131.
+// Four lanes exchanging their rows' units and storing 64 bytes of eight rows per instruction gave E4M3 152 and dense K = 512 168;
+// reading a 512-row tile out into registers first and handing its accumulator back before storing (the stores then run beside
+// the next main loop, which they slow) 151; an evict-first hint nothing.
+// 32 x 32 chunk of a tile, rounded (w: this lane's row), through one of the warp's buffers to C; rows of 64 bytes, swizzled as
+// the store's tensor map expects it (64-byte swizzle), so that a thread per row writes without bank conflicts.
+template <int kBufs>
+__device__ __forceinline__ void store_chunk(const CUtensorMap* tmapC, uint8_t* bufs, uint32_t& buf, const uint32_t* w, int col, int row,
+                                            int lane) {
+  if (lane == 0) bulk_wait_read<kBufs - 1>();                              // the chunk before (or the one before that) has left
+  __syncwarp();
+  uint8_t* b = bufs + buf * kEpiWarpBytes;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    *reinterpret_cast<uint4*>(b + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+  fence_proxy_async_smem();
+  __syncwarp();
+  if (lane == 0) {
+    tma_store_2d(tmapC, b, col, row);
+    bulk_commit();
+  }
+  if (kBufs == 2) buf ^= 1u;
+}
+// kEarly, last_first: as in epi_tile.
+template <int kTileN, int kBufs, bool kEarly>
+__device__ __forceinline__ void epi_store_tile(const GemmArgs& args, const CUtensorMap* tmapC, uint32_t taddr, int64_t m0, int64_t n0,
+                                               int64_t n_limit, int q, int lane, uint8_t* bufs, uint32_t& buf, int part, int parts,
+                                               uint64_t* tmem_empty_bar) {
+  const int live = (int)min((int64_t)(kTileN / 32), (n_limit - n0) >> 5);
+  const int ch0 = live * part / parts, nch = live * (part + 1) / parts;
+  if (ch0 >= nch) {
+    if (kEarly) release_accumulator(lane, tmem_empty_bar);
+    return;
+  }
+  const float al = args.out_scale != 0.f ? args.out_scale : 1.f;           // x 1 is exact: bf16 products unchanged
+  const int row = (int)m0 + q * 32;
+  auto pack = [&](float lo, float hi) { return pack_bf16x2(__fmul_rn(lo, al), __fmul_rn(hi, al)); };
+  auto at = [&](int i) { return kEarly && part == 1 ? nch - 1 - (i - ch0) : i; };
+  auto chunk = [&](int i, uint32_t (&v)[32], uint32_t (&next)[32]) {
+    tmem_ld_wait_on(v);
+    if (kEarly && i == ch0) release_accumulator(lane, tmem_empty_bar);
+    if (i + 1 < nch) tmem_ld_32x32b_x32(taddr + at(i + 1) * 32, next);
+    uint32_t w[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) w[j] = pack(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+    store_chunk<kBufs>(tmapC, bufs, buf, w, (int)n0 + at(i) * 32, row, lane);
+  };
+  uint32_t va[32], vb[32];
+  tmem_ld_32x32b_x32(taddr + at(ch0) * 32, va);
+#pragma unroll 1
+  for (int i = ch0; i < nch; i += 2) {
+    chunk(i, va, vb);
+    if (i + 1 < nch) chunk(i + 1, vb, va);
+  }
+}
 
 // ---- fused SquaredReLU + V:N:M selection (groups of eight) ---------------------------------------------
 // Epilogue of the y1 product: the accumulator tile is y1^T (TMEM lane = feature, column = token), so a
@@ -1024,8 +1125,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant_
 constexpr int kThreads2 = 192;
 constexpr int kThreads2Expand = 448;                     // + eight warps that expand a packed operand into its stage
 constexpr int kThreads2Sets = 320;                       // + a second set of four epilogue warps
-__host__ __device__ constexpr int threads2(int mode, int epi, int expand, bool one) {
-  return expand ? kThreads2Expand : (two_sets(epi) || split_sets(mode, epi, expand, one) ? kThreads2Sets : kThreads2);
+__host__ __device__ constexpr int threads2(int mode, int epi, int expand, bool var) {
+  return expand ? kThreads2Expand : (two_sets(epi) || split_sets(mode, epi, expand, var) ? kThreads2Sets : kThreads2);
 }
 constexpr int kPkStageBytes = 8192 + 1024;               // packed values [64 tokens][64] + metadata bytes [64][16]
 // 8-bit operands (fp8 = true) keep the byte geometry of a stage (128-byte rows now hold 128 elements, so a
@@ -1037,15 +1138,20 @@ __host__ __device__ constexpr int stage_bytes2(bool sparse, int bn = BN, bool fp
 __host__ __device__ constexpr int num_stages2(bool sparse, int bn = BN, bool expand = false) {
   return sparse ? 4 : (expand ? 5 : 6);
 }
-__host__ __device__ constexpr int epi_bytes2(int epi, int bn = BN) {
-  return epi == EPI_VNM8 ? kVnmEpiBytes
+// Plain stores of full-width tiles go through TMA, two chunk buffers to a warp (2:4 products, whose stages leave less room, one); narrow tiles (run-time width), where the latency
+// of a chunk counts, and the kernels that expand an operand store from registers.
+__host__ __device__ constexpr bool tma_store2(int epi, bool expand, bool var) { return epi == EPI_STORE && !expand && !var; }
+__host__ __device__ constexpr int store_bufs2(bool sparse) { return sparse ? 1 : 2; }
+__host__ __device__ constexpr int epi_bytes2(int epi, int bn = BN, int store_bufs = 0) {
+  return store_bufs > 0   ? store_bufs * kEpiWarpBytes
+         : epi == EPI_VNM8 ? kVnmEpiBytes
          : is_drelu_t(epi) ? kSetWarps * kDreluWarpBytes / (bn == 256 ? 2 : 1)
          : epi == EPI_STORE || epi == EPI_ROUTE ? 0 : kSetWarps * kEpiWarpBytes;
 }
 __host__ __device__ constexpr int smem_bytes2(bool sparse, int bn = BN, int epi = EPI_STORE, bool expand = false,
-                                              bool fp8 = false) {
+                                              bool fp8 = false, int store_bufs = 0) {
   return 1024 + num_stages2(sparse, bn, expand) * (stage_bytes2(sparse, bn, fp8) + (expand ? kPkStageBytes : 0)) +
-         epi_bytes2(epi, bn) + 1024;
+         epi_bytes2(epi, bn, store_bufs) + 1024;
 }
 
 struct SmemCtl2 {
@@ -1092,14 +1198,13 @@ __device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) {
 // more SMs to work and shorten what one of them does: the eight kernels of a step at T 1024, D 256, F 1024 take 50 us
 // instead of 61 (graph replay). A kernel of its own, because the run-time width costs the issuing threads instructions
 // that the large products do not have (dense, 256 wide: 1.5 % and more).
-// kOneSet: dense products that store their tiles with one set of epilogue warps instead of two.
 // kDual: two independent products with the same reduction length in one launch (the weight gradients). The second one's
 // operands are tmapMeta (A) and tmapPk (B), its output args.C2.
-template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false, bool kDual = false, bool kOneSet = false>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kMode, kEpi, kExpand, kOneSet), 1)
+template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false, bool kDual = false>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kMode, kEpi, kExpand, kVar), 1)
 gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB,
                 const __grid_constant__ CUtensorMap tmapMeta, const __grid_constant__ CUtensorMap tmapPk,
-                const GemmArgs args) {
+                const __grid_constant__ CUtensorMap tmapC, const __grid_constant__ CUtensorMap tmapC2, const GemmArgs args) {
   extern __shared__ uint8_t smem_dyn[];
   uint8_t* smem = smem_dyn + align_pad(smem_dyn, 1024);
   constexpr bool kSparse = kMode == MODE_SPARSE24;
@@ -1130,7 +1235,9 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   static_assert(!kBMN || kBN == BN, "MN-major B is loaded in 64-column chunks");
   uint8_t* pk_stage = smem + kStages * kStageBytes;       // kExpand: ring of packed tiles, one per stage
   uint8_t* epi_stage = pk_stage + (kExpand ? kStages * kPkStageBytes : 0);
-  SmemCtl2* ctl = reinterpret_cast<SmemCtl2*>(epi_stage + epi_bytes2(kEpi, kBN));
+  constexpr bool kTmaStore = tma_store2(kEpi, kExpand != 0, kVar);
+  constexpr int kStoreBufs = kTmaStore ? (threads2(kMode, kEpi, kExpand, kVar) / 32 - 2) * store_bufs2(kSparse) : 0;
+  SmemCtl2* ctl = reinterpret_cast<SmemCtl2*>(epi_stage + epi_bytes2(kEpi, kBN, kStoreBufs));
   volatile int* abort_flag = &ctl->abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1155,7 +1262,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     for (int b = 0; b < 2; ++b) {
       mbar_init(&ctl->tmem_full[b], 1);
       // the epilogue warps of both CTAs that read the accumulator
-      mbar_init(&ctl->tmem_empty[b], split_sets(kMode, kEpi, kExpand, kOneSet) || (two_sets(kEpi) && kAccBufs == 1) ? 16 : 8);
+      mbar_init(&ctl->tmem_empty[b], split_sets(kMode, kEpi, kExpand, kVar) || (two_sets(kEpi) && kAccBufs == 1) ? 16 : 8);
     }
     ctl->abort_flag = 0;
     fence_mbar_init();
@@ -1388,9 +1495,9 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   } else {
     // =========================== epilogue (warps 2..5 or 2..9, both CTAs) ===========================
     const int q = warp & 3, set = (warp - 2) >> 2;
-    constexpr int kParts = split_sets(kMode, kEpi, kExpand, kOneSet) ? 2 : 1;
-    uint8_t* my_stage = epi_stage + (set * 4 + q) * kEpiWarpBytes;
-    uint32_t acc = 0, acc_phase = 0;
+    constexpr int kParts = split_sets(kMode, kEpi, kExpand, kVar) ? 2 : 1;
+    uint8_t* my_stage = epi_stage + (set * 4 + q) * (kTmaStore ? store_bufs2(kSparse) : 1) * kEpiWarpBytes;
+    uint32_t acc = 0, acc_phase = 0, buf = 0;
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
       const GemmTile tc = get_tile<kBN, kVar, kDual>(args, tile, num_m_tiles, num_n_tiles_, nkb_full);
@@ -1401,11 +1508,17 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
       const bool live = args.tile_table != nullptr || m0 < (second ? args.M2 : args.M);
       if (!mbar_wait_warp(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      if (live) epi_tile<kEpi, kBN, kOverlap>(args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts, second, acc_phase == 0,
-                                              &ctl->tmem_empty[0]);
+      if (kTmaStore && live && !args.row_map) {
+        epi_store_tile<kBN, store_bufs2(kSparse), kOverlap>(args, second ? &tmapC2 : &tmapC, taddr, m0, n0, n_limit, q, lane, my_stage,
+                                                            buf, set, kParts, &ctl->tmem_empty[0]);
+      } else if (live) {
+        epi_tile<kEpi, kBN, kOverlap, false, kTmaStore>(args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts, second,
+                                                        &ctl->tmem_empty[0]);
+      }
       if (!kOverlap || !live) release_accumulator(lane, &ctl->tmem_empty[acc]);
       if (++acc == (uint32_t)kAccBufs) { acc = 0; acc_phase ^= 1; }
     }
+    if (kTmaStore && lane == 0) bulk_wait_all();
   }
 
   // =========================== teardown ===========================
@@ -1438,7 +1551,7 @@ constexpr int kTallThreads = 320;                         // producer, MMA issue
 __host__ __device__ constexpr int tall_b_bytes(bool bmn) { return bmn ? 32768 : 28672; }
 __host__ __device__ constexpr int tall_stage_bytes(bool bmn, bool fp8) { return tall_b_bytes(bmn) + 2 * (16384 + meta_stage_bytes2(fp8)); }
 __host__ __device__ constexpr int tall_epi_bytes(int epi) {
-  return is_drelu_t(epi) ? kSetWarps * kDreluWarpBytes : epi == EPI_STORE ? 0 : kSetWarps * kEpiWarpBytes;
+  return kSetWarps * (is_drelu_t(epi) ? kDreluWarpBytes : kEpiWarpBytes);
 }
 __host__ __device__ constexpr int tall_smem(int epi, bool bmn, bool fp8) {
   return 1024 + kTallStages * tall_stage_bytes(bmn, fp8) + tall_epi_bytes(epi) + 1024;
@@ -1489,7 +1602,8 @@ __device__ __forceinline__ TallTile tall_tile(const GemmArgs& args, int tile) {
 template <bool kBMN, int kEpi, bool kFp8>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTallThreads, 1)
 gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB,
-                 const __grid_constant__ CUtensorMap tmapBn, const __grid_constant__ CUtensorMap tmapMeta, const GemmArgs args) {
+                 const __grid_constant__ CUtensorMap tmapBn, const __grid_constant__ CUtensorMap tmapMeta,
+                 const __grid_constant__ CUtensorMap tmapC, const GemmArgs args) {
   extern __shared__ uint8_t smem_dyn[];
   uint8_t* smem = smem_dyn + align_pad(smem_dyn, 1024);
   constexpr int kBBytes = tall_b_bytes(kBMN), kMetaBytes = meta_stage_bytes2(kFp8), kStageBytes = tall_stage_bytes(kBMN, kFp8);
@@ -1628,7 +1742,7 @@ gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constan
     const int q = warp & 3, h = (warp - 2) >> 2;
     uint8_t* wsm = epi_stage + (h * 4 + q) * (tall_epi_bytes(kEpi) / kSetWarps);
     const uint32_t taddr = tmem_base + (uint32_t)(h * kTallBN) + ((uint32_t)(q * 32) << 16);
-    uint32_t phase = 0;
+    uint32_t phase = 0, buf = 0;
     for (int l = 0, tile; (tile = tall_nth(args, l, pair, num_pairs)) >= 0; ++l) {
       const TallTile t = tall_tile(args, tile);
       if (h >= t.halves) continue;
@@ -1642,11 +1756,16 @@ gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constan
       } else {
         if (!mbar_wait_warp(&ctl->tmem_full[h], phase, abort_flag)) break;
         tc_fence_after();
-        if (live) epi_tile<kEpi, kTallBN, false, true>(args, taddr, m0, n0, n_limit, q, lane, wsm);
+        if (kEpi == EPI_STORE && live) {
+          epi_store_tile<kTallBN, 1, false>(args, &tmapC, taddr, m0, n0, n_limit, q, lane, wsm, buf, 0, 1, nullptr);
+        } else if (live) {
+          epi_tile<kEpi, kTallBN, false, true>(args, taddr, m0, n0, n_limit, q, lane, wsm);
+        }
         release_accumulator(lane, &ctl->tmem_empty[h]);
       }
       phase ^= 1;
     }
+    if (kEpi == EPI_STORE && lane == 0) bulk_wait_all();
   }
 
   // =========================== teardown ===========================
@@ -1705,6 +1824,11 @@ int make_tmap(CUtensorMap* m, const void* base, int64_t rows, int64_t cols, int6
   return SF_OK;
 }
 
+// Map of a plain store: C [rows, cols] bf16, chunks of 32 x 32 (see store_chunk).
+int make_store_map(CUtensorMap* m, void* C, int64_t rows, int64_t cols, int64_t ld) {
+  return make_tmap(m, C, rows, cols, ld, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
+}
+
 int sm_count() {
   static int n[64] = {0};
   int dev = 0;
@@ -1733,12 +1857,13 @@ int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const GemmArgs& a, 
                     ta, tb, a);
 }
 
-template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false, bool kDual = false,
-          bool kOneSet = false>
+template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false, bool kDual = false>
 int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tm, GemmArgs a, cudaStream_t s,
-               const CUtensorMap* tpk = nullptr) {
-  auto kern = gemm_tc2_kernel<kMode, kAMN, kBMN, kEpi, kBN, kExpand, kFp8, kVar, kDual, kOneSet>;
-  constexpr int smem = smem_bytes2(kMode != MODE_DENSE, kBN, kEpi, kExpand != 0, kFp8);
+               const CUtensorMap* tpk = nullptr, const CUtensorMap* tc = nullptr, const CUtensorMap* tc2 = nullptr) {
+  auto kern = gemm_tc2_kernel<kMode, kAMN, kBMN, kEpi, kBN, kExpand, kFp8, kVar, kDual>;
+  constexpr int threads = threads2(kMode, kEpi, kExpand, kVar);
+  constexpr bool tma_store = tma_store2(kEpi, kExpand != 0, kVar);
+  constexpr int smem = smem_bytes2(kMode != MODE_DENSE, kBN, kEpi, kExpand != 0, kFp8, tma_store ? (threads / 32 - 2) * store_bufs2(kMode != MODE_DENSE) : 0);
   static_assert(smem <= 232448 && smem >= kExclusiveSmem, "shared memory per CTA: fits, and one CTA per SM");
   static bool attr_done[64] = {false};
   int dev = 0;
@@ -1755,7 +1880,8 @@ int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
                                  : a.num_m_tiles * a.num_n_tiles + (kDual ? a.num_m_tiles2 * a.num_n_tiles2 : 0);
   const int max_pairs = sm_count() / 2;
   const int pairs = tiles < max_pairs ? tiles : max_pairs;
-  return launch_pdl(kern, dim3(2 * pairs), threads2(kMode, kEpi, kExpand, kOneSet), smem, s, ta, tb, tm, tpk ? *tpk : ta, a);
+  if (tma_store && !a.row_map && (!tc || (kDual && !tc2))) return SF_ERR_UNSUPPORTED;
+  return launch_pdl(kern, dim3(2 * pairs), threads, smem, s, ta, tb, tm, tpk ? *tpk : ta, tc ? *tc : ta, tc2 ? *tc2 : ta, a);
 }
 
 int64_t l2_bytes() {
@@ -1770,14 +1896,6 @@ int64_t l2_bytes() {
   return n[dev];
 }
 
-// Dense products: does one set of epilogue warps store a tile sooner than two that share it? Two halve an epilogue, and where
-// the output stays in the L2 they are the faster ones (12288 x 4096, K = 128 37.5 us, one set 39.9). Where it does not and the
-// reduction is short, the kernel lasts as long as its writes, and those of twice as many warps go slower: 8192 x 16384, K = 128
-// 132.9 us with two and 113.6 with one, K = 512 170.8 and 159.9, K = 1024 237.9 and 234.5, K = 2048 419 and 426; E4M3, K = 512
-// 146.3 and 125.6, K = 1024 176 and 165. (stages: 64 of K, E4M3 128; the dense step's two-operand epilogues keep two sets: y1 at
-// T 8192, D 256, F 16384 121 us with two and 135 with one, dy1 158 and 195)
-bool one_epilogue_set(int64_t out_elements, int64_t stages) { return stages <= 8 && 2 * out_elements > l2_bytes(); }
-
 // Tile width of the two-accumulator 2:4 variant (transposed-output products): 2 x 224 accumulator
 // columns + 8 metadata columns fit the 512 TMEM columns.
 #ifndef SF_NARROW_BN
@@ -1787,7 +1905,8 @@ constexpr int kNarrowBN = SF_NARROW_BN;
 
 template <bool kBMN, int kEpi, bool kFp8 = false>
 int launch_tall(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tbn, const CUtensorMap& tm, GemmArgs a,
-                cudaStream_t s) {
+                cudaStream_t s, const CUtensorMap* tc = nullptr) {
+  if (kEpi == EPI_STORE && !tc) return SF_ERR_UNSUPPORTED;
   auto kern = gemm_tall_kernel<kBMN, kEpi, kFp8>;
   constexpr int smem = tall_smem(kEpi, kBMN, kFp8);
   static_assert(smem <= 232448 && smem >= kExclusiveSmem, "shared memory per CTA: fits, and one CTA per SM");
@@ -1801,7 +1920,7 @@ int launch_tall(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap&
   a.num_m_tiles = (int)((a.M + 511) / 512);
   a.num_n_tiles = (int)(a.N / kTallBN);                                       // full-width columns
   const int tiles = a.num_m_tiles * (a.num_n_tiles + (a.N % kTallBN ? 1 : 0)), max_pairs = sm_count() / 2;
-  return launch_pdl(kern, dim3(2 * (tiles < max_pairs ? tiles : max_pairs)), kTallThreads, smem, s, ta, tb, tbn, tm, a);
+  return launch_pdl(kern, dim3(2 * (tiles < max_pairs ? tiles : max_pairs)), kTallThreads, smem, s, ta, tb, tbn, tm, tc ? *tc : ta, a);
 }
 
 // Tensor maps of a tall product, lengths in 2-byte words (8-bit operands: two codes): vals [M, kw / 2] packed A, B [N, kw]
@@ -1876,15 +1995,12 @@ bool use_tall(int64_t M, int64_t N, int64_t stages, int bn, double flat_epi, dou
   return q * full + rest < 0.99 * flat;
 }
 
-// The same for the products that store row-major (y3, dX; E4M3). With a short reduction and an output beyond the L2 the kernel
-// lasts as long as its writes, which the clocks above do not hold, and the two sets of epilogue warps of a 512-row tile write
-// slower than the one of a 256-row tile: 8192 x 16384 K = 128 130 us on 512-row tiles and 117 on 256-row ones, K = 256 134 and
-// 123, K = 512 152 and 137; E4M3 K = 256 131 and 118, K = 512 138 and 123, K = 1024 168 and 147.
-// The line could lie higher: in bursts 256-row tiles also win at 8 to 16 stages (8192 x 16384, K = 1024 207 and 189 us, E4M3 K = 2048
-// 237 and 219), but not under the power cap: 4096 x 16384 x 4096 in E4M3, 16 stages, 175 and 167 us in a burst, and 213 and
-// 220 us for prune, quantise and product call after call.
+// The same for the products that store row-major (y3, dX; E4M3). With an output beyond the L2 and a short reduction the kernel
+// lasts as long as its writes, which the clocks above do not hold. With one stage 512-row tiles end first (8192 x 16384 67.5 us
+// against 76.7), with two to six the two are equal in bf16 (K = 256 83.0 and 85.2, K = 512 109.5 and 109.1, K = 768 136.3
+// and 136.1) and in E4M3 (K = 1024 113.7 and 113.9), and 256-row tiles are kept, which leave fewer idle at the end.
 bool use_tall_plain(int64_t M, int64_t N, int64_t stages) {
-  const bool write_bound = stages < 7 && 2 * M * N > l2_bytes();
+  const bool write_bound = stages > 1 && stages < 7 && 2 * M * N > l2_bytes();
   return !write_bound && use_tall(M, N, stages, BN, 2500.0, 2500.0);
 }
 
@@ -1917,6 +2033,9 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
   if (b_kmajor) st = make_tmap(&tb, B, N, K, K, 64, two ? bn / 2 : 256, CU_TENSOR_MAP_SWIZZLE_128B);
   else          st = make_tmap(&tb, B, K, N, N, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st != SF_OK) return st;
+  const bool tma = two && bn == BN && epi == EPI_STORE;
+  CUtensorMap tc;
+  if (tma && (st = make_store_map(&tc, C, M, N, ldc)) != SF_OK) return st;
   GemmArgs a{};
   a.M = M; a.N = N; a.K = K;
   a.C = C; a.ldc = ldc; a.C2 = C2; a.ldc2 = ldc2; a.aux = aux; a.ldaux = ldaux;
@@ -1925,25 +2044,20 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
   a.bn = bn;
 #define SF_DENSE_CASE(AMN, BMN, EPI)                                                                \
   return !two       ? launch_one<MODE_DENSE, AMN, BMN, EPI>(ta, tb, a, s)                             \
-         : bn == BN ? launch_two<MODE_DENSE, AMN, BMN, EPI>(ta, tb, ta, a, s)                         \
+         : bn == BN ? launch_two<MODE_DENSE, AMN, BMN, EPI>(ta, tb, ta, a, s, nullptr, tma ? &tc : nullptr) \
                     : launch_two<MODE_DENSE, AMN, BMN, EPI, BN, 0, false, true>(ta, tb, ta, a, s)
-#define SF_DENSE_STORE(AMN, BMN)                                                                                              \
-  if (two && bn == BN && one_epilogue_set(M * N, K / 64))                                                                     \
-    return launch_two<MODE_DENSE, AMN, BMN, EPI_STORE, BN, 0, false, false, false, true>(ta, tb, ta, a, s);                   \
-  SF_DENSE_CASE(AMN, BMN, EPI_STORE)
   const bool amn = !a_kmajor, bmn = !b_kmajor;
   if (epi == EPI_STORE) {
-    if (!amn && !bmn) { SF_DENSE_STORE(false, false); }
-    if (!amn && bmn) { SF_DENSE_STORE(false, true); }
-    if (amn && !bmn) { SF_DENSE_STORE(true, false); }
-    SF_DENSE_STORE(true, true);
+    if (!amn && !bmn) SF_DENSE_CASE(false, false, EPI_STORE);
+    if (!amn && bmn) SF_DENSE_CASE(false, true, EPI_STORE);
+    if (amn && !bmn) SF_DENSE_CASE(true, false, EPI_STORE);
+    SF_DENSE_CASE(true, true, EPI_STORE);
   } else if (epi == EPI_SQRELU) {
     if (!amn && !bmn) SF_DENSE_CASE(false, false, EPI_SQRELU);
   } else if (epi == EPI_DRELU) {
     if (!amn && bmn) SF_DENSE_CASE(false, true, EPI_DRELU);
     if (!amn && !bmn) SF_DENSE_CASE(false, false, EPI_DRELU);
   }
-#undef SF_DENSE_STORE
 #undef SF_DENSE_CASE
   return SF_ERR_UNSUPPORTED;
 }
@@ -1980,9 +2094,13 @@ int gemm_dual_tn(const void* A1, const void* B1, int64_t M1, int64_t N1, void* C
   a.num_m_tiles2 = (int)((M2 + 255) / 256);
   a.num_n_tiles2 = (int)((N2 + a.bn - 1) / a.bn);
   a.status = status;
-  if (a.bn == BN && one_epilogue_set(M1 * N1 + M2 * N2, K / 64))
-    return launch_two<MODE_DENSE, true, true, EPI_STORE, BN, 0, false, false, true, true>(ta, tb, ta2, a, s, &tb2);
-  return a.bn == BN ? launch_two<MODE_DENSE, true, true, EPI_STORE, BN, 0, false, false, true>(ta, tb, ta2, a, s, &tb2)
+  CUtensorMap tc, tc2;
+  if (a.bn == BN) {
+    st = make_store_map(&tc, C1, M1, N1, N1);
+    if (st == SF_OK) st = make_store_map(&tc2, C2, M2, N2, N2);
+    if (st != SF_OK) return st;
+  }
+  return a.bn == BN ? launch_two<MODE_DENSE, true, true, EPI_STORE, BN, 0, false, false, true>(ta, tb, ta2, a, s, &tb2, &tc, &tc2)
                     : launch_two<MODE_DENSE, true, true, EPI_STORE, BN, 0, false, true, true>(ta, tb, ta2, a, s, &tb2);
 }
 
@@ -2001,8 +2119,12 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   if (M == 0 || N == 0) return SF_OK;
   const bool plain = (epi == EPI_STORE);                 // row-major output, either B layout: two-CTA kernel only
   if ((plain || !b_kmajor) && !two) return SF_ERR_UNSUPPORTED;
-  CUtensorMap ta, tb, tm;
+  CUtensorMap ta, tb, tm, tc;
   const TileShape tile = two ? gemm_sparse24_tile(M, N, K, epi) : TileShape{BM, BN};
+  if (plain) {
+    const int st = make_store_map(&tc, C, M, N, ldc);
+    if (st != SF_OK) return st;
+  }
   if (tile.rows == 512) {
     CUtensorMap tbn;
     const int st = tall_maps(a_vals, meta_hw, B, b_kmajor, M, N, K, 0, 2, &ta, &tb, &tbn, &tm);
@@ -2011,7 +2133,7 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
     a.M = M; a.N = N; a.K = K;
     a.C = C; a.ldc = ldc; a.status = status;
     if (!plain) return launch_tall<false, EPI_STORE_T>(ta, tb, tbn, tm, a, s);
-    return b_kmajor ? launch_tall<false, EPI_STORE>(ta, tb, tbn, tm, a, s) : launch_tall<true, EPI_STORE>(ta, tb, tbn, tm, a, s);
+    return b_kmajor ? launch_tall<false, EPI_STORE>(ta, tb, tbn, tm, a, s, &tc) : launch_tall<true, EPI_STORE>(ta, tb, tbn, tm, a, s, &tc);
   }
   int st = two ? make_tmap(&ta, a_vals, M, K / 2, K / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B)
                : make_tmap(&ta, a_vals, M, K / 2, K / 2, 32, 128, CU_TENSOR_MAP_SWIZZLE_64B);
@@ -2035,9 +2157,9 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   const bool var = two && bn != (plain ? BN : kNarrowBN);
   if (epi == EPI_STORE) {
     if (b_kmajor) return var ? launch_two<MODE_SPARSE24, false, false, EPI_STORE, BN, 0, false, true>(ta, tb, tm, a, s)
-                             : launch_two<MODE_SPARSE24, false, false, EPI_STORE>(ta, tb, tm, a, s);
+                             : launch_two<MODE_SPARSE24, false, false, EPI_STORE>(ta, tb, tm, a, s, nullptr, &tc);
     return var ? launch_two<MODE_SPARSE24, false, true, EPI_STORE, BN, 0, false, true>(ta, tb, tm, a, s)
-               : launch_two<MODE_SPARSE24, false, true, EPI_STORE>(ta, tb, tm, a, s);
+               : launch_two<MODE_SPARSE24, false, true, EPI_STORE>(ta, tb, tm, a, s, nullptr, &tc);
   }
   if (epi == EPI_STORE_T)
     return !two ? launch_one<MODE_SPARSE24, false, false, EPI_STORE_T>(ta, tb, a, s)
@@ -2146,17 +2268,19 @@ int gemm_fp8(bool sparse, const void* A, const uint8_t* meta_hw, const void* B, 
   if (M == 0 || N == 0) return SF_OK;
   // the operands in 2-byte units: [M, K/2] (dense) or [M, K/4] (2:4 values), [N, K/2]
   const int64_t K2 = K / 2;
-  CUtensorMap ta, tb, tm;
+  CUtensorMap ta, tb, tm, tc;
+  int st = make_store_map(&tc, C, M, N, ldc);
+  if (st != SF_OK) return st;
   if (sparse && use_tall_plain(M, N, K / 256)) {
     CUtensorMap tbn;
-    const int st = tall_maps(A, meta_hw, B, true, M, N, K2, 2, 4, &ta, &tb, &tbn, &tm);
+    st = tall_maps(A, meta_hw, B, true, M, N, K2, 2, 4, &ta, &tb, &tbn, &tm);
     if (st != SF_OK) return st;
     GemmArgs a{};
     a.M = M; a.N = N; a.K = K2;
     a.C = C; a.ldc = ldc; a.status = status; a.out_scale = alpha;
-    return launch_tall<false, EPI_STORE, true>(ta, tb, tbn, tm, a, s);
+    return launch_tall<false, EPI_STORE, true>(ta, tb, tbn, tm, a, s, &tc);
   }
-  int st = sparse ? make_tmap(&ta, A, M, K2 / 2, K2 / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2)
+  st = sparse ? make_tmap(&ta, A, M, K2 / 2, K2 / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2)
                   : make_tmap(&ta, A, M, K2, K2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2);
   if (st != SF_OK) return st;
   const int bn = best_width(M, N, K2 / (sparse ? 128 : 64), sparse, BN, 32, sparse ? 400.0 : 200.0, sparse, sparse ? 700.0 : 0.0);
@@ -2174,13 +2298,11 @@ int gemm_fp8(bool sparse, const void* A, const uint8_t* meta_hw, const void* B, 
   a.C = C; a.ldc = ldc; a.meta_hw = meta_hw; a.status = status; a.out_scale = alpha;
   a.num_k_blocks = (int)(K2 / 64);
   a.bn = bn;
-  if (!sparse && bn == BN && one_epilogue_set(M * N, K2 / 64))
-    return launch_two<MODE_DENSE, false, false, EPI_STORE, BN, 0, true, false, false, true>(ta, tb, tm, a, s);
   if (bn != BN)
     return sparse ? launch_two<MODE_SPARSE24, false, false, EPI_STORE, BN, 0, true, true>(ta, tb, tm, a, s)
                   : launch_two<MODE_DENSE, false, false, EPI_STORE, BN, 0, true, true>(ta, tb, tm, a, s);
-  return sparse ? launch_two<MODE_SPARSE24, false, false, EPI_STORE, BN, 0, true>(ta, tb, tm, a, s)
-                : launch_two<MODE_DENSE, false, false, EPI_STORE, BN, 0, true>(ta, tb, tm, a, s);
+  return sparse ? launch_two<MODE_SPARSE24, false, false, EPI_STORE, BN, 0, true>(ta, tb, tm, a, s, nullptr, &tc)
+                : launch_two<MODE_DENSE, false, false, EPI_STORE, BN, 0, true>(ta, tb, tm, a, s, nullptr, &tc);
 }
 
 bool gemm_sparse24_vnm8_supported(int64_t F, int64_t T, int64_t D, int V) {
@@ -2276,19 +2398,21 @@ int gemm_grouped_sparse24_rm(const void* a_vals, const uint8_t* meta_hw, const v
   return launch_two<MODE_SPARSE24, false, true, EPI_STORE>(ta, tb, tm, a, s);
 }
 
-int gemm_grouped_dense_tn(const void* A, int64_t Ma, const void* B, int64_t Nb, int64_t rows, void* C, int64_t ldc,
+int gemm_grouped_dense_tn(const void* A, int64_t Ma, const void* B, int64_t Nb, int64_t rows, void* C, int64_t c_rows, int64_t ldc,
                           const GemmTile* tiles, const int* num_tiles, int max_tiles, int* status, cudaStream_t s) {
   if (Ma % 256 || Nb % 256 || rows % 64 || max_tiles <= 0) return SF_ERR_SHAPE;
   CUtensorMap ta, tb;
   int st = make_tmap(&ta, A, rows, Ma, Ma, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st != SF_OK) return st;
   st = make_tmap(&tb, B, rows, Nb, Nb, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
+  CUtensorMap tc;
+  if (st == SF_OK) st = make_store_map(&tc, C, c_rows, ldc, ldc);
   if (st != SF_OK) return st;
   GemmArgs a{};
   a.M = Ma; a.N = ldc; a.K = rows;                         // N bounds the stored columns: the whole output row
   a.C = C; a.ldc = ldc; a.status = status;
   a.tile_table = tiles; a.num_tiles_dev = num_tiles; a.num_k_blocks = max_tiles;
-  return launch_two<MODE_DENSE, true, true, EPI_STORE>(ta, tb, ta, a, s);
+  return launch_two<MODE_DENSE, true, true, EPI_STORE>(ta, tb, ta, a, s, nullptr, &tc);
 }
 
 int gemm_dense_expand(const void* dense_op, int packed_operand, const void* pk_vals, const void* pk_meta, int64_t M,

@@ -145,9 +145,9 @@ int gemm_grouped_drelu24(const void* a_vals, const uint8_t* meta_hw, const void*
 int gemm_grouped_sparse24_rm(const void* a_vals, const uint8_t* meta_hw, const void* B, bool b_kmajor, int64_t rows,
                              int64_t N, int64_t Fe, int64_t Ktot, void* C, const int* row_map, const GemmTile* tiles,
                              const int* num_tiles, int max_tiles, int* status, cudaStream_t s);
-// C[M, N] (leading dimension ldc) accumulates A^T B over each tile's own range of rows: A [rows, Ma], B [rows, Nb]
+// C[c_rows, ldc] accumulates A^T B over each tile's own range of rows: A [rows, Ma], B [rows, Nb]
 // row-major (both reduced over rows).
-int gemm_grouped_dense_tn(const void* A, int64_t Ma, const void* B, int64_t Nb, int64_t rows, void* C, int64_t ldc,
+int gemm_grouped_dense_tn(const void* A, int64_t Ma, const void* B, int64_t Nb, int64_t rows, void* C, int64_t c_rows, int64_t ldc,
                           const GemmTile* tiles, const int* num_tiles, int max_tiles, int* status, cudaStream_t s);
 // A_s[M,K] 2:4-packed times B (b_kmajor: [N,K] row-major, else [K,N] row-major).
 // epi EPI_STORE_T: transposed output Ct[N,M] (b_kmajor only); EPI_STORE: C[M,N]

@@ -489,10 +489,10 @@ int sf_routed_ffn_bwd(const sf_router_desc* desc, const void* dY, const void* X,
                                   status, s));
   trace_mark(s);
   // line 3: dW2[:, expert block] = dY_e^T y2_e;  line 6: dW1[expert block, :] = dy1_e^T X_e
-  SF_TRY(gemm_grouped_dense_tn(at(workspace, L.dyp), d.D, at(fwd_ctx, L.y2_dense), L.Fe, L.rows_max, dW2, d.F,
+  SF_TRY(gemm_grouped_dense_tn(at(workspace, L.dyp), d.D, at(fwd_ctx, L.y2_dense), L.Fe, L.rows_max, dW2, d.D, d.F,
                                (const GemmTile*)at(fwd_ctx, L.tabC), counts + 2, L.max_tiles[2], status, s));
   trace_mark(s);
-  SF_TRY(gemm_grouped_dense_tn(at(workspace, L.dy1_dense), L.Fe, at(fwd_ctx, L.xp), d.D, L.rows_max, dW1, d.D,
+  SF_TRY(gemm_grouped_dense_tn(at(workspace, L.dy1_dense), L.Fe, at(fwd_ctx, L.xp), d.D, L.rows_max, dW1, d.F, d.D,
                                (const GemmTile*)at(fwd_ctx, L.tabD), counts + 3, L.max_tiles[3], status, s));
   trace_mark(s);
   return SF_OK;

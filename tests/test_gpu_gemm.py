@@ -100,6 +100,37 @@ def _integer_24_product(Mr, Nc, K, b_k, run):
     return bits(C), synth.f32_to_bf16_bits(oracle.bf16_to_f32(p.dense) @ B.T)
 
 
+# The stores through TMA of full-width tiles: one buffer set or two, half-empty last tiles, several tiles to a CTA pair, the shortest
+# reduction. Exact on small integers, nothing written outside the result.
+@pytest.mark.parametrize("kind,Mr,Nc,K", [("dense", 2688, 4864, 64), ("dense", 5248, 2304, 320),           # two sets of warps share a tile
+                                          ("sparse24", 256, 18944, 128), ("sparse24", 9728, 512, 256),     # 256-row tiles, overlapping accumulators
+                                          ("sparse24", 6400, 4352, 128), ("sparse24", 512, 1792, 384),  # 512-row tiles
+                                          ("fp8", 4096, 4608, 256), ("fp8", 256, 18944, 512), ("fp8_dense", 2560, 4864, 128)])
+def test_full_width_stores_stay_inside_the_result(kind, Mr, Nc, K):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(Mr + K)
+    ints = lambda *s: torch.randint(-3, 4, s, generator=g, device="cuda")
+    A, B = ints(Mr, K), ints(Nc, K)
+    out = Guarded((Mr, Nc), torch.bfloat16)
+    bf = lambda t: t.to(torch.bfloat16)
+    if kind == "dense":
+        _, ws = binding.sf_gemm_dense(bf(A), True, bf(B), True, C_out=out.t)
+    elif kind == "sparse24":
+        vals, meta, A = binding.sf_prune24_compress(bf(A), 1, 0, want_dense=True)
+        _, ws = binding.sf_gemm_sparse24_rm(vals, meta, bf(B), True, C_out=out.t)
+    else:
+        q = lambda t: binding.sf_fp8_quantize(bf(t), 1.0)
+        if kind == "fp8":
+            vals, meta, A = binding.sf_prune24_compress_fp8(bf(A), 0, 1.0, want_dense=True)
+            A = A.view(torch.float8_e4m3fn)
+            _, ws = binding.sf_gemm_fp8_sparse24(vals, meta, q(B), 1.0, C_out=out.t)
+        else:
+            _, ws = binding.sf_gemm_fp8_dense(q(A), q(B), 1.0, C_out=out.t)
+    assert binding.sf_check_status(ws) == binding.SF_OK
+    out.check(kind)
+    assert torch.equal(out.t, bf(A.double() @ B.double().T))
+
+
 @pytest.mark.parametrize("b_k", [True, False])
 @pytest.mark.parametrize("Mr,Nc,K", [(8192, 8192, 512),    # 512-row tiles, a narrow last column of 128
                                      (8448, 4352, 512),    # the same, last tile row half empty, narrow column of 96
