@@ -101,20 +101,6 @@ prune24_fp8_kernel(const uint4* __restrict__ W, int64_t rows, int cols, int64_t 
   }
 }
 
-// Canonical metadata [R, K/16] to the order of the 8-bit 2:4 instruction (meta_hw8_offset): the eight words of 128 columns
-// stay together, so the unit is 16 bytes. One thread each, chunks of a row fastest: with one 2-byte word per thread the
-// conversion and the product took 146.4 us together at 4096 x 16384 x 4096, with this 143.9.
-__global__ void __launch_bounds__(256)
-meta_reorder8_kernel(const uint4* __restrict__ meta, uint8_t* __restrict__ meta_hw, uint32_t R, uint32_t K) {
-  pdl_wait();
-  pdl_trigger();
-  const uint32_t chunks = K >> 7;                                  // even: K % 256 == 0
-  const uint32_t idx = blockIdx.x * 256u + threadIdx.x;
-  if (idx >= R * chunks) return;
-  const uint32_t m = idx / chunks, c = idx - m * chunks;
-  *reinterpret_cast<uint4*>(meta_hw + meta_hw8_offset(m, (int64_t)c * 8, K)) = __ldg(meta + idx);
-}
-
 }  // namespace
 
 }  // namespace sf
@@ -190,13 +176,8 @@ int sf_gemm_fp8_sparse24(const void* a_vals, const void* a_meta, const void* B, 
   if (!aligned16(a_vals) || !aligned16(a_meta) || !aligned16(B) || !aligned16(C) || !aligned16(workspace))
     return SF_ERR_ALIGN;
   SF_TRY(check_arch());
-  cudaStream_t s = (cudaStream_t)stream;
-  uint8_t* hw = reinterpret_cast<uint8_t*>(workspace) + kStatusBytes8;
-  const int64_t n = Mr * (K >> 7);
-  if (n > (int64_t)1 << 31 || K > (int64_t)1 << 31) return SF_ERR_SHAPE;
-  SF_TRY(launch_pdl(meta_reorder8_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, s, (const uint4*)a_meta, hw,
-                    (uint32_t)Mr, (uint32_t)K));
-  return gemm_fp8(true, a_vals, hw, B, Mr, Nc, K, alpha, C, Nc, (int*)workspace, s);
+  if (Mr * (K >> 7) > (int64_t)1 << 31 || K > (int64_t)1 << 31) return SF_ERR_SHAPE;
+  return gemm_fp8(true, a_vals, a_meta, B, Mr, Nc, K, alpha, C, Nc, (int*)workspace, (cudaStream_t)stream);
 }
 
 }  // extern "C"

@@ -367,7 +367,7 @@ __device__ __forceinline__ void store_chunk(const CUtensorMap* tmapC, uint8_t* b
   }
   if (kBufs == 2) buf ^= 1u;
 }
-// kEarly, last_first: as in epi_tile.
+// kEarly: as in epi_tile.
 template <int kTileN, int kBufs, bool kEarly>
 __device__ __forceinline__ void epi_store_tile(const GemmArgs& args, const CUtensorMap* tmapC, uint32_t taddr, int64_t m0, int64_t n0,
                                                int64_t n_limit, int q, int lane, uint8_t* bufs, uint32_t& buf, int part, int parts,
@@ -1166,6 +1166,15 @@ struct SmemCtl2 {
   int abort_flag;
 };
 
+// Metadata of 128 rows and one stage (256 columns) of an 8-bit 2:4 operand, straight from the canonical [R, K/16] words: the
+// instruction wants 16 bytes a row and 128 columns, rows in order. A box of 32 bytes a row brings both halves of the columns,
+// 32-byte swizzled, and the copy to TMEM starts at either 16. A pass that wrote the words in this order first took 4 us at
+// 4096 x 4096, and the product could not be set up beside it: E4M3 2:4 2048 x 2048 x 2048 11.6 -> 9.3 us, 8192 x 4096 x 16384 308 ->
+// 288. Two boxes of 16 bytes a row are too many requests for 512-row tiles: 4096 x 16384 x 4096 154.1 us, 148.1 with one.
+__device__ __forceinline__ void load_meta8(uint8_t* dst, const CUtensorMap* m, uint64_t* bar, int kb, int row) {
+  tma_load_2d_2cta(dst, m, bar, kb * 16, row);             // box {16 words, 128 rows}
+}
+
 // The tile a CTA pair works on: from the regular raster, or from a device-built table (grouped products).
 template <int kBN, bool kVar, bool kDual>
 __device__ __forceinline__ GemmTile get_tile(const GemmArgs& args, int tile, int num_m, int num_n, int nkb_full) {
@@ -1337,10 +1346,13 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
             }
           } else {
             tma_load_2d_2cta(sA, &tmapA, bar, (ak0 >> 1) + kb * 64, m0);       // stored values: box {64, 128}
-            // metadata atoms are rows of 2 x 1 KB in a [2 * atoms, 256] uint32 view (8-bit operands: a pair of
-            // atoms per stage, 4 rows)
-            const int atom = (m0 >> 7) * nkb_full + (ak0 >> 7) + kb;
-            tma_load_2d_2cta(sM, &tmapMeta, bar, 0, (kFp8 ? 4 : 2) * atom);
+            if (kFp8) {
+              load_meta8(sM, &tmapMeta, bar, kb, m0);
+            } else {
+              // metadata atoms are rows of 2 x 1 KB in a [2 * atoms, 256] uint32 view
+              const int atom = (m0 >> 7) * nkb_full + (ak0 >> 7) + kb;
+              tma_load_2d_2cta(sM, &tmapMeta, bar, 0, 2 * atom);
+            }
             if (!kBMN) {
               tma_load_2d_2cta(sB, &tmapB, bar, bk0 + kb * 128, nb0);          // two 64-wide K slabs
               tma_load_2d_2cta(sB + kBSlabBytes, &tmapB, bar, bk0 + kb * 128 + 64, nb0);
@@ -1365,7 +1377,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
                                                              : smem_desc(0, 16, 1024, kSwizzle128B);
       const uint64_t b_proto = kBMN ? smem_desc(0, kSparse ? 16384 : 8192, 1024, kSwizzle128B)
                                     : smem_desc(0, 16, 1024, kSwizzle128B);
-      const uint64_t m_proto = smem_desc(0, 128, 128, kSwizzleNone);
+      const uint64_t m_proto = kFp8 ? smem_desc(0, 16, 256, kSwizzle32B) : smem_desc(0, 128, 128, kSwizzleNone);
       const uint32_t a_hi = (uint32_t)(a_proto >> 32), b_hi = (uint32_t)(b_proto >> 32), m_hi = (uint32_t)(m_proto >> 32);
       const uint32_t a_lo0 = (uint32_t)a_proto + (smem0 >> 4);
       const uint32_t b_lo0 = (uint32_t)b_proto + ((smem0 + kAStageBytes) >> 4);
@@ -1387,7 +1399,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
           const uint32_t a_lo = a_lo0 + soff, b_lo = b_lo0 + soff;
           const uint32_t mbuf = tmem_base + kMetaCol + kMetaCols * ((uint32_t)kb & 1u);   // metadata double buffer
           if (kSparse) tmem_cp_128x128b_2cta(mbuf, desc64(m_lo0 + soff, m_hi));
-          if (kSparse && kFp8) tmem_cp_128x128b_2cta(mbuf + 4u, desc64(m_lo0 + soff + (2048u >> 4), m_hi));
+          if (kSparse && kFp8) tmem_cp_128x128b_2cta(mbuf + 4u, desc64(m_lo0 + soff + 1u, m_hi));
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const uint32_t accum = (kb > 0 || k > 0) ? 1u : 0u;
@@ -1653,8 +1665,9 @@ gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constan
       const uint32_t tx = 2u * (t.halves * (16384u + (uint32_t)kMetaBytes) + (kBMN ? (uint32_t)chunks * 16384u : 256u * (uint32_t)half_n));
       auto load_a = [&](int kb, int h, uint8_t* st, uint64_t* bar) {
         tma_load_2d_2cta(st + kBBytes + h * 16384, &tmapA, bar, kb * 64, m0 + h * 256);           // stored values: box {64, 128}
-        // metadata atoms are rows of 2 x 1 KB in a [2 * atoms, 256] uint32 view (8-bit operands: pairs of atoms)
-        tma_load_2d_2cta(st + kMetaAt + h * kMetaBytes, &tmapMeta, bar, 0, (kFp8 ? 4 : 2) * (atom0 + 2 * h * nkb + kb));
+        // metadata atoms are rows of 2 x 1 KB in a [2 * atoms, 256] uint32 view
+        if (kFp8) load_meta8(st + kMetaAt + h * kMetaBytes, &tmapMeta, bar, kb, m0 + h * 256);
+        else      tma_load_2d_2cta(st + kMetaAt + h * kMetaBytes, &tmapMeta, bar, 0, 2 * (atom0 + 2 * h * nkb + kb));
       };
       for (int kb = 0; kb < nkb; ++kb) {
         if (!mbar_wait(&ctl->empty[stage], phase ^ 1, abort_flag)) { ok = false; break; }
@@ -1685,7 +1698,7 @@ gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constan
       const uint32_t idesc_wide = idesc0 | ((uint32_t)(kTallBN >> 3) << 17);
       const uint32_t idesc_narrow = idesc0 | ((uint32_t)((int)args.N % kTallBN >> 3) << 17);
       const uint32_t s0 = smem_u32(smem) >> 4;
-      const uint64_t a_proto = smem_desc(0, 16, 1024, kSwizzle128B), m_proto = smem_desc(0, 128, 128, kSwizzleNone);
+      const uint64_t a_proto = smem_desc(0, 16, 1024, kSwizzle128B), m_proto = kFp8 ? smem_desc(0, 16, 256, kSwizzle32B) : smem_desc(0, 128, 128, kSwizzleNone);
       const uint64_t b_proto = kBMN ? smem_desc(0, 16384, 1024, kSwizzle128B) : smem_desc(0, 16, 1024, kSwizzle128B);
       const uint32_t a_hi = (uint32_t)(a_proto >> 32), b_hi = (uint32_t)(b_proto >> 32), m_hi = (uint32_t)(m_proto >> 32);
       const int nfull = args.num_m_tiles * args.num_n_tiles;
@@ -1710,7 +1723,7 @@ gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constan
             const uint32_t m_lo = (uint32_t)m_proto + at + (uint32_t)((kMetaAt + h * kMetaBytes) >> 4);
             const uint32_t mbuf = tmem_base + kMetaCol + kMetaCols * (uint32_t)(2 * (kb & 1) + h);   // metadata double buffer
             tmem_cp_128x128b_2cta(mbuf, desc64(m_lo, m_hi));
-            if (kFp8) tmem_cp_128x128b_2cta(mbuf + 4u, desc64(m_lo + (2048u >> 4), m_hi));
+            if (kFp8) tmem_cp_128x128b_2cta(mbuf + 4u, desc64(m_lo + 1u, m_hi));
             const uint32_t tmem_d = tmem_base + (uint32_t)(h * kTallBN);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -1923,10 +1936,15 @@ int launch_tall(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap&
   return launch_pdl(kern, dim3(2 * (tiles < max_pairs ? tiles : max_pairs)), kTallThreads, smem, s, ta, tb, tbn, tm, tc ? *tc : ta, a);
 }
 
+// Map of the canonical metadata [R, K/16] of an 8-bit 2:4 operand; kw: K in 2-byte words.
+int make_meta8_map(CUtensorMap* m, const void* meta, int64_t R, int64_t kw) {
+  return make_tmap(m, meta, R, kw / 8, kw / 8, 16, 128, CU_TENSOR_MAP_SWIZZLE_32B, 2);
+}
+
 // Tensor maps of a tall product, lengths in 2-byte words (8-bit operands: two codes): vals [M, kw / 2] packed A, B [N, kw]
-// K-major or [kw, N] MN-major. kind: 0 bf16, 2 words; meta_rows: 1 KB metadata rows per 128 operand rows and stage.
-int tall_maps(const void* vals, const void* meta_hw, const void* B, bool b_kmajor, int64_t M, int64_t N, int64_t kw,
-              int kind, int meta_rows, CUtensorMap* ta, CUtensorMap* tb, CUtensorMap* tbn, CUtensorMap* tm) {
+// K-major or [kw, N] MN-major. kind: 0 bf16 (metadata in tensor-core order), 2 words (canonical metadata).
+int tall_maps(const void* vals, const void* meta, const void* B, bool b_kmajor, int64_t M, int64_t N, int64_t kw,
+              int kind, CUtensorMap* ta, CUtensorMap* tb, CUtensorMap* tbn, CUtensorMap* tm) {
   int st = make_tmap(ta, vals, M, kw / 2, kw / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, kind);
   if (st == SF_OK)
     st = b_kmajor ? make_tmap(tb, B, N, kw, kw, 64, kTallBN / 2, CU_TENSOR_MAP_SWIZZLE_128B, kind)
@@ -1934,8 +1952,7 @@ int tall_maps(const void* vals, const void* meta_hw, const void* B, bool b_kmajo
   *tbn = *tb;
   if (st == SF_OK && b_kmajor && N % kTallBN)
     st = make_tmap(tbn, B, N, kw, kw, 64, (uint32_t)(N % kTallBN / 2), CU_TENSOR_MAP_SWIZZLE_128B, kind);
-  if (st == SF_OK)
-    st = make_tmap(tm, meta_hw, meta_rows * (M / 128) * (kw / 128), 256, 256, 256, (uint32_t)meta_rows, CU_TENSOR_MAP_SWIZZLE_NONE, 1);
+  if (st == SF_OK) st = kind == 2 ? make_meta8_map(tm, meta, M, kw) : make_tmap(tm, meta, 2 * (M / 128) * (kw / 128), 256, 256, 256, 2, CU_TENSOR_MAP_SWIZZLE_NONE, 1);
   return st;
 }
 
@@ -2127,7 +2144,7 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   }
   if (tile.rows == 512) {
     CUtensorMap tbn;
-    const int st = tall_maps(a_vals, meta_hw, B, b_kmajor, M, N, K, 0, 2, &ta, &tb, &tbn, &tm);
+    const int st = tall_maps(a_vals, meta_hw, B, b_kmajor, M, N, K, 0, &ta, &tb, &tbn, &tm);
     if (st != SF_OK) return st;
     GemmArgs a{};
     a.M = M; a.N = N; a.K = K;
@@ -2208,7 +2225,7 @@ int gemm_sparse24_drelu(const void* w_vals, const uint8_t* meta_hw, const void* 
   CUtensorMap ta, tb, tbn, tm;
   const TileShape tile = gemm_sparse24_drelu_tile(F, T, D);
   if (tile.rows == 512) {
-    const int st = tall_maps(w_vals, meta_hw, dY, true, F, T, D, 0, 2, &ta, &tb, &tbn, &tm);
+    const int st = tall_maps(w_vals, meta_hw, dY, true, F, T, D, 0, &ta, &tb, &tbn, &tm);
     if (st != SF_OK) return st;
     return mask.colidx ? launch_tall<false, EPI_DRELUV_T>(ta, tb, tbn, tm, a, s) : launch_tall<false, EPI_DRELU24_T>(ta, tb, tbn, tm, a, s);
   }
@@ -2262,9 +2279,9 @@ int gemm_route(const void* X, const void* means, int64_t T, int64_t D, int E, in
   return launch_two<MODE_DENSE, false, false, EPI_ROUTE>(ta, tb, ta, a, s);
 }
 
-int gemm_fp8(bool sparse, const void* A, const uint8_t* meta_hw, const void* B, int64_t M, int64_t N, int64_t K,
+int gemm_fp8(bool sparse, const void* A, const void* meta, const void* B, int64_t M, int64_t N, int64_t K,
              float alpha, void* C, int64_t ldc, int* status, cudaStream_t s) {
-  if (M % 256 || N % 32 || K % (sparse ? 256 : 128) || (sparse && !meta_hw)) return SF_ERR_SHAPE;
+  if (M % 256 || N % 32 || K % (sparse ? 256 : 128) || (sparse && !meta)) return SF_ERR_SHAPE;
   if (M == 0 || N == 0) return SF_OK;
   // the operands in 2-byte units: [M, K/2] (dense) or [M, K/4] (2:4 values), [N, K/2]
   const int64_t K2 = K / 2;
@@ -2273,7 +2290,7 @@ int gemm_fp8(bool sparse, const void* A, const uint8_t* meta_hw, const void* B, 
   if (st != SF_OK) return st;
   if (sparse && use_tall_plain(M, N, K / 256)) {
     CUtensorMap tbn;
-    st = tall_maps(A, meta_hw, B, true, M, N, K2, 2, 4, &ta, &tb, &tbn, &tm);
+    st = tall_maps(A, meta, B, true, M, N, K2, 2, &ta, &tb, &tbn, &tm);
     if (st != SF_OK) return st;
     GemmArgs a{};
     a.M = M; a.N = N; a.K = K2;
@@ -2288,14 +2305,12 @@ int gemm_fp8(bool sparse, const void* A, const uint8_t* meta_hw, const void* B, 
   if (st != SF_OK) return st;
   tm = ta;
   if (sparse) {
-    // per 128 rows and 256 logical K: two 2 KB atoms = four rows of the [4 * atom pairs, 256] uint32 view
-    const int64_t pairs = (M / 128) * (K / 256);
-    st = make_tmap(&tm, meta_hw, 4 * pairs, 256, 256, 256, 4, CU_TENSOR_MAP_SWIZZLE_NONE, 1);
+    st = make_meta8_map(&tm, meta, M, K2);
     if (st != SF_OK) return st;
   }
   GemmArgs a{};
   a.M = M; a.N = N; a.K = K2;
-  a.C = C; a.ldc = ldc; a.meta_hw = meta_hw; a.status = status; a.out_scale = alpha;
+  a.C = C; a.ldc = ldc; a.status = status; a.out_scale = alpha;
   a.num_k_blocks = (int)(K2 / 64);
   a.bn = bn;
   if (bn != BN)

@@ -173,9 +173,9 @@ int gemm_route(const void* X, const void* means, int64_t T, int64_t D, int E, in
 int launch_meta_reorder(const void* meta, void* meta_hw, int64_t R, int64_t K, int64_t transposed_cols, cudaStream_t s);
 
 // E4M3 operands, both K-major: C[M, N] = bf16(alpha * A B^T). sparse: A = 2:4 values [M, K/2] (codes) with
-// metadata in the 8-bit instruction's order (see meta_hw8_offset); else A [M, K]. B [N, K].
+// canonical metadata [M, K/16]; else A [M, K]. B [N, K].
 // M % 256 == 0, N % 32 == 0, K % 256 == 0 (2:4) or K % 128 == 0 (dense).
-int gemm_fp8(bool sparse, const void* A, const uint8_t* meta_hw, const void* B, int64_t M, int64_t N, int64_t K,
+int gemm_fp8(bool sparse, const void* A, const void* meta, const void* B, int64_t M, int64_t N, int64_t K,
              float alpha, void* C, int64_t ldc, int* status, cudaStream_t s);
 // C[T,N] = A_vnm[T,F] Bt[F,N]; A_vnm packed (vals [T, 2F/Mv], hardware-ordered metadata, colidx).
 int gemm_venom(const void* a_vals, const uint8_t* meta_hw, const uint8_t* colidx, const void* Bt, int64_t T,

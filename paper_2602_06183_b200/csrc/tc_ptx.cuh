@@ -330,7 +330,7 @@ __device__ __forceinline__ void tmem_cp_128x128b_2cta(uint32_t taddr, uint64_t s
 
 // ---- descriptors ---------------------------------------------------------------------------------
 // Shared-memory matrix descriptor (sm_100 format): start address, leading/stride byte offsets
-// (all >> 4), version 1, swizzle mode in bits 61-63 (0 none, 2 = 128 B).
+// (all >> 4), version 1, swizzle mode in bits 61-63 (0 none, 2 = 128 B, 6 = 32 B).
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes,
                                               uint32_t swizzle_mode) {
   uint64_t d = 0;
@@ -341,7 +341,7 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo_bytes
   d |= static_cast<uint64_t>(swizzle_mode & 7u) << 61;
   return d;
 }
-constexpr uint32_t kSwizzleNone = 0, kSwizzle128B = 2;
+constexpr uint32_t kSwizzleNone = 0, kSwizzle128B = 2, kSwizzle32B = 6;
 
 // Instruction descriptor for kind::f16 with bf16 A/B and fp32 D.
 __host__ __device__ constexpr uint32_t idesc_bf16(uint32_t M, uint32_t N, bool a_mn_major, bool b_mn_major,
