@@ -137,6 +137,35 @@ __device__ __forceinline__ void quad_transpose(uint32_t (&x)[16], int lane) {
     }
 }
 
+// ---- stores through TMA -----------------------------------------------------------------------------
+// What bounded the plain store: an epilogue thread holds a row, so a 16-byte store of a warp went to 32 rows, 32 cycles of the
+// load/store unit each (7000 clocks for the 256 x 224 outputs of an SM in a 512-row tile), on the chain from one main loop to the
+// next and in the way of the MMAs' shared-memory reads. Here a warp puts 32 x 32 results into shared memory, 64 bytes a row, and one
+// thread hands them to TMA. Same box, call after call: 2:4 row-major 8192 x 16384, K = 128 115 -> 67 us, K = 1024 215 -> 167,
+// K = 4096 535 -> 503; E4M3 2:4 4096 x 16384 x 4096 170 -> 150; dense 8192 x 16384, K = 128 119 -> 79, 16384 x 8192, K = 512 168 -> 131.
+// Four lanes exchanging their rows' units and storing 64 bytes of eight rows per instruction gave E4M3 152 and dense K = 512 168;
+// reading a 512-row tile out into registers first and handing its accumulator back before storing (the stores then run beside
+// the next main loop, which they slow) 151; an evict-first hint nothing.
+// 32 x 32 chunk of a tile, rounded (w: this lane's row), through one of the warp's buffers to C; rows of 64 bytes, swizzled as
+// the store's tensor map expects it (64-byte swizzle), so that a thread per row writes without bank conflicts.
+template <int kBufs>
+__device__ __forceinline__ void store_chunk(const CUtensorMap* tmapC, uint8_t* bufs, uint32_t& buf, const uint32_t* w, int col, int row,
+                                            int lane) {
+  if (lane == 0) bulk_wait_read<kBufs - 1>();                              // the chunk before (or the one before that) has left
+  __syncwarp();
+  uint8_t* b = bufs + buf * kEpiWarpBytes;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    *reinterpret_cast<uint4*>(b + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+  fence_proxy_async_smem();
+  __syncwarp();
+  if (lane == 0) {
+    tma_store_2d(tmapC, b, col, row);
+    bulk_commit();
+  }
+  if (kBufs == 2) buf ^= 1u;
+}
+
 // ---- epilogue (shared by the one-CTA and the two-CTA kernels) ---------------------------------------
 // One epilogue warp owns TMEM lanes [32q, 32q+32) of a 128 x 256 accumulator tile whose first row is
 // m0 and first column n0; `taddr` is the TMEM address of (lane 32q, column 0) of that accumulator.
@@ -151,11 +180,12 @@ __device__ __forceinline__ void quad_transpose(uint32_t (&x)[16], int lane) {
 // eight rows per instruction: y1 + SquaredReLU at T 4096, D 2048, F 8192 129 -> 96 us.
 // kEarly: the accumulator is handed back when the first chunk has been read; the second part starts with its last chunk, so that
 // the columns at either end of the tile are the first to be read.
-// kPairs: the transposed store goes through shared memory as words of two tokens (see there).
-template <int kEpi, int kTileN = BN, bool kEarly = false, bool kPairs = false, bool kQuad = false>
+// kTma: the two-operand epilogues hand their chunks to TMA (T 10496, D 384, F 7424, the dense step 504 -> 488 us).
+template <int kEpi, int kTileN = BN, bool kEarly = false, bool kQuad = false, bool kTma = false>
 __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit,
                                          int q, int lane, uint8_t* my_stage, int part = 0, int parts = 1, bool second = false,
-                                         uint64_t* tmem_empty_bar = nullptr) {
+                                         uint64_t* tmem_empty_bar = nullptr, const CUtensorMap* tmapC = nullptr,
+                                         const CUtensorMap* tmapC2 = nullptr, uint32_t* buf = nullptr) {
   if constexpr (kEpi == EPI_ROUTE) {
     const int64_t row = m0 + q * 32 + lane;                                // this thread's D row
     // the row is a token, the first route_E columns its logits
@@ -277,44 +307,29 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
         for (int j = 0; j < 4; ++j) c[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
       }
     } else if (kEpi != EPI_STORE_T) {
-      store_rows(w, args.C, args.ldc, col0);
+      // kTma: EPI_SQRELU has both buffers for its outputs, EPI_DRELU stages y1 in the first
+      if constexpr (kTma && kEpi == EPI_SQRELU) store_chunk<2>(tmapC, my_stage, *buf, w, (int)col0, (int)m0 + q * 32, lane);
+      else if constexpr (kTma) store_chunk<1>(tmapC, my_stage + kEpiWarpBytes, *buf, w, (int)col0, (int)m0 + q * 32, lane);
+      else store_rows(w, args.C, args.ldc, col0);
       if (kEpi == EPI_SQRELU) {
 #pragma unroll
         for (int j = 0; j < 16; ++j) w[j] = bf2_sq(bf2_relu(w[j]));
-        store_rows(w, args.C2, args.ldc2, col0);
+        if constexpr (kTma) store_chunk<2>(tmapC2, my_stage, *buf, w, (int)col0, (int)m0 + q * 32, lane);
+        else store_rows(w, args.C2, args.ldc2, col0);
       }
     } else {
-      // Transposed output: D row = feature (lane), D column = token. C is [N, M] row-major. Through shared memory token by token
-      // (32 16-bit stores, four 16-byte loads), or as words of two neighbouring tokens: half the stores, but the rows have to be
-      // taken apart on the chain from a load to the global store. A warp walks its chunks one after another, so where the
-      // epilogue is the tile's time (256-row tiles with a short reduction) the first is the faster one: 8192 x 16384,
-      // K = 128 71.7 us and 96.5, 28672 x 2048, K = 128 37.7 and 47.0, 4096 x 4096, K = 1024 24.0 and 24.8. (The order of the global
-      // stores is the smaller part: the pairs' order, every second one of 16 tokens, 76.7; pairs read so that eight consecutive
-      // tokens leave at once, 98.4.) 512-row tiles, whose long main loop shares the shared memory with it, take the second
-      // (kPairs): 4096 x 16384, K = 2048 140.5 us and 144.6, K = 4096 245.2 and 249.0, 8192 x 16384, K = 2048 282 and 287.
+      // Transposed output: D row = feature (lane), D column = token. C is [N, M] row-major; through shared memory token by token
+      // (32 16-bit stores, four 16-byte loads). With a short reduction a warp's walk from chunk to chunk is the tile's time, and this is
+      // the shortest: 8192 x 16384, K = 128 74.6 us, by fragments and TMA (epi_store_t_tile) 108, by words of two tokens that are
+      // taken apart again 96.5; 28672 x 2048, K = 128 38.1, 51.8 and 47.0; 4096 x 4096, K = 1024 24.9, 24.8 and 24.8.
       __syncwarp();
-      if constexpr (kPairs) {
-        uint32_t* st = reinterpret_cast<uint32_t*>(my_stage);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) st[j * 32 + lane] = w[j];
-        __syncwarp();
+      for (int t = 0; t < 32; ++t)
+        reinterpret_cast<uint16_t*>(unit(t, lane >> 3))[lane & 7] = (uint16_t)(w[t >> 1] >> (16 * (t & 1)));
+      __syncwarp();
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          uint32_t r0[4], r1[4];
-          pair_rows(st + (i * 8 + t8) * 32 + u * 8, lane, r0, r1);
-          uint16_t* c = reinterpret_cast<uint16_t*>(args.C) + (col0 + i * 16 + t8 * 2) * args.ldc + m0 + q * 32 + u * 8;
-          *reinterpret_cast<uint4*>(c) = make_uint4(r0[0], r0[1], r0[2], r0[3]);
-          *reinterpret_cast<uint4*>(c + args.ldc) = make_uint4(r1[0], r1[1], r1[2], r1[3]);
-        }
-      } else {
-#pragma unroll
-        for (int t = 0; t < 32; ++t)
-          reinterpret_cast<uint16_t*>(unit(t, lane >> 3))[lane & 7] = (uint16_t)(w[t >> 1] >> (16 * (t & 1)));
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(args.C) + (col0 + i * 8 + t8) * args.ldc + m0 + q * 32 + u * 8) = *unit(t8 + 8 * i, u);
-      }
+      for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(args.C) + (col0 + i * 8 + t8) * args.ldc + m0 + q * 32 + u * 8) = *unit(t8 + 8 * i, u);
     }
   };
   // two register buffers: the TMEM load of the next 32 columns is in flight while this chunk is converted
@@ -339,34 +354,7 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
 }
 
 
-// ---- the plain store through TMA -----------------------------------------------------------------------
-// What bounded the plain store: an epilogue thread holds a row, so a 16-byte store of a warp went to 32 rows, 32 cycles of the
-// load/store unit each (7000 clocks for the 256 x 224 outputs of an SM in a 512-row tile), on the chain from one main loop to the
-// next and in the way of the MMAs' shared-memory reads. Here a warp puts 32 x 32 results into shared memory, 64 bytes a row, and one
-// thread hands them to TMA. Same box, call after call: 2:4 row-major 8192 x 16384, K = 128 115 -> 67 us, K = 1024 215 -> 167,
-// K = 4096 535 -> 503; E4M3 2:4 4096 x 16384 x 4096 170 -> 150; dense 8192 x 16384, K = 128 119 -> 79, 16384 x 8192, K = 512 168 -> 131.
-// Four lanes exchanging their rows' units and storing 64 bytes of eight rows per instruction gave E4M3 152 and dense K = 512 168;
-// reading a 512-row tile out into registers first and handing its accumulator back before storing (the stores then run beside
-// the next main loop, which they slow) 151; an evict-first hint nothing.
-// 32 x 32 chunk of a tile, rounded (w: this lane's row), through one of the warp's buffers to C; rows of 64 bytes, swizzled as
-// the store's tensor map expects it (64-byte swizzle), so that a thread per row writes without bank conflicts.
-template <int kBufs>
-__device__ __forceinline__ void store_chunk(const CUtensorMap* tmapC, uint8_t* bufs, uint32_t& buf, const uint32_t* w, int col, int row,
-                                            int lane) {
-  if (lane == 0) bulk_wait_read<kBufs - 1>();                              // the chunk before (or the one before that) has left
-  __syncwarp();
-  uint8_t* b = bufs + buf * kEpiWarpBytes;
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    *reinterpret_cast<uint4*>(b + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
-  fence_proxy_async_smem();
-  __syncwarp();
-  if (lane == 0) {
-    tma_store_2d(tmapC, b, col, row);
-    bulk_commit();
-  }
-  if (kBufs == 2) buf ^= 1u;
-}
+// ---- plain and transposed stores of a whole tile -------------------------------------------------------
 // kEarly: as in epi_tile.
 template <int kTileN, int kBufs, bool kEarly>
 __device__ __forceinline__ void epi_store_tile(const GemmArgs& args, const CUtensorMap* tmapC, uint32_t taddr, int64_t m0, int64_t n0,
@@ -397,6 +385,52 @@ __device__ __forceinline__ void epi_store_tile(const GemmArgs& args, const CUten
   for (int i = ch0; i < nch; i += 2) {
     chunk(i, va, vb);
     if (i + 1 < nch) chunk(i + 1, vb, va);
+  }
+}
+
+// The transposed store: D row = feature, D column = token, C is [tokens, features] row-major. The accumulator is read as the 8 x 8
+// fragments that stmatrix transposes on its way to shared memory, [32 tokens][32 features], and leaves through TMA as above: the
+// fewest passes over the shared memory that the main loop works on. For 512-row tiles; against words of two tokens staged by
+// lane and taken apart again 16384 x 8192, K = 4096 502.9 -> 499.2 us, 4096 x 16384, K = 2048 140.4 -> 138.8.
+template <int kTileN, int kBufs>
+__device__ __forceinline__ void epi_store_t_tile(const CUtensorMap* tmapC, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit, int q,
+                                                 int lane, uint8_t* bufs, uint32_t& buf) {
+  const int nch = (int)min((int64_t)(kTileN / 32), (n_limit - n0) >> 5);
+  auto load = [&](int ch, uint32_t (&v)[32]) {
+    tmem_ld_16x256b_x4(taddr + ch * 32, v);
+    tmem_ld_16x256b_x4(taddr + ch * 32 + (16u << 16), v + 16);
+  };
+  // lane 8 k + j addresses eight features (16-byte unit k) of token j of eight: units swizzled as in store_chunk
+  const uint32_t at = smem_u32(bufs) + (lane & 7) * 64 + (((lane >> 3) ^ ((lane >> 1) & 3)) << 4);
+  auto chunk = [&](int ch, uint32_t (&v)[32], uint32_t (&next)[32]) {
+    tmem_ld_wait_on(v);
+    if (ch + 1 < nch) load(ch + 1, next);
+    uint32_t w[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t* x = v + 16 * (k >> 1) + 4 * i + 2 * (k & 1);
+        w[i][k] = pack_bf16x2(__uint_as_float(x[0]), __uint_as_float(x[1]));
+      }
+    if (lane == 0) bulk_wait_read<kBufs - 1>();
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) stmatrix_x4_trans(at + buf * kEpiWarpBytes + i * 512, w[i][0], w[i][1], w[i][2], w[i][3]);
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) {
+      tma_store_2d(tmapC, bufs + buf * kEpiWarpBytes, (int)m0 + q * 32, (int)n0 + ch * 32);
+      bulk_commit();
+    }
+    if (kBufs == 2) buf ^= 1u;
+  };
+  uint32_t va[32], vb[32];
+  load(0, va);
+#pragma unroll 1
+  for (int ch = 0; ch < nch; ch += 2) {
+    chunk(ch, va, vb);
+    if (ch + 1 < nch) chunk(ch + 1, vb, va);
   }
 }
 
@@ -1140,8 +1174,10 @@ __host__ __device__ constexpr int num_stages2(bool sparse, int bn = BN, bool exp
 }
 // Plain stores of full-width tiles go through TMA, two chunk buffers to a warp (2:4 products, whose stages leave less room, one); narrow tiles (run-time width), where the latency
 // of a chunk counts, and the kernels that expand an operand store from registers.
-__host__ __device__ constexpr bool tma_store2(int epi, bool expand, bool var) { return epi == EPI_STORE && !expand && !var; }
-__host__ __device__ constexpr int store_bufs2(bool sparse) { return sparse ? 1 : 2; }
+__host__ __device__ constexpr bool tma_store2(int epi, bool expand, bool var) {
+  return (epi == EPI_STORE || epi == EPI_SQRELU || epi == EPI_DRELU) && !expand && !var;
+}
+__host__ __device__ constexpr int store_bufs2(bool sparse, int epi) { return sparse && epi == EPI_STORE ? 1 : 2; }
 __host__ __device__ constexpr int epi_bytes2(int epi, int bn = BN, int store_bufs = 0) {
   return store_bufs > 0   ? store_bufs * kEpiWarpBytes
          : epi == EPI_VNM8 ? kVnmEpiBytes
@@ -1245,7 +1281,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   uint8_t* pk_stage = smem + kStages * kStageBytes;       // kExpand: ring of packed tiles, one per stage
   uint8_t* epi_stage = pk_stage + (kExpand ? kStages * kPkStageBytes : 0);
   constexpr bool kTmaStore = tma_store2(kEpi, kExpand != 0, kVar);
-  constexpr int kStoreBufs = kTmaStore ? (threads2(kMode, kEpi, kExpand, kVar) / 32 - 2) * store_bufs2(kSparse) : 0;
+  constexpr int kStoreBufs = kTmaStore ? (threads2(kMode, kEpi, kExpand, kVar) / 32 - 2) * store_bufs2(kSparse, kEpi) : 0;
   SmemCtl2* ctl = reinterpret_cast<SmemCtl2*>(epi_stage + epi_bytes2(kEpi, kBN, kStoreBufs));
   volatile int* abort_flag = &ctl->abort_flag;
 
@@ -1508,7 +1544,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
     // =========================== epilogue (warps 2..5 or 2..9, both CTAs) ===========================
     const int q = warp & 3, set = (warp - 2) >> 2;
     constexpr int kParts = split_sets(kMode, kEpi, kExpand, kVar) ? 2 : 1;
-    uint8_t* my_stage = epi_stage + (set * 4 + q) * (kTmaStore ? store_bufs2(kSparse) : 1) * kEpiWarpBytes;
+    uint8_t* my_stage = epi_stage + (set * 4 + q) * (kTmaStore ? store_bufs2(kSparse, kEpi) : 1) * kEpiWarpBytes;
     uint32_t acc = 0, acc_phase = 0, buf = 0;
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
@@ -1520,12 +1556,12 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
       const bool live = args.tile_table != nullptr || m0 < (second ? args.M2 : args.M);
       if (!mbar_wait_warp(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      if (kTmaStore && live && !args.row_map) {
-        epi_store_tile<kBN, store_bufs2(kSparse), kOverlap>(args, second ? &tmapC2 : &tmapC, taddr, m0, n0, n_limit, q, lane, my_stage,
-                                                            buf, set, kParts, &ctl->tmem_empty[0]);
+      if (kEpi == EPI_STORE && kTmaStore && live && !args.row_map) {
+        epi_store_tile<kBN, store_bufs2(kSparse, kEpi), kOverlap>(args, second ? &tmapC2 : &tmapC, taddr, m0, n0, n_limit, q, lane,
+                                                                  my_stage, buf, set, kParts, &ctl->tmem_empty[0]);
       } else if (live) {
-        epi_tile<kEpi, kBN, kOverlap, false, kTmaStore>(args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts, second,
-                                                        &ctl->tmem_empty[0]);
+        epi_tile<kEpi, kBN, kOverlap, kEpi == EPI_STORE && kTmaStore, kTmaStore>(
+            args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts, second, &ctl->tmem_empty[0], &tmapC, &tmapC2, &buf);
       }
       if (!kOverlap || !live) release_accumulator(lane, &ctl->tmem_empty[acc]);
       if (++acc == (uint32_t)kAccBufs) { acc = 0; acc_phase ^= 1; }
@@ -1769,16 +1805,16 @@ gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constan
       } else {
         if (!mbar_wait_warp(&ctl->tmem_full[h], phase, abort_flag)) break;
         tc_fence_after();
-        if (kEpi == EPI_STORE && live) {
-          epi_store_tile<kTallBN, 1, false>(args, &tmapC, taddr, m0, n0, n_limit, q, lane, wsm, buf, 0, 1, nullptr);
+        if (kEpi == EPI_STORE_T && live) {
+          epi_store_t_tile<kTallBN, 1>(&tmapC, taddr, m0, n0, n_limit, q, lane, wsm, buf);
         } else if (live) {
-          epi_tile<kEpi, kTallBN, false, true>(args, taddr, m0, n0, n_limit, q, lane, wsm);
+          epi_store_tile<kTallBN, 1, false>(args, &tmapC, taddr, m0, n0, n_limit, q, lane, wsm, buf, 0, 1, nullptr);
         }
         release_accumulator(lane, &ctl->tmem_empty[h]);
       }
       phase ^= 1;
     }
-    if (kEpi == EPI_STORE && lane == 0) bulk_wait_all();
+    if (!is_drelu_t(kEpi) && lane == 0) bulk_wait_all();
   }
 
   // =========================== teardown ===========================
@@ -1876,7 +1912,7 @@ int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
   auto kern = gemm_tc2_kernel<kMode, kAMN, kBMN, kEpi, kBN, kExpand, kFp8, kVar, kDual>;
   constexpr int threads = threads2(kMode, kEpi, kExpand, kVar);
   constexpr bool tma_store = tma_store2(kEpi, kExpand != 0, kVar);
-  constexpr int smem = smem_bytes2(kMode != MODE_DENSE, kBN, kEpi, kExpand != 0, kFp8, tma_store ? (threads / 32 - 2) * store_bufs2(kMode != MODE_DENSE) : 0);
+  constexpr int smem = smem_bytes2(kMode != MODE_DENSE, kBN, kEpi, kExpand != 0, kFp8, tma_store ? (threads / 32 - 2) * store_bufs2(kMode != MODE_DENSE, kEpi) : 0);
   static_assert(smem <= 232448 && smem >= kExclusiveSmem, "shared memory per CTA: fits, and one CTA per SM");
   static bool attr_done[64] = {false};
   int dev = 0;
@@ -1893,7 +1929,7 @@ int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
                                  : a.num_m_tiles * a.num_n_tiles + (kDual ? a.num_m_tiles2 * a.num_n_tiles2 : 0);
   const int max_pairs = sm_count() / 2;
   const int pairs = tiles < max_pairs ? tiles : max_pairs;
-  if (tma_store && !a.row_map && (!tc || (kDual && !tc2))) return SF_ERR_UNSUPPORTED;
+  if (tma_store && !a.row_map && (!tc || ((kDual || kEpi == EPI_SQRELU) && !tc2))) return SF_ERR_UNSUPPORTED;
   return launch_pdl(kern, dim3(2 * pairs), threads, smem, s, ta, tb, tm, tpk ? *tpk : ta, tc ? *tc : ta, tc2 ? *tc2 : ta, a);
 }
 
@@ -1919,7 +1955,7 @@ constexpr int kNarrowBN = SF_NARROW_BN;
 template <bool kBMN, int kEpi, bool kFp8 = false>
 int launch_tall(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tbn, const CUtensorMap& tm, GemmArgs a,
                 cudaStream_t s, const CUtensorMap* tc = nullptr) {
-  if (kEpi == EPI_STORE && !tc) return SF_ERR_UNSUPPORTED;
+  if (!is_drelu_t(kEpi) && !tc) return SF_ERR_UNSUPPORTED;
   auto kern = gemm_tall_kernel<kBMN, kEpi, kFp8>;
   constexpr int smem = tall_smem(kEpi, kBMN, kFp8);
   static_assert(smem <= 232448 && smem >= kExclusiveSmem, "shared memory per CTA: fits, and one CTA per SM");
@@ -2050,9 +2086,10 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
   if (b_kmajor) st = make_tmap(&tb, B, N, K, K, 64, two ? bn / 2 : 256, CU_TENSOR_MAP_SWIZZLE_128B);
   else          st = make_tmap(&tb, B, K, N, N, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st != SF_OK) return st;
-  const bool tma = two && bn == BN && epi == EPI_STORE;
-  CUtensorMap tc;
+  const bool tma = two && bn == BN;
+  CUtensorMap tc, tc2;
   if (tma && (st = make_store_map(&tc, C, M, N, ldc)) != SF_OK) return st;
+  if (tma && C2 && (st = make_store_map(&tc2, C2, M, N, ldc2)) != SF_OK) return st;
   GemmArgs a{};
   a.M = M; a.N = N; a.K = K;
   a.C = C; a.ldc = ldc; a.C2 = C2; a.ldc2 = ldc2; a.aux = aux; a.ldaux = ldaux;
@@ -2061,7 +2098,7 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
   a.bn = bn;
 #define SF_DENSE_CASE(AMN, BMN, EPI)                                                                \
   return !two       ? launch_one<MODE_DENSE, AMN, BMN, EPI>(ta, tb, a, s)                             \
-         : bn == BN ? launch_two<MODE_DENSE, AMN, BMN, EPI>(ta, tb, ta, a, s, nullptr, tma ? &tc : nullptr) \
+         : bn == BN ? launch_two<MODE_DENSE, AMN, BMN, EPI>(ta, tb, ta, a, s, nullptr, &tc, C2 ? &tc2 : nullptr) \
                     : launch_two<MODE_DENSE, AMN, BMN, EPI, BN, 0, false, true>(ta, tb, ta, a, s)
   const bool amn = !a_kmajor, bmn = !b_kmajor;
   if (epi == EPI_STORE) {
@@ -2138,8 +2175,8 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   if ((plain || !b_kmajor) && !two) return SF_ERR_UNSUPPORTED;
   CUtensorMap ta, tb, tm, tc;
   const TileShape tile = two ? gemm_sparse24_tile(M, N, K, epi) : TileShape{BM, BN};
-  if (plain) {
-    const int st = make_store_map(&tc, C, M, N, ldc);
+  if (plain || tile.rows == 512) {
+    const int st = plain ? make_store_map(&tc, C, M, N, ldc) : make_store_map(&tc, C, N, M, ldc);
     if (st != SF_OK) return st;
   }
   if (tile.rows == 512) {
@@ -2149,7 +2186,7 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
     GemmArgs a{};
     a.M = M; a.N = N; a.K = K;
     a.C = C; a.ldc = ldc; a.status = status;
-    if (!plain) return launch_tall<false, EPI_STORE_T>(ta, tb, tbn, tm, a, s);
+    if (!plain) return launch_tall<false, EPI_STORE_T>(ta, tb, tbn, tm, a, s, &tc);
     return b_kmajor ? launch_tall<false, EPI_STORE>(ta, tb, tbn, tm, a, s, &tc) : launch_tall<true, EPI_STORE>(ta, tb, tbn, tm, a, s, &tc);
   }
   int st = two ? make_tmap(&ta, a_vals, M, K / 2, K / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B)

@@ -222,6 +222,22 @@ __device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&v)
       : "r"(taddr)
       : "memory");
 }
+// Sixteen of this warp's lanes (those of the address and the next fifteen) x 32 columns, laid out as the 8 x 8 fragments of
+// stmatrix: v[4 i], v[4 i + 1] are columns 8 i + 2 (lane % 4) and the next of lane (lane / 4), v[4 i + 2], v[4 i + 3] those of lane (lane / 4 + 8).
+__device__ __forceinline__ void tmem_ld_16x256b_x4(uint32_t taddr, uint32_t* v) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+      : "r"(taddr)
+      : "memory");
+}
+// Four 8 x 8 matrices of 16-bit elements, transposed, to shared memory: lane 8 k + j gives the address of row j of matrix k.
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t saddr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(a), "r"(b), "r"(c), "r"(d)
+               : "memory");
+}
 // Waits for the loads, with the loaded registers as in/out operands so that no use of them can be scheduled before the wait
 // (needed when another load is issued between this load and its wait).
 __device__ __forceinline__ void tmem_ld_wait_on(uint32_t (&v)[32]) {
