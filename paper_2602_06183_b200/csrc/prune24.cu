@@ -5,8 +5,8 @@
 //     metadata word): two 128-bit loads, one 128-bit store of packed values, one 16-bit store;
 //     a warp owns 32 consecutive chunks of a row, so no index is ever divided.
 //   * strided groups (groups along dim 0, output K-major): a CTA stages a [128 x 64] panel in
-//     shared memory, selects per column, and writes the transposed packed panel with 128-bit
-//     stores through a padded staging buffer.
+//     shared memory, selects per column, and writes the transposed packed panel through a staging
+//     buffer: one TMA store.
 #include "sf_common.cuh"
 #include "fp8_fmt.cuh"
 #include "tc_ptx.cuh"
@@ -91,42 +91,49 @@ prune24_rows_kernel(const uint4* __restrict__ W, int64_t rows, int cols, int64_t
 // vals [Rc, Kd/2], meta [Rc, Kd/16]. Panel: 128 reduction rows x 64 columns.
 // Persistent CTAs walk the panels. One TMA load brings the next panel into a two-slot ring
 // (out-of-range rows and columns arrive as zeros), so no thread computes load addresses; selection runs
-// on column pairs; packed values and metadata words of a panel are collected in shared memory and leave as
-// 128-bit stores, the metadata in either order.
+// on column pairs; packed values and metadata words of a panel are collected in shared memory; the values leave
+// through TMA, the metadata as 128-bit stores in either order.
 // What bounds it: no unit is full. Issue (0.64 of the slots), the round trip through shared memory (a panel is written once
-// by TMA, read and written once by the selection, read by the stores; 40 % of the LSU data pipe) and the barriers share it,
+// by TMA, read and written once by the selection, read by the store) and the barriers share it,
 // with HBM at half its rate. Two barriers a panel: the one behind the wait for the load also says that the previous panel
 // is stored. With a third one before the wait, metadata placed by 16-bit stores and columns staged in order, 4096 x 16384
 // took 47.7 us soft / 40.8 hard, 8192 x 28672 hard 167, 2048 x 8192 soft 15.6 (events around each launch, buffers larger than
 // the L2); without them 44.4 / 37.7, 153 and 14.1, and with the stores of whole panels unrolled 42.8 / 36.6, 151 and 13.7
 // (4.9 TB/s at 8192 x 28672). Called back to back on one matrix the last of these takes 4096 x 16384 soft from 45.9 to 44.7.
+// The packed bf16 values of a panel then leave as one TMA store instead of being read back and stored by the threads: 4096 x 16384
+// soft 44.4 -> 42.1 us, other sizes 116.4 -> 108.9, 13.5 -> 13.1, 12.9 -> 12.4 (calls back to back). The stage holds even columns, then odd
+// ones, so that the threads' swizzled 16-byte writes (two columns each) meet no bank twice; the tensor map takes the two apart
+// again. A second stage leaves room for four CTAs an SM instead of five: 42.4, 13.0, 11.8. E4M3 codes keep the threads' stores:
+// their rows need not be multiples of 16 bytes.
 constexpr int kPanelK = 128, kPanelC = 64;
 constexpr int kColsSlots = 2;                       // the next panel loads while this one is worked on
-constexpr int kStageRow = (kPanelK / 2) * 2 + 16;   // packed bytes per column + 16 B pad
-constexpr int kColsTileBytes = kPanelK * kPanelC * 2, kColsStageBytes = kPanelC * kStageRow;
+constexpr int kStageRow = kPanelK / 2 + 16;         // E4M3: packed bytes per column + 16 B pad
+constexpr int kColsTileBytes = kPanelK * kPanelC * 2, kColsStageBytes = kPanelC * kPanelK;
 constexpr int kColsMetaBytes = kPanelC * (kPanelK / 16) * 2;       // metadata words [chunk][column]
-constexpr int kColsSmemBytes = 128 + kColsSlots * kColsTileBytes + kColsStageBytes + kColsMetaBytes + 64;
+constexpr int kColsSmemBytes = 1024 + kColsSlots * kColsTileBytes + kColsStageBytes + kColsMetaBytes + 64;
+static_assert(kPanelC * kStageRow <= kColsStageBytes, "the E4M3 stage is the smaller one");
 constexpr int kColsCtasPerSm = 5;                   // 43 KB each; measured best among 3..5 with two or three slots
 static_assert(kPanelK / 16 == 8 && kPanelC == 64, "index shifts in prune24_cols_kernel assume a 128 x 64 panel");
 
-// Row of the stage buffer that holds a column: even columns first. A warp writes 32 columns of one parity, 144 bytes
-// apart in this order, so its 16-byte stores touch every bank once a quarter warp (288 bytes apart they met two by two).
+// E4M3: row of the stage buffer that holds a column: even columns first. A warp writes 32 columns of one parity, 80 bytes
+// apart in this order, so that its 8-byte stores meet two by two (160 bytes apart, four by four).
 __device__ __forceinline__ int stage_row(int c) { return (c >> 1) + (c & 1) * (kPanelC / 2); }
 
 // kFp8: the kept values leave as E4M3 codes of float(value) * scale (vals = uint8 [Rc, Kd/2]); no masked copy.
 template <bool kSoft, bool kFp8 = false>
 __global__ void __launch_bounds__(256)
-prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64_t Rc,
-                    uint16_t* __restrict__ vals, uint16_t* __restrict__ meta, uint8_t* __restrict__ meta_hw,
+prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, const __grid_constant__ CUtensorMap tmapV, int64_t Kd, int64_t Rc,
+                    uint8_t* __restrict__ vals, uint16_t* __restrict__ meta, uint8_t* __restrict__ meta_hw,
                     uint16_t* __restrict__ dense_out, int panels_x, int num_panels, float scale) {
   using namespace ptx;
   extern __shared__ uint8_t cols_smem_raw[];
-  uint8_t* cols_smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(cols_smem_raw) + 127) & ~uintptr_t(127));
+  uint8_t* cols_smem = cols_smem_raw + align_pad(cols_smem_raw, 1024);
   typedef uint16_t TileRow[kPanelC];
   typedef uint8_t StageRow[kStageRow];
   typedef uint16_t MetaRow[kPanelC];
-  StageRow* stage = reinterpret_cast<StageRow*>(cols_smem + kColsSlots * kColsTileBytes);              // [kPanelC]
-  MetaRow* mstage = reinterpret_cast<MetaRow*>(cols_smem + kColsSlots * kColsTileBytes + kColsStageBytes);   // [kPanelK / 16]
+  uint8_t* vstage = cols_smem + kColsSlots * kColsTileBytes;            // bf16: [parity][column pair][128 B], 128-byte swizzled
+  StageRow* stage = reinterpret_cast<StageRow*>(vstage);                // E4M3: [kPanelC]
+  MetaRow* mstage = reinterpret_cast<MetaRow*>(vstage + kColsStageBytes);               // [kPanelK / 16]
   uint64_t* full = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(mstage) + kColsMetaBytes);    // [kColsSlots]
   int* abort_flag = reinterpret_cast<int*>(full + kColsSlots);
   const int tid = threadIdx.x;
@@ -160,6 +167,7 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64
     // one warp waits for the load (bounded), the block follows through the barrier
     bool ok = true;
     if (tid < 32) ok = mbar_wait(&full[slot], (uint32_t)(it / kColsSlots) & 1u, abort_flag);
+    if (!kFp8 && tid == 0) bulk_wait_read<0>();                         // the stage has left
     if (!ok) drain_after_expiry();      // (here and not behind the loop: there it cost eight registers and 2 % of the time)
     if (__syncthreads_or(!ok)) break;
     // every warp has stored the previous panel: its stage buffers and its slot are free
@@ -212,25 +220,28 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64
           const uint32_t q2 = quant2(packed[e][2], scale), q3 = quant2(packed[e][3], scale);
           *reinterpret_cast<uint2*>(&stage[stage_row(c + e)][ch * 8]) = make_uint2(q0 | (q1 << 16), q2 | (q3 << 16));
         } else {
-          *reinterpret_cast<uint4*>(&stage[stage_row(c + e)][ch * 16]) = make_uint4(packed[e][0], packed[e][1], packed[e][2], packed[e][3]);
+          *reinterpret_cast<uint4*>(vstage + e * (kColsStageBytes / 2) + cp * 128 + ((ch ^ (cp & 7)) << 4)) =
+              make_uint4(packed[e][0], packed[e][1], packed[e][2], packed[e][3]);
         }
       }
       *reinterpret_cast<uint32_t*>(&mstage[ch][c]) = m[0] | (m[1] << 16);
     }
+    if (!kFp8) fence_proxy_async_smem();
     __syncthreads();
 
-    // store packed values: per column kvalid/2 elements = kvalid bytes, 16 B per thread
+    // store packed values: bf16 through TMA (the map ends where the matrix does); E4M3 per column kvalid/2 bytes, 8 B per thread
     const int chunks = kvalid >> 4;
     const bool full_k = chunks == kPanelK / 16;
     auto put = [&](int c, int ch) {
       const int64_t at = (c0 + c) * (Kd >> 1) + (k0 >> 1) + ch * 8;
-      if (kFp8) {
-        *reinterpret_cast<uint2*>(reinterpret_cast<uint8_t*>(vals) + at) = *reinterpret_cast<const uint2*>(&stage[stage_row(c)][ch * 8]);
-      } else {
-        *reinterpret_cast<uint4*>(vals + at) = *reinterpret_cast<const uint4*>(&stage[stage_row(c)][ch * 16]);
-      }
+      *reinterpret_cast<uint2*>(vals + at) = *reinterpret_cast<const uint2*>(&stage[stage_row(c)][ch * 8]);
     };
-    if (full_k) {
+    if (!kFp8) {
+      if (tid == 0) {
+        tma_store_3d(&tmapV, vstage, (int)(k0 >> 1), (int)(c0 >> 1), 0);
+        bulk_commit();
+      }
+    } else if (full_k) {
 #pragma unroll
       for (int j = 0; j < kPanelC / 32; ++j) {
         const int c = (tid >> 3) + 32 * j;
@@ -282,6 +293,7 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, int64_t Kd, int64
       }
     }
   }
+  if (!kFp8 && tid == 0) bulk_wait_all();
 }
 
 // Plain tiled transpose of a bf16 matrix: out[c][r] = in[r][c].
@@ -384,13 +396,14 @@ int launch_prune24(const void* W, int64_t rows, int64_t cols, int64_t ld, int gr
       SF_CUDA_TRY(cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev));
       attr_done[dev] = true;
     }
-    alignas(64) CUtensorMap tm;
+    alignas(64) CUtensorMap tm, tv;
     int st = make_tmap_2d(&tm, W, rows, cols, ld, kPanelC, kPanelK, false);
+    if (st == SF_OK) st = make_tmap_parity(&tv, vals, cols, rows / 2, kPanelK / 2, kPanelC / 2);
     if (st != SF_OK) return st;
     const int resident = sms[dev] * kColsCtasPerSm;
     const unsigned grid = (unsigned)(num_panels < resident ? num_panels : resident);
     return launch_pdl(prune_mode == 0 ? prune24_cols_kernel<false> : prune24_cols_kernel<true>, dim3(grid), 256,
-                      kColsSmemBytes, s, tm, rows, cols, (uint16_t*)vals, (uint16_t*)meta, (uint8_t*)meta_hw,
+                      kColsSmemBytes, s, tm, tv, rows, cols, (uint8_t*)vals, (uint16_t*)meta, (uint8_t*)meta_hw,
                       (uint16_t*)dense_out, (int)px, num_panels, 1.f);
   }
 }
@@ -418,7 +431,7 @@ int launch_prune24_cols_fp8(const void* W, int64_t rows, int64_t cols, int64_t l
   const int resident = sms[dev] * kColsCtasPerSm;
   const unsigned grid = (unsigned)(num_panels < resident ? num_panels : resident);
   return launch_pdl(prune_mode == 0 ? prune24_cols_kernel<false, true> : prune24_cols_kernel<true, true>, dim3(grid), 256,
-                    kColsSmemBytes, s, tm, rows, cols, (uint16_t*)vals, (uint16_t*)meta, (uint8_t*)nullptr,
+                    kColsSmemBytes, s, tm, tm, rows, cols, (uint8_t*)vals, (uint16_t*)meta, (uint8_t*)nullptr,
                     (uint16_t*)nullptr, (int)px, num_panels, scale);
 }
 

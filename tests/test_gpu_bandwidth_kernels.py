@@ -5,7 +5,7 @@ import torch
 
 import oracle
 from paper_2602_06183_b200 import binding, synth
-from util import to_dev, bits
+from util import to_dev, bits, Guarded
 
 pytestmark = pytest.mark.gpu
 
@@ -44,6 +44,21 @@ def test_prune24_cols_several_panels_per_cta(rows, cols, mode, want_dense):
     assert np.array_equal(bits(meta), ref.meta)
     assert np.array_equal(bits(vals), ref.vals)
     assert not want_dense or np.array_equal(bits(dense), ref.dense)
+
+
+# The packed values leave panel by panel through TMA: panels cut by either edge, a last panel of one chunk or one column pair's worth,
+# several turns of a CTA, a strided input. Nothing is written outside the results.
+@pytest.mark.parametrize("rows,cols,pad", [(16, 8, 0), (112, 56, 8), (144, 72, 0), (2064, 8, 0), (16, 8200, 24), (1168, 8264, 0)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_prune24_cols_values_stay_inside_the_result(rows, cols, pad, mode):
+    w = synth.prune_sweep_matrix(rows, cols, seed=2600 + rows + mode, tie_frac=0.1, axis=0)
+    ref = oracle.prune24(w, group_dim=0, mode=mode)
+    W = to_dev(np.concatenate([w, w[:, :pad]], axis=1))[:, :cols]
+    vals, meta = Guarded((cols, rows // 2), torch.bfloat16), Guarded((cols, rows // 16), torch.int16)
+    binding.sf_prune24_compress(W, 0, mode, out=(vals.t, meta.t, None))
+    vals.check("values")
+    meta.check("metadata")
+    assert np.array_equal(bits(meta.t), ref.meta) and np.array_equal(bits(vals.t), ref.vals)
 
 
 def test_prune24_strided_input_and_special_values():
