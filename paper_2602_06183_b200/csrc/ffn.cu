@@ -195,7 +195,7 @@ struct WeightGradShapes {
 };
 
 // dW2 = dY^T h in the layout of W2 ([D, F], or [F, D] = h^T dY with w2_fd) and dW1 = dy1^T X [F, D]: in one launch where
-// that saves rounds of tiles. The host-buffer step keeps them apart: it downloads dW2 while dW1 is computed.
+// that saves rounds of tiles or there are few of them. The host-buffer step keeps them apart: it downloads dW2 while dW1 is computed.
 int weight_grads(const sf_ffn_desc& d, const void* dY, const void* h, const void* dy1, const void* X, void* dW2, void* dW1,
                  int* status, cudaStream_t s) {
   const bool w2_fd = (d.flags & SF_FFN_W2_FD) != 0;

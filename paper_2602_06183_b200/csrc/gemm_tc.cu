@@ -2133,16 +2133,17 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
   return SF_ERR_UNSUPPORTED;
 }
 
-// By rounds of 256-column tiles, whatever width either side then runs, and without the launch that is saved: the shared
-// launch is never the slower one by the estimate where this takes it (165 000 drawn sizes), but it would also pay at sizes that
-// are left apart: whole step at T 1920, D 1408, F 5504 168.8 us apart and 160.6 together, T 512, D 1024, F 4096 77.6 and 72.4,
-// T 256, D 256, F 9728 99.4 and 92.1.
+// By rounds of 256-column tiles, whatever width either side then runs. Never more of them together than apart; where they are as many,
+// the launch that is saved, with its last round and set-up, is what counts, and with many rounds nothing is left of it. Whole
+// steps, apart and together: T 1920, D 1408, F 5504 (4 rounds either way) 181.7 and 178.3 us, drawn sizes of that order 240.4 and
+// 234.6, 121.7 and 116.9, 109.9 and 105.6, 315.5 and 311.6; T 8192, D 4096, F 16384 (28 rounds) the same within the noise, M = 16
+// there 3535 and 3544.
 bool gemm_dual_tn_pays(int64_t M1, int64_t N1, int64_t M2, int64_t N2) {
   if (M1 < 256 || M2 < 256) return false;
   const int64_t P = sm_count() / 2;
   const int64_t t1 = ((M1 + 255) / 256) * ((N1 + 255) / 256), t2 = ((M2 + 255) / 256) * ((N2 + 255) / 256);
   const int64_t apart = (t1 + P - 1) / P + (t2 + P - 1) / P, together = (t1 + t2 + P - 1) / P;
-  return (double)together <= 0.97 * (double)apart;
+  return apart <= 12 || (double)together <= 0.97 * (double)apart;
 }
 
 TileShape gemm_dual_tn_tile(int64_t M1, int64_t N1, int64_t M2, int64_t N2, int64_t K) {
