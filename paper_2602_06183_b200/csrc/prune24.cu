@@ -93,9 +93,8 @@ prune24_rows_kernel(const uint4* __restrict__ W, int64_t rows, int cols, int64_t
 // (out-of-range rows and columns arrive as zeros), so no thread computes load addresses; selection runs
 // on column pairs; packed values and metadata words of a panel are collected in shared memory; the values leave
 // through TMA, the metadata as 128-bit stores in either order.
-// What bounds it: no unit is full. Issue (0.64 of the slots), the round trip through shared memory (a panel is written once
-// by TMA, read and written once by the selection, read by the store) and the barriers share it,
-// with HBM at half its rate. Two barriers a panel: the one behind the wait for the load also says that the previous panel
+// What bounds it: no unit is full. The selection on the integer pipe (0.64 of the busiest pipe's peak, 0.53 of the issue slots) and
+// the barriers share it (math pipe throttle and barrier, 2.4 stalled warps an issue each), the LSU data pipe is at 34 %. Two barriers a panel: the one behind the wait for the load also says that the previous panel
 // is stored. With a third one before the wait, metadata placed by 16-bit stores and columns staged in order, 4096 x 16384
 // took 47.7 us soft / 40.8 hard, 8192 x 28672 hard 167, 2048 x 8192 soft 15.6 (events around each launch, buffers larger than
 // the L2); without them 44.4 / 37.7, 153 and 14.1, and with the stores of whole panels unrolled 42.8 / 36.6, 151 and 13.7
