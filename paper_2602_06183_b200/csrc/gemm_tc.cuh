@@ -185,8 +185,5 @@ int gemm_venom(const void* a_vals, const uint8_t* meta_hw, const uint8_t* colidx
 // elements with leading dimension ld; box = {box_cols, box_rows}.
 int make_tmap_2d(void* map, const void* base, int64_t rows, int64_t cols, int64_t ld, uint32_t box_cols,
                  uint32_t box_rows, bool swizzle128);
-// The same matrix (contiguous rows, an even number of them) with its even and odd rows apart, [2][rows / 2][cols]: box
-// {box_cols, box_pairs, 2}, 128-byte swizzled.
-int make_tmap_parity(void* map, const void* base, int64_t rows, int64_t cols, uint32_t box_cols, uint32_t box_pairs);
 
 }  // namespace sf
