@@ -437,7 +437,7 @@ SF_API int sf_selftest_wait_expiry(void* workspace, int64_t budget_clocks, void*
  *               with the selection fused into the y1 product: no V:N:M kernel)
  *   sparse bwd: 7 events (prune W2 | dy1 product | pack | dX product | dW2 product | dW1 product);
  *               dy1 leaves its product packed, so the pack interval is empty; where the two weight gradients
- *               share one launch (on small and middle sizes), the dW2 interval
+ *               share one launch (weight_grad_launches of sf_ffn_step_plan), the dW2 interval
  *               holds both and the dW1 interval is empty (dense bwd: the same)
  *   dense fwd: 3 events, dense bwd: 5 events.
  *   routed fwd: 6 events (prune W1 | route | group + tile tables + gather X | y1 product | y3 product)

@@ -195,14 +195,14 @@ struct WeightGradShapes {
 };
 
 // dW2 = dY^T h in the layout of W2 ([D, F], or [F, D] = h^T dY with w2_fd) and dW1 = dy1^T X [F, D]: in one launch where
-// that saves rounds of tiles or there are few of them. The host-buffer step keeps them apart: it downloads dW2 while dW1 is computed.
+// that ends sooner by the estimate. The host-buffer step keeps them apart: it downloads dW2 while dW1 is computed.
 int weight_grads(const sf_ffn_desc& d, const void* dY, const void* h, const void* dy1, const void* X, void* dW2, void* dW1,
                  int* status, cudaStream_t s) {
   const bool w2_fd = (d.flags & SF_FFN_W2_FD) != 0;
   const void *a2 = w2_fd ? h : dY, *b2 = w2_fd ? dY : h;
   const WeightGradShapes g(d);
   const int64_t m2 = g.m2, n2 = g.n2;
-  if (!g_hooks && gemm_dual_tn_pays(m2, n2, d.F, d.D)) {
+  if (!g_hooks && gemm_dual_tn_pays(m2, n2, d.F, d.D, d.T)) {
     const int st = gemm_dual_tn(a2, b2, m2, n2, dW2, dy1, X, d.F, d.D, dW1, d.T, status, s);
     trace_mark(s);
     trace_mark(s);      // (one launch: the dW1 interval is empty)
@@ -338,7 +338,7 @@ int sf_ffn_step_plan(const sf_ffn_desc* desc, sf_ffn_plan* plan) {
   const TileShape dy1 = gemm_sparse24_drelu_tile(d.F, d.T, d.D);
   const TileShape y3 = L.plain24 ? gemm_sparse24_tile(d.T, d.D, d.F, EPI_STORE) : TileShape{0, 0};
   const WeightGradShapes g(d);
-  const bool shared = !L.expand && gemm_dual_tn_pays(g.m2, g.n2, d.F, d.D);
+  const bool shared = !L.expand && gemm_dual_tn_pays(g.m2, g.n2, d.F, d.D, d.T);
   *plan = sf_ffn_plan{gemm_cta_pairs(), L.fused || d.M == 4, y1.rows, y1.cols, dy1.rows, dy1.cols, shared ? 1 : 2,
                       shared ? gemm_dual_tn_tile(g.m2, g.n2, d.F, d.D, d.T).cols : 0, y3.rows, y3.cols};
   return SF_OK;

@@ -2004,8 +2004,9 @@ int tall_maps(const void* vals, const void* meta, const void* B, bool b_kmajor, 
 // took without it, 4096 x 4096 14.7 and 22.1, K = 256 15.9 and 19.1 (64 columns); row-major 2048 x 5632, K = 512 19.9 and 21.1.
 // A narrower width has to gain 10 %: its kernel takes the width at run time (at 6 % the weight gradients of D 2048 took 224
 // columns, 0.94 by the estimate, and 1.02 of the time).
-int best_width(int64_t M, int64_t N, int64_t stages, bool sparse, int max_bn, int step, double chunk, bool exposed,
-               double tile = 0.0, int64_t M2 = 0, int64_t N2 = 0) {
+struct TileWidth { int cols; double clocks; };
+TileWidth best_width(int64_t M, int64_t N, int64_t stages, bool sparse, int max_bn, int step, double chunk, bool exposed,
+                     double tile = 0.0, int64_t M2 = 0, int64_t N2 = 0) {
   const int64_t P = sm_count() / 2, nm = (M + 255) / 256, nm2 = (M2 + 255) / 256;
   auto cost = [&](int w) {
     const int64_t tiles = nm * ((N + w - 1) / w) + nm2 * ((N2 + w - 1) / w);
@@ -2017,7 +2018,7 @@ int best_width(int64_t M, int64_t N, int64_t stages, bool sparse, int max_bn, in
   double least = 0.90 * cost(max_bn);
   for (int w = max_bn - step; w >= step; w -= step)
     if (cost(w) < least) { least = cost(w); best = w; }
-  return best;
+  return {best, cost(best)};
 }
 
 // 512 x 224 tiles, or 256-row tiles of `bn` columns (bn = 256: one accumulator, its epilogue exposed)? Estimated clocks
@@ -2078,7 +2079,7 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
                void* C, int64_t ldc, void* C2, int64_t ldc2, const void* aux, int64_t ldaux, int* status,
                cudaStream_t s) {
   const bool two = use_two_cta(M);
-  const int bn = two ? best_width(M, N, K / 64, false, BN, 32, epi == EPI_STORE ? 200.0 : 400.0, false) : BN;
+  const int bn = two ? best_width(M, N, K / 64, false, BN, 32, epi == EPI_STORE ? 200.0 : 400.0, false).cols : BN;
   if (M % BM || N % (two ? 128 : BN) || K % 64) return SF_ERR_SHAPE;     // pairs: a ragged last tile of whole 32-column chunks
   if (M == 0 || N == 0) return SF_OK;
   CUtensorMap ta, tb;
@@ -2119,21 +2120,36 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
   return SF_ERR_UNSUPPORTED;
 }
 
-// By rounds of 256-column tiles, whatever width either side then runs. Never more of them together than apart; where they are as many,
-// the launch that is saved, with its last round and set-up, is what counts, and with many rounds nothing is left of it. Whole
-// steps, apart and together: T 1920, D 1408, F 5504 (4 rounds either way) 181.7 and 178.3 us, drawn sizes of that order 240.4 and
-// 234.6, 121.7 and 116.9, 109.9 and 105.6, 315.5 and 311.6; T 8192, D 4096, F 16384 (28 rounds) the same within the noise, M = 16
-// there 3535 and 3544.
-bool gemm_dual_tn_pays(int64_t M1, int64_t N1, int64_t M2, int64_t N2) {
+namespace {
+// One or both weight gradients (M2 = N2 = 0: one), reduced over K.
+TileWidth weight_grad_width(int64_t M1, int64_t N1, int64_t M2, int64_t N2, int64_t K) {
+  return best_width(M1, N1, K / 64, false, BN, 32, 200.0, false, 0.0, M2, N2);
+}
+}  // namespace
+
+// By the estimated clocks of the two launches, each on the width that suits it, and of the shared one, whose width is one for both.
+// kLaunch is what the second launch costs next to its tiles. Whole steps, apart and together, with M = 8:
+//   as many rounds: T 1920, D 1408, F 5504 174.4 us and 169.8;
+//   together longer, by less than a launch: T 4096, D 1024, F 2816 (1000 clocks) 152.5 and 148.8, T 6272, D 512, F 7040 (5100)
+//   296.2 and 292.0, T 10240, D 1920, F 1792 (9000) 323.6 and 319.1;
+//   by more (one of the two fits fewer columns better): T 4096, D 384, F 28032 (11 100) 694 and 694, T 10112, D 384, F 18048 (19 000)
+//   1013 and 1017, T 16256, D 384, F 28032 (47 600) 2331 and 2352.
+// kShort: of two launches of that many clocks the one that is saved is half a percent; from there on nothing of it is measured, and
+// the power cap takes something back (together fewer clocks, at a lower rate). Together over apart, as many rounds: T 1536, D 2560,
+// F 22272 (0.30 million) 0.995, T 4096, D 3072, F 12288 (0.5) 0.996, T 2560, D 3584, F 26624, M = 32 (0.82) 0.997, T 8192, D 4096,
+// F 16384 (1.8) 0.998 and 0.999, T 11776, D 2560, F 20480, M = 16 (2.1) 0.999, T 4096, D 8192, F 28672 (3.2) 0.997, T 16384, D 4096,
+// F 16384 (3.7) 1.004, T 8192, D 8192, F 28672 (6.4) 1.002, T 16384, D 8192, F 28672 (12.8) 1.011. Where rounds are saved they
+// are a gain at any length: T 16384, D 1536, F 23040 (15 instead of 16) 0.985, T 16384, D 2048, F 28672 (25 instead of 26) 0.994.
+bool gemm_dual_tn_pays(int64_t M1, int64_t N1, int64_t M2, int64_t N2, int64_t K) {
+  constexpr double kLaunch = 10000.0, kShort = 1.6e6;
   if (M1 < 256 || M2 < 256) return false;
-  const int64_t P = sm_count() / 2;
-  const int64_t t1 = ((M1 + 255) / 256) * ((N1 + 255) / 256), t2 = ((M2 + 255) / 256) * ((N2 + 255) / 256);
-  const int64_t apart = (t1 + P - 1) / P + (t2 + P - 1) / P, together = (t1 + t2 + P - 1) / P;
-  return apart <= 12 || (double)together <= 0.97 * (double)apart;
+  const double apart = weight_grad_width(M1, N1, 0, 0, K).clocks + weight_grad_width(M2, N2, 0, 0, K).clocks;
+  const double together = weight_grad_width(M1, N1, M2, N2, K).clocks;
+  return together <= 0.97 * apart || (apart <= kShort && together < apart + kLaunch);
 }
 
 TileShape gemm_dual_tn_tile(int64_t M1, int64_t N1, int64_t M2, int64_t N2, int64_t K) {
-  return TileShape{256, best_width(M1, N1, K / 64, false, BN, 32, 200.0, false, 0.0, M2, N2)};
+  return TileShape{256, weight_grad_width(M1, N1, M2, N2, K).cols};
 }
 
 int gemm_dual_tn(const void* A1, const void* B1, int64_t M1, int64_t N1, void* C1, const void* A2, const void* B2, int64_t M2,
@@ -2167,7 +2183,7 @@ TileShape gemm_sparse24_tile(int64_t M, int64_t N, int64_t K, int epi) {
   const bool plain = (epi == EPI_STORE);
   const int max_bn = plain ? BN : kNarrowBN;
   if (plain ? use_tall_plain(M, N, K / 128) : use_tall(M, N, K / 128, max_bn, 0.0, 2500.0)) return TileShape{512, kTallBN};
-  return TileShape{256, best_width(M, N, K / 128, true, max_bn, 32, 400.0, plain, 700.0)};
+  return TileShape{256, best_width(M, N, K / 128, true, max_bn, 32, 400.0, plain, 700.0).cols};
 }
 
 int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, bool b_kmajor, int64_t M, int64_t N,
@@ -2248,7 +2264,7 @@ TileShape gemm_sparse24_drelu_tile(int64_t F, int64_t T, int64_t D) {
   // D 896, F 11392 from 49.1 to 47.2 and T 768, D 768, F 23808 from 38.9 to 38.7, so the line could be lower.
   const int64_t stages = D / 128, P = sm_count() / 2, nm = (F + 255) / 256;
   auto rounds = [&](int64_t w) { return (double)((nm * ((T + w - 1) / w) + P - 1) / P); };
-  const int bn = best_width(F, T, stages, true, kNarrowBN, 32, 500.0, false);
+  const int bn = best_width(F, T, stages, true, kNarrowBN, 32, 500.0, false).cols;
   const bool wide = stages >= 8 && bn == kNarrowBN && rounds(256) * (stages * 735.0 + 1000.0) < 0.95 * rounds(kNarrowBN) * (stages * 680.0);
   if (use_tall(F, T, stages, wide ? 256 : kNarrowBN, wide ? 1000.0 : 0.0, 4000.0)) return TileShape{512, kTallBN};
   return TileShape{256, wide ? 256 : bn};
@@ -2284,7 +2300,7 @@ int gemm_sparse24_drelu(const void* w_vals, const uint8_t* meta_hw, const void* 
 }
 
 TileShape gemm_sparse24_act4_tile(int64_t F, int64_t T, int64_t D) {
-  return TileShape{256, best_width(F, T, D / 128, true, kNarrowBN, 32, 500.0, false)};
+  return TileShape{256, best_width(F, T, D / 128, true, kNarrowBN, 32, 500.0, false).cols};
 }
 
 int gemm_sparse24_act4(const void* w_vals, const uint8_t* meta_hw, const void* X, int64_t F, int64_t T, int64_t D, int V,
@@ -2341,7 +2357,7 @@ int gemm_fp8(bool sparse, const void* A, const void* meta, const void* B, int64_
   st = sparse ? make_tmap(&ta, A, M, K2 / 2, K2 / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2)
                   : make_tmap(&ta, A, M, K2, K2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2);
   if (st != SF_OK) return st;
-  const int bn = best_width(M, N, K2 / (sparse ? 128 : 64), sparse, BN, 32, sparse ? 400.0 : 200.0, sparse, sparse ? 700.0 : 0.0);
+  const int bn = best_width(M, N, K2 / (sparse ? 128 : 64), sparse, BN, 32, sparse ? 400.0 : 200.0, sparse, sparse ? 700.0 : 0.0).cols;
   st = make_tmap(&tb, B, N, K2, K2, 64, bn / 2, CU_TENSOR_MAP_SWIZZLE_128B, 2);
   if (st != SF_OK) return st;
   tm = ta;
@@ -2374,7 +2390,7 @@ bool gemm_sparse24_vnm8_supported(int64_t F, int64_t T, int64_t D, int V) {
 TileShape gemm_sparse24_vnm8_tile(int64_t F, int64_t T, int64_t D, int V) {
   const int64_t stages = D / 128, P = sm_count() / 2, nm = (F + 255) / 256;
   auto rounds = [&](int w) { return (double)((nm * ((T + w - 1) / w) + P - 1) / P); };
-  const int narrow = V == 128 ? 128 : best_width(F, T, stages, true, 192, 64, 1500.0, false);
+  const int narrow = V == 128 ? 128 : best_width(F, T, stages, true, 192, 64, 1500.0, false).cols;
   const double epi = 1500.0 * (narrow / 32), main = stages * 0.93 * (272 + 2 * narrow), wide = stages * 735.0 + 2500.0;
   const double cost_narrow = rounds(narrow) * (main > epi ? main : epi) + epi;
   const double cost_wide = rounds(256) * (wide > 13000.0 ? wide : 13000.0) + 9000.0;
