@@ -30,6 +30,8 @@ CASES = {
     "drelu_m16_160_columns": ((768, 512, 9728, 64, 16, W2_FD), dict(dy1_rows=256, dy1_cols=160)),
     "drelu_m32_224_columns": ((1024, 768, 10240, 128, 32, 0), dict(dy1_rows=256, dy1_cols=224)),
     "drelu_m32_256_columns": ((1024, 1024, 12288, 64, 32, W2_FD), dict(dy1_rows=256, dy1_cols=256)),
+    # y3 and dX at 256 columns with the accumulators alternating, half-empty last row and column, four tiles to a pair
+    "plain_256_columns": ((4224, 4224, 512, 64, 8, 0), dict(y3_rows=256, y3_cols=256)),
     # both weight gradients in one launch, CTA pairs that go from the first product's tiles to the second's
     "shared_gradients_256_columns": ((256, 640, 7040, 64, 8, 0), dict(weight_grad_launches=1, weight_grad_cols=256)),
     "shared_gradients_160_columns": ((256, 640, 6272, 64, 8, 0), dict(weight_grad_launches=1, weight_grad_cols=160)),
@@ -53,6 +55,9 @@ def test_the_rules_give_each_case_the_tiles_it_is_for(name):
         first = _tiles(m2, n2, 256, plan.weight_grad_cols)
         tiles = first + _tiles(F, D, 256, plan.weight_grad_cols)
         assert first % plan.cta_pairs != 0 and first > plan.cta_pairs       # some pairs take tiles of both products
+    elif name.startswith("plain"):
+        tiles = _tiles(T, D, plan.y3_rows, plan.y3_cols)
+        assert T % plan.y3_rows == 128 and D % plan.y3_cols == 128
     elif name.startswith("drelu"):
         tiles = _tiles(F, T, plan.dy1_rows, plan.dy1_cols)
     else:
@@ -103,8 +108,9 @@ def test_short_reductions_with_many_tiles_keep_wide_tiles(T, F, D):
 @pytest.mark.parametrize("T,D", [(8192, 16384), (16384, 8192), (4096, 16640)])
 @pytest.mark.parametrize("F", [256, 512, 768])
 def test_short_reductions_beyond_the_l2_stay_on_256_row_tiles(T, D, F):
-    """y3 and dX with up to six k-stages and an output larger than the L2 last as long as their writes, and 512-row tiles write
-    slower (measured 1.08 to 1.1 times the time); longer reductions go to 512-row tiles, smaller outputs by the clocks."""
+    """y3 and dX with two to six k-stages and an output larger than the L2 last as long as their writes, on 512-row tiles as on
+    256-row ones, and the smaller tiles leave fewer pairs idle at the end; longer reductions go to 512-row tiles, smaller
+    outputs by the clocks."""
     y3_rows = lambda *a: binding.sf_ffn_step_plan(binding.make_desc(*a, 64, 8)).y3_rows
     assert y3_rows(T, D, F) == 256
     assert y3_rows(T, D, 16 * F) == 512
@@ -190,3 +196,37 @@ def test_step_on_these_tiles_is_exact(name):
         got = _step(X, W1, W2, dY, T, D, F, V, M, flags | binding.SF_FFN_UNFUSED_ACT)
         for k in ref:
             assert np.array_equal(got[k], ref[k]), ("two kernels", k)
+
+
+# y1 with SquaredReLU and dy1 of the dense step write two results a tile through TMA at full width only. 522 tiles on 74 pairs are eight
+# rounds of ten k-stages, so that no estimate takes a narrower one; the last row and the last column of tiles are half empty.
+@pytest.mark.gpu
+@pytest.mark.parametrize("flags", [0, W2_FD])
+def test_dense_step_on_full_width_tiles_is_exact(flags):
+    T, D, F = 2176, 640, 14720
+    X, dY, W1, W2 = (_integers(shape, 1, seed) for seed, shape in enumerate([(T, D), (T, D), (F, D), (D, F)], 11))
+    w2_fd = bool(flags & W2_FD)
+    desc = binding.make_desc(T, D, F, 64, 8, flags=flags)
+    nctx, nws = binding.sf_ffn_workspace_size(desc)
+    bufs = dict(context=Guarded(nctx, zero=True), workspace=Guarded(nws, zero=True), Y=Guarded((T, D), torch.bfloat16),
+                dX=Guarded((T, D), torch.bfloat16), dW1=Guarded((F, D), torch.bfloat16),
+                dW2=Guarded((F, D) if w2_fd else (D, F), torch.bfloat16))
+    ctx, ws, Y, dX, dW1, dW2 = (b.t for b in bufs.values())
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda().to(torch.bfloat16)
+    x, w1, w2, dy = dev(X), dev(W1), dev(W2.T if w2_fd else W2), dev(dY)
+    binding.sf_dense_ffn_fwd(desc, x, w1, w2, Y, ctx, ws)
+    binding.sf_dense_ffn_bwd(desc, dy, x, w1, w2, ctx, dX, dW1, dW2, ws)
+    assert binding.sf_check_status(ws) == binding.SF_OK
+    for name, b in bufs.items():
+        b.check(name)
+    y1 = _round(_exact_product(X, W1.T, "y1"))
+    relu = np.maximum(y1, 0)
+    h = _round(relu * relu)
+    dy1 = _round(2.0 * _exact_product(dY, W2, "dy2") * relu)
+    n = T * F * 2
+    assert np.array_equal(f32(ctx[:n].view(torch.bfloat16)).reshape(T, F), y1)
+    assert np.array_equal(f32(ctx[n:2 * n].view(torch.bfloat16)).reshape(T, F), h)
+    assert np.array_equal(f32(Y), _round(_exact_product(h, W2.T, "Y")))
+    assert np.array_equal(f32(dX), _round(_exact_product(dy1, W1, "dX")))
+    assert np.array_equal(f32(dW1), _round(_exact_product(dy1.T, X, "dW1")))
+    assert np.array_equal(f32(dW2).T if w2_fd else f32(dW2), _round(_exact_product(dY.T, h, "dW2")))
