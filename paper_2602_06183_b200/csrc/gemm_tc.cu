@@ -172,16 +172,16 @@ __device__ __forceinline__ void store_chunk(const CUtensorMap* tmapC, uint8_t* b
 // kTileN: accumulator columns of the tile (a multiple of 32). Columns at or beyond n_limit (a ragged last
 // tile, whole 32-column chunks only since N % 32 == 0) are not stored. `part` of `parts`: the share of the tile's
 // columns that this warp takes.
-// A thread holds one row. EPI_STORE stores from there (16 bytes of 32 rows per instruction), or with kQuad 64 bytes of eight rows
-// after an exchange among four lanes; tiles of full width go out through TMA instead (epi_store_tile), except where the rows
-// are scattered (row_map). Narrow tiles (run-time width), where the latency of a chunk is what counts, keep the first: with the
-// exchange the step at T 1024, D 256, F 1024 took 40.4 us instead of 40.0. kQuad in the routed step at T 8192, D 4096, F 16384 in
+// A thread holds one row. EPI_STORE stores from there (16 bytes of 32 rows per instruction), or 64 bytes of eight rows after an
+// exchange among four lanes where the rows are scattered (kScatter: row_map); other tiles of full width go out through TMA instead
+// (epi_store_tile). Narrow tiles (run-time width), where the latency of a chunk is what counts, keep the first: with the
+// exchange the step at T 1024, D 256, F 1024 took 40.4 us instead of 40.0. The exchange in the routed step at T 8192, D 4096, F 16384 in
 // four experts: 1277 -> 1257 us. The two-operand epilogues of the dense step move a chunk through shared memory, 64 contiguous bytes of
 // eight rows per instruction: y1 + SquaredReLU at T 4096, D 2048, F 8192 129 -> 96 us.
 // kEarly: the accumulator is handed back when the first chunk has been read; the second part starts with its last chunk, so that
 // the columns at either end of the tile are the first to be read.
 // kTma: the two-operand epilogues hand their chunks to TMA (T 10496, D 384, F 7424, the dense step 504 -> 488 us).
-template <int kEpi, int kTileN = BN, bool kEarly = false, bool kQuad = false, bool kTma = false>
+template <int kEpi, int kTileN = BN, bool kEarly = false, bool kScatter = false, bool kTma = false>
 __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit,
                                          int q, int lane, uint8_t* my_stage, int part = 0, int parts = 1, bool second = false,
                                          uint64_t* tmem_empty_bar = nullptr, const CUtensorMap* tmapC = nullptr,
@@ -215,24 +215,16 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
     if (kEarly) release_accumulator(lane, tmem_empty_bar);
     return;
   }
-  int64_t row = m0 + q * 32 + lane;                                        // this thread's D row
-  bool row_live = true;
-  if (kEpi == EPI_STORE && args.row_map) {                                 // scattered output rows
-    const int r = __ldg(args.row_map + row);
-    row_live = r >= 0;
-    row = r;
-  }
-  // kQuad: this thread stores 16-byte unit `lane & 3` of the four rows of its four lanes
+  // EPI_STORE: this thread's row (formed here: inside the chunk loop the step at T 1024, D 256, F 1024 takes 38.58 us instead of 38.42)
+  const int64_t row = m0 + q * 32 + lane;
+  uint16_t* const crow = reinterpret_cast<uint16_t*>(second ? args.C2 : args.C) + row * (second ? args.ldc2 : args.ldc);
+  // kScatter: this thread stores 16-byte unit `lane & 3` of the four rows of its four lanes
   int rows4[4];
-  const int64_t ldq = second ? args.ldc2 : args.ldc;
-  uint16_t* cq = reinterpret_cast<uint16_t*>(second ? args.C2 : args.C) + (lane & 3) * 8;
-  if (kQuad) {
-    if (args.row_map) {
+  uint16_t* const cq = reinterpret_cast<uint16_t*>(args.C) + (lane & 3) * 8;
+  if (kScatter) {
+    const int r = __ldg(args.row_map + row);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) rows4[i] = __shfl_sync(0xFFFFFFFFu, (int)row, (lane & 28) + i);
-    } else {
-      cq += (m0 + q * 32 + (lane & 28)) * ldq;
-    }
+    for (int i = 0; i < 4; ++i) rows4[i] = __shfl_sync(0xFFFFFFFFu, r, (lane & 28) + i);
   }
   // EPI_SQRELU, EPI_DRELU: this thread moves 16-byte unit `u` of the rows `t8 + 8 i` of a chunk.
   const int t8 = lane >> 2, u = lane & 3;
@@ -295,14 +287,14 @@ __device__ __forceinline__ void epi_tile(const GemmArgs& args, uint32_t taddr, i
       for (int j = 0; j < 16; ++j) w[j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
     }
     if (kEpi == EPI_STORE) {
-      if constexpr (kQuad) {
+      if constexpr (kScatter) {
         quad_transpose(w, lane);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          if (!args.row_map || rows4[i] >= 0)
-            *reinterpret_cast<uint4*>(cq + (args.row_map ? rows4[i] : i) * ldq + col0) = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
-      } else if (row_live) {
-        uint4* c = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(second ? args.C2 : args.C) + row * (second ? args.ldc2 : args.ldc) + col0);
+          if (rows4[i] >= 0)
+            *reinterpret_cast<uint4*>(cq + rows4[i] * args.ldc + col0) = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+      } else {
+        uint4* c = reinterpret_cast<uint4*>(crow + col0);
 #pragma unroll
         for (int j = 0; j < 4; ++j) c[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
       }
@@ -392,16 +384,16 @@ __device__ __forceinline__ void epi_store_tile(const GemmArgs& args, const CUten
 // fragments that stmatrix transposes on its way to shared memory, [32 tokens][32 features], and leaves through TMA as above: the
 // fewest passes over the shared memory that the main loop works on. For 512-row tiles; against words of two tokens staged by
 // lane and taken apart again 16384 x 8192, K = 4096 502.9 -> 499.2 us, 4096 x 16384, K = 2048 140.4 -> 138.8.
-template <int kTileN, int kBufs>
+template <int kTileN>
 __device__ __forceinline__ void epi_store_t_tile(const CUtensorMap* tmapC, uint32_t taddr, int64_t m0, int64_t n0, int64_t n_limit, int q,
-                                                 int lane, uint8_t* bufs, uint32_t& buf) {
+                                                 int lane, uint8_t* stage) {
   const int nch = (int)min((int64_t)(kTileN / 32), (n_limit - n0) >> 5);
   auto load = [&](int ch, uint32_t (&v)[32]) {
     tmem_ld_16x256b_x4(taddr + ch * 32, v);
     tmem_ld_16x256b_x4(taddr + ch * 32 + (16u << 16), v + 16);
   };
   // lane 8 k + j addresses eight features (16-byte unit k) of token j of eight: units swizzled as in store_chunk
-  const uint32_t at = smem_u32(bufs) + (lane & 7) * 64 + (((lane >> 3) ^ ((lane >> 1) & 3)) << 4);
+  const uint32_t at = smem_u32(stage) + (lane & 7) * 64 + (((lane >> 3) ^ ((lane >> 1) & 3)) << 4);
   auto chunk = [&](int ch, uint32_t (&v)[32], uint32_t (&next)[32]) {
     tmem_ld_wait_on(v);
     if (ch + 1 < nch) load(ch + 1, next);
@@ -413,17 +405,16 @@ __device__ __forceinline__ void epi_store_t_tile(const CUtensorMap* tmapC, uint3
         const uint32_t* x = v + 16 * (k >> 1) + 4 * i + 2 * (k & 1);
         w[i][k] = pack_bf16x2(__uint_as_float(x[0]), __uint_as_float(x[1]));
       }
-    if (lane == 0) bulk_wait_read<kBufs - 1>();
+    if (lane == 0) bulk_wait_read<0>();
     __syncwarp();
 #pragma unroll
-    for (int i = 0; i < 4; ++i) stmatrix_x4_trans(at + buf * kEpiWarpBytes + i * 512, w[i][0], w[i][1], w[i][2], w[i][3]);
+    for (int i = 0; i < 4; ++i) stmatrix_x4_trans(at + i * 512, w[i][0], w[i][1], w[i][2], w[i][3]);
     fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) {
-      tma_store_2d(tmapC, bufs + buf * kEpiWarpBytes, (int)m0 + q * 32, (int)n0 + ch * 32);
+      tma_store_2d(tmapC, stage, (int)m0 + q * 32, (int)n0 + ch * 32);
       bulk_commit();
     }
-    if (kBufs == 2) buf ^= 1u;
   };
   uint32_t va[32], vb[32];
   load(0, va);
@@ -1281,6 +1272,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   uint8_t* pk_stage = smem + kStages * kStageBytes;       // kExpand: ring of packed tiles, one per stage
   uint8_t* epi_stage = pk_stage + (kExpand ? kStages * kPkStageBytes : 0);
   constexpr bool kTmaStore = tma_store2(kEpi, kExpand != 0, kVar);
+  constexpr bool kMapped = kTmaStore && kSparse && kEpi == EPI_STORE && !kFp8;   // may be given a row_map
   constexpr int kStoreBufs = kTmaStore ? (threads2(kMode, kEpi, kExpand, kVar) / 32 - 2) * store_bufs2(kSparse, kEpi) : 0;
   SmemCtl2* ctl = reinterpret_cast<SmemCtl2*>(epi_stage + epi_bytes2(kEpi, kBN, kStoreBufs));
   volatile int* abort_flag = &ctl->abort_flag;
@@ -1559,11 +1551,11 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
       const bool live = args.tile_table != nullptr || m0 < (second ? args.M2 : args.M);
       if (!mbar_wait_warp(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      if (kEpi == EPI_STORE && kTmaStore && live && !args.row_map) {
+      if (kEpi == EPI_STORE && kTmaStore && live && !(kMapped && args.row_map)) {
         epi_store_tile<kBN, store_bufs2(kSparse, kEpi), kOverlap>(args, second ? &tmapC2 : &tmapC, taddr, m0, n0, n_limit, q, lane,
                                                                   my_stage, buf, set, kParts, &ctl->tmem_empty[0]);
       } else if (live) {
-        epi_tile<kEpi, kBN, kOverlap, kEpi == EPI_STORE && kTmaStore, kTmaStore>(
+        epi_tile<kEpi, kBN, kOverlap, kMapped, kTmaStore>(
             args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts, second, &ctl->tmem_empty[0], &tmapC, &tmapC2, &buf);
       }
       if (!kOverlap || !live) release_accumulator(lane, &ctl->tmem_empty[acc]);
@@ -1809,7 +1801,7 @@ gemm_tall_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constan
         if (!mbar_wait_warp(&ctl->tmem_full[h], phase, abort_flag)) break;
         tc_fence_after();
         if (kEpi == EPI_STORE_T && live) {
-          epi_store_t_tile<kTallBN, 1>(&tmapC, taddr, m0, n0, n_limit, q, lane, wsm, buf);
+          epi_store_t_tile<kTallBN>(&tmapC, taddr, m0, n0, n_limit, q, lane, wsm);
         } else if (live) {
           epi_store_tile<kTallBN, 1, false>(args, &tmapC, taddr, m0, n0, n_limit, q, lane, wsm, buf, 0, 1, nullptr);
         }
