@@ -202,8 +202,8 @@ SF_API int sf_gemm_sparse24_noalloc(const void* a_vals, const void* a_meta, cons
  * sf_gemm_fp8_sparse24: the same with A given 2:4-packed: a_vals uint8 [Mr,K/2], a_meta canonical
  *     uint16 [Mr,K/16]. alpha is normally 1 / (scale_A * scale_B).
  *     Mr % 256 == 0, Nc % 256 == 0, K % 128 == 0 (dense) or K % 256 == 0 (2:4). fp32 accumulation.
- * `workspace`: sf_gemm_fp8_workspace_size(Mr, K) bytes (status word; the rest is reserved); read its
- *     status with sf_check_status.
+ * `workspace`: sf_gemm_fp8_workspace_size(Mr, K) bytes (a status word; the rest is not used at
+ *     present, and the size stays as it is); read its status with sf_check_status.
  * Errors as everywhere: SF_ERR_SHAPE / NULL / ALIGN / ARCH before anything is launched. */
 SF_API int sf_fp8_quantize(const void* X, int64_t rows, int64_t cols, int64_t ld, float scale, void* Xq, void* stream);
 SF_API int sf_prune24_fp8_sizes(int64_t rows, int64_t cols, int group_dim, size_t* vals_bytes, size_t* meta_bytes);

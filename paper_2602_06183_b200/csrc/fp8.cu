@@ -154,7 +154,7 @@ int sf_prune24_compress_fp8(const void* W, int64_t rows, int64_t cols, int64_t l
 int sf_gemm_fp8_workspace_size(int64_t Mr, int64_t K, size_t* bytes) {
   if (!bytes) return SF_ERR_NULL;
   if (Mr < 0 || K < 0) return SF_ERR_SHAPE;
-  *bytes = kStatusBytes8 + (size_t)Mr * K / 8;
+  *bytes = kStatusBytes8 + (size_t)Mr * K / 8;          // used: the status word. Callers keep the buffers that they were told to make
   return SF_OK;
 }
 
@@ -176,6 +176,7 @@ int sf_gemm_fp8_sparse24(const void* a_vals, const void* a_meta, const void* B, 
   if (!aligned16(a_vals) || !aligned16(a_meta) || !aligned16(B) || !aligned16(C) || !aligned16(workspace))
     return SF_ERR_ALIGN;
   SF_TRY(check_arch());
+  // (256 GB of codes: refused before, and still)
   if (Mr * (K >> 7) > (int64_t)1 << 31 || K > (int64_t)1 << 31) return SF_ERR_SHAPE;
   return gemm_fp8(true, a_vals, a_meta, B, Mr, Nc, K, alpha, C, Nc, (int*)workspace, (cudaStream_t)stream);
 }
