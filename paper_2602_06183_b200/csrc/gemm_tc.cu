@@ -139,8 +139,9 @@ __device__ __forceinline__ void quad_transpose(uint32_t (&x)[16], int lane) {
 
 // ---- stores through TMA -----------------------------------------------------------------------------
 // What bounded the plain store: an epilogue thread holds a row, so a 16-byte store of a warp went to 32 rows, 32 cycles of the
-// load/store unit each (7000 clocks for the 256 x 224 outputs of an SM in a 512-row tile), on the chain from one main loop to the
-// next and in the way of the MMAs' shared-memory reads. Here a warp puts 32 x 32 results into shared memory, 64 bytes a row, and one
+// load/store unit's data pipe each (counted: 33 wavefronts a store; 7200 clocks for the 256 x 224 outputs of an SM in a 512-row tile;
+// 56 % of the pipe's peak at 8192 x 16384, K = 128, now 14.5 %, and every sector written to the L2 in two halves), on the chain from one
+// main loop to the next and in the way of the MMAs' shared-memory reads. Here a warp puts 32 x 32 results into shared memory, 64 bytes a row, and one
 // thread hands them to TMA. Same box, call after call: 2:4 row-major 8192 x 16384, K = 128 115 -> 67 us, K = 1024 215 -> 167,
 // K = 4096 535 -> 503; E4M3 2:4 4096 x 16384 x 4096 170 -> 150; dense 8192 x 16384, K = 128 119 -> 79, 16384 x 8192, K = 512 168 -> 131.
 // Four lanes exchanging their rows' units and storing 64 bytes of eight rows per instruction gave E4M3 152 and dense K = 512 168;
@@ -1393,8 +1394,9 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
       }
     }
     // The next launch is let in when the last loads are on their way. Let in at the start, its CTAs sat in their wait on the SMs
-    // that were free (what that cost is measured, its cause is not): T 1024, D 256, F 1024, whole step 39.9 -> 38.4 us; T 1920,
-    // D 1408, F 5504 183.1 -> 181.8; T 4096, D 2048, F 8192 557 -> 554. No early start at all costs the small step 3 us.
+    // that were free (what that cost is measured, its cause is not). Whole steps, libraries in turn: T 1024, D 256, F 1024 39.85 -> 38.29
+    // us, T 1920, D 1408, F 5504 183.1 -> 181.8, T 4096, D 2048, F 8192 549 -> 547, T 8192, D 4096, F 16384 3848 -> 3838 (0.997 +- 0.0007),
+    // M = 16 there 3500 -> 3494, T 16384, D 8192, F 28672 equal (25.34 and 25.39 ms, +- 0.08). No early start at all costs the first 3 us.
     pdl_trigger();
   } else if (warp == 1) {
     // =========================== MMA issuer (leader CTA only) ===========================
