@@ -1169,6 +1169,20 @@ __host__ __device__ constexpr int num_stages2(bool sparse, int bn = BN, bool exp
 __host__ __device__ constexpr bool tma_store2(int epi, bool expand, bool var) {
   return (epi == EPI_STORE || epi == EPI_SQRELU || epi == EPI_DRELU) && !expand && !var;
 }
+// The store maps of a kernel: none, one, or two (two products, or two outputs). Only what it uses is a parameter, and only that is
+// encoded: both cost the host's side of a launch, which is all of the smallest calls (dense 512 x 512 x 256 5.33 us with two maps
+// that are not used and 5.21 without, 2:4 512 x 1280 x 512 7.44 and 7.21, E4M3 dense 512 x 1024 x 512 5.28 and 5.09). Without the
+// alignment the arguments behind an empty one start inside a line of 64 bytes: T 1024, D 256, F 1024 38.66 us a step instead of 38.43.
+template <int N> struct StoreMaps { CUtensorMap m[N]; };
+template <> struct alignas(64) StoreMaps<0> {};
+__host__ __device__ constexpr int store_maps2(int epi, bool expand, bool var, bool dual) {
+  return !tma_store2(epi, expand, var) ? 0 : dual || epi == EPI_SQRELU ? 2 : 1;
+}
+template <int N>
+__device__ __forceinline__ const CUtensorMap* store_map(const StoreMaps<N>& maps, int i) {
+  if constexpr (N == 0) return nullptr;
+  else return &maps.m[N > 1 ? i : 0];
+}
 __host__ __device__ constexpr int store_bufs2(bool sparse, int epi) { return sparse && epi == EPI_STORE ? 1 : 2; }
 __host__ __device__ constexpr int epi_bytes2(int epi, int bn = BN, int store_bufs = 0) {
   return store_bufs > 0   ? store_bufs * kEpiWarpBytes
@@ -1241,7 +1255,7 @@ template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand =
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kMode, kEpi, kExpand, kVar), 1)
 gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB,
                 const __grid_constant__ CUtensorMap tmapMeta, const __grid_constant__ CUtensorMap tmapPk,
-                const __grid_constant__ CUtensorMap tmapC, const __grid_constant__ CUtensorMap tmapC2, const GemmArgs args) {
+                const __grid_constant__ StoreMaps<store_maps2(kEpi, kExpand != 0, kVar, kDual)> tmapsC, const GemmArgs args) {
   extern __shared__ uint8_t smem_dyn[];
   uint8_t* smem = smem_dyn + align_pad(smem_dyn, 1024);
   constexpr bool kSparse = kMode == MODE_SPARSE24;
@@ -1554,11 +1568,11 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
       if (!mbar_wait_warp(&ctl->tmem_full[acc], acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
       if (kEpi == EPI_STORE && kTmaStore && live && !(kMapped && args.row_map)) {
-        epi_store_tile<kBN, store_bufs2(kSparse, kEpi), kOverlap>(args, second ? &tmapC2 : &tmapC, taddr, m0, n0, n_limit, q, lane,
+        epi_store_tile<kBN, store_bufs2(kSparse, kEpi), kOverlap>(args, store_map(tmapsC, second), taddr, m0, n0, n_limit, q, lane,
                                                                   my_stage, buf, set, kParts, &ctl->tmem_empty[0]);
       } else if (live) {
         epi_tile<kEpi, kBN, kOverlap, kMapped, kTmaStore>(
-            args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts, second, &ctl->tmem_empty[0], &tmapC, &tmapC2, &buf);
+            args, taddr, m0, n0, n_limit, q, lane, my_stage, set, kParts, second, &ctl->tmem_empty[0], store_map(tmapsC, 0), store_map(tmapsC, 1), &buf);
       }
       if (!kOverlap || !live) release_accumulator(lane, &ctl->tmem_empty[acc]);
       if (++acc == (uint32_t)kAccBufs) { acc = 0; acc_phase ^= 1; }
@@ -1926,8 +1940,12 @@ int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
                                  : a.num_m_tiles * a.num_n_tiles + (kDual ? a.num_m_tiles2 * a.num_n_tiles2 : 0);
   const int max_pairs = sm_count() / 2;
   const int pairs = tiles < max_pairs ? tiles : max_pairs;
-  if (tma_store && !a.row_map && (!tc || ((kDual || kEpi == EPI_SQRELU) && !tc2))) return SF_ERR_UNSUPPORTED;
-  return launch_pdl(kern, dim3(2 * pairs), threads, smem, s, ta, tb, tm, tpk ? *tpk : ta, tc ? *tc : ta, tc2 ? *tc2 : ta, a);
+  constexpr int maps = store_maps2(kEpi, kExpand != 0, kVar, kDual);
+  if (!a.row_map && ((maps > 0 && !tc) || (maps > 1 && !tc2))) return SF_ERR_UNSUPPORTED;
+  StoreMaps<maps> cm;
+  if constexpr (maps > 0) cm.m[0] = tc ? *tc : ta;
+  if constexpr (maps > 1) cm.m[1] = *tc2;
+  return launch_pdl(kern, dim3(2 * pairs), threads, smem, s, ta, tb, tm, tpk ? *tpk : ta, cm, a);
 }
 
 int64_t l2_bytes() {
@@ -2189,7 +2207,9 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   if ((plain || !b_kmajor) && !two) return SF_ERR_UNSUPPORTED;
   CUtensorMap ta, tb, tm, tc;
   const TileShape tile = two ? gemm_sparse24_tile(M, N, K, epi) : TileShape{BM, BN};
-  if (plain || tile.rows == 512) {
+  const int bn = tile.cols;
+  const bool var = two && tile.rows != 512 && bn != (plain ? BN : kNarrowBN);
+  if ((plain && !var) || tile.rows == 512) {
     const int st = plain ? make_store_map(&tc, C, M, N, ldc) : make_store_map(&tc, C, N, M, ldc);
     if (st != SF_OK) return st;
   }
@@ -2206,7 +2226,6 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   int st = two ? make_tmap(&ta, a_vals, M, K / 2, K / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B)
                : make_tmap(&ta, a_vals, M, K / 2, K / 2, 32, 128, CU_TENSOR_MAP_SWIZZLE_64B);
   if (st != SF_OK) return st;
-  const int bn = tile.cols;
   if (b_kmajor) st = make_tmap(&tb, B, N, K, K, 64, two ? bn / 2 : 256, CU_TENSOR_MAP_SWIZZLE_128B);
   else          st = make_tmap(&tb, B, K, N, N, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st != SF_OK) return st;
@@ -2222,7 +2241,6 @@ int gemm_sparse24(const void* a_vals, const uint8_t* meta_hw, const void* B, boo
   a.C = C; a.ldc = ldc; a.meta_hw = meta_hw; a.status = status;
   a.num_m_tiles = (int)(M / BM); a.num_n_tiles = (int)(N / BN); a.num_k_blocks = (int)(K / 64);
   a.bn = bn;
-  const bool var = two && bn != (plain ? BN : kNarrowBN);
   if (epi == EPI_STORE) {
     if (b_kmajor) return var ? launch_two<MODE_SPARSE24, false, false, EPI_STORE, BN, 0, false, true>(ta, tb, tm, a, s)
                              : launch_two<MODE_SPARSE24, false, false, EPI_STORE>(ta, tb, tm, a, s, nullptr, &tc);
@@ -2337,9 +2355,11 @@ int gemm_fp8(bool sparse, const void* A, const void* meta, const void* B, int64_
   // the operands in 2-byte units: [M, K/2] (dense) or [M, K/4] (2:4 values), [N, K/2]
   const int64_t K2 = K / 2;
   CUtensorMap ta, tb, tm, tc;
-  int st = make_store_map(&tc, C, M, N, ldc);
-  if (st != SF_OK) return st;
-  if (sparse && use_tall_plain(M, N, K / 256)) {
+  const bool tall = sparse && use_tall_plain(M, N, K / 256);
+  const int bn = tall ? kTallBN : best_width(M, N, K2 / (sparse ? 128 : 64), sparse, BN, 32, sparse ? 400.0 : 200.0, sparse, sparse ? 700.0 : 0.0).cols;
+  int st = SF_OK;
+  if ((tall || bn == BN) && (st = make_store_map(&tc, C, M, N, ldc)) != SF_OK) return st;
+  if (tall) {
     CUtensorMap tbn;
     st = tall_maps(A, meta, B, true, M, N, K2, 2, &ta, &tb, &tbn, &tm);
     if (st != SF_OK) return st;
@@ -2349,9 +2369,8 @@ int gemm_fp8(bool sparse, const void* A, const void* meta, const void* B, int64_
     return launch_tall<false, EPI_STORE, true>(ta, tb, tbn, tm, a, s, &tc);
   }
   st = sparse ? make_tmap(&ta, A, M, K2 / 2, K2 / 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2)
-                  : make_tmap(&ta, A, M, K2, K2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2);
+              : make_tmap(&ta, A, M, K2, K2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B, 2);
   if (st != SF_OK) return st;
-  const int bn = best_width(M, N, K2 / (sparse ? 128 : 64), sparse, BN, 32, sparse ? 400.0 : 200.0, sparse, sparse ? 700.0 : 0.0).cols;
   st = make_tmap(&tb, B, N, K2, K2, 64, bn / 2, CU_TENSOR_MAP_SWIZZLE_128B, 2);
   if (st != SF_OK) return st;
   tm = ta;
