@@ -1336,6 +1336,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
   pdl_wait();                                            // everything above overlaps the previous kernel's tail
   const int num_tiles = args.tile_table ? __ldg(args.num_tiles_dev)
                                         : num_m_tiles * num_n_tiles_ + (kDual ? args.num_m_tiles2 * args.num_n_tiles2 : 0);
+  if (kMode == MODE_DENSE && !kVar && args.early_next) pdl_trigger();
   const uint32_t tmem_base = ctl->tmem_base;
 
   if (warp == 0) {
@@ -1407,10 +1408,10 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
         if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
     }
-    // The next launch is let in when the last loads are on their way. Let in at the start, its CTAs sat in their wait on the SMs
-    // that were free (what that cost is measured, its cause is not). Whole steps, libraries in turn: T 1024, D 256, F 1024 39.85 -> 38.29
-    // us, T 1920, D 1408, F 5504 183.1 -> 181.8, T 4096, D 2048, F 8192 549 -> 547, T 8192, D 4096, F 16384 3848 -> 3838 (0.997 +- 0.0007),
-    // M = 16 there 3500 -> 3494, T 16384, D 8192, F 28672 equal (25.34 and 25.39 ms, +- 0.08). No early start at all costs the first 3 us.
+    // The next launch is let in when the last loads are on their way (long dense products: at the start, see long_dense). Let in at
+    // the start, its CTAs sat in their wait on the SMs that were free (what that cost is measured, its cause is not). Whole steps:
+    // T 1024, D 256, F 1024 39.85 -> 38.29 us, T 1920, D 1408, F 5504 180.2 -> 178.1, T 4096, D 2048, F 8192 554.6 -> 551.2. No early
+    // start at all costs the first 3 us.
     pdl_trigger();
   } else if (warp == 1) {
     // =========================== MMA issuer (leader CTA only) ===========================
@@ -1917,6 +1918,15 @@ int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const GemmArgs& a, 
                     ta, tb, a);
 }
 
+// Dense products of several rounds of full-width tiles, 128 k-stages and more to a CTA pair (65 000 clocks): the next launch is let in
+// at their start. Behind their last loads, call after call at the power cap, they took longer, at the same clocks and a lower rate: 8192
+// x 8192 x 8192 874 us, at the start 846, 2048 x 12544 x 7360 309 and 296, 4096 x 16384 x 4096 424 and 421, E4M3 2048 x 12544 x 7424 165
+// and 160; steps T 16384, D 8192, F 28672 26.73 ms and 26.05, the dense one at T 8192, D 4096, F 16384 5.16 and 5.08. 300 drawn sizes, at
+// the start over behind the last loads: up to 64 stages 1.01, to 128 1.003, to 192 0.995, to 384 0.993, above 0.985 (4864 x 6144 x 448, 49
+// stages, 28.9 us and 29.3; the step at T 1920, D 1408, F 5504, whose weight gradients have 120, 178.1 and 179.4). The 2:4 products gained
+// nothing from it (0.996 to 1.005) and T 4096, D 2048, F 8192 lost 0.5 %; of its weight gradients (448 stages) it loses 0.2 %.
+bool long_dense(int tiles, int pairs, int64_t stages) { return tiles > pairs && (int64_t)((tiles + pairs - 1) / pairs) * stages >= 128; }
+
 template <int kMode, bool kAMN, bool kBMN, int kEpi, int kBN = BN, int kExpand = 0, bool kFp8 = false, bool kVar = false, bool kDual = false>
 int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tm, GemmArgs a, cudaStream_t s,
                const CUtensorMap* tpk = nullptr, const CUtensorMap* tc = nullptr, const CUtensorMap* tc2 = nullptr) {
@@ -1940,6 +1950,7 @@ int launch_two(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
                                  : a.num_m_tiles * a.num_n_tiles + (kDual ? a.num_m_tiles2 * a.num_n_tiles2 : 0);
   const int max_pairs = sm_count() / 2;
   const int pairs = tiles < max_pairs ? tiles : max_pairs;
+  a.early_next = kMode == MODE_DENSE && kEpi != EPI_ROUTE && kExpand == 0 && !kVar && !a.tile_table && long_dense(tiles, max_pairs, a.K / 64);
   constexpr int maps = store_maps2(kEpi, kExpand != 0, kVar, kDual);
   if (!a.row_map && ((maps > 0 && !tc) || (maps > 1 && !tc2))) return SF_ERR_UNSUPPORTED;
   StoreMaps<maps> cm;

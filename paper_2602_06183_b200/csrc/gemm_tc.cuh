@@ -53,6 +53,7 @@ struct GemmArgs {
   int64_t M2, N2;           // second product of a launch of two (output C2)
   int num_m_tiles2, num_n_tiles2;
   int gather_tma_groups;    // Venom: groups (of 16 per stage) fetched by TMA row gather; the rest by cp.async
+  int early_next;           // CTA-pair dense kernels: the next launch is let in at the start (see long_dense)
   // EPI_DRELU24_T / EPI_DRELUV_T: metadata of the activation's mask and the packed output (see ActMask)
   const void* pack_meta;
   void* pack_vals;

@@ -88,6 +88,28 @@ def test_dense_gemm_output_beyond_the_l2(a_k, b_k, M, N, K):
     assert torch.equal(C, (A.double() @ B.double().T).to(torch.bfloat16))
 
 
+@pytest.mark.parametrize("K", [768, 1088])         # nine rounds of 12 k-stages (the next launch is let in late) and of 17 (at the start)
+def test_dense_gemm_read_by_the_next_launch(K):
+    """Each product is the operand of the next launch, which is set up while it runs; three turns through one pair of buffers."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(K)
+    ints = lambda *s: torch.randint(-1, 2, s, generator=g, device="cuda").to(torch.bfloat16)
+    M, N = 2688, 14848
+    C, D = (torch.empty(s, dtype=torch.bfloat16, device="cuda") for s in ((M, N), (M, 256)))
+    ws = torch.zeros(binding.sf_gemm_workspace_size(M, K), dtype=torch.uint8, device="cuda")
+    operands = [(ints(M, K), ints(N, K), ints(256, N)) for _ in range(3)]
+    got = []
+    for A, B, E in operands:
+        binding.sf_gemm_dense(A, True, B, True, C_out=C, workspace=ws)
+        binding.sf_gemm_dense(C, True, E, True, C_out=D, workspace=ws)
+        got.append(D.clone())
+    assert binding.sf_check_status(ws) == binding.SF_OK
+    for (A, B, E), d in zip(operands, got):
+        c = (A.double() @ B.double().T).to(torch.bfloat16)             # integers: exact in float32, one rounding to bf16
+        assert float((c.double().abs() @ E.double().abs().T).max()) < 2.0 ** 24
+        assert torch.equal(d, (c.double() @ E.double().T).to(torch.bfloat16))
+
+
 def _integer_24_product(Mr, Nc, K, b_k, run):
     """Small integers: every partial sum is exact in float32, so only the bf16 rounding of the result is left."""
     rng = np.random.default_rng(Mr + Nc)
