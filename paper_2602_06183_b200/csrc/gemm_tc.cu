@@ -2152,23 +2152,23 @@ TileWidth weight_grad_width(int64_t M1, int64_t N1, int64_t M2, int64_t N2, int6
 
 // By the estimated clocks of the two launches, each on the width that suits it, and of the shared one, whose width is one for both.
 // kLaunch is what the second launch costs next to its tiles. Whole steps, apart and together, with M = 8:
-//   as many rounds: T 1920, D 1408, F 5504 174.4 us and 169.8;
-//   together longer, by less than a launch: T 4096, D 1024, F 2816 (1000 clocks) 152.5 and 148.8, T 6272, D 512, F 7040 (5100)
-//   296.2 and 292.0, T 10240, D 1920, F 1792 (9000) 323.6 and 319.1;
-//   by more (one of the two fits fewer columns better): T 4096, D 384, F 28032 (11 100) 694 and 694, T 10112, D 384, F 18048 (19 000)
-//   1013 and 1017, T 16256, D 384, F 28032 (47 600) 2331 and 2352.
-// kShort: of two launches of that many clocks the one that is saved is half a percent; from there on nothing of it is measured, and
-// the power cap takes something back (together fewer clocks, at a lower rate). Together over apart, as many rounds: T 1536, D 2560,
-// F 22272 (0.30 million) 0.995, T 4096, D 3072, F 12288 (0.5) 0.996, T 2560, D 3584, F 26624, M = 32 (0.82) 0.997, T 8192, D 4096,
-// F 16384 (1.8) 0.998 and 0.999, T 11776, D 2560, F 20480, M = 16 (2.1) 0.999, T 4096, D 8192, F 28672 (3.2) 0.997, T 16384, D 4096,
-// F 16384 (3.7) 1.004, T 8192, D 8192, F 28672 (6.4) 1.002, T 16384, D 8192, F 28672 (12.8) 1.011. Where rounds are saved they
-// are a gain at any length: T 16384, D 1536, F 23040 (15 instead of 16) 0.985, T 16384, D 2048, F 28672 (25 instead of 26) 0.994.
+//   as many rounds: T 1920, D 1408, F 5504 174.7 us and 170.3;
+//   together longer, by less than a launch: T 4096, D 1024, F 2816 (1000 clocks) 155.2 and 151.1, T 6272, D 512, F 7040 (5100)
+//   296.2 and 292.0, T 10240, D 1920, F 1792 (9000) 326.4 and 324.7;
+//   by more (one of the two fits fewer columns better): T 4096, D 384, F 28032 (11 100) 708 and 707, T 10112, D 384, F 18048 (19 000)
+//   1031 and 1038, T 16256, D 384, F 28032 (47 600) 2390 and 2413.
+// kShort: of two launches of that many clocks the one that is saved is half a percent; from there on nothing of it is left, and at the
+// power cap the shared one takes fewer clocks at a lower rate. Together over apart, as many rounds: T 1536, D 2560, F 22272 (0.30
+// million) 0.996, T 4096, D 3072, F 12288 (0.5) 1.000, T 8192, D 4096, F 16384 (1.8) 1.004, T 4096, D 8192, F 28672 (3.2) 1.005,
+// T 16384, D 4096, F 16384 (3.7) 1.017, T 8192, D 8192, F 28672 (6.4) 1.033, T 16384, D 8192, F 28672 (12.8) 1.022. kLong: the same
+// where rounds are saved: T 16384, D 1536, F 23040 (2.1; 15 instead of 16) 0.985 on one box and 1.004 on another, T 16384, D 2048,
+// F 28672 (3.4; 25 instead of 26) 1.015.
 bool gemm_dual_tn_pays(int64_t M1, int64_t N1, int64_t M2, int64_t N2, int64_t K) {
-  constexpr double kLaunch = 10000.0, kShort = 1.6e6;
+  constexpr double kLaunch = 10000.0, kShort = 1.6e6, kLong = 2.4e6;
   if (M1 < 256 || M2 < 256) return false;
   const double apart = weight_grad_width(M1, N1, 0, 0, K).clocks + weight_grad_width(M2, N2, 0, 0, K).clocks;
   const double together = weight_grad_width(M1, N1, M2, N2, K).clocks;
-  return together <= 0.97 * apart || (apart <= kShort && together < apart + kLaunch);
+  return apart <= kShort ? together < apart + kLaunch : apart <= kLong && together <= 0.97 * apart;
 }
 
 TileShape gemm_dual_tn_tile(int64_t M1, int64_t N1, int64_t M2, int64_t N2, int64_t K) {
