@@ -2098,6 +2098,20 @@ int make_tmap_2d(void* map, const void* base, int64_t rows, int64_t cols, int64_
                    swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
+int make_tmap_pairs(void* map, const void* base, int64_t rows, int64_t cols, uint32_t box_cols, uint32_t box_pairs) {
+  EncodeTiledFn fn = get_encode_fn();
+  if (!fn) return cuda_fail(cudaErrorUnknown);
+  cuuint64_t dims[3] = {(cuuint64_t)cols, 2, (cuuint64_t)rows / 2};
+  cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * 4};
+  cuuint32_t box[3] = {box_cols, 1, box_pairs}, estr[3] = {1, 1, 1};
+  const CUresult r = fn(reinterpret_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides,
+                        box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r == CUDA_SUCCESS) return SF_OK;
+  g_last_cuda_error = (int)r;
+  return SF_ERR_CUDA;
+}
+
 int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64_t M, int64_t N, int64_t K, int epi,
                void* C, int64_t ldc, void* C2, int64_t ldc2, const void* aux, int64_t ldaux, int* status,
                cudaStream_t s) {

@@ -187,4 +187,8 @@ int gemm_venom(const void* a_vals, const uint8_t* meta_hw, const uint8_t* colidx
 int make_tmap_2d(void* map, const void* base, int64_t rows, int64_t cols, int64_t ld, uint32_t box_cols,
                  uint32_t box_rows, bool swizzle128);
 
+// The same matrix (contiguous rows, an even number of them) by pairs of rows, [rows / 2][2][cols]: box {box_cols, 1, box_pairs}, every
+// second row, 128-byte swizzled.
+int make_tmap_pairs(void* map, const void* base, int64_t rows, int64_t cols, uint32_t box_cols, uint32_t box_pairs);
+
 }  // namespace sf

@@ -101,9 +101,11 @@ prune24_rows_kernel(const uint4* __restrict__ W, int64_t rows, int cols, int64_t
 // (4.9 TB/s at 8192 x 28672). Called back to back on one matrix the last of these takes 4096 x 16384 soft from 45.9 to 44.7.
 // The packed bf16 values of a panel then leave through TMA instead of being read back and stored by the threads: 4096 x 16384
 // soft 44.4 -> 42.1 us, other sizes 116.4 -> 108.9, 13.5 -> 13.1, 12.9 -> 12.4 (calls back to back). The stage holds even columns, then odd
-// ones, so that the threads' swizzled 16-byte writes (two columns each) meet no bank twice; each half has a tensor map and a store of
-// its own (one three-dimensional map for both, with strides that do not ascend, took the same time: 40.8 us and 40.8, 8192 x 16384
-// 80.8 and 80.8). A second stage leaves room for four CTAs an SM instead of five: 42.4, 13.0, 11.8. E4M3 codes keep the threads' stores:
+// ones, so that the threads' swizzled 16-byte writes (two columns each) meet no bank twice; each half has a store of its own, both on
+// one map of column pairs [pair][parity][K] (two plain maps cost a host-bound call 0.1 us of 5.1). The map is not prefetched: with that, or
+// with two maps, the hard variant takes 48 registers instead of 40, five CTAs leave no room for the next launch's beside them, and the
+// routed step at T 2560, D 4352, F 4096 in eight experts takes 211 us instead of 207; held to 40 by launch bounds 4352 x 4096 takes 10.2
+// instead of 9.7. A second stage leaves room for four CTAs an SM instead of five: 42.4, 13.0, 11.8. E4M3 codes keep the threads' stores:
 // their rows need not be multiples of 16 bytes.
 constexpr int kPanelK = 128, kPanelC = 64;
 constexpr int kColsSlots = 2;                       // the next panel loads while this one is worked on
@@ -122,8 +124,7 @@ __device__ __forceinline__ int stage_row(int c) { return (c >> 1) + (c & 1) * (k
 // kFp8: the kept values leave as E4M3 codes of float(value) * scale (vals = uint8 [Rc, Kd/2]); no masked copy.
 template <bool kSoft, bool kFp8 = false>
 __global__ void __launch_bounds__(256)
-prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, const __grid_constant__ CUtensorMap tmapEven,
-                    const __grid_constant__ CUtensorMap tmapOdd, int64_t Kd, int64_t Rc,
+prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, const __grid_constant__ CUtensorMap tmapV, int64_t Kd, int64_t Rc,
                     uint8_t* __restrict__ vals, uint16_t* __restrict__ meta, uint8_t* __restrict__ meta_hw,
                     uint16_t* __restrict__ dense_out, int panels_x, int num_panels, float scale) {
   using namespace ptx;
@@ -151,7 +152,6 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, const __grid_cons
   top2_lut_init(lut, tid);
   if (tid == 0) {
     prefetch_tmap(&tmapW);
-    if (!kFp8) { prefetch_tmap(&tmapEven); prefetch_tmap(&tmapOdd); }
     for (int sl = 0; sl < kColsSlots; ++sl) mbar_init(&full[sl], 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -231,7 +231,7 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, const __grid_cons
     if (!kFp8) fence_proxy_async_smem();
     __syncthreads();
 
-    // store packed values: bf16 through TMA (the maps end where the matrix does); E4M3 per column kvalid/2 bytes, 8 B per thread
+    // store packed values: bf16 through TMA (the map ends where the matrix does); E4M3 per column kvalid/2 bytes, 8 B per thread
     const int chunks = kvalid >> 4;
     const bool full_k = chunks == kPanelK / 16;
     auto put = [&](int c, int ch) {
@@ -240,8 +240,8 @@ prune24_cols_kernel(const __grid_constant__ CUtensorMap tmapW, const __grid_cons
     };
     if (!kFp8) {
       if (tid == 0) {
-        tma_store_2d(&tmapEven, vstage, (int)(k0 >> 1), (int)(c0 >> 1));
-        tma_store_2d(&tmapOdd, vstage + kColsStageBytes / 2, (int)(k0 >> 1), (int)(c0 >> 1));
+        tma_store_3d(&tmapV, vstage, (int)(k0 >> 1), 0, (int)(c0 >> 1));
+        tma_store_3d(&tmapV, vstage + kColsStageBytes / 2, (int)(k0 >> 1), 1, (int)(c0 >> 1));
         bulk_commit();
       }
     } else if (full_k) {
@@ -399,17 +399,14 @@ int launch_prune24(const void* W, int64_t rows, int64_t cols, int64_t ld, int gr
       SF_CUDA_TRY(cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev));
       attr_done[dev] = true;
     }
-    alignas(64) CUtensorMap tm, te, to;
+    alignas(64) CUtensorMap tm, tv;
     int st = make_tmap_2d(&tm, W, rows, cols, ld, kPanelC, kPanelK, false);
-    // values of the even and of the odd columns, [cols / 2, rows / 2] each: a map's strides have to ascend, so one map cannot
-    // have the columns' parity as its last dimension
-    if (st == SF_OK) st = make_tmap_2d(&te, vals, cols / 2, rows / 2, rows, kPanelK / 2, kPanelC / 2, true);
-    if (st == SF_OK) st = make_tmap_2d(&to, (const uint16_t*)vals + rows / 2, cols / 2, rows / 2, rows, kPanelK / 2, kPanelC / 2, true);
+    if (st == SF_OK) st = make_tmap_pairs(&tv, vals, cols, rows / 2, kPanelK / 2, kPanelC / 2);
     if (st != SF_OK) return st;
     const int resident = sms[dev] * kColsCtasPerSm;
     const unsigned grid = (unsigned)(num_panels < resident ? num_panels : resident);
     return launch_pdl(prune_mode == 0 ? prune24_cols_kernel<false> : prune24_cols_kernel<true>, dim3(grid), 256,
-                      kColsSmemBytes, s, tm, te, to, rows, cols, (uint8_t*)vals, (uint16_t*)meta, (uint8_t*)meta_hw,
+                      kColsSmemBytes, s, tm, tv, rows, cols, (uint8_t*)vals, (uint16_t*)meta, (uint8_t*)meta_hw,
                       (uint16_t*)dense_out, (int)px, num_panels, 1.f);
   }
 }
@@ -437,7 +434,7 @@ int launch_prune24_cols_fp8(const void* W, int64_t rows, int64_t cols, int64_t l
   const int resident = sms[dev] * kColsCtasPerSm;
   const unsigned grid = (unsigned)(num_panels < resident ? num_panels : resident);
   return launch_pdl(prune_mode == 0 ? prune24_cols_kernel<false, true> : prune24_cols_kernel<true, true>, dim3(grid), 256,
-                    kColsSmemBytes, s, tm, tm, tm, rows, cols, (uint8_t*)vals, (uint16_t*)meta, (uint8_t*)nullptr,
+                    kColsSmemBytes, s, tm, tm, rows, cols, (uint8_t*)vals, (uint16_t*)meta, (uint8_t*)nullptr,
                     (uint16_t*)nullptr, (int)px, num_panels, scale);
 }
 
