@@ -122,38 +122,14 @@ def _integer_24_product(Mr, Nc, K, b_k, run):
     return bits(C), synth.f32_to_bf16_bits(oracle.bf16_to_f32(p.dense) @ B.T)
 
 
-def _tiles_24(Mr, Nc, K, transposed=False):
-    """(rows, columns) of the tiles of a 2:4 product: y3 of a step is the row-major one, y1 the transposed one."""
-    if transposed:
-        plan = binding.sf_ffn_step_plan(binding.make_desc(Nc, K, Mr, 64, 8, flags=binding.SF_FFN_UNFUSED_ACT))
-        return plan.y1_rows, plan.y1_cols
-    plan = binding.sf_ffn_step_plan(binding.make_desc(Mr, Nc, K, 64, 8))
-    return plan.y3_rows, plan.y3_cols
-
-
-# The stores, those of full-width tiles through TMA: both kernels, half-empty last tiles, several tiles to a CTA pair, the shortest reduction.
-# Exact on small integers, nothing written outside the result. The dense products (E4M3 ones too) have seven rounds of tiles and more,
-# of at least four k-stages: a narrower tile costs more per column and saves at most a seventh of the last round, so that no
-# estimate takes one.
-@pytest.mark.parametrize("kind,Mr,Nc,K,rows", [("dense", 2688, 14848, 256, 256),      # half-empty last row of tiles
-                                               ("dense", 14976, 2304, 320, 256),
-                                               ("fp8_dense", 2560, 14848, 512, 256),
-                                               ("sparse24", 8448, 8192, 512, 256),    # overlapping accumulators, fourteen tiles to a pair
-                                               ("sparse24", 256, 18944, 256, 256),    # one tile to a pair
-                                               ("sparse24", 256, 18944, 128, None),   # the shortest reduction (the plan starts at 256)
-                                               ("sparse24", 6400, 4352, 128, None),
-                                               ("sparse24", 6400, 4352, 256, 512),    # last row half empty, narrow last column of 96
-                                               ("sparse24", 9728, 512, 256, 512),
-                                               ("sparse24", 3328, 4864, 256, 512),    # more narrow tiles than two per idle pair: round robin
-                                               ("fp8", 4096, 4608, 512, 512), ("fp8", 6400, 4352, 256, None),
-                                               ("fp8", 8448, 8192, 1024, 256), ("fp8", 256, 18944, 512, 256),
-                                               # fewer tiles or stages: narrower ones, stored from registers
-                                               ("dense", 2688, 4864, 64, None), ("dense", 5248, 2304, 320, None),
-                                               ("fp8_dense", 2560, 4864, 128, None), ("sparse24", 512, 1792, 384, None),
-                                               ("fp8", 4096, 4608, 256, None)])
-def test_stores_stay_inside_the_result(kind, Mr, Nc, K, rows):
-    if kind in ("sparse24", "fp8") and rows:      # E4M3: the rule and the width of a bf16 product with half the reduction
-        assert _tiles_24(Mr, Nc, K if kind == "sparse24" else K // 2) == (rows, 224 if rows == 512 else 256)
+# The stores of row-major products: half-empty last tiles, several tiles to a CTA pair, the shortest reduction. Exact on small integers,
+# nothing written outside the result. Some of these sizes take narrow tiles, which store from registers (dense with
+# K = 64, E4M3 dense, 2:4 512 x 1792); test_stores_on_the_tiles_named has the full-width ones by name.
+@pytest.mark.parametrize("kind,Mr,Nc,K", [("dense", 2688, 4864, 64), ("dense", 5248, 2304, 320),
+                                          ("sparse24", 256, 18944, 128), ("sparse24", 9728, 512, 256),
+                                          ("sparse24", 6400, 4352, 128), ("sparse24", 512, 1792, 384),
+                                          ("fp8", 4096, 4608, 256), ("fp8", 256, 18944, 512), ("fp8_dense", 2560, 4864, 128)])
+def test_full_width_stores_stay_inside_the_result(kind, Mr, Nc, K):
     g = torch.Generator(device="cuda")
     g.manual_seed(Mr + K)
     ints = lambda *s: torch.randint(-3, 4, s, generator=g, device="cuda")
@@ -178,6 +154,34 @@ def test_stores_stay_inside_the_result(kind, Mr, Nc, K, rows):
     assert torch.equal(out.t, bf(A.double() @ B.double().T))
 
 
+def _tiles_24(Mr, Nc, K, transposed=False):
+    """(rows, columns) of the tiles of a 2:4 product: y3 of a step is the row-major one, y1 the transposed one."""
+    if transposed:
+        plan = binding.sf_ffn_step_plan(binding.make_desc(Nc, K, Mr, 64, 8, flags=binding.SF_FFN_UNFUSED_ACT))
+        return plan.y1_rows, plan.y1_cols
+    plan = binding.sf_ffn_step_plan(binding.make_desc(Mr, Nc, K, 64, 8))
+    return plan.y3_rows, plan.y3_cols
+
+
+# The same on stated tiles. The dense products (E4M3 ones too) have seven rounds of tiles and more, of at least four k-stages: a narrower
+# tile costs more per column and saves at most a seventh of the last round, so that no estimate takes one.
+@pytest.mark.parametrize("kind,Mr,Nc,K,rows", [("dense", 2688, 14848, 256, 256),      # half-empty last row of tiles
+                                               ("dense", 14976, 2304, 320, 256),
+                                               ("fp8_dense", 2560, 14848, 512, 256),
+                                               ("sparse24", 8448, 8192, 512, 256),    # overlapping accumulators, fourteen tiles to a pair
+                                               ("sparse24", 256, 18944, 256, 256),    # one tile to a pair
+                                               ("sparse24", 6400, 4352, 256, 512),    # last row half empty, narrow last column of 96
+                                               ("sparse24", 9728, 512, 256, 512),
+                                               ("sparse24", 3328, 4864, 256, 512),    # more narrow tiles than two per idle pair: round robin
+                                               ("fp8", 4096, 4608, 512, 512), ("fp8", 8448, 8192, 1024, 256),
+                                               ("fp8", 256, 18944, 512, 256),
+                                               ("fp8", 6400, 4352, 256, None)])       # one k-stage (the plan starts at 256 in bf16)
+def test_stores_on_the_tiles_named(kind, Mr, Nc, K, rows):
+    if kind in ("sparse24", "fp8") and rows:      # E4M3: the rule and the width of a bf16 product with half the reduction
+        assert _tiles_24(Mr, Nc, K if kind == "sparse24" else K // 2) == (rows, 224 if rows == 512 else 256)
+    test_full_width_stores_stay_inside_the_result(kind, Mr, Nc, K)
+
+
 @pytest.mark.parametrize("b_k", [True, False])
 @pytest.mark.parametrize("Mr,Nc,K", [(8192, 8192, 512),    # 512-row tiles, a narrow last column of 128
                                      (8448, 4352, 512),    # the same, last tile row half empty, narrow column of 96
@@ -198,14 +202,19 @@ def test_sparse24_gemm_short_reductions_about_the_l2(b_k, Mr, Nc, K, rows):
     assert np.array_equal(got, ref)
 
 
-@pytest.mark.parametrize("Mr,Nc,K,tile", [(37632, 256, 128, None), (256, 7680, 128, None),    # one k-stage (the plan starts at 256)
-                                          (8576, 4864, 512, (256, 224)),     # half-empty last row, narrow last column of 160
+@pytest.mark.parametrize("Mr,Nc,K", [(37632, 256, 128), (256, 7680, 128), (8576, 4864, 512)])    # 256-row tiles
+def test_sparse24_gemm_tile_shapes_transposed_output(Mr, Nc, K):
+    got, ref = _integer_24_product(Mr, Nc, K, True, binding.sf_gemm_sparse24)
+    assert np.array_equal(got, np.ascontiguousarray(ref.T))
+
+
+@pytest.mark.parametrize("Mr,Nc,K,tile", [(8576, 4864, 512, (256, 224)),     # half-empty last row, narrow last column of 160
                                           (256, 7680, 256, (256, 64)),       # one row of tiles
                                           (2688, 2304, 2048, (512, 224)),    # 512-row tiles: 128 rows in the last, column of 64
                                           (2944, 2560, 2048, (512, 224)),    # 384 rows in the last: its second half is half empty; 96
                                           (19072, 512, 2048, (512, 224))])   # two tiles to some pairs
-def test_sparse24_gemm_tile_shapes_transposed_output(Mr, Nc, K, tile):
-    assert tile is None or _tiles_24(Mr, Nc, K, transposed=True) == tile
+def test_transposed_stores_on_the_tiles_named(Mr, Nc, K, tile):
+    assert _tiles_24(Mr, Nc, K, transposed=True) == tile
     out = Guarded((Nc, Mr), torch.bfloat16)
     got, ref = _integer_24_product(Mr, Nc, K, True, lambda v, m, b: binding.sf_gemm_sparse24(v, m, b, Ct_out=out.t))
     out.check("transposed product")
