@@ -104,7 +104,7 @@ int gemm_dense(const void* A, bool a_kmajor, const void* B, bool b_kmajor, int64
                cudaStream_t s);
 // Two products C1[M1,N1] = A1[K,M1]^T B1[K,N1] and C2[M2,N2] = A2[K,M2]^T B2[K,N2] in one launch. _pays: whether that ends sooner
 // by the estimate: it saves rounds of tiles (a launch of its own leaves its last round part empty; D 2048, F 8192: 4 + 4 rounds against 7),
-// or there are so few that the launch counts. M >= 256, all sizes multiples of 128.
+// or there are so few that the launch counts; long ones stay apart. M >= 256, all sizes multiples of 128.
 bool gemm_dual_tn_pays(int64_t M1, int64_t N1, int64_t M2, int64_t N2, int64_t K);
 int gemm_dual_tn(const void* A1, const void* B1, int64_t M1, int64_t N1, void* C1, const void* A2, const void* B2, int64_t M2,
                  int64_t N2, void* C2, int64_t K, int* status, cudaStream_t s);
